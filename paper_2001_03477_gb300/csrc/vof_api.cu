@@ -135,7 +135,7 @@ static vof_status sweep_common(int axis, const vof_grid* g, const double* c_in, 
   // stand-alone sweep: diag[0] += clipped volume
   static const signed char kMap[kNSums] = {-1, -1, 0, -1, -1, -1};
   SweepScratch sc = carve_sweep_scratch(axis, d, workspace, sums_to_diag(diag, kMap));
-  return cuda_status(launch_sweep(axis, d, c_in, e_in, c_out, e_in ? e_out : nullptr, uf, state, theta, flux_out, sc, true,
+  return cuda_status(launch_sweep(axis, d, c_in, e_in, c_out, e_in ? e_out : nullptr, uf, state, theta, flux_out, sc,
                                   (cudaStream_t)stream));
 }
 
@@ -202,49 +202,53 @@ vof_status vof_phase_change_shift(const vof_grid* g, const double* c_in, const d
   static const signed char kMap[kNSums] = {3, 4, -1, 0, 1, 2};
   const SumOut so = sums_to_diag(diag, kMap);
   return cuda_status(launch_shift(d, c_in, e_in, c_out, e_out, dd, dd_uniform, state, carve_shift_scratch(d, workspace),
-                                  so, so, true, (cudaStream_t)stream));
+                                  so, so, (cudaStream_t)stream));
 }
 
-// workspace layout: theta | state | sum rows (tile pass, the three sweeps'
-// update kernels, the shift's sums kernel; kNSums doubles per CTA) |
-// reduction scratch | work counts (12 ints) and, 128 bytes in, the passes'
-// list counters (kStepCounters ints, cleared by the tile pass) | tiles |
-// scratch (reused by the three sweeps, then the shift).  The sweeps and the
-// shift all run in place on c and e; the tile pass sums c and e at the start
-// and every later kernel adds the changes it makes, so one fixed-order
-// reduction of all rows gives the sums at the end of the step.
+// workspace layout: theta | sum rows (kNSums doubles per tile) |
+// reduction scratch | work counts (12 ints) and, 128 bytes in, the step's
+// counters (kStepCounters ints, cleared by the tile pass) | tiles | scratch
+// fields c, e | the mixed cells' fluxes | ghost fluxes | planes | lists |
+// active tiles | clipped volumes.  The step's last kernel sums every
+// active tile's cells, the tile pass the quiet ones', so one fixed-order
+// reduction of the rows gives the sums.  The size is at least that of the
+// stand-alone sweeps' and shift's scratch and a byte per cell behind the first five regions.
 struct StepLayout {
-  size_t off_th, off_st, off_rows, off_red, off_stats, off_tiles, off_sw, total;
-  int nb_tiles, nb_sw[3], nb_sh, nrows;
+  size_t off_th, off_rows, off_red, off_stats, off_tiles, off_sc, off_se, off_fl, off_fr, off_gf, off_plane,
+      off_l0, off_l1, off_tlist, off_clip, total;
+  int ntiles;
 };
 
 static StepLayout step_layout(const vof_grid* g) {
   StepLayout L;
   GridDev d = to_dev(g, 0.0);
-  size_t N = cells(g);
-  L.off_th = 0;
-  L.off_st = L.off_th + align256(N * 8);
-  L.off_rows = L.off_st + align256(N);
-  L.nb_tiles = tile_blocks(d);
-  L.nrows = L.nb_tiles;
-  for (int a = 0; a < 3; ++a) {
-    L.nb_sw[a] = sweep_blocks(a, d);
-    L.nrows += L.nb_sw[a];
-  }
-  L.nb_sh = shift_sum_blocks(d);
-  L.nrows += L.nb_sh;
-  L.off_red = L.off_rows + align256((size_t)L.nrows * kNSums * 8);
-  L.off_stats = L.off_red + align256(reduce_scratch_bytes());
-  L.off_tiles = L.off_stats + 256;
-  L.off_sw = L.off_tiles + align256(tile_scratch_bytes(d));
+  const size_t N = cells(g);
+  size_t lines = 0;
+  for (int a = 0; a < 3; ++a) lines = N / (size_t)d.n[a] > lines ? N / (size_t)d.n[a] : lines;
+  L.ntiles = tile_total(d);
+  const size_t T = (size_t)L.ntiles;
+  size_t o = 0;
+  auto take = [&](size_t b) { const size_t at = o; o += align256(b); return at; };
+  L.off_th = take(N * 8);
+  L.off_rows = take(T * kNSums * 8);
+  L.off_red = take(reduce_scratch_bytes());
+  L.off_stats = take(256);
+  L.off_tiles = take(tile_scratch_bytes(d));
+  const size_t base = o;
+  L.off_sc = take(N * 8);
+  L.off_se = take(N * 8);
+  L.off_fl = take(N * 8);
+  L.off_fr = take(N * 8);
+  L.off_gf = take(2 * lines * 8);
+  L.off_plane = take(N * 32);
+  L.off_l0 = take(N * 4);
+  L.off_l1 = take(N * 4);
+  L.off_tlist = take(T * 4);
+  L.off_clip = take(12 * T * 8);
   const size_t sw = sweep_scratch_bytes(d), sh = shift_scratch_bytes(d);
-  L.total = L.off_sw + align256(sw > sh ? sw : sh);
+  const size_t other = base + align256(N) + align256(sw > sh ? sw : sh);
+  L.total = o > other ? o : other;
   return L;
-}
-
-// the passes' list counters: 128 bytes into the work-count block
-static int* step_counters(char* ws, const StepLayout& L) {
-  return reinterpret_cast<int*>(ws + L.off_stats + 128);
 }
 
 size_t vof_step_workspace_bytes(const vof_grid* g) {
@@ -256,92 +260,43 @@ size_t vof_step_workspace_bytes(const vof_grid* g) {
 
 namespace vofgb {
 
-// One box's arguments for the grouped step: the same carving, sum rows and
-// launch shapes as vof_step below (keep the two in step).
 bool step_box(const vof_grid* g, double* c, double* e, const double* u, const double* v, const double* w,
               double dt, const double* dd, double dd_uniform, double* sums, char* ws, StepBox* out) {
   if (!grid_ok(g) || !c || !e || !u || !v || !w || !(dt >= 0.0) || !ws) return false;
-  if (g->normal == VOF_NORMAL_MLP) return false;  // the learned normal runs per grid (vof_step)
   const StepLayout L = step_layout(g);
   const GridDev d = to_dev(g, dt);
-  const size_t N = cells(g);
   StepBox& B = *out;
-  B.cells = N;
-  double* th = reinterpret_cast<double*>(ws + L.off_th);
-  uint8_t* state = reinterpret_cast<uint8_t*>(ws + L.off_st);
-  double* rows = reinterpret_cast<double*>(ws + L.off_rows);
-  int* cnt = step_counters(ws, L);
-  // tile pass
-  const TileScratch ts = carve_tile_scratch(d, ws + L.off_tiles);
-  int nt[3];
-  tile_counts(d, nt);
-  B.tiles.g = d;
-  B.tiles.c = c;
-  B.tiles.e = e;
-  B.tiles.ts = ts;
-  B.tiles.nt[0] = nt[0]; B.tiles.nt[1] = nt[1]; B.tiles.nt[2] = nt[2];
-  B.tiles.sums = sums_to_partials(rows, kNSums);
-  B.tiles.state = state;
-  B.tiles.counters = cnt;
-  B.grid_tiles = dim3((unsigned)((nt[0] + 3) / 4), (unsigned)nt[1], (unsigned)nt[2]);
-  B.grid_quiet = quiet_blocks(d);
-  size_t r = (size_t)L.nb_tiles;
-  TileMap tm{nullptr, {0, 0, 0}};
-  if (tiles_usable(d)) {
-    tm.quiet = ts.quiet;
-    tile_counts(d, tm.nt);
-  }
-  const double* uf[3] = {u, v, w};
-  // sum rows in the order of the axes of an even step (x, y, z): the rows of
-  // a sweep belong to its axis, as in vof_step
-  size_t row_of_axis[3];  // fixed per axis, as in vof_step
-  {
-    size_t rr = r;
-    for (int a = 0; a < 3; ++a) {
-      row_of_axis[a] = rr;
-      rr += (size_t)L.nb_sw[a];
-    }
-  }
-  for (int a = 0; a < 3; ++a) {
-    SweepScratch sc = carve_sweep_scratch(a, d, ws + L.off_sw, sums_to_partials(rows + row_of_axis[a] * kNSums, kNSums));
-    sc.tiles = tm;
-    sc.stats = reinterpret_cast<int*>(ws + L.off_stats) + 2 * a;
-    sc.mlp_stat = reinterpret_cast<int*>(ws + L.off_stats) + 9 + a;
-    sc.counters = cnt + 4 * a;
-    const SweepPlan p = sweep_plan(a, d);
-    SweepArgs& A = B.sweep[a];
-    A.g = d;
-    A.c = c;
-    A.e = e;
-    A.uf = uf[a];
-    A.state = state;
-    A.theta = th;
-    A.sc = sc;
-    A.cap = p.cap;
-    A.nsub = (int)p.nsub;
-    A.ngrp = p.lpc / kUpdLists;
-    A.status = device_status_ptr();
-    B.grid_stream[a] = p.gridA;
-    B.grid_update[a] = p.gridB;
-    r += (size_t)L.nb_sw[a];
-  }
-  ShiftScratch shs = carve_shift_scratch(d, ws + L.off_sw);
-  shs.tiles = tm;
-  shs.stats = reinterpret_cast<int*>(ws + L.off_stats) + 6;
-  shs.counters = cnt + 12;
-  ShiftArgs& S = B.shift;
-  S.g = d;
-  S.c = c;
-  S.e = e;
-  S.dd = dd;
-  S.dd_uniform = dd_uniform;
-  S.sc = shs;
-  S.sums = sums_to_partials(rows + r * kNSums, kNSums);
-  S.nw = shift_warps_of(d);
-  B.grid_shift_stream = shift_stream_grid_of(d);
-  B.grid_shift_sums = (unsigned)shift_sum_blocks(d);
-  r += (size_t)L.nb_sh;
-  B.red = ReduceBox{rows, (int)r, sums, reinterpret_cast<double*>(ws + L.off_red)};
+  B.cells = cells(g);
+  StepArgs& A = B.args;
+  A.g = d;
+  A.c = c;
+  A.e = e;
+  A.s_c = reinterpret_cast<double*>(ws + L.off_sc);
+  A.s_e = reinterpret_cast<double*>(ws + L.off_se);
+  A.uf[0] = u; A.uf[1] = v; A.uf[2] = w;
+  A.theta = reinterpret_cast<double*>(ws + L.off_th);
+  A.fl = reinterpret_cast<double*>(ws + L.off_fl);
+  A.fr = reinterpret_cast<double*>(ws + L.off_fr);
+  A.gf = reinterpret_cast<double*>(ws + L.off_gf);
+  A.plane = reinterpret_cast<double*>(ws + L.off_plane);
+  A.list[0] = reinterpret_cast<uint32_t*>(ws + L.off_l0);
+  A.list[1] = reinterpret_cast<uint32_t*>(ws + L.off_l1);
+  A.tlist = reinterpret_cast<uint32_t*>(ws + L.off_tlist);
+  A.clip = reinterpret_cast<double*>(ws + L.off_clip);
+  A.rows = reinterpret_cast<double*>(ws + L.off_rows);
+  A.ts = carve_tile_scratch(d, ws + L.off_tiles);
+  tile_counts(d, A.nt);
+  A.usable = tiles_usable(d) ? 1 : 0;
+  A.stats = reinterpret_cast<int*>(ws + L.off_stats);
+  A.cnt = reinterpret_cast<int*>(ws + L.off_stats + 128);
+  A.status = device_status_ptr();
+  A.dd = dd;
+  A.dd_uniform = dd_uniform;
+  A.pairs = reinterpret_cast<uint2*>(A.theta);
+  A.pair_cap = (int)B.cells;
+  A.chain = 0;
+  B.grid_tiles = dim3((unsigned)((A.nt[0] + 3) / 4), (unsigned)A.nt[1], (unsigned)A.nt[2]);
+  B.red = ReduceBox{A.rows, L.ntiles, sums, reinterpret_cast<double*>(ws + L.off_red)};
   return true;
 }
 
@@ -361,59 +316,18 @@ vof_status vof_step(const vof_grid* g, double* c, double* e, const double* u, co
   if (overlap(c, B, e, B) || overlap(c, B, workspace, L.total) || overlap(e, B, workspace, L.total))
     return VOF_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  char* ws = static_cast<char*>(workspace);
-  double* th = reinterpret_cast<double*>(ws + L.off_th);
-  uint8_t* state = reinterpret_cast<uint8_t*>(ws + L.off_st);
-  double* rows = reinterpret_cast<double*>(ws + L.off_rows);
-  GridDev d = to_dev(g, dt);
-  const double* uf[3] = {u, v, w};
-  int* cnt = step_counters(ws, L);
-  // tile pass: quiet tiles and the sums of c, e at the start of the step;
-  // it also clears the frozen-state flags and the passes' list counters
-  const TileScratch ts = carve_tile_scratch(d, ws + L.off_tiles);
-  size_t r = 0;
-  cudaError_t err = launch_tiles(d, c, e, ts, sums_to_partials(rows, kNSums), state, cnt, st);
-  if (err != cudaSuccess) return cuda_status(err);
-  r += (size_t)L.nb_tiles;
-  TileMap tm{nullptr, {0, 0, 0}};
-  if (tiles_usable(d)) {
-    tm.quiet = ts.quiet;
-    tile_counts(d, tm.nt);
-  }
-  // each axis' sum rows have a fixed place (x, y, z after the tile rows),
-  // whatever the order the sweeps run in
-  size_t row_of_axis[3];
-  for (int a = 0; a < 3; ++a) {
-    row_of_axis[a] = r;
-    r += (size_t)L.nb_sw[a];
-  }
-  for (int s = 0; s < 3; ++s) {
-    const int ax = (step_index % 2 == 0) ? s : 2 - s;
-    SweepScratch sc =
-        carve_sweep_scratch(ax, d, ws + L.off_sw, sums_to_partials(rows + row_of_axis[ax] * kNSums, kNSums));
-    sc.tiles = tm;
-    sc.stats = reinterpret_cast<int*>(ws + L.off_stats) + 2 * ax;
-    sc.mlp_stat = reinterpret_cast<int*>(ws + L.off_stats) + 9 + ax;
-    sc.counters = cnt + 4 * ax;
-    err = launch_sweep(ax, d, c, e, c, e, uf[ax], state, th, nullptr, sc, false, st);
-    if (err != cudaSuccess) return cuda_status(err);
-  }
-  ShiftScratch shs = carve_shift_scratch(d, ws + L.off_sw);
-  shs.tiles = tm;
-  shs.stats = reinterpret_cast<int*>(ws + L.off_stats) + 6;
-  shs.counters = cnt + 12;
-  const SumOut none = sums_to_partials(nullptr, kNSums);
-  err = launch_shift(d, c, e, c, e, dd, dd_uniform, nullptr, shs, none, sums_to_partials(rows + r * kNSums, kNSums),
-                     false, st);
-  if (err != cudaSuccess) return cuda_status(err);
-  r += (size_t)L.nb_sh;
-  if (sums) {
-    // sums[0..1] = sum c, sum e; sums[2] = clip; sums[3..5] = shift diagnostics
-    err = launch_reduce_fused(ReduceJob{rows, (int)r, kNSums, 0, kNSums, sums},
-                              reinterpret_cast<double*>(ws + L.off_red), cnt + (kStepCounters - 1), st);
-    if (err != cudaSuccess) return cuda_status(err);
-  }
-  return VOF_OK;
+  StepBox bx;
+  if (!step_box(g, c, e, u, v, w, dt, dd, dd_uniform, sums, static_cast<char*>(workspace), &bx)) return VOF_EINVAL;
+  const StepArgs& A = bx.args;
+  cudaError_t err = launch_tiles(A, st);
+  const int odd = (int)(step_index % 2);
+  for (int s = 0; s < 3 && err == cudaSuccess; ++s) err = launch_stage(A, odd ? 2 - s : s, s, st);
+  if (err == cudaSuccess) err = launch_shift_step(A, odd, st);
+  // sums[0..1] = sum c, sum e; sums[2] = clip; sums[3..5] = shift diagnostics
+  if (err == cudaSuccess && sums)
+    err = launch_reduce_fused(ReduceJob{bx.red.rows, bx.red.nblocks, kNSums, 0, kNSums, sums}, bx.red.scratch,
+                              A.cnt + (kStepCounters - 1), st);
+  return cuda_status(err);
 }
 
 vof_status vof_step_work_counts(const vof_grid* g, const void* workspace, int* counts, void* stream) {

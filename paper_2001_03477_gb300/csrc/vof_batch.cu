@@ -190,7 +190,7 @@ vof_status vof_batched_step(const vof_box* boxes, int nbox, long step_index, dou
 // vof_group_create() carves each box's own step workspace out of the
 // caller's buffer, builds every kernel's per-box arguments (exactly as
 // vof_step would) and the CTA -> box maps of every grouped launch, and copies
-// them into the same buffer once; vof_group_step() then issues ~22 launches
+// them into the same buffer once; vof_group_step() then issues 13 launches
 // whatever the number of boxes (no host work per box, capturable).
 // ---------------------------------------------------------------------------
 namespace {
@@ -224,11 +224,9 @@ struct LaunchPlan {
 struct vof_group {
   int nbox = 0;
   int f32 = 0, youngs = 0;
-  const TileArgs* tiles = nullptr;
-  const SweepArgs* sweep[3] = {nullptr, nullptr, nullptr};
-  const ShiftArgs* shift = nullptr;
+  const StepArgs* args = nullptr;
   const ReduceBox* red = nullptr;
-  Launch l_tiles, l_quiet, l_stream[3], l_prep[3], l_faces[3], l_update[3], l_sh[5], l_red1;
+  Launch l_tiles, l_quiet, l_mix, l_walk, l_planes, l_sweep, l_apply, l_red1;
   bool sums = false;
 };
 
@@ -267,7 +265,7 @@ static vof_status group_plan(const vof_box* boxes, int nbox, double* sums, int w
   const size_t tables = off;
   std::vector<StepBox> sb(nbox);
   // launch plans
-  LaunchPlan p_tiles, p_quiet, p_stream[3], p_prep[3], p_faces[3], p_update[3], p_sh[5], p_red1;
+  LaunchPlan p_tiles, p_quiet, p_mix, p_walk, p_planes, p_sweep, p_apply, p_red1;
   size_t base = 0;
   for (int b = 0; b < nbox; ++b) {
     const vof_box& x = boxes[b];
@@ -279,29 +277,19 @@ static vof_status group_plan(const vof_box* boxes, int nbox, double* sums, int w
     base += align256(ws[b]);
     const StepBox& B = sb[b];
     p_tiles.add(B.grid_tiles.x, B.grid_tiles.y, B.grid_tiles.z);
-    p_quiet.add(B.grid_quiet, 1, 1);
-    for (int a = 0; a < 3; ++a) {
-      p_stream[a].add(B.grid_stream[a].x, B.grid_stream[a].y, B.grid_stream[a].z);
-      p_prep[a].add(gs_ctas(B.cells, work, prep_ctas()), 1, 1);
-      p_faces[a].add(gs_ctas(B.cells, work, prep_ctas()), 1, 1);
-      p_update[a].add(B.grid_update[a], 1, 1);
-    }
-    p_sh[0].add(B.grid_shift_stream.x, B.grid_shift_stream.y, 1);
-    for (int k = 1; k < 4; ++k) p_sh[k].add(gs_ctas(B.cells, work, shift_list_ctas()), 1, 1);
-    p_sh[4].add(B.grid_shift_sums, 1, 1);
+    p_quiet.add(quiet_ctas(B.args.g), 1, 1);
+    p_mix.add(gs_ctas(B.cells, work, mix_ctas(B.args.g)), 1, 1);
+    p_walk.add(walk_ctas(B.args.g), 1, 1);
+    p_planes.add(gs_ctas(B.cells, work, shift_plane_ctas()), 1, 1);
+    p_sweep.add(gs_ctas(B.cells, work, shift_plane_ctas()), 1, 1);
+    p_apply.add(apply_ctas(B.args.g), 1, 1);
     p_red1.add(kReduceCTAs, 1, 1);
   }
   // table region after the boxes' workspaces
-  LaunchPlan* plans[] = {&p_tiles,     &p_quiet,     &p_stream[0], &p_stream[1], &p_stream[2], &p_prep[0],
-                         &p_prep[1],   &p_prep[2],   &p_faces[0],  &p_faces[1],  &p_faces[2],  &p_update[0],
-                         &p_update[1], &p_update[2], &p_sh[0],     &p_sh[1],     &p_sh[2],     &p_sh[3],
-                         &p_sh[4],     &p_red1};
+  LaunchPlan* plans[] = {&p_tiles, &p_quiet, &p_mix, &p_walk, &p_planes, &p_sweep, &p_apply, &p_red1};
   const size_t nb = (size_t)nbox;
   size_t t = tables;
-  const size_t o_tiles = t;  t += align256(nb * sizeof(TileArgs));
-  size_t o_sweep[3];
-  for (int a = 0; a < 3; ++a) { o_sweep[a] = t; t += align256(nb * sizeof(SweepArgs)); }
-  const size_t o_shift = t;  t += align256(nb * sizeof(ShiftArgs));
+  const size_t o_args = t;   t += align256(nb * sizeof(StepArgs));
   const size_t o_red = t;    t += align256(nb * sizeof(ReduceBox));
   const size_t o_maps = t;
   for (LaunchPlan* lp : plans) t += lp->bytes();
@@ -313,26 +301,24 @@ static vof_status group_plan(const vof_box* boxes, int nbox, double* sums, int w
   std::vector<unsigned char> img(t - tables, 0);
   auto put = [&](size_t o, const void* src, size_t n) { std::memcpy(img.data() + (o - tables), src, n); };
   {
-    std::vector<TileArgs> ta(nb);
-    std::vector<SweepArgs> sa(nb);
-    std::vector<ShiftArgs> sh(nb);
+    std::vector<StepArgs> sa(nb);
     std::vector<ReduceBox> rb(nb);
-    for (size_t b = 0; b < nb; ++b) ta[b] = sb[b].tiles;
-    put(o_tiles, ta.data(), nb * sizeof(TileArgs));
-    for (int a = 0; a < 3; ++a) {
-      for (size_t b = 0; b < nb; ++b) sa[b] = sb[b].sweep[a];
-      put(o_sweep[a], sa.data(), nb * sizeof(SweepArgs));
+    // the boxes' walks share the machine: chains short enough for a dozen
+    // items a resident warp over the whole batch, at most 4 tiles (48 ... 96
+    // cells an edge hold 6 ... 12)
+    size_t tiles = 0;
+    for (size_t b = 0; b < nb; ++b) tiles += (size_t)tile_total(sb[b].args.g);
+    const size_t items = 2 * tiles / (12ull * 152 * 16);
+    for (size_t b = 0; b < nb; ++b) {
+      sa[b] = sb[b].args;
+      sa[b].chain = items < 1 ? 1 : (items > 4 ? 4 : (int)items);
     }
-    for (size_t b = 0; b < nb; ++b) sh[b] = sb[b].shift;
-    put(o_shift, sh.data(), nb * sizeof(ShiftArgs));
+    put(o_args, sa.data(), nb * sizeof(StepArgs));
     for (size_t b = 0; b < nb; ++b) rb[b] = sb[b].red;
     put(o_red, rb.data(), nb * sizeof(ReduceBox));
   }
-  Launch* launches[] = {&out->l_tiles,     &out->l_quiet,     &out->l_stream[0], &out->l_stream[1],
-                        &out->l_stream[2], &out->l_prep[0],   &out->l_prep[1],   &out->l_prep[2],
-                        &out->l_faces[0],  &out->l_faces[1],  &out->l_faces[2],  &out->l_update[0],
-                        &out->l_update[1], &out->l_update[2], &out->l_sh[0],     &out->l_sh[1],
-                        &out->l_sh[2],     &out->l_sh[3],     &out->l_sh[4],     &out->l_red1};
+  Launch* launches[] = {&out->l_tiles,  &out->l_quiet, &out->l_mix,   &out->l_walk,
+                        &out->l_planes, &out->l_sweep, &out->l_apply, &out->l_red1};
   size_t o = o_maps;
   for (size_t i = 0; i < sizeof(plans) / sizeof(plans[0]); ++i) {
     const LaunchPlan& lp = *plans[i];
@@ -362,9 +348,7 @@ static vof_status group_plan(const vof_box* boxes, int nbox, double* sums, int w
   out->nbox = nbox;
   out->f32 = prec == VOF_F32_FLUX ? 1 : 0;
   out->youngs = nrm == VOF_NORMAL_YOUNGS ? 1 : 0;
-  out->tiles = reinterpret_cast<const TileArgs*>(dev + o_tiles);
-  for (int a = 0; a < 3; ++a) out->sweep[a] = reinterpret_cast<const SweepArgs*>(dev + o_sweep[a]);
-  out->shift = reinterpret_cast<const ShiftArgs*>(dev + o_shift);
+  out->args = reinterpret_cast<const StepArgs*>(dev + o_args);
   out->red = reinterpret_cast<const ReduceBox*>(dev + o_red);
   out->sums = sums != nullptr;
   return VOF_OK;
@@ -410,25 +394,15 @@ vof_status vof_group_create(const vof_box* boxes, int nbox, double* sums, int wo
 vof_status vof_group_step(vof_group* grp, long step_index, void* stream) {
   if (!grp || grp->nbox < 1 || step_index < 0) return VOF_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  // the tile pass also clears every box's frozen-state flags and counters
+  // the tile pass also clears every box's counters
   cudaError_t err =
-      launch_tiles_grp(grp->l_tiles.m, grp->l_quiet.m, grp->tiles, grp->l_tiles.ctas, grp->l_quiet.ctas, st);
-  for (int s = 0; s < 3 && err == cudaSuccess; ++s) {
-    const int ax = (step_index % 2 == 0) ? s : 2 - s;
-    const GroupMap maps[4] = {grp->l_stream[ax].m, grp->l_prep[ax].m, grp->l_faces[ax].m, grp->l_update[ax].m};
-    const unsigned ctas[4] = {grp->l_stream[ax].ctas, grp->l_prep[ax].ctas, grp->l_faces[ax].ctas,
-                              grp->l_update[ax].ctas};
-    err = launch_sweep_grp(ax, grp->f32, grp->youngs, maps, grp->sweep[ax], ctas, st);
-  }
-  if (err == cudaSuccess) {
-    GroupMap maps[5];
-    unsigned ctas[5];
-    for (int k = 0; k < 5; ++k) {
-      maps[k] = grp->l_sh[k].m;
-      ctas[k] = grp->l_sh[k].ctas;
-    }
-    err = launch_shift_grp(maps, grp->shift, ctas, st);
-  }
+      launch_tiles_grp(grp->l_tiles.m, grp->l_quiet.m, grp->args, grp->l_tiles.ctas, grp->l_quiet.ctas, st);
+  const int odd = (int)(step_index % 2);
+  const GroupMap sweep[2] = {grp->l_mix.m, grp->l_walk.m}, shift[3] = {grp->l_planes.m, grp->l_sweep.m, grp->l_apply.m};
+  const unsigned nsweep[2] = {grp->l_mix.ctas, grp->l_walk.ctas}, nshift[3] = {grp->l_planes.ctas, grp->l_sweep.ctas, grp->l_apply.ctas};
+  for (int s = 0; s < 3 && err == cudaSuccess; ++s)
+    err = launch_stage_grp(odd ? 2 - s : s, s, grp->f32, grp->youngs, sweep, nsweep, grp->args, st);
+  if (err == cudaSuccess) err = launch_shift_grp(shift, nshift, grp->args, odd, st);
   if (err == cudaSuccess && grp->sums)
     err = launch_reduce_grp(grp->l_red1.m, grp->red, grp->l_red1.ctas, (unsigned)grp->nbox, st);
   if (err != cudaSuccess) {

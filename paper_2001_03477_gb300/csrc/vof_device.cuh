@@ -43,11 +43,6 @@ struct GridDev {
 // oracle's double compares.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
-// a == b (IEEE: +0 == -0)
-__device__ __forceinline__ bool deq(double a, double b) {
-  unsigned long long x = (unsigned long long)dbits(a), y = (unsigned long long)dbits(b);
-  return x == y || ((x | y) << 1) == 0ull;
-}
 // a != 0 on the integer pipe.  The halves are taken with an opaque move: the
 // one-word form ((bits << 1) != 0) is exactly an FP64 "not equal to zero"
 // compare, and the compiler may emit it as one, which costs an FP64 unit
@@ -57,6 +52,8 @@ __device__ __forceinline__ bool dnz(double a) {
   asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(a));
   return ((hi & 0x7fffffffu) | lo) != 0u;
 }
+// a == b (IEEE: +0 == -0)
+__device__ __forceinline__ bool deq(double a, double b) { return dbits(a) == dbits(b) || (!dnz(a) && !dnz(b)); }
 __device__ __forceinline__ bool dgt0(double a) { return dbits(a) > 0; }
 __device__ __forceinline__ bool dlt0(double a) { return dbits(a) < 0 && dnz(a); }
 // a > 1.0
@@ -73,8 +70,13 @@ __device__ __forceinline__ double dtwice(double x) {
   const unsigned long long sg = b & 0x8000000000000000ull, mg = b & 0x7FFFFFFFFFFFFFFFull;
   return __longlong_as_double((long long)((mg >> 52) ? b + (1ull << 52) : (sg | (mg << 1))));
 }
-// -x (the sign bit flipped)
-__device__ __forceinline__ double dneg(double x) { return __longlong_as_double(dbits(x) ^ (long long)0x8000000000000000ull); }
+// -x (the sign bit flipped), through an opaque move: the one-word form is an
+// FP64 negation, which the compiler emits as an FP64 add
+__device__ __forceinline__ double dneg(double x) {
+  unsigned lo, hi;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(x));
+  return __hiloint2double((int)(hi ^ 0x80000000u), (int)lo);
+}
 // x / 2 where that is exact without rounding: x = 0, or the half a normal
 // number (exponent field >= 2); ok = false otherwise (the caller multiplies)
 __device__ __forceinline__ double dhalf_exact(double x, bool& ok) {
@@ -103,8 +105,7 @@ __device__ __forceinline__ double heat_cap(double Cp_l, double Cp_g, double c) {
 // (c, e) always give equal T.
 __device__ __forceinline__ double temp_of(const GridDev& g, double e, double c) {
   const long long b = __double_as_longlong(c);
-  if (b == 0x3FF0000000000000LL) return e * g.rCp_l;
-  if (b == 0) return e * g.rCp_g;
+  if (b == 0x3FF0000000000000LL || b == 0) return e * (b ? g.rCp_l : g.rCp_g);  // one multiply for both phases
   return e / heat_cap(g.Cp_l, g.Cp_g, c);
 }
 
@@ -907,7 +908,7 @@ __device__ __forceinline__ void myc_normal(const double* s, double m[3]) {
 
 // ---------------------------------------------------------------------------
 // WENO5 face value (Jiang-Shu weights, eps 1e-6), upwind-ordered stencil:
-// weno5_df (vof_df.cuh), the weights and the correction to the donor value
+// weno5_corr6_df (vof_df.cuh), the weights and the correction to the donor value
 // in double-float pairs (FP64-accurate, a fraction of the FP64 instructions).
 // Five equal values return the donor value exactly.
 // ---------------------------------------------------------------------------
@@ -1059,11 +1060,31 @@ __device__ __forceinline__ double slab_volume_f(const double m[3], double alpha,
   return v;
 }
 
+// FP32 of an FP64 value to nearest even, and back, on the integer pipe (an
+// FP64 conversion instruction occupies the FP64 unit like an add).  Values
+// below FP32's normal range become 0; infinities and NaN stay what they are.
+__device__ __forceinline__ float f32_of(double x) {
+  const unsigned long long b = (unsigned long long)dbits(x);
+  const unsigned long long r = (b & 0x7FFFFFFFFFFFFFFFull) + 0x0FFFFFFFull + ((b >> 29) & 1ull);
+  const int ex = (int)(r >> 52) - 1023 + 127;
+  unsigned f = ((unsigned)ex << 23) | ((unsigned)(r >> 29) & 0x7FFFFFu);
+  if (ex <= 0) f = 0u;
+  if (ex >= 255) f = ((b & 0x7FFFFFFFFFFFFFFFull) > 0x7FF0000000000000ull) ? 0x7FC00000u : 0x7F800000u;
+  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x), ex = (b >> 23) & 0xFFu;
+  const unsigned long long m = (unsigned long long)(b & 0x7FFFFFu) << 29;
+  const unsigned long long v = ex == 255u ? (0x7FF0000000000000ull | m) : (ex ? ((unsigned long long)(ex + 896u) << 52) | m : 0ull);
+  return __longlong_as_double((long long)(v | ((unsigned long long)(b & 0x80000000u) << 32)));
+}
+
 // WENO5 with the neighbour differences in FP64 and the nonlinear weights and
-// the correction to v0 in FP32: T_f = v0 + correction
-__device__ __forceinline__ double weno5_f(double vm2, double vm1, double v0, double vp1, double vp2) {
-  if (deq(vm2, v0) && deq(vm1, v0) && deq(vp1, v0) && deq(vp2, v0)) return v0;
-  const float D0 = (float)(vm1 - vm2), D1 = (float)(v0 - vm1), D2 = (float)(vp1 - v0), D3 = (float)(vp2 - vp1);
+// the correction to the donor value in FP32, from the four differences in
+// upwind order: T_f = v0 + correction (weno5_add)
+__device__ __forceinline__ double weno5_corr_f(double E0, double E1, double E2, double E3) {
+  if (!dnz(E0) && !dnz(E1) && !dnz(E2) && !dnz(E3)) return 0.0;
+  const float D0 = f32_of(E0), D1 = f32_of(E1), D2 = f32_of(E2), D3 = f32_of(E3);
   const float epsw = 1e-6f;
   const float d0 = D1 - D0, d1 = D2 - D1, d2 = D3 - D2;
   const float e0 = 3.f * D1 - D0, e1 = D1 + D2, e2 = D3 - 3.f * D2;
@@ -1075,8 +1096,9 @@ __device__ __forceinline__ double weno5_f(double vm2, double vm1, double v0, dou
   const float i0 = 1.f / (epsw + b0), i1 = 1.f / (epsw + b1), i2 = 1.f / (epsw + b2);
   const float w0 = 0.1f * i0 * i0, w1 = 0.6f * i1 * i1, w2 = 0.3f * i2 * i2;
   const float r0 = 5.f * D1 - 2.f * D0, r1 = 2.f * D2 + D1, r2 = 4.f * D2 - D3;
-  const float corr = (w0 * r0 + w1 * r1 + w2 * r2) / (6.f * (w0 + w1 + w2));
-  return v0 + (double)corr;
+  return f64_of((w0 * r0 + w1 * r1 + w2 * r2) / (6.f * (w0 + w1 + w2)));
 }
+// donor value plus its correction; a zero correction leaves the value's bits
+__device__ __forceinline__ double weno5_add(double v0, double corr) { return dnz(corr) ? v0 + corr : v0; }
 
 }  // namespace vofgb

@@ -76,27 +76,39 @@ VOF_HD float fma_f(float a, float b, float c) {
 #endif
 }
 
-// FP32 value of x * 2^-k with x's significand truncated to 24 bits, from the
-// bits (sign, exponent shifted by -k, top 23 stored bits); 0 when the result
-// would be below the normal FP32 range.  The caller keeps x * 2^-k below
-// 2^127.
-VOF_HD float trunc_scale(double x, int k) {
+// The two words of an FP64 value, through an opaque move on the device: masks
+// of the 64-bit pattern are recognised as FP64 absolute values and negations,
+// which are FP64 instructions.
+struct words {
+  uint32_t hi, lo;
+};
+VOF_HD words words_of(double x) {
+#ifdef __CUDA_ARCH__
+  words w;
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(w.lo), "=r"(w.hi) : "d"(x));
+  return w;
+#else
   const uint64_t b = d_bits(x);
-  const int e = (int)((b >> 52) & 0x7FF) - 1023 - k + 127;
-  if (e <= 0) return 0.0f;
-  if (e >= 255) return bits_f((uint32_t)((b >> 32) & 0x80000000u) | 0x7F800000u);  // beyond FP32: infinity
-  const uint32_t f = (uint32_t)((b >> 32) & 0x80000000u) | ((uint32_t)e << 23) | (uint32_t)((b >> 29) & 0x7FFFFFu);
-  return bits_f(f);
+  return {(uint32_t)(b >> 32), (uint32_t)b};
+#endif
 }
 
 // x * 2^-k as a pair: hi = x with its significand truncated to 24 bits
-// (exact in FP32), lo = the rest (one FP64 subtraction, exact), truncated to
-// 24 bits: |x 2^-k - (hi + lo)| <= 2^-47 |x 2^-k| (and below 2^-126 for
-// parts under the FP32 normal range)
-VOF_HD f2 split_scaled(double x, int k) {
-  const double xh = bits_d(d_bits(x) & 0xFFFFFFFFE0000000ull);
-  const double xl = x - xh;
-  return {trunc_scale(xh, k), trunc_scale(xl, k)};
+// (exact in FP32, from the bits; 0 below the normal FP32 range; the caller
+// keeps x 2^-k below 2^127), lo = the rest (the 29 bits below, an integer in
+// units of x's last place), rounded to 24 bits: |x 2^-k - (hi + lo)| <= 2^-48
+// |x 2^-k| (and below 2^-125 for parts under the FP32 normal range).  No FP64
+// instruction.
+VOF_HD f2 split_scaled(words x, int k) {
+  const int e = (int)((x.hi >> 20) & 0x7FF) - 1023 - k + 127;  // FP32 exponent field of x 2^-k
+  const uint32_t sg = x.hi & 0x80000000u;
+  const uint32_t man = ((x.hi & 0xFFFFFu) << 3) | (x.lo >> 29);
+  uint32_t h = ((uint32_t)e << 23) | man;
+  uint32_t u = (uint32_t)(e - 52) << 23;  // x's last place, scaled
+  if (e <= 0) h = 0u;
+  if (e <= 52) u = 0u;
+  if (e >= 255) h = u = 0x7F800000u;  // beyond FP32: infinity
+  return {bits_f(h | sg), (float)(x.lo & 0x1FFFFFFFu) * bits_f(u | sg)};
 }
 
 // FP64 value of the FP32 number f * 2^k (exact; f normal or zero)
@@ -107,6 +119,29 @@ VOF_HD double widen_scaled(float f, int k) {
   const uint64_t d = ((uint64_t)(b & 0x80000000u) << 32) | ((uint64_t)(ef + k - 127 + 1023) << 52) |
                      ((uint64_t)(b & 0x7FFFFFu) << 29);
   return bits_d(d);
+}
+
+VOF_HD int rint_i(float x) {
+#ifdef __CUDA_ARCH__
+  return __float2int_rn(x);
+#else
+  return (int)std::lrintf(x);
+#endif
+}
+// FP64 value of the pair (hi + lo) * 2^k (|lo| at most half a last place of
+// hi): hi widened exactly, then lo added to the bit pattern as an integer
+// number of FP64 last places, to the nearest (to two of them when the sum
+// drops below a power of two).  A lo whose last places are out of FP32's
+// range (hi below 2^-74) is left out.
+VOF_HD double widen_pair(f2 q, int k) {
+  const uint64_t h = d_bits(widen_scaled(q.hi, k));
+  const int eh = (int)((f_bits(q.hi) >> 23) & 0xFF);
+  if (eh == 0 || eh == 255) return bits_d(h);
+  const int es = 52 + 127 - (eh - 127);
+  const float up = es > 254 ? 0.0f : bits_f((uint32_t)es << 23);
+  // towards larger magnitude when the signs agree
+  const float l = bits_f(f_bits(q.lo) ^ (f_bits(q.hi) & 0x80000000u));
+  return bits_d(h + (uint64_t)(int64_t)rint_i(l * up));
 }
 
 // error-free transformations
@@ -134,8 +169,15 @@ VOF_HD f2 add(f2 x, f2 y) {
   s.lo += t.lo;
   return fast_two_sum(s.hi, s.lo);
 }
+// the same in 11 operations instead of 20, the error bounded by ~2^-46 of the
+// operands' magnitudes (no bound relative to a cancelled sum)
+VOF_HD f2 add_c(f2 x, f2 y) {
+  f2 s = two_sum(x.hi, y.hi);
+  s.lo += x.lo + y.lo;
+  return fast_two_sum(s.hi, s.lo);
+}
 VOF_HD f2 neg(f2 x) { return {-x.hi, -x.lo}; }
-VOF_HD f2 sub(f2 x, f2 y) { return add(x, neg(y)); }
+VOF_HD f2 twice(f2 x) { return {2.0f * x.hi, 2.0f * x.lo}; }  // exact
 VOF_HD f2 mul(f2 x, f2 y) {
   f2 p = two_prod(x.hi, y.hi);
   p.lo = fma_f(x.hi, y.lo, fma_f(x.lo, y.hi, p.lo));
@@ -152,57 +194,174 @@ VOF_HD f2 sqr(f2 x) {
   p.lo = fma_f(2.0f * x.hi, x.lo, p.lo);
   return fast_two_sum(p.hi, p.lo);
 }
-// x / y: the FP32 quotient, its remainder by one pair product, a correction
-VOF_HD f2 div(f2 x, f2 y) {
-  const float q1 = x.hi / y.hi;
-  const f2 r = sub(x, mul({q1, 0.0f}, y));
-  const float q2 = r.hi / y.hi;
-  return fast_two_sum(q1, q2);
+
+// Two FP32 values side by side: one packed instruction per operation on this
+// architecture (the same roundings as two separate ones).
+struct v2 {
+#ifdef __CUDA_ARCH__
+  unsigned long long b;
+#else
+  float x, y;
+#endif
+};
+VOF_HD v2 vset(float x, float y) {
+#ifdef __CUDA_ARCH__
+  v2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.b) : "f"(x), "f"(y));
+  return r;
+#else
+  return {x, y};
+#endif
 }
+VOF_HD void vget(v2 a, float& x, float& y) {
+#ifdef __CUDA_ARCH__
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.b));
+#else
+  x = a.x;
+  y = a.y;
+#endif
+}
+VOF_HD v2 vadd(v2 a, v2 b) {
+#ifdef __CUDA_ARCH__
+  v2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(a.b), "l"(b.b));
+  return r;
+#else
+  return {a.x + b.x, a.y + b.y};
+#endif
+}
+VOF_HD v2 vmul(v2 a, v2 b) {
+#ifdef __CUDA_ARCH__
+  v2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.b) : "l"(a.b), "l"(b.b));
+  return r;
+#else
+  return {a.x * b.x, a.y * b.y};
+#endif
+}
+VOF_HD v2 vfma(v2 a, v2 b, v2 c) {
+#ifdef __CUDA_ARCH__
+  v2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.b) : "l"(a.b), "l"(b.b), "l"(c.b));
+  return r;
+#else
+  return {std::fmaf(a.x, b.x, c.x), std::fmaf(a.y, b.y, c.y)};
+#endif
+}
+// a - b as one fused multiply-add: the same rounding
+VOF_HD v2 vsub(v2 a, v2 b) { return vfma(b, vset(-1.0f, -1.0f), a); }
+
+// two pairs side by side
+struct f2x2 {
+  v2 hi, lo;
+};
+VOF_HD f2x2 both(f2 x, f2 y) { return {vset(x.hi, y.hi), vset(x.lo, y.lo)}; }
+VOF_HD void each(f2x2 a, f2& x, f2& y) {
+  vget(a.hi, x.hi, y.hi);
+  vget(a.lo, x.lo, y.lo);
+}
+VOF_HD f2x2 two_sum(v2 a, v2 b) {
+  const v2 s = vadd(a, b), bb = vsub(s, a);
+  return {s, vadd(vsub(a, vsub(s, bb)), vsub(b, bb))};
+}
+VOF_HD f2x2 fast_two_sum(v2 a, v2 b) {
+  const v2 s = vadd(a, b);
+  return {s, vsub(b, vsub(s, a))};
+}
+VOF_HD f2x2 add(f2x2 x, f2x2 y) {
+  f2x2 s = two_sum(x.hi, y.hi);
+  const f2x2 t = two_sum(x.lo, y.lo);
+  s.lo = vadd(s.lo, t.hi);
+  s = fast_two_sum(s.hi, s.lo);
+  s.lo = vadd(s.lo, t.lo);
+  return fast_two_sum(s.hi, s.lo);
+}
+VOF_HD f2x2 add_c(f2x2 x, f2x2 y) {
+  f2x2 s = two_sum(x.hi, y.hi);
+  s.lo = vadd(s.lo, vadd(x.lo, y.lo));
+  return fast_two_sum(s.hi, s.lo);
+}
+VOF_HD f2x2 mul(f2x2 x, f2x2 y) {
+  const v2 p = vmul(x.hi, y.hi);
+  v2 e = vfma(x.hi, y.hi, vmul(p, vset(-1.0f, -1.0f)));
+  e = vfma(x.hi, y.lo, vfma(x.lo, y.hi, e));
+  return fast_two_sum(p, e);
+}
+VOF_HD f2x2 sqr(f2x2 x) {
+  const v2 p = vmul(x.hi, x.hi), m = vmul(p, vset(-1.0f, -1.0f));
+  return fast_two_sum(p, vfma(vadd(x.hi, x.hi), x.lo, vfma(x.hi, x.hi, m)));
+}
+VOF_HD f2x2 twice(f2x2 x) { return {vadd(x.hi, x.hi), vadd(x.lo, x.lo)}; }  // exact
 
 }  // namespace df
 
-// WENO5 face value (Jiang-Shu weights, eps = 1e-6, linear weights 0.1, 0.6,
-// 0.3) of the upwind-ordered stencil: the four neighbour differences in FP64,
-// the weights and the correction to v0 in pairs, T_f = v0 + correction in
-// FP64.  The same reformulation as the FP64 form: candidate values 6 v0 +
-// r_k, smoothness indicators scaled by 12/13 with eps (weights unchanged),
-// linear weights scaled by 10.  The differences are scaled by a power of
-// two 2^-k with the largest near 1 (k >= -20) and eps by 2^-2k, both exact,
-// so that no pair overflows or underflows where it matters; the correction
-// is scaled back exactly.  Error: ~1e-14 of the largest difference, far
-// below the FP64 form's parity bound.
-VOF_HD double weno5_df(double vm2, double vm1, double v0, double vp1, double vp2) {
+// Six times the WENO5 correction to the donor value (Jiang-Shu weights, eps =
+// 1e-6, linear weights 0.1, 0.6, 0.3) from the four neighbour differences D_0
+// .. D_3 in upwind order (D_1 = v0 - v_-1): T_f = v0 + correction, one FP64
+// fused multiply-add; exactly 0 when all four are 0.  With the second differences d_i = D_(i+1) - D_i the three
+// candidates are v0 + r_k / 6, r_1 = D_1 + 2 D_2, r_0 - r_1 = 2 (d_0 - d_1), r_2
+// - r_1 = d_1 - d_2, so six times the correction is
+//   r_1 + (2 w_0 (d_0 - d_1) + w_2 (d_1 - d_2)) / (w_0 + w_1 + w_2):
+// only the third differences pass through the weights, and the smoothness
+// indicators' first differences are 2 D_1 + d_0, D_1 + D_2 and d_2 - 2 D_2.
+// Indicators scaled by 12/13 with eps (weights unchanged), linear weights by
+// 10.  The differences are scaled by a power of two 2^-k with the largest near
+// 1 (k >= -20) and eps by 2^-2k, both exact, so that no pair overflows or
+// underflows where it matters; the correction is scaled back exactly.  Error:
+// ~1e-14 of the largest difference, far below the FP64 form's parity bound.
+// Indicators 0 and 2 mirror each other, so their arithmetic runs side by side:
+// (d_0, -d_2), (e_0, -e_2), (s_0, s_2).
+VOF_HD double weno5_corr6_df(double D0, double D1, double D2, double D3) {
   using namespace df;
-  const double D0 = vm1 - vm2, D1 = v0 - vm1, D2 = vp1 - v0, D3 = vp2 - vp1;
+  const words x0 = words_of(D0), x1 = words_of(D1), x2 = words_of(D2), x3 = words_of(D3);
   // exponent of the largest |D| (from the bits)
-  uint64_t mb = d_bits(D0) & 0x7FFFFFFFFFFFFFFFull;
-  uint64_t b1 = d_bits(D1) & 0x7FFFFFFFFFFFFFFFull, b2 = d_bits(D2) & 0x7FFFFFFFFFFFFFFFull,
-           b3 = d_bits(D3) & 0x7FFFFFFFFFFFFFFFull;
-  mb = mb > b1 ? mb : b1;
-  mb = mb > b2 ? mb : b2;
-  mb = mb > b3 ? mb : b3;
-  if (mb == 0) return v0;
-  int k = (int)(mb >> 52) - 1023 + 1;  // max |D| < 2^k
+  const uint32_t h0 = x0.hi & 0x7FFFFFFFu, h1 = x1.hi & 0x7FFFFFFFu, h2 = x2.hi & 0x7FFFFFFFu, h3 = x3.hi & 0x7FFFFFFFu;
+  const uint32_t m01 = h0 > h1 ? h0 : h1, m23 = h2 > h3 ? h2 : h3, mh = m01 > m23 ? m01 : m23;
+  if ((mh | x0.lo | x1.lo | x2.lo | x3.lo) == 0) return 0.0;
+  int k = (int)(mh >> 20) - 1023 + 1;  // max |D| < 2^k
   if (k < -20) k = -20;
-  const f2 a0 = split_scaled(D0, k), a1 = split_scaled(D1, k), a2 = split_scaled(D2, k), a3 = split_scaled(D3, k);
+  // (the outer two negated, by their sign bits)
+  const f2 n0 = split_scaled({x0.hi ^ 0x80000000u, x0.lo}, k), a1 = split_scaled(x1, k), a2 = split_scaled(x2, k),
+           n3 = split_scaled({x3.hi ^ 0x80000000u, x3.lo}, k);
   // eps' = 1e-6 * 12/13 * 2^-2k, exact scaling of the FP32 pair of eps'
-  const double epsd = 1e-6 * (12.0 / 13.0);
-  const f2 eps = split_scaled(epsd, 2 * k);
-  const f2 d0 = sub(a1, a0), d1 = sub(a2, a1), d2 = sub(a3, a2);
-  const f2 e0 = sub(mul_k(a1, 3.0f), a0), e1 = add(a1, a2), e2 = sub(a3, mul_k(a2, 3.0f));
-  const f2 c3 = split_scaled(3.0 / 13.0, 0);  // the ratio of the indicators' two terms, to pair accuracy
-  const f2 t0 = add(add(sqr(d0), mul(sqr(e0), c3)), eps);
-  const f2 t1 = add(add(sqr(d1), mul(sqr(e1), c3)), eps);
-  const f2 t2 = add(add(sqr(d2), mul(sqr(e2), c3)), eps);
-  const f2 s0 = sqr(t0), s1 = sqr(t1), s2 = sqr(t2);
-  const f2 w0 = mul(s1, s2), w1 = mul_k(mul(s0, s2), 6.0f), w2 = mul_k(mul(s0, s1), 3.0f);
-  const f2 r0 = sub(mul_k(a1, 5.0f), mul_k(a0, 2.0f)), r1 = add(mul_k(a2, 2.0f), a1),
-           r2 = sub(mul_k(a2, 4.0f), a3);
-  const f2 num = add(add(mul(w0, r0), mul(w1, r1)), mul(w2, r2));
-  const f2 den = mul_k(add(add(w0, w1), w2), 6.0f);
-  const f2 q = div(num, den);
-  return v0 + (widen_scaled(q.hi, k) + widen_scaled(q.lo, k));
+  const f2 eps = split_scaled(words_of(1e-6 * (12.0 / 13.0)), 2 * k);
+  const f2 c3 = split_scaled(words_of(3.0 / 13.0), 0);  // the ratio of the indicators' two terms, to pair accuracy
+  const f2x2 A = both(a1, a2);
+  const f2x2 d02 = add(A, both(n0, n3));  // (relative accuracy: they cancel)
+  const f2x2 e02 = add_c(twice(A), d02);
+  const f2x2 c33 = both(c3, c3), ee = both(eps, eps);
+  const f2x2 s02 = sqr(add_c(add_c(sqr(d02), mul(sqr(e02), c33)), ee));
+  const f2x2 de1 = add(both(a2, a2), both(neg(a1), a1));  // d_1, e_1
+  f2 q0, q1, d1, e1, s0, s2;
+  each(sqr(de1), q0, q1);
+  const f2 s1 = sqr(add_c(add_c(q0, mul(q1, c3)), eps));
+  each(s02, s0, s2);
+  each(de1, d1, e1);
+  // w_0 = s1 s2, w_2 / 3 = s0 s1, w_1 = 6 s0 s2
+  const f2x2 w02 = mul(both(s2, s0), both(s1, s1));
+  f2 w0, w2, p0, p2;
+  each(w02, w0, w2);
+  const f2 W = add_c(add_c(w0, mul_k(mul(s0, s2), 6.0f)), mul_k(w2, 3.0f));
+  // (d_0 - d_1, d_1 - d_2) times (w_0, w_2 / 3)
+  each(mul(w02, add_c(d02, both(neg(d1), d1))), p0, p2);
+  const f2 num = add_c(twice(p0), mul_k(p2, 3.0f));
+  // num / W: the FP32 quotient and one correction from its remainder
+  const float qh = num.hi / W.hi;
+  const f2 p = two_prod(qh, W.hi);
+  const float rem = ((num.hi - p.hi) - p.lo) + (num.lo - qh * W.lo);
+  const f2 q = fast_two_sum(qh, rem / W.hi);
+  return widen_pair(add(add_c(twice(a2), a1), q), k);
+}
+
+// Donor value plus a sixth of x, one rounding; x = 0 leaves the value's bits.
+VOF_HD double weno5_add6(double v0, double x) {
+#ifdef __CUDA_ARCH__
+  const double t = fma(x, 1.0 / 6.0, v0);
+#else
+  const double t = std::fma(x, 1.0 / 6.0, v0);
+#endif
+  const df::words w = df::words_of(x);
+  return ((w.hi & 0x7FFFFFFFu) | w.lo) == 0 ? v0 : t;
 }
 
 }  // namespace vofgb

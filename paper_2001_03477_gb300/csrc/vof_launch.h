@@ -113,10 +113,6 @@ inline SumOut sums_to_diag(double* diag, const signed char (&map)[kNSums]) {
 // is mixed when the shift runs, so the streaming kernels of an in-place step
 // skip them.  quiet == nullptr: no tile is skipped.
 constexpr int kTile = 8;
-struct TileMap {
-  const uint8_t* quiet;
-  int nt[3];  // tiles per axis
-};
 
 // Scratch of one sweep (kernel A -> kernels M, F, U): T of the cells whose
 // (c, e) differs from the previous cell of their line (kernel F adds the
@@ -130,8 +126,6 @@ struct SweepScratch {
   uint32_t* list;
   int* count;
   SumOut sums;       // per-CTA sums of kernel U: Delta c, Delta e, clipped volume
-  TileMap tiles;     // quiet tiles (in-place steps only)
-  int* stats;        // nullable: kernel U copies counters[0..1] here
   uint32_t* mlist;   // per-warp staging lists of mixed cells
   uint32_t* rlist;   // per-warp staging lists of run ends
   int* counters;     // [0] mixed cells, [1] face items at the front, [2] at the
@@ -144,8 +138,6 @@ struct SweepScratch {
   double* gplane;    // [2][N / n_axis][4]: planes of the ghost donors beyond the
                      // low / high zero-gradient end of each line (boundary
                      // cells that are mixed only)
-  int* mlp_stat;     // nullable: kernel U copies counters[3] (learned normals
-                     // replaced by MYC in this sweep) here
   double* F;         // face arrays of the axis (face layout of the velocities)
   double* G;
 };
@@ -166,8 +158,6 @@ struct SweepPlan {
 SweepPlan sweep_plan(int axis, const GridDev& g);
 size_t sweep_scratch_bytes(const GridDev& g);
 SweepScratch carve_sweep_scratch(int axis, const GridDev& g, void* ws, SumOut sums);
-
-int sweep_blocks(int axis, const GridDev& g);
 
 // Scratch of the shift: per-warp lists of moving mixed cells with their
 // counts (fixed order; a warp owns up to 256 cells of one x row), a
@@ -190,20 +180,19 @@ struct ShiftScratch {
   // every cell it visits; the cells of quiet tiles it skips are never read
   uint8_t* reach; // [N] 1: moving mixed cell with shift < 0, 2: > 0, else 0
   uint32_t* claim;  // [N] receivers: bit 31 - b set by the reaching neighbour at offset index b
-  TileMap tiles;  // quiet tiles (in-place steps only)
-  int* stats;     // nullable: the sums kernel copies counters[0..2] here
+  double* mark;   // nullable: the tagged c words (c_in), where receivers are marked instead of
+                  // claimed; then also the pairs whose plane may enter the receiver
+  uint2* pairs;
+  int pair_cap;
+  int* npairs;
 };
 
 // The shift's kernels: stream (lists; out of place also copies; sums c, e
 // when `stream_sums` is given) and sums (applies and sums the changes).
-// sum_blocks: CTAs of the sums kernel (rows it writes to its SumOut).
-int shift_sum_blocks(const GridDev& g);
-int shift_stream_blocks(const GridDev& g);
 size_t shift_scratch_bytes(const GridDev& g);
 ShiftScratch carve_shift_scratch(const GridDev& g, void* ws);
 
-// Tiles: per-tile uniform flag and values, then the quiet map; the tile
-// pass also sums c and e over the grid (per-CTA rows).
+// Tiles: per-tile uniform flag and values, then the quiet map.
 struct TileScratch {
   uint8_t* uni;
   double* vc;
@@ -212,19 +201,66 @@ struct TileScratch {
 };
 void tile_counts(const GridDev& g, int nt[3]);
 bool tiles_usable(const GridDev& g);
-int tile_blocks(const GridDev& g);
+int tile_total(const GridDev& g);
 size_t tile_scratch_bytes(const GridDev& g);
 TileScratch carve_tile_scratch(const GridDev& g, void* ws);
-// The tile pass of a time step also clears the step's frozen-state flags
-// (state[N], nullable) and its list counters (counters[kStepCounters],
-// nullable), so that the step needs no memset.
-constexpr int kStepCounters = 16;  // 4 per sweep axis, then the shift's 3; the last: the reduction's ticket
-cudaError_t launch_tiles(const GridDev& g, const double* c, const double* e, TileScratch ts, SumOut sums,
-                         uint8_t* state, int* counters, cudaStream_t st);
+
+// Counters of a time step (StepArgs::cnt), cleared by the tile pass: per
+// stage s = 0, 1, 2 (the sweeps in the order they run) [4 s] mixed cells in
+// the stage's list, [4 s + 1] faces evaluated, [4 s + 3] learned normals
+// replaced by MYC; [12], [13] the shift's list (other cells, edge cells),
+// [14] active tiles, [2] the shift's pairs, [15] the reduction's ticket.
+constexpr int kStepCounters = 16;
+
+// One grid's time step in place: everything its kernels need.
+struct StepArgs {
+  GridDev g;
+  double* c;             // the caller's fields: read by stages 0 and 2, written by stage 1 and the shift
+  double* e;
+  double* s_c;           // [N] scratch fields: written by stages 0 and 2, read by stage 1 and the shift;
+                         // between the stages the c words carry two tag bits (vof_fused.cu)
+  double* s_e;
+  const double* uf[3];
+  double* theta;         // [N] frozen Theta, written by stage 0 for every cell of an active tile
+  double* fl;            // [N] VOF flux a mixed cell sends through its left face (negative)
+  double* fr;            // [N] and through its right face; the shift reuses both
+  double* gf;            // [2][lines] the same of the ghost donors behind zero-gradient walls
+  double* plane;         // [N][4] learned normals (sweeps), planes (shift)
+  uint32_t* list[2];     // [N] mixed cells of the even / odd stages (the shift's is odd: non-edge
+                         // cells from the front, edge cells from the back), no fixed order
+  uint32_t* tlist;       // [tiles] the tiles that are not quiet, no fixed order
+  double* clip;          // [12][tiles] clipped volume per stage and quarter of a tile
+  double* rows;          // [tiles][kNSums] sum rows
+  TileScratch ts;
+  int nt[3];
+  int usable;            // quiet tiles may be skipped (tiles_usable)
+  int* cnt;              // [kStepCounters]
+  int* stats;            // [VOF_NCOUNTS] work counts, by axis
+  int* status;
+  const double* dd;
+  double dd_uniform;
+  uint2* pairs;          // [N] the shift's (source, neighbour) pairs (Theta's storage)
+  int pair_cap;
+  int chain;             // 0: one grid; else the walks' chain length in a batch of boxes
+};
+
+// tile pass: quiet map, active list, mixed cells of stage 0, the quiet
+// tiles' sum rows
+cudaError_t launch_tiles(const StepArgs& A, cudaStream_t st);
+// one sweep along `axis` as stage 0, 1 or 2
+cudaError_t launch_stage(const StepArgs& A, int axis, int stage, cudaStream_t st);
+// the shift of the state in the scratch fields, back into the caller's, and
+// the active tiles' sum rows; odd: the sweeps ran z, y, x
+cudaError_t launch_shift_step(const StepArgs& A, int odd, cudaStream_t st);
+unsigned quiet_ctas(const GridDev& g);
+unsigned mix_ctas(const GridDev& g);
+unsigned walk_ctas(const GridDev& g);
+unsigned shift_plane_ctas();
+unsigned apply_ctas(const GridDev& g);
 
 cudaError_t launch_sweep(int axis, const GridDev& g, const double* c_in, const double* e_in, double* c_out,
                          double* e_out, const double* uf, uint8_t* state, double* theta, double* flux_out,
-                         SweepScratch sc, bool zero_counters, cudaStream_t st);
+                         SweepScratch sc, cudaStream_t st);
 
 cudaError_t launch_energy(int axis, const GridDev& g, const double* c_before, const double* c_after,
                           const double* e_in, double* e_out, const double* F, const double* uf, uint8_t* state,
@@ -232,7 +268,7 @@ cudaError_t launch_energy(int axis, const GridDev& g, const double* c_before, co
 
 cudaError_t launch_shift(const GridDev& g, const double* c_in, const double* e_in, double* c_out, double* e_out,
                          const double* dd, double dd_uniform, uint8_t* state, ShiftScratch sc, SumOut stream_sums,
-                         SumOut sums, bool zero_counters, cudaStream_t st);
+                         SumOut sums, cudaStream_t st);
 
 cudaError_t launch_reconstruct(const GridDev& g, const double* c, double* m, double* alpha, uint8_t* mixed,
                                cudaStream_t st);
@@ -258,73 +294,34 @@ cudaError_t launch_reduce_fused(const ReduceJob& job, double* scratch, int* tick
 // of a batch (vof_group_*), each CTA on its box's arguments (from a table in
 // device memory) with its virtual block index in the box's own launch shape.
 // ---------------------------------------------------------------------------
-struct SweepArgs {  // one box's in-place sweep along one axis
-  GridDev g;
-  double* c;
-  double* e;
-  const double* uf;
-  uint8_t* state;
-  double* theta;
-  SweepScratch sc;
-  int cap, nsub, ngrp;
-  int* status;
-};
-struct TileArgs {
-  GridDev g;
-  const double* c;
-  const double* e;
-  TileScratch ts;
-  int nt[3];
-  SumOut sums;
-  uint8_t* state;  // cleared by the tile pass
-  int* counters;   // kStepCounters, cleared by the tile pass
-};
-struct ShiftArgs {
-  GridDev g;
-  double* c;
-  double* e;
-  const double* dd;
-  double dd_uniform;
-  ShiftScratch sc;
-  SumOut sums;
-  long long nw;
-};
 struct ReduceBox {  // one box's sum rows and its output
   const double* rows;
   int nblocks;
   double* out;
   double* scratch;  // kReduceCTAs x kMaxReduceK partials
 };
-cudaError_t launch_tiles_grp(const GroupMap& mt, const GroupMap& mq, const TileArgs* a, unsigned ct, unsigned cq,
+cudaError_t launch_tiles_grp(const GroupMap& mt, const GroupMap& mq, const StepArgs* a, unsigned ct, unsigned cq,
                              cudaStream_t st);
-// maps / ctas: [0] kernel A, [1] prep, [2] faces, [3] update
-cudaError_t launch_sweep_grp(int axis, int f32, int youngs, const GroupMap* maps, const SweepArgs* a,
-                             const unsigned* ctas, cudaStream_t st);
-// maps / ctas: [0] stream, [1] planes, [2] own, [3] receivers, [4] sums
-cudaError_t launch_shift_grp(const GroupMap* maps, const ShiftArgs* a, const unsigned* ctas, cudaStream_t st);
+// maps / ctas: [0] mix, [1] walk
+cudaError_t launch_stage_grp(int axis, int stage, int f32, int youngs, const GroupMap* maps, const unsigned* ctas,
+                             const StepArgs* a, cudaStream_t st);
+// maps / ctas: [0] planes, [1] swept volumes, [2] apply
+cudaError_t launch_shift_grp(const GroupMap* maps, const unsigned* ctas, const StepArgs* a, int odd, cudaStream_t st);
 // m1: (box, part) CTAs of the first level; the second level runs one CTA per box
 cudaError_t launch_reduce_grp(const GroupMap& m1, const ReduceBox* rb, unsigned ctas1, unsigned nbox,
                               cudaStream_t st);
-// One box's arguments and launch shapes for every kernel of a grouped time
-// step (vof_api.cu builds them exactly as vof_step carves its workspace).
+// One box's arguments and launch shapes for the kernels of a time step
+// (vof_api.cu; vof_step uses the same).
 struct StepBox {
   size_t cells;
-  TileArgs tiles;
-  SweepArgs sweep[3];
-  ShiftArgs shift;
+  StepArgs args;
   ReduceBox red;
-  dim3 grid_tiles, grid_stream[3], grid_shift_stream;
-  unsigned grid_quiet, grid_update[3], grid_shift_sums;
+  dim3 grid_tiles;
 };
 // false for a grid vof_step refuses; ws: the box's step workspace
 // (vof_step_workspace_bytes), sums: device double[VOF_NSUMS] or null
 bool step_box(const vof_grid* g, double* c, double* e, const double* u, const double* v, const double* w,
               double dt, const double* dd, double dd_uniform, double* sums, char* ws, StepBox* out);
-int shift_list_ctas();
-long long shift_warps_of(const GridDev& g);
-int prep_ctas();
-dim3 shift_stream_grid_of(const GridDev& g);
-unsigned quiet_blocks(const GridDev& g);
 
 // per-launch timing (vof_profile_begin/end): records an event after a launch
 void prof_mark(const char* name, cudaStream_t st);
@@ -363,7 +360,11 @@ cudaError_t launch_mlp_pack(const float* master, void* packed, cudaStream_t st);
 cudaError_t launch_mlp_forward(const void* params, const double* X, long n, float* y, cudaStream_t st);
 cudaError_t launch_mlp_normals(const void* params, const double* X, long n, double* m, uint8_t* flag,
                                int* nfallback, cudaStream_t st);
-cudaError_t launch_mlp_sweep_normals(const GridDev& g, const double* c, const SweepScratch& sc, cudaStream_t st);
+// tagged: the words of c carry a step's tag bits; list: the mixed cells,
+// counters[0] of them (device); normals into
+// plane[cell][0..2], counters[3] += fallbacks
+cudaError_t launch_mlp_sweep_normals(const GridDev& g, const double* c, bool tagged, const uint32_t* list,
+                                     int* counters, double* plane, cudaStream_t st);
 cudaError_t launch_mlp_train_step(const double* X, const double* N, long ntrain, int batch, unsigned long long seed,
                                   long step, float* master, float* mom, float* vel, void* packed, float* partial,
                                   float* loss_part, const long* idx_fixed, float lr, float beta1, float beta2,

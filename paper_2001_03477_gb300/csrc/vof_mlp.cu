@@ -260,6 +260,7 @@ struct SrcGrid {
   GridDev g;
   const double* c;
   const uint32_t* gmix;
+  unsigned mask;  // of the high words: all ones, or without a time step's tag bits (vof_fused.cu)
   __device__ __forceinline__ double at(long i, int k) const {
     const size_t id = gmix[i];
     int x, y, z;
@@ -267,7 +268,8 @@ struct SrcGrid {
     const int xx = map_idx(x + k % 3 - 1, g.n[0], g.bc[0]);
     const int yy = map_idx(y + (k / 3) % 3 - 1, g.n[1], g.bc[1]);
     const int zz = map_idx(z + k / 9 - 1, g.n[2], g.bc[2]);
-    return __ldg(c + ((size_t)zz * g.n[1] + yy) * g.n[0] + xx);
+    const double w = __ldg(c + ((size_t)zz * g.n[1] + yy) * g.n[0] + xx);
+    return __hiloint2double((int)((unsigned)__double2hiint(w) & mask), __double2loint(w));
   }
 };
 
@@ -887,13 +889,13 @@ cudaError_t launch_mlp_normals(const void* params, const double* X, long n, doub
   return launch_infer_t<1>(mlp::SrcX{X}, nullptr, n, n, params, nullptr, m, flag, nullptr, nfallback, st);
 }
 
-cudaError_t launch_mlp_sweep_normals(const GridDev& g, const double* c, const SweepScratch& sc, cudaStream_t st) {
+cudaError_t launch_mlp_sweep_normals(const GridDev& g, const double* c, bool tagged, const uint32_t* list,
+                                     int* counters, double* plane, cudaStream_t st) {
   const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-  mlp::SrcGrid src{g, c, sc.gmix};
+  mlp::SrcGrid src{g, c, list, tagged ? 0x3FFFFFFFu : 0xFFFFFFFFu};
   // the mixed-cell count (counters[0]) is read on the device; fallbacks are
   // counted in counters[3]
-  return launch_infer_t<2>(src, sc.counters, 0, (long)N, g.mlp_params, nullptr, nullptr, nullptr, sc.plane,
-                           sc.counters + 3, st);
+  return launch_infer_t<2>(src, counters, 0, (long)N, g.mlp_params, nullptr, nullptr, nullptr, plane, counters + 3, st);
 }
 
 cudaError_t launch_mlp_train_step(const double* X, const double* N, long ntrain, int batch, unsigned long long seed,

@@ -13,12 +13,11 @@
 // visit a compact list of the moving mixed cells instead of the grid.
 #include "vof_launch.h"
 #include "vof_sums.cuh"
+#include "vof_sweep.cuh"
 
 namespace vofgb {
 
 constexpr int kShBX = 32, kShBY = 4, kShBZ = 2, kShThreads = kShBX * kShBY * kShBZ;
-
-__device__ __forceinline__ bool same_bits_dev(double a, double b) { return dbits(a) == dbits(b); }
 
 // ---------------------------------------------------------------------------
 // Shift in four kernels.
@@ -51,6 +50,9 @@ __device__ __forceinline__ void decode(const GridDev& g, size_t id, int& x, int&
 __device__ __forceinline__ size_t cell_id(const GridDev& g, int x, int y, int z) {
   return ((size_t)z * g.n[1] + y) * g.n[0] + x;
 }
+
+// tag bits of a step's c word (vof_fused.cu)
+__device__ __forceinline__ unsigned c_tag_of(double w) { return (unsigned)__double2hiint(w) >> 30; }
 
 // c within 1e-3 of 0 or 1: alpha(c) is ill-conditioned and the plane is
 // extrapolated into neighbours, so its constant takes the bisection
@@ -85,21 +87,11 @@ __device__ __forceinline__ void k_shift_stream_body(const GridDev& g, const doub
   const int cap = nx < kWarpCells ? nx : kWarpCells;
   uint32_t* list = sc.list + w * cap;
   const bool do_sums = sums.partials || sums.diag;
-  // quiet tiles of the row segment (in place only): bit l = tile l quiet
-  unsigned qmask = 0u;
-  if (sc.tiles.quiet && !copy && !do_sums && rowok) {
-    const int txi = (x0 >> 3) + lane;
-    const int y = row % ny, z = row / ny;
-    const bool q = txi * kTile < x1 &&
-                   sc.tiles.quiet[((size_t)(z >> 3) * sc.tiles.nt[1] + (y >> 3)) * sc.tiles.nt[0] + txi] != 0;
-    qmask = __ballot_sync(kFullMask, q);
-  }
   int n = 0, ne = 0;
   double v[kNSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   const bool uni_moving = dnz(dd_uniform);
   if (rowok) {
     for (int it = 0; it < kWarpCells / 32 && x0 + 32 * it < x1; ++it) {
-      if (((qmask >> (4 * it)) & 0xFu) == 0xFu) continue;  // four quiet tiles: no mixed cell
       const int X = x0 + 32 * it + lane;
       const bool ok = X < x1;
       const size_t id = rbase + X;
@@ -122,9 +114,8 @@ __device__ __forceinline__ void k_shift_stream_body(const GridDev& g, const doub
         if (dd) ddv = __ldg(dd + id);
         moving = dd ? dnz(ddv) : uni_moving;
       }
-      // every visited cell's reach byte and claim word are written here, so
-      // the later kernels (which read them only next to moving cells, never
-      // in a skipped quiet tile) need no cleared arrays
+      // every cell's reach byte and claim word are written here, so the later
+      // kernels need no cleared arrays
       if (ok) {
         sc.reach[id] = moving ? (dlt0(ddv) ? 1 : 2) : 0;
         sc.claim[id] = 0u;
@@ -194,6 +185,10 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
       }
     }
   }
+  if (sc.mark) {  // a time step's c words carry tag bits
+#pragma unroll
+    for (int i = 0; i < 27; ++i) st[i] = c_value(st[i]);
+  }
   const double ct = st[13];
   double m[3];
   myc_normal(st, m);
@@ -222,12 +217,40 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
   // one that settles the receiver -- holds the highest set bit whatever
   // the order of the atomics
   const bool full = dlt0(ddv);  // the kind of pure cell this shift reaches
+  // In a time step: only marks, and a list of the pairs whose plane may enter
+  // the neighbour.  Most stay outside (the shift is a few hundredths of a cell),
+  // which FP32 decides with a margin far above its rounding; the exact test and
+  // the volumes are k_shift_sweep's.
+  float fm[3] = {0.f, 0.f, 0.f}, fa = 0.f, flo = 0.f, fhi = 0.f, mg = 0.f;
+  if (sc.mark) {
+    fm[0] = f32_of(m[0]); fm[1] = f32_of(m[1]); fm[2] = f32_of(m[2]);
+    const float al_f = f32_of(al), sft_f = f32_of(sft);
+    fa = al_f + sft_f;
+    flo = fminf(fm[0], 0.f) + fminf(fm[1], 0.f) + fminf(fm[2], 0.f);
+    fhi = fmaxf(fm[0], 0.f) + fmaxf(fm[1], 0.f) + fmaxf(fm[2], 0.f);
+    mg = 1e-5f * (4.f + fabsf(al_f) + fabsf(sft_f));
+  }
   for (int oz = -1; oz <= 1; ++oz)
     for (int oy = -1; oy <= 1; ++oy)
       for (int ox = -1; ox <= 1; ++ox) {
         if (!ox && !oy && !oz) continue;
         size_t pid;
         if (!neighbour(g, x, y, z, ox, oy, oz, pid)) continue;
+        if (sc.mark) {
+          const double cp = c_value(__ldg(c_in + pid));
+          if (is_mixed_b(cp, g) || is_full_b(cp, g) != full) continue;
+          // (every store of a word writes the same bits, and its readers here
+          // drop the tag)
+          reinterpret_cast<unsigned*>(sc.mark + pid)[1] = (unsigned)__double2hiint(cp) | 0xC0000000u;
+          sc.cnew[pid] = 0.0;  // no change so far
+          const float an = fa - (fm[0] * (float)ox + fm[1] * (float)oy + fm[2] * (float)oz);
+          const bool outside = full ? an >= fhi + mg : an <= flo - mg;
+          if (!outside && sub == 0 && dnz(sft)) {
+            const int k = atomicAdd(sc.npairs, 1);
+            if (k < sc.pair_cap) sc.pairs[k] = make_uint2((uint32_t)id, (unsigned)offset_bit(ox, oy, oz));
+          }
+          continue;
+        }
         const double cp = __ldg(c_in + pid);
         if (is_mixed_b(cp, g) || is_full_b(cp, g) != full) continue;
         atomicOr(sc.claim + pid, 0x80000000u >> offset_bit(-ox, -oy, -oz));
@@ -422,7 +445,7 @@ __device__ __forceinline__ void k_shift_sums_body(const GridDev& g, const double
     for (int i = lane; i < cnt; i += 32) {
       const size_t qid = list[i];
       const double ct = c_in[qid], cn = sc.cnew[qid];
-      if (!same_bits_dev(cn, ct)) {
+      if (!same_bits(cn, ct)) {
         const double dc = cn - ct;
         const double de = dc * (g.Cp_l - g.Cp_g) * g.T_sat;
         const double eq = e_in[qid];
@@ -446,7 +469,7 @@ __device__ __forceinline__ void k_shift_sums_body(const GridDev& g, const double
         const double v = cp + best;
         const double vc = dlt0(v) ? 0.0 : (dgt1(v) ? 1.0 : v);
         if (!deq(v, vc)) acc[1] += v - vc;
-        if (!same_bits_dev(vc, cp)) {
+        if (!same_bits(vc, cp)) {
           const double dc = vc - cp;
           const double de = dc * (g.Cp_l - g.Cp_g) * g.T_sat;
           const double ep = e_in[pid];
@@ -465,11 +488,6 @@ __device__ __forceinline__ void k_shift_sums_body(const GridDev& g, const double
   v[kSumShDc] = acc[0];
   v[kSumUnpl] = acc[1];
   v[kSumShDe] = acc[2];
-  if (sc.stats && vb.bx == 0 && threadIdx.x == 0) {
-    sc.stats[0] = sc.counters[0];
-    sc.stats[1] = sc.counters[1];
-    sc.stats[2] = sc.counters[2];
-  }
   block_sums(v, sums, vb.bx);
 }
 
@@ -532,15 +550,10 @@ static long long shift_warps(const GridDev& g) {
   return (long long)((g.n[0] + kWarpCells - 1) / kWarpCells) * g.n[1] * g.n[2];
 }
 
-int shift_sum_blocks(const GridDev& g) { return (int)((shift_warps(g) + 7) / 8); }
+static int shift_sum_blocks(const GridDev& g) { return (int)((shift_warps(g) + 7) / 8); }
 
 static dim3 shift_stream_grid(const GridDev& g) {
   return dim3((unsigned)((g.n[1] * g.n[2] + 7) / 8), (unsigned)((g.n[0] + kWarpCells - 1) / kWarpCells), 1);
-}
-
-int shift_stream_blocks(const GridDev& g) {
-  const dim3 d = shift_stream_grid(g);
-  return (int)(d.x * d.y);
 }
 
 static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -581,76 +594,288 @@ ShiftScratch carve_shift_scratch(const GridDev& g, void* ws) {
   s.own = reinterpret_cast<uint32_t*>(b);    b += al256(N * 4);
   s.reach = reinterpret_cast<uint8_t*>(b);   b += al256(N);
   s.claim = reinterpret_cast<uint32_t*>(b);
-  s.tiles = TileMap{nullptr, {0, 0, 0}};
-  s.stats = nullptr;
+  s.mark = nullptr;
   return s;
 }
 
-__global__ void __launch_bounds__(256) k_shift_stream_grp(GroupMap m, const ShiftArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ ShiftArgs sA;
-  const ShiftArgs& A = cta_args(args, b, sA);
-  const SumOut none = sums_to_partials(nullptr, kNSums);
-  k_shift_stream_body(A.g, A.c, A.e, A.c, A.e, A.dd, A.dd_uniform, A.sc, none, 0, vb);
-}
-__global__ void __launch_bounds__(kListThreads) k_shift_planes_grp(GroupMap m, const ShiftArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ ShiftArgs sA;
-  const ShiftArgs& A = cta_args(args, b, sA);
-  k_shift_planes_body(A.g, A.c, A.dd, A.dd_uniform, A.sc, vb);
-}
-__global__ void __launch_bounds__(kListThreads) k_shift_own_grp(GroupMap m, const ShiftArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ ShiftArgs sA;
-  const ShiftArgs& A = cta_args(args, b, sA);
-  k_shift_own_body(A.g, A.c, A.dd, A.dd_uniform, A.sc, vb);
-}
-__global__ void __launch_bounds__(kListThreads) k_shift_receivers_grp(GroupMap m, const ShiftArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ ShiftArgs sA;
-  const ShiftArgs& A = cta_args(args, b, sA);
-  k_shift_receivers_body(A.g, A.c, A.dd, A.dd_uniform, A.sc, vb);
-}
-__global__ void __launch_bounds__(256) k_shift_sums_grp(GroupMap m, const ShiftArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ ShiftArgs sA;
-  const ShiftArgs& A = cta_args(args, b, sA);
-  k_shift_sums_body(A.g, A.c, A.e, A.c, A.e, A.sc, A.nw, A.sums, vb);
+// ---------------------------------------------------------------------------
+// The shift of a time step: the planes kernel on the list the last sweep left
+// (moving mixed cells of the scratch fields) also marks the receivers and lists
+// the (source, neighbour) pairs whose moved plane may enter the neighbour; a
+// kernel over the pairs, one per lane, evaluates the swept volumes; one over the
+// active tiles applies every change, writes the tile's cells to the caller's
+// fields and sums them.  (The stand-alone shift's own, receivers and sums
+// kernels took 21, 48 and 32 us of the 256^3 bubble step, each a few ten
+// thousand cells' latency; the tile kernel also replaces the sums of the whole
+// grid at the step's start.)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ ShiftScratch step_shift_scratch(const StepArgs& A) {
+  ShiftScratch s{};
+  s.counters = A.cnt + 12;
+  s.gmix = A.list[1];
+  s.plane = A.plane;
+  s.shift = A.fl;
+  s.cnew = A.fr;
+  s.mark = A.s_c;
+  s.pairs = A.pairs;
+  s.pair_cap = A.pair_cap;
+  s.npairs = A.cnt + 2;
+  return s;
 }
 
-cudaError_t launch_shift_grp(const GroupMap* m, const ShiftArgs* a, const unsigned* n, cudaStream_t st) {
-  if (n[0]) k_shift_stream_grp<<<n[0], dim3(32, 8), 0, st>>>(m[0], a);
-  prof_mark("group.shift_stream", st);
-  if (n[1]) k_shift_planes_grp<<<n[1], kListThreads, 0, st>>>(m[1], a);
-  prof_mark("group.shift_planes", st);
-  if (n[2]) k_shift_own_grp<<<n[2], kListThreads, 0, st>>>(m[2], a);
-  prof_mark("group.shift_own", st);
-  if (n[3]) k_shift_receivers_grp<<<n[3], kListThreads, 0, st>>>(m[3], a);
-  prof_mark("group.shift_receivers", st);
-  if (n[4]) k_shift_sums_grp<<<n[4], 256, 0, st>>>(m[4], a);
-  prof_mark("group.shift_sums", st);
+__global__ void __launch_bounds__(kListThreads) k_shift_mark(StepArgs A) {
+  pdl_wait();
+  k_shift_planes_body(A.g, A.s_c, A.dd, A.dd_uniform, step_shift_scratch(A), vb_self());
+}
+
+// the change by one neighbour's plane (m, al, shift sft) extended into the
+// receiver at offset (ox, oy, oz) from it; 0 when it stays outside
+__device__ __forceinline__ double swept_change(const double4& pl, double sft, bool full, int ox, int oy, int oz) {
+  const double m0 = pl.x, m1 = pl.y, m2 = pl.z, al = pl.w;
+  // m . o with o of -1, 0, 1: signs and zeros, no multiply
+  auto term = [](double m, int o) { return o == 0 ? 0.0 : (o > 0 ? m : dneg(m)); };
+  const double shiftv = dneg((term(m0, ox) + term(m1, oy)) + term(m2, oz));
+  const double a_old = al + shiftv;
+  const double a_new = (al + sft) + shiftv;
+  double lo = 0.0, hi = 0.0;
+  if (dlt0(m0)) lo += m0; else hi += m0;
+  if (dlt0(m1)) lo += m1; else hi += m1;
+  if (dlt0(m2)) lo += m2; else hi += m2;
+  // the extended plane stays outside the receiver: both volumes are exactly
+  // 1 (or 0); the margin clears the rounding of that test
+  if (full ? (a_new >= hi + 1e-9) : (a_new <= lo - 1e-9)) return 0.0;
+  const VolNormal vn = volume_normal_nn(m0, m1, m2);
+  return volume_at_nn(vn, a_new) - volume_at_nn(vn, a_old);
+}
+
+// One pair per lane.  A receiver takes the largest change: the maximum of
+// (|change|, positive) as an integer in its word of fr, the same whatever the
+// order.  A list that did not hold every pair (dense interfaces on tiny grids)
+// is left aside, and every neighbour of every moving cell is looked at.
+__device__ __forceinline__ void sweep_pairs_body(const StepArgs& A, const VB vb) {
+  const GridDev& g = A.g;
+  const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
+  const int np = A.cnt[2], nn = A.cnt[12], ne = A.cnt[13];
+  const bool listed = np <= A.pair_cap;
+  const long long total = listed ? np : 27ll * (nn + ne);
+  for (long long i = (long long)vb.bx * blockDim.x + threadIdx.x; i < total; i += (long long)vb.gx * blockDim.x) {
+    size_t id;
+    int b;
+    if (listed) {
+      const uint2 pr = A.pairs[i];
+      id = pr.x;
+      b = (int)pr.y;
+    } else {
+      const int j = (int)(i / 27);
+      b = (int)(i % 27);
+      id = j < nn ? A.list[1][j] : A.list[1][N - 1 - (size_t)(j - nn)];
+    }
+    const double sft = A.fl[id];
+    if (b == 13 || !dnz(sft)) continue;
+    int x, y, z;
+    decode(g, id, x, y, z);
+    const int ox = b % 3 - 1, oy = (b / 3) % 3 - 1, oz = b / 9 - 1;
+    size_t pid;
+    if (!neighbour(g, x, y, z, ox, oy, oz, pid)) continue;
+    const double w = A.s_c[pid];
+    if (c_tag_of(w) != 3u) continue;
+    const bool full = is_full_b(c_value(w), g);
+    if (full != (c_tag_of(A.s_c[id]) == 1u)) continue;  // tag 1: dd < 0
+    const double sw = swept_change(reinterpret_cast<const double4*>(A.plane)[id], sft, full, ox, oy, oz);
+    if (dnz(sw))
+      atomicMax(reinterpret_cast<unsigned long long*>(A.fr + pid),
+                (unsigned long long)dbits(sw) << 1 | (dlt0(sw) ? 0ull : 1ull));
+  }
+}
+
+__global__ void __launch_bounds__(kListThreads) k_shift_sweep(StepArgs A) {
+  pdl_wait();
+  sweep_pairs_body(A, vb_self());
+}
+
+constexpr int kAppThreads = 128;
+constexpr int kAppCells = kTile * kTile * kTile / kAppThreads;  // cells per thread
+
+struct AppSmem {
+  double red[5][kAppThreads];
+  int ones[4];
+  unsigned moved[4], cmix[4];
+};
+
+// One CTA per active tile: the moving mixed cells' and the receivers' new
+// values, the tile's cells to the caller's fields, its sum row.
+__device__ __forceinline__ void apply_body(const StepArgs& A, int odd, const VB vb, AppSmem& S) {
+  const GridDev& g = A.g;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int ntx = A.nt[0], nty = A.nt[1], T_all = ntx * nty * A.nt[2];
+  const int nact = A.cnt[14];
+  if (vb.bx == 0 && tid == 0) {  // the step's work counts, by axis
+    for (int s = 0; s < 3; ++s) {
+      const int ax = odd ? 2 - s : s;
+      A.stats[2 * ax] = A.cnt[4 * s];
+      A.stats[2 * ax + 1] = A.cnt[4 * s + 1];
+      A.stats[9 + ax] = A.cnt[4 * s + 3];
+    }
+    A.stats[6] = A.cnt[12];
+    A.stats[7] = A.cnt[13];
+  }
+  int nrecv = 0;
+  for (int it = (int)vb.bx; it < nact; it += (int)vb.gx) {
+    const int t = (int)A.tlist[it];
+    const int x0 = (t % ntx) * kTile, y0 = ((t / ntx) % nty) * kTile, z0 = (t / (ntx * nty)) * kTile;
+    double cv[kAppCells], ev[kAppCells];
+    unsigned tg[kAppCells];
+    size_t id[kAppCells];
+    bool ok[kAppCells];
+#pragma unroll
+    for (int r = 0; r < kAppCells; ++r) {
+      const int j = r * kAppThreads + tid;
+      const int x = x0 + (j & 7), y = y0 + ((j >> 3) & 7), z = z0 + (j >> 6);
+      ok[r] = x < g.n[0] && y < g.n[1] && z < g.n[2];
+      id[r] = ok[r] ? ((size_t)z * g.n[1] + y) * g.n[0] + x : 0;
+      const double w = ok[r] ? __ldcs(A.s_c + id[r]) : 0.0;
+      ev[r] = ok[r] ? __ldcs(A.s_e + id[r]) : 0.0;
+      cv[r] = c_value(w);
+      tg[r] = c_tag_of(w);  // 1, 2: moving mixed cell (dd < 0, > 0), 3: receiver
+    }
+    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};  // c of the mixed cells, e, dc, clamped, de
+    int ones = 0;
+    unsigned any = 0u;
+#pragma unroll
+    for (int r = 0; r < kAppCells; ++r) {
+      any |= tg[r];
+      if (__any_sync(kFullMask, tg[r] != 0)) {
+        double cn = cv[r];
+        if (tg[r] == 1 || tg[r] == 2) {
+          cn = A.fr[id[r]];
+        } else if (tg[r] == 3) {
+          ++nrecv;
+          const long long key = dbits(A.fr[id[r]]);
+          if (key) {
+            const double mag = __longlong_as_double((long long)((unsigned long long)key >> 1));
+            const double w = (key & 1) ? cv[r] + mag : cv[r] - mag;
+            cn = dlt0(w) ? 0.0 : (dgt1(w) ? 1.0 : w);
+            if (!deq(w, cn)) v[3] += w - cn;
+          }
+        }
+        if (!same_bits(cn, cv[r])) {
+          const double dc = cn - cv[r];
+          const double de = dc * (g.Cp_l - g.Cp_g) * g.T_sat;
+          cv[r] = cn;
+          ev[r] = ev[r] + de;
+          v[2] += dc;
+          v[4] += de;
+        }
+      }
+      if (ok[r]) {
+        A.c[id[r]] = cv[r];
+        A.e[id[r]] = ev[r];
+      }
+      const long long cb = dbits(cv[r]);
+      if (cb == kOneBits) ++ones;
+      const bool other = cb != 0 && cb != kOneBits;
+      if (__any_sync(kFullMask, other)) v[0] += other ? cv[r] : 0.0;
+    }
+    // pairwise; each sum once per CTA, by one warp, and only where a cell
+    // contributes (an FP64 addition costs a warp ~76 cycles of its FP64 unit)
+    static_assert(kAppCells == 4, "the sum of a thread's cells below");
+    v[1] = (ev[0] + ev[1]) + (ev[2] + ev[3]);
+    ones = __reduce_add_sync(kFullMask, ones);
+    const bool wmoved = __any_sync(kFullMask, any != 0), wmix = __any_sync(kFullMask, dnz(v[0]));
+    if (lane == 0) {
+      S.ones[warp] = ones;
+      S.moved[warp] = wmoved;
+      S.cmix[warp] = wmix;
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) S.red[k][tid] = v[k];
+    __syncthreads();
+    const bool moved = (S.moved[0] | S.moved[1] | S.moved[2] | S.moved[3]) != 0;
+    const bool cmix = (S.cmix[0] | S.cmix[1] | S.cmix[2] | S.cmix[3]) != 0;
+    double* row = A.rows + (size_t)t * kNSums;
+    for (int k = warp; k < 5; k += kAppThreads / 32) {
+      double x = 0.0;
+      if (k == 1 || (k == 0 ? cmix : moved)) {  // uniform over the CTA
+        x = (S.red[k][lane] + S.red[k][lane + 32]) + (S.red[k][lane + 64] + S.red[k][lane + 96]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFullMask, x, o);
+      }
+      if (k == 0) x += (double)(S.ones[0] + S.ones[1] + S.ones[2] + S.ones[3]);
+      if (lane == 0) row[k == 0 ? kSumC : (k == 1 ? kSumE : (k == 2 ? kSumShDc : (k == 3 ? kSumUnpl : kSumShDe)))] = x;
+    }
+    if (warp == 3) {  // the sweeps' clipped volume of this tile
+      const double x = lane < 12 ? A.clip[(size_t)lane * T_all + t] : 0.0;
+      double s = 0.0;
+      if (__any_sync(kFullMask, dnz(x)))
+        for (int q = 0; q < 12; ++q) s += __shfl_sync(kFullMask, x, q);
+      if (lane == 0) row[kSumClip] = s;
+    }
+    __syncthreads();  // the shared values are rewritten for the next tile
+  }
+  nrecv = __reduce_add_sync(kFullMask, nrecv);
+  if (lane == 0 && nrecv) atomicAdd(A.stats + 8, nrecv);
+}
+
+__global__ void __launch_bounds__(kAppThreads) k_shift_apply(StepArgs A, int odd) {
+  __shared__ AppSmem S;
+  pdl_wait();
+  apply_body(A, odd, vb_self(), S);
+}
+
+__global__ void __launch_bounds__(kListThreads) k_shift_mark_grp(GroupMap m, const StepArgs* __restrict__ args) {
+  unsigned b;
+  const VB vb = vb_group(m, b);
+  __shared__ StepArgs sA;
+  const StepArgs& A = cta_args(args, b, sA);
+  k_shift_planes_body(A.g, A.s_c, A.dd, A.dd_uniform, step_shift_scratch(A), vb);
+}
+__global__ void __launch_bounds__(kListThreads) k_shift_sweep_grp(GroupMap m, const StepArgs* __restrict__ args) {
+  unsigned b;
+  const VB vb = vb_group(m, b);
+  __shared__ StepArgs sA;
+  sweep_pairs_body(cta_args(args, b, sA), vb);
+}
+__global__ void __launch_bounds__(kAppThreads) k_shift_apply_grp(GroupMap m, const StepArgs* __restrict__ args, int odd) {
+  __shared__ AppSmem S;
+  unsigned b;
+  const VB vb = vb_group(m, b);
+  __shared__ StepArgs sA;
+  apply_body(cta_args(args, b, sA), odd, vb, S);
+}
+
+unsigned shift_plane_ctas() { return kListCTAs; }
+unsigned apply_ctas(const GridDev& g) {
+  const int T = tile_total(g);
+  return (unsigned)(T < 152 * 8 ? T : 152 * 8);
+}
+
+cudaError_t launch_shift_step(const StepArgs& A, int odd, cudaStream_t st) {
+  launch_pdl(k_shift_mark, kListCTAs, kListThreads, st, A);
+  prof_mark("shift.planes", st);
+  launch_pdl(k_shift_sweep, kListCTAs, kListThreads, st, A);
+  prof_mark("shift.sweep", st);
+  launch_pdl(k_shift_apply, apply_ctas(A.g), kAppThreads, st, A, odd);
+  prof_mark("shift.apply", st);
   return cudaGetLastError();
 }
 
-int shift_list_ctas() { return kListCTAs; }
-long long shift_warps_of(const GridDev& g) { return shift_warps(g); }
-dim3 shift_stream_grid_of(const GridDev& g) { return shift_stream_grid(g); }
+cudaError_t launch_shift_grp(const GroupMap* m, const unsigned* n, const StepArgs* a, int odd, cudaStream_t st) {
+  if (n[0]) k_shift_mark_grp<<<n[0], kListThreads, 0, st>>>(m[0], a);
+  prof_mark("group.shift_planes", st);
+  if (n[1]) k_shift_sweep_grp<<<n[1], kListThreads, 0, st>>>(m[1], a);
+  prof_mark("group.shift_sweep", st);
+  if (n[2]) k_shift_apply_grp<<<n[2], kAppThreads, 0, st>>>(m[2], a, odd);
+  prof_mark("group.shift_apply", st);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_shift(const GridDev& g, const double* c_in, const double* e_in, double* c_out, double* e_out,
                          const double* dd, double dd_uniform, uint8_t* state, ShiftScratch sc, SumOut stream_sums,
-                         SumOut sums, bool zero_counters, cudaStream_t st) {
+                         SumOut sums, cudaStream_t st) {
   const long long nw = shift_warps(g);
-  cudaError_t err = cudaSuccess;
-  if (zero_counters) {  // else the caller's tile pass cleared them
-    err = cudaMemsetAsync(sc.counters, 0, 3 * sizeof(int), st);
-    if (err != cudaSuccess) return err;
-    prof_mark("shift.memset", st);
-  }
+  cudaError_t err = cudaMemsetAsync(sc.counters, 0, 3 * sizeof(int), st);
+  if (err != cudaSuccess) return err;
+  prof_mark("shift.memset", st);
   launch_pdl(k_shift_stream, shift_stream_grid(g), dim3(32, 8), st, g, c_in, e_in, c_out, e_out, dd, dd_uniform,
              sc, stream_sums, c_out != c_in);
   prof_mark("shift.stream", st);

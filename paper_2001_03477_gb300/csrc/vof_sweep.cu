@@ -31,6 +31,7 @@
 // (the scarce unit on this part) runs lane-dense over compact lists.
 #include "vof_launch.h"
 #include "vof_sums.cuh"
+#include "vof_sweep.cuh"
 
 namespace vofgb {
 
@@ -50,75 +51,6 @@ __device__ __forceinline__ size_t face_index(int ax, int f, int i, int j, int k,
   if (ax == 0) return ((size_t)k * ny + j) * (nx + 1) + f;
   if (ax == 1) return ((size_t)k * (ny + 1) + f) * nx + i;
   return ((size_t)f * ny + j) * nx + i;
-}
-
-// ---------------------------------------------------------------------------
-// No-op cells.  A cell's c and e come out bit-identical when the 7 cells
-// around it along the sweep axis have the same (c, e) bits, c is exactly 0 or
-// 1 and the cell has not changed earlier in the step: both donors are then
-// pure with the same c, F = c a, both face temperatures equal T, and
-// (G - Theta a) vanishes exactly on both faces.
-// ---------------------------------------------------------------------------
-
-constexpr unsigned kFull = 0xffffffffu;
-constexpr long long kOneBits = 0x3FF0000000000000LL;
-
-__device__ __forceinline__ bool same_bits(double a, double b) { return dbits(a) == dbits(b); }
-__device__ __forceinline__ bool is01(double c) { long long b = dbits(c); return b == 0 || b == kOneBits; }
-
-__device__ __forceinline__ size_t cell_at(const GridDev& g, int x, int y, int z) {
-  return ((size_t)z * g.n[1] + y) * g.n[0] + x;
-}
-
-// energy flux G = T_f (C_pl F + C_pg (a - F)) with T_f = WENO5 of the
-// upwind-ordered stencil
-__device__ __forceinline__ double face_energy_flux(double Cp_l, double Cp_g, double Fv, double a, double t0, double t1,
-                                                double t2, double t3, double t4, bool f32) {
-  const double Tf = f32 ? weno5_f(t0, t1, t2, t3, t4) : weno5_df(t0, t1, t2, t3, t4);
-  // one rounding of (T_f C_pl) F, as in the separate product: a pure cell
-  // (F = a or 0) still gives (T_f C_pl) a or (T_f C_pg) a exactly
-  return fma(Tf * Cp_l, Fv, (Tf * Cp_g) * (a - Fv));
-}
-
-// WY update of one cell from its two faces; returns the clipped volume
-// LAG: the Lagrangian-explicit form (a compile-time choice, so that the
-// Weymouth-Yue kernel carries none of its FP64 arithmetic)
-template <bool ENERGY, bool LAG>
-__device__ __forceinline__ double update_cell(const GridDev& g, size_t id, double c, double e, double T, uint8_t stv,
-                                              double Fl, double Gl, double al, double Fr, double Gr, double ar,
-                                              double* __restrict__ c_out, double* __restrict__ e_out,
-                                              uint8_t* __restrict__ state, double* __restrict__ theta, double& dc,
-                                              double& de) {
-  // Lagrangian-explicit sweeps: the dilatation terms use the cell's own
-  // c and Theta; no frozen state
-  constexpr bool lag = LAG;
-  const bool dirty = !lag && (stv & 1);
-  const bool ccb = dirty ? ((stv >> 1) & 1) != 0 : dgthalf(c);
-  // Weymouth-Yue: cc is 0 or 1, so cc a is a or 0 exactly (no multiply);
-  // Lagrangian explicit: the cell's own c
-  const double lf = lag ? Fl - c * al : (ccb ? Fl - al : Fl);
-  const double rf = lag ? Fr - c * ar : (ccb ? Fr - ar : Fr);
-  const double cn = (c + lf) - rf;
-  double cc2 = cn, clip = 0.0;
-  if (dlt0(cn)) { cc2 = 0.0; clip = cn; }
-  else if (dgt1(cn)) { cc2 = 1.0; clip = cn - 1.0; }
-  c_out[id] = cc2;
-  dc = cc2 - c;
-  de = 0.0;
-  if (ENERGY) {
-    // C_p(cc) with cc in {0, 1} is C_pl or C_pg exactly
-    const double th = lag ? (T * g.Cp_l) * c + (T * g.Cp_g) * (1.0 - c)
-                         : (dirty ? theta[id] : (ccb ? g.Cp_l : g.Cp_g) * T);
-    const double le = Gl - th * al, re = Gr - th * ar;
-    const double en = (e + le) - re;
-    e_out[id] = en;
-    de = en - e;
-    if (!lag && state && !dirty && (!deq(cc2, c) || !deq(en, e))) {
-      state[id] = (uint8_t)(1 | (ccb ? 2 : 0));
-      theta[id] = th;
-    }
-  }
-  return clip;
 }
 
 // ---------------------------------------------------------------------------
@@ -207,21 +139,6 @@ __device__ __forceinline__ void k_stream_col_body(const GridDev& g, const double
   uint32_t* mlist = sc.mlist + sub * (size_t)cap;
   uint32_t* rlist = sc.rlist + sub * (size_t)cap;
   const unsigned lt = (1u << lane) - 1u;
-  if (sc.tiles.quiet && !force_all) {
-    // in place: a warp whose 32 x 32 cells lie in quiet tiles has no work
-    // (lanes 0..15 check its 4 x 4 tiles; t is the same for the warp)
-    bool q = true;
-    const int txi = vb.bx * 4 + (lane & 3), tai = (s0 >> 3) + (lane >> 2);
-    if (lane < 16 && txi * kTile < nx && tai * kTile < s1 && t < n_t) {
-      const int tt = t >> 3;
-      const int ty_ = AX == 1 ? tai : tt, tz_ = AX == 1 ? tt : tai;
-      q = sc.tiles.quiet[((size_t)tz_ * sc.tiles.nt[1] + ty_) * sc.tiles.nt[0] + txi] != 0;
-    }
-    if (__all_sync(kFull, q)) {
-      if (lane == 0) sc.count[sub] = 0;
-      return;
-    }
-  }
   int nlist = 0, nmixed = 0, nrun = 0, nlist_m = 0, nrun_m = 0;
   bool prev_listed = false;  // cell k-1 of this segment listed
   double cm1 = 0.0;          // c of cell s0 - 1
@@ -350,23 +267,6 @@ __device__ __forceinline__ void k_stream_row_body(const GridDev& g, const double
   uint32_t* mlist = sc.mlist + sub * (size_t)cap;
   uint32_t* rlist = sc.rlist + sub * (size_t)cap;
   const unsigned lt = (1u << lane) - 1u;
-  // quiet tiles of the segment (bit l: its l-th tile)
-  unsigned qmask = 0u;
-  if (sc.tiles.quiet && !force_all) {
-    // in place: a warp whose row segment lies in quiet tiles has no work
-    // (lane l checks the l-th tile of the segment)
-    bool q = true;
-    const int txi = (x0 >> 3) + lane;
-    if (txi * kTile < x1) {
-      const int y = row % ny, z = row / ny;
-      q = sc.tiles.quiet[((size_t)(z >> 3) * sc.tiles.nt[1] + (y >> 3)) * sc.tiles.nt[0] + txi] != 0;
-    }
-    if (__all_sync(kFull, q)) {
-      if (lane == 0) sc.count[sub] = 0;
-      return;
-    }
-    qmask = __ballot_sync(kFull, q);
-  }
   int nlist = 0, nmixed = 0, nrun = 0, nlist_m = 0, nrun_m = 0;
   auto ldc = [&](int X) { return __ldg(c_in + rbase + map_idx(X, nx, bcx)); };
   auto lde = [&](int X) { return ENERGY ? __ldg(e_in + rbase + map_idx(X, nx, bcx)) : 0.0; };
@@ -393,20 +293,6 @@ __device__ __forceinline__ void k_stream_row_body(const GridDev& g, const double
   for (; base < x1; base += 32) {
     const double cNN = ldc(base + 64 + lane), eNN = lde(base + 64 + lane);
     const uint8_t stN = lds_(base + 32 + lane);
-    if (((qmask >> ((base - x0) >> 3)) & 0xFu) == 0xFu) {
-      // a chunk of quiet tiles: no-op cells only, none listed or mixed (the
-      // previous chunk's run ends were found looking into this one); the
-      // pipeline moves on
-      const double c31 = __shfl_sync(kFull, cN, 31), e31 = __shfl_sync(kFull, eN, 31);
-      const unsigned eqNN = eqmask(c31, e31, cNN, eNN);
-      mixed_carry = false;
-      cP = cC; eP = eC;
-      cC = cN; eC = eN;
-      cN = cNN; eN = eNN;
-      eqP = eqC; eqC = eqN; eqN = eqNN;
-      stC = stN;
-      continue;
-    }
     const int X = base + lane;
     const bool cell_ok = X < x1;
     const uint8_t stv = cell_ok ? stC : (uint8_t)0;
@@ -486,37 +372,6 @@ k_stream_row(GridDev g, const double* __restrict__ c_in, const double* __restric
 // the only T values kernel F reads back -- and for every listed cell, which
 // kernel U reads.
 // ---------------------------------------------------------------------------
-// PLIC plane (MYC normal, plane constant) of the 3x3x3 stencil centred on
-// position (qx, qy, qz), each index mapped by the boundary conditions.
-// F32: the precision form's FP32 MYC normal (its own instance, so that the
-// FP64 form keeps its register budget); YOUNGS: Youngs' normal instead
-template <bool F32, bool YOUNGS = false>
-__device__ __forceinline__ double4 stencil_plane(const GridDev& g, const double* __restrict__ c_in, int qx, int qy,
-                                                 int qz) {
-  double s[27];
-#pragma unroll
-  for (int oz = 0; oz < 3; ++oz) {
-    const int zz = map_idx(qz + oz - 1, g.n[2], g.bc[2]);
-#pragma unroll
-    for (int oy = 0; oy < 3; ++oy) {
-      const int yy = map_idx(qy + oy - 1, g.n[1], g.bc[1]);
-#pragma unroll
-      for (int ox = 0; ox < 3; ++ox) {
-        const int xx = map_idx(qx + ox - 1, g.n[0], g.bc[0]);
-        s[(oz * 3 + oy) * 3 + ox] = __ldg(c_in + cell_at(g, xx, yy, zz));
-      }
-    }
-  }
-  double m[3];
-  if (YOUNGS) youngs_normal(s, m);
-  else if (F32) myc_normal_f(s, m);
-  else myc_normal(s, m);
-  double4 pl;
-  pl.x = m[0]; pl.y = m[1]; pl.z = m[2];
-  pl.w = plane_alpha(m[0], m[1], m[2], s[13]);
-  return pl;
-}
-
 // Items: the mixed cells (their planes), then with e_in the T items, then,
 // on a zero-gradient sweep axis `ax`, the two ends of every line: where the
 // end cell is mixed, the plane of the ghost donor beyond it (position -1 or
@@ -590,13 +445,6 @@ k_prep(GridDev g, const double* __restrict__ c_in, const double* __restrict__ e_
 constexpr int kFaceThreads = 128;
 constexpr int kFaceCTAs = 152 * 8;
 
-template <int AX>
-__device__ __forceinline__ size_t face_of(const GridDev& g, int f, int x, int y, int z) {
-  if (AX == 0) return ((size_t)z * g.n[1] + y) * (g.n[0] + 1) + f;
-  if (AX == 1) return ((size_t)z * (g.n[1] + 1) + f) * g.n[0] + x;
-  return ((size_t)f * g.n[1] + y) * g.n[0] + x;
-}
-
 template <int AX, bool ENERGY>
 __device__ __forceinline__ void k_faces_body(const GridDev& g, const double* __restrict__ c_in, const double* __restrict__ e_in, const double* __restrict__ uf, double* __restrict__ flux_out, const SweepScratch& sc, int* __restrict__ status, const VB vb) {
   const int nx = g.n[0], ny = g.n[1];
@@ -631,10 +479,11 @@ __device__ __forceinline__ void k_faces_body(const GridDev& g, const double* __r
     const size_t fid = face_of<AX>(g, fr, x, y, z);
     const double a = __ldg(uf + fid) * g.lam;
     double Fv = 0.0, Gv = 0.0;
+    const bool pos = dgt0(a);
+    const double cd = pos ? cw[3] : cw[4];  // donor f-1 (a > 0) or f (a < 0)
+    const bool mixd = is_mixed_b(cd, g);
     if (dnz(a)) {
-      const bool pos = dgt0(a);
-      const double cd = pos ? cw[3] : cw[4];  // donor f-1 (a > 0) or f (a < 0)
-      if (is_mixed_b(cd, g)) {
+      if (mixd) {
         const int dq = pos ? f - 1 : f;  // donor position along the axis
         double4 pl;
         if (bca != 0 && (dq < 0 || dq >= n_ax)) {
@@ -645,32 +494,17 @@ __device__ __forceinline__ void k_faces_body(const GridDev& g, const double* __r
         } else {
           pl = reinterpret_cast<const double4*>(sc.plane)[lbase + stride * map_idx(dq, n_ax, bca)];
         }
-        const double mv[3] = {pl.x, pl.y, pl.z};
-        const double da = fabs(a);
-        if (da > 1.0 && status) atomicOr(status, DEV_CFL);
-        // Weymouth-Yue: the donor slab of width |a|; Lagrangian explicit:
-        // the preimage of width |a| / J, J = 1 + (a_r - a_l) of the donor,
-        // its liquid stretched by J (the width capped at 1)
-        double w = da, J = 1.0;
+        double adl = 0.0, adr = 0.0;
         if (g.le) {
-          const int dk = map_idx(pos ? f - 1 : f, n_ax, bca);
+          const int dk = map_idx(dq, n_ax, bca);
           const int dk1 = (bca == 0 && dk + 1 == n_ax) ? 0 : dk + 1;
-          const double adl = __ldg(uf + face_of<AX>(g, dk, x, y, z)) * g.lam;
-          const double adr = __ldg(uf + face_of<AX>(g, dk1, x, y, z)) * g.lam;
-          J = 1.0 + (adr - adl);
-          if (J > da) {
-            w = da / J;
-          } else {
-            w = 1.0;
-            if (status) atomicOr(status, DEV_CFL);
-          }
+          adl = __ldg(uf + face_of<AX>(g, dk, x, y, z)) * g.lam;
+          adr = __ldg(uf + face_of<AX>(g, dk1, x, y, z)) * g.lam;
         }
-        double vol = g.f32 ? slab_volume_f(mv, pl.w, AX, pos ? 1.0 - w : 0.0, w, cd)
-                           : slab_volume_nn(mv, pl.w, AX, pos ? 1.0 - w : 0.0, w);
-        if (g.le) vol = J * vol;
+        const double vol = donor_volume(g, AX, pl, cd, fabs(a), pos, adl, adr, status);
         Fv = pos ? vol : -vol;
       } else {
-        Fv = cd * a;
+        Fv = pure_flux(cd, a);
       }
       if (ENERGY) {
         // upwind-ordered stencil around the donor
@@ -679,7 +513,9 @@ __device__ __forceinline__ void k_faces_body(const GridDev& g, const double* __r
         const double t2 = pos ? Tw[3] : Tw[4];
         const double t3 = pos ? Tw[4] : Tw[3];
         const double t4 = pos ? Tw[5] : Tw[2];
-        Gv = face_energy_flux(g.Cp_l, g.Cp_g, Fv, a, t0, t1, t2, t3, t4, g.f32 != 0);
+        const double D0 = t1 - t0, D1 = t2 - t1, D2 = t3 - t2, D3 = t4 - t3;
+        const double Tf = face_temperature(g.f32 != 0, t2, D0, D1, D2, D3);
+        Gv = energy_flux(g, Tf, cd, Fv, a);
       }
     }
     sc.F[fid] = Fv;
@@ -765,11 +601,24 @@ __device__ __forceinline__ void update_groups(const GridDev& g, const double* c_
       const double e = ENERGY ? e_in[id] : 0.0;
       const double T = ENERGY ? sc.T[id] : 0.0;
       const uint8_t stv = state ? state[id] : (uint8_t)0;
-      double dc, de;
-      v[kSumClip] += update_cell<ENERGY, LAG>(g, id, c, e, T, stv, Fl, Gl, al, Fr, Gr, ar, c_out, e_out, state,
-                                              theta, dc, de);
-      v[kSumC] += dc;
-      v[kSumE] += de;
+      const bool dirty = !LAG && (stv & 1);
+      const bool cc = dirty ? ((stv >> 1) & 1) != 0 : dgthalf(c);
+      const double2 r = update_c(c, Fl, al, Fr, ar, cc, LAG);
+      c_out[id] = r.x;
+      if (!same_bits(r.x, c) || dnz(r.y)) {
+        v[kSumClip] += r.y;
+        v[kSumC] += r.x - c;
+      }
+      if (ENERGY) {
+        const double th = dirty ? theta[id] : theta_now(g, T, c, cc, LAG);
+        const double en = (e + (Gl - th * al)) - (Gr - th * ar);
+        e_out[id] = en;
+        v[kSumE] += en - e;
+        if (!LAG && state && !dirty && (!deq(r.x, c) || !deq(en, e))) {
+          state[id] = (uint8_t)(1 | (cc ? 2 : 0));
+          theta[id] = th;
+        }
+      }
     }
     __syncthreads();  // pre[] and lst[] are rewritten by the next batch
   }
@@ -786,14 +635,6 @@ __device__ __forceinline__ void k_update_body(const GridDev& g, const double* c_
   else
     update_groups<AX, ENERGY, false>(g, c_in, e_in, c_out, e_out, uf, state, theta, sc, nsub, cap, ngrp, vb, pre,
                                      lst, v);
-  // work counts of this sweep (kernel A's counters are final by now)
-  if (sc.stats && vb.bx == 0 && threadIdx.x == 0) {
-    sc.stats[0] = sc.counters[0];
-    sc.stats[1] = sc.counters[1] + sc.counters[2];
-  }
-  if (sc.mlp_stat && vb.bx == 0 && threadIdx.x == 0) {
-    sc.mlp_stat[0] = sc.counters[3];
-  }
   block_sums(v, sc.sums, vb.bx);
 }
 
@@ -864,7 +705,9 @@ k_energy(GridDev g, const double* __restrict__ c_before, const double* __restric
           v[r + 2] = sT[(pz * TY + py) * TX + px];
         }
         // the fused sweep's face energy flux, bit for bit
-        Gv = face_energy_flux(g.Cp_l, g.Cp_g, Fv, a, v[0], v[1], v[2], v[3], v[4], g.f32 != 0);
+        const double D0 = v[1] - v[0], D1 = v[2] - v[1], D2 = v[3] - v[2], D3 = v[4] - v[3];
+        const double Tf = face_temperature(g.f32 != 0, v[2], D0, D1, D2, D3);
+        Gv = energy_mix(Tf, g.Cp_l, g.Cp_g, Fv, a);
       }
     }
     sG[q] = Gv;
@@ -984,9 +827,6 @@ SweepScratch carve_sweep_scratch(int axis, const GridDev& g, void* ws, SumOut su
   s.list = reinterpret_cast<uint32_t*>(b);      b += al256((size_t)p.nsub * p.cap * 4);
   s.count = reinterpret_cast<int*>(b);          b += al256((size_t)p.nsub * 4);
   s.sums = sums;
-  s.tiles = TileMap{nullptr, {0, 0, 0}};
-  s.stats = nullptr;
-  s.mlp_stat = nullptr;
   s.mlist = reinterpret_cast<uint32_t*>(b);     b += al256((size_t)p.nsub * p.cap * 4);
   s.rlist = reinterpret_cast<uint32_t*>(b);     b += al256((size_t)p.nsub * p.cap * 4);
   s.counters = reinterpret_cast<int*>(b);       b += 256;
@@ -999,8 +839,6 @@ SweepScratch carve_sweep_scratch(int axis, const GridDev& g, void* ws, SumOut su
   s.G = reinterpret_cast<double*>(b);
   return s;
 }
-
-int sweep_blocks(int axis, const GridDev& g) { return (int)sweep_plan(axis, g).gridB; }
 
 template <int AX, bool ENERGY>
 static void launch_ab(const SweepPlan& p, const GridDev& g, const double* c_in, const double* e_in, double* c_out,
@@ -1015,7 +853,7 @@ static void launch_ab(const SweepPlan& p, const GridDev& g, const double* c_in, 
   prof_mark(AX == 0 ? "sweep_x.stream" : (AX == 1 ? "sweep_y.stream" : "sweep_z.stream"), st);
   if (g.mlp == 1) {
     // learned normals of the mixed cells (tensor cores), then their planes
-    launch_mlp_sweep_normals(g, c_in, sc, st);
+    (void)launch_mlp_sweep_normals(g, c_in, false, sc.gmix, sc.counters, sc.plane, st);  // errors: cudaGetLastError()
     if (g.f32) launch_pdl(k_prep<true, 1>, kPlaneCTAs, kPlaneThreads, st, g, c_in, e_in, sc, AX);
     else launch_pdl(k_prep<false, 1>, kPlaneCTAs, kPlaneThreads, st, g, c_in, e_in, sc, AX);
   } else if (g.mlp == 2) {
@@ -1035,14 +873,12 @@ static void launch_ab(const SweepPlan& p, const GridDev& g, const double* c_in, 
 
 cudaError_t launch_sweep(int axis, const GridDev& g, const double* c_in, const double* e_in, double* c_out,
                          double* e_out, const double* uf, uint8_t* state, double* theta, double* flux_out,
-                         SweepScratch sc, bool zero_counters, cudaStream_t st) {
+                         SweepScratch sc, cudaStream_t st) {
   int* status = device_status_ptr();
   const SweepPlan p = sweep_plan(axis, g);
-  if (zero_counters) {  // else the caller's tile pass cleared them
-    const cudaError_t err = cudaMemsetAsync(sc.counters, 0, 4 * sizeof(int), st);
-    if (err != cudaSuccess) return err;
-    prof_mark("sweep.memset", st);
-  }
+  const cudaError_t err = cudaMemsetAsync(sc.counters, 0, 4 * sizeof(int), st);
+  if (err != cudaSuccess) return err;
+  prof_mark("sweep.memset", st);
   if (e_in) {
     if (axis == 0) launch_ab<0, true>(p, g, c_in, e_in, c_out, e_out, uf, state, theta, flux_out, sc, status, st);
     else if (axis == 1) launch_ab<1, true>(p, g, c_in, e_in, c_out, e_out, uf, state, theta, flux_out, sc, status, st);
@@ -1055,73 +891,6 @@ cudaError_t launch_sweep(int axis, const GridDev& g, const double* c_in, const d
   }
   return cudaGetLastError();
 }
-
-// ---------------------------------------------------------------------------
-// Grouped sweep kernels: every box of a batch in one launch (in place, with
-// energy, no exported fluxes); each CTA takes its box's arguments.
-// ---------------------------------------------------------------------------
-template <int AX>
-__global__ void __launch_bounds__(256) k_stream_grp(GroupMap m, const SweepArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ SweepArgs sA;
-  const SweepArgs& A = cta_args(args, b, sA);
-  if (AX == 0)
-    k_stream_row_body<true>(A.g, A.c, A.e, A.c, A.e, A.state, A.sc, 0, A.cap, 0, vb);
-  else
-    k_stream_col_body<AX == 0 ? 1 : AX, true>(A.g, A.c, A.e, A.c, A.e, A.state, A.sc, 0, A.cap, 0, vb);
-}
-template <bool F32, int NRM>
-__global__ void __launch_bounds__(kPlaneThreads) k_prep_grp(GroupMap m, const SweepArgs* __restrict__ args, int ax) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ SweepArgs sA;
-  const SweepArgs& A = cta_args(args, b, sA);
-  k_prep_body<F32, NRM>(A.g, A.c, A.e, A.sc, ax, vb);
-}
-template <int AX>
-__global__ void __launch_bounds__(kFaceThreads) k_faces_grp(GroupMap m, const SweepArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ SweepArgs sA;
-  const SweepArgs& A = cta_args(args, b, sA);
-  k_faces_body<AX, true>(A.g, A.c, A.e, A.uf, nullptr, A.sc, A.status, vb);
-}
-template <int AX>
-__global__ void __launch_bounds__(256) k_update_grp(GroupMap m, const SweepArgs* __restrict__ args) {
-  unsigned b;
-  const VB vb = vb_group(m, b);
-  __shared__ SweepArgs sA;
-  const SweepArgs& A = cta_args(args, b, sA);
-  k_update_body<AX, true>(A.g, A.c, A.e, A.c, A.e, A.uf, A.state, A.theta, A.sc, A.nsub, A.cap, A.ngrp, vb);
-}
-
-template <int AX>
-static void launch_sweep_grp_t(int f32, int youngs, const GroupMap* m, const SweepArgs* a, const unsigned* n,
-                               cudaStream_t st) {
-  if (n[0]) k_stream_grp<AX><<<n[0], dim3(32, 8), 0, st>>>(m[0], a);
-  prof_mark("group.stream", st);
-  if (n[1]) {
-    if (youngs) k_prep_grp<false, 2><<<n[1], kPlaneThreads, 0, st>>>(m[1], a, AX);
-    else if (f32) k_prep_grp<true, 0><<<n[1], kPlaneThreads, 0, st>>>(m[1], a, AX);
-    else k_prep_grp<false, 0><<<n[1], kPlaneThreads, 0, st>>>(m[1], a, AX);
-  }
-  prof_mark("group.prep", st);
-  if (n[2]) k_faces_grp<AX><<<n[2], kFaceThreads, 0, st>>>(m[2], a);
-  prof_mark("group.faces", st);
-  if (n[3]) k_update_grp<AX><<<n[3], 256, 0, st>>>(m[3], a);
-  prof_mark("group.update", st);
-}
-
-cudaError_t launch_sweep_grp(int axis, int f32, int youngs, const GroupMap* maps, const SweepArgs* a,
-                             const unsigned* ctas, cudaStream_t st) {
-  if (axis == 0) launch_sweep_grp_t<0>(f32, youngs, maps, a, ctas, st);
-  else if (axis == 1) launch_sweep_grp_t<1>(f32, youngs, maps, a, ctas, st);
-  else launch_sweep_grp_t<2>(f32, youngs, maps, a, ctas, st);
-  return cudaGetLastError();
-}
-
-int prep_ctas() { return kPlaneCTAs; }
 
 cudaError_t launch_energy(int axis, const GridDev& g, const double* c_before, const double* c_after,
                           const double* e_in, double* e_out, const double* F, const double* uf, uint8_t* state,

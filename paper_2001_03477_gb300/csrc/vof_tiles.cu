@@ -1,6 +1,7 @@
 // vof_tiles.cu -- the tile pass at the start of an in-place time step: which
 // 8^3 tiles are quiet (no cell of them can change in this step, so the
-// streaming kernels skip them), and the sums of c and e over the grid.
+// step's kernels skip them), the list of the others, the mixed cells the first
+// sweep starts from, and the quiet tiles' shares of the sums of c and e.
 //
 // A tile is uniform when all its cells hold the same (c, e) bits; it is quiet
 // when it is uniform with c exactly 0 or 1 and every one of its 26 neighbour
@@ -27,7 +28,7 @@ constexpr unsigned kFullT = 0xffffffffu;
 // and one along z (the threads walk its 8 planes).  Each tile's flag and
 // reference values; integer compares only (no FP64 work and nothing kept
 // beyond registers), so the pass streams c and e at the memory's rate.
-__device__ __forceinline__ void k_tiles_body(const GridDev& g, const double* __restrict__ c, const double* __restrict__ e, const TileScratch& ts, int ntx, int nty, uint8_t* __restrict__ state, int* __restrict__ counters, const VB vb) {
+__device__ __forceinline__ void k_tiles_body(const GridDev& g, const double* __restrict__ c, const double* __restrict__ e, const TileScratch& ts, int ntx, int nty, int* __restrict__ counters, int* __restrict__ stats, const VB vb) {
   __shared__ unsigned uni_w[8];
   __shared__ double ref[4][2];
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -45,9 +46,11 @@ __device__ __forceinline__ void k_tiles_body(const GridDev& g, const double* __r
     const size_t id = ((size_t)z * ny + y) * nx + x;
     cb[zi] = ok ? dbits(__ldg(c + id)) : 0;
     eb[zi] = ok ? dbits(__ldg(e + id)) : 0;
-    if (ok && state) state[id] = 0;  // the step's frozen-state flags start clear
   }
-  if (counters && (vb.bx | vb.by | vb.bz) == 0 && ty == 0 && tx < kStepCounters) counters[tx] = 0;
+  if ((vb.bx | vb.by | vb.bz) == 0 && ty == 0 && tx < kStepCounters) {
+    counters[tx] = 0;
+    if (tx == 0) stats[8] = 0;  // receivers, counted by the step's last kernel
+  }
   // reference of each tile: its first cell, which this CTA's thread
   // (8 j, 0) holds as its first value
   if (ty == 0 && (tx & 7) == 0 && tile_ok) {
@@ -75,11 +78,9 @@ __device__ __forceinline__ void k_tiles_body(const GridDev& g, const double* __r
   }
 }
 
-__global__ void __launch_bounds__(256)
-k_tiles(GridDev g, const double* __restrict__ c, const double* __restrict__ e, TileScratch ts, int ntx, int nty,
-        uint8_t* state, int* counters) {
+__global__ void __launch_bounds__(256) k_tiles(StepArgs A) {
   pdl_wait();
-  k_tiles_body(g, c, e, ts, ntx, nty, state, counters, vb_self());
+  k_tiles_body(A.g, A.c, A.e, A.ts, A.nt[0], A.nt[1], A.cnt, A.stats, vb_self());
 }
 
 // neighbour tile index along one axis: -1 when it lies beyond a
@@ -89,33 +90,6 @@ __device__ __forceinline__ int tile_nb(int p, int n, int bc) {
   if (p < 0) return bc ? -1 : p + n;
   if (p >= n) return bc ? -1 : p - n;
   return p;
-}
-
-// Sums of c and e over a tile whose cells differ: each lane its cells
-// q = lane + 32 r (x fastest within the tile) in order, then the lanes in a
-// fixed tree; lane 0 holds the result.  Not inlined and called under a
-// warp-uniform branch, so that uniform tiles issue none of its FP64 adds
-// (an FP64 instruction costs its full issue time whatever its active lanes).
-__device__ __noinline__ double2 tile_cell_sums(int nx, int ny, int nz, const double* __restrict__ c,
-                                               const double* __restrict__ e, int x0, int y0, int z0) {
-  const int lane = threadIdx.x & 31;
-  double sc = 0.0, se = 0.0;
-#pragma unroll 4
-  for (int r = 0; r < kTile * kTile * kTile / 32; ++r) {
-    const int q = lane + 32 * r;
-    const int x = x0 + (q & 7), y = y0 + ((q >> 3) & 7), z = z0 + (q >> 6);
-    if (x < nx && y < ny && z < nz) {
-      const size_t id = ((size_t)z * ny + y) * nx + x;
-      sc += __ldg(c + id);
-      se += __ldg(e + id);
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sc += __shfl_down_sync(kFullT, sc, o);
-    se += __shfl_down_sync(kFullT, se, o);
-  }
-  return make_double2(sc, se);
 }
 
 // n x v for the bit pattern v (the same for every lane of the warp): a
@@ -134,17 +108,19 @@ __device__ __forceinline__ double times_cells(int n, long long v) {
 }
 
 // One warp per tile: quiet flag (lanes 0..26 check the tile and its 26
-// neighbours at once) and the tile's sum row -- a uniform tile's is
-// (cells) x value, another's the sum of its cells.  Rows are placed at
-// (tz nty + ty) 4 ceil(ntx / 4) + tx; the slots past the last tile of an
-// x-row of tiles hold zero rows.
-__device__ __forceinline__ void k_quiet_body(const GridDev& g, const double* __restrict__ c, const double* __restrict__ e, const TileScratch& ts, int ntx, int nty, int ntz, const SumOut& sums, const VB vb) {
+// neighbours at once).  A quiet tile's sum row is (cells) x value; any other
+// tile joins the active list, and its mixed cells the first stage's list
+// (one atomic per tile and list; both orders vary from run to run).
+__device__ __forceinline__ void k_quiet_body(const StepArgs& A, const VB vb) {
+  const GridDev& g = A.g;
+  const TileScratch& ts = A.ts;
+  const int ntx = A.nt[0], nty = A.nt[1], ntz = A.nt[2];
   const long long nt = (long long)ntx * nty * ntz;
   const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
   const long long wpb = blockDim.x >> 5;
-  const int rstride = 4 * ((ntx + 3) / 4);
   // tile t goes to CTA t mod gx: neighbouring tiles (the interface's, whose
-  // sums take FP64 adds) spread over the SMs
+  // cells are read) spread over the SMs
   for (long long t = vb.bx + (long long)vb.gx * (threadIdx.x >> 5); t < nt; t += (long long)vb.gx * wpb) {
     const int tx = (int)(t % ntx), ty = (int)((t / ntx) % nty), tz = (int)(t / ((long long)ntx * nty));
     // lane o < 27: the tile at offset (o % 3 - 1, o / 3 % 3 - 1, o / 9 - 1);
@@ -166,44 +142,48 @@ __device__ __forceinline__ void k_quiet_body(const GridDev& g, const double* __r
     const long long cr = __shfl_sync(kFullT, nb_c, 13), er = __shfl_sync(kFullT, nb_e, 13);
     const bool same = !nb_ok || (nb_uni && nb_c == cr && nb_e == er);
     const bool all = __all_sync(kFullT, lane >= 27 || same);
-    const bool q = uni && (cr == 0 || cr == 0x3FF0000000000000LL) && all;
+    const bool pure = cr == 0 || cr == 0x3FF0000000000000LL;
+    const bool q = A.usable && uni && pure && all;
+    const int x0 = tx * kTile, y0 = ty * kTile, z0 = tz * kTile;
     if (lane == 0) ts.quiet[t] = q ? 1 : 0;
-    if (!sums.partials) continue;
-    double sc, se;
-    if (uni) {
-      const int cx = min(kTile, g.n[0] - tx * kTile), cy = min(kTile, g.n[1] - ty * kTile),
-                cz = min(kTile, g.n[2] - tz * kTile);
-      const int n = cx * cy * cz;
-      sc = times_cells(n, cr);
-      se = times_cells(n, er);
-    } else {
-      const double2 s2 = tile_cell_sums(g.n[0], g.n[1], g.n[2], c, e, tx * kTile, ty * kTile, tz * kTile);
-      sc = s2.x;
-      se = s2.y;
+    if (q) {
+      const int n = min(kTile, g.n[0] - x0) * min(kTile, g.n[1] - y0) * min(kTile, g.n[2] - z0);
+      const double sc = times_cells(n, cr), se = times_cells(n, er);
+      if (lane < kNSums) A.rows[(size_t)t * kNSums + lane] = lane == kSumC ? sc : (lane == kSumE ? se : 0.0);
+      continue;
     }
-    const size_t slot = ((size_t)tz * nty + ty) * rstride + tx;
-    if (lane == 0) {
-      double* row = sums.partials + slot * sums.stride;
-      row[kSumC] = sc;
-      row[kSumE] = se;
-      row[kSumClip] = 0.0;
-      row[kSumShDc] = 0.0;
-      row[kSumUnpl] = 0.0;
-      row[kSumShDe] = 0.0;
+    if (lane == 0) A.tlist[atomicAdd(A.cnt + 14, 1)] = (uint32_t)t;
+    if (uni && pure) continue;  // no mixed cell
+    unsigned mine = 0u;  // bit r: this lane's r-th cell is mixed
+#pragma unroll
+    for (int r = 0; r < kTile * kTile * kTile / 32; ++r) {
+      const int o = lane + 32 * r, x = x0 + (o & 7), y = y0 + ((o >> 3) & 7), z = z0 + (o >> 6);
+      if (x < g.n[0] && y < g.n[1] && z < g.n[2] &&
+          is_mixed_b(__ldg(A.c + ((size_t)z * g.n[1] + y) * g.n[0] + x), g))
+        mine |= 1u << r;
     }
-    if (tx == ntx - 1 && lane >= 1 && lane < rstride - ntx + 1) {
-      // zero rows of the slots past the row's last tile
-      double* row = sums.partials + (slot + lane) * sums.stride;
-      for (int k = 0; k < kNSums; ++k) row[k] = 0.0;
+    const int k = __popc(mine);
+    const int total = __reduce_add_sync(kFullT, k);
+    if (total == 0) continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(A.cnt + 0, total);
+    base = __shfl_sync(kFullT, base, 0);
+#pragma unroll 1
+    for (int r = 0; r < kTile * kTile * kTile / 32; ++r) {
+      const unsigned m = __ballot_sync(kFullT, (mine >> r) & 1u);
+      if ((mine >> r) & 1u) {
+        const int o = lane + 32 * r;
+        A.list[0][base + __popc(m & lt)] =
+            (uint32_t)(((size_t)(z0 + (o >> 6)) * g.n[1] + y0 + ((o >> 3) & 7)) * g.n[0] + x0 + (o & 7));
+      }
+      base += __popc(m);
     }
   }
 }
 
-__global__ void __launch_bounds__(256)
-k_quiet(GridDev g, const double* __restrict__ c, const double* __restrict__ e, TileScratch ts, int ntx, int nty,
-        int ntz, SumOut sums) {
+__global__ void __launch_bounds__(256) k_quiet(StepArgs A) {
   pdl_wait();
-  k_quiet_body(g, c, e, ts, ntx, nty, ntz, sums, vb_self());
+  k_quiet_body(A, vb_self());
 }
 
 size_t al256t(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -222,11 +202,10 @@ bool tiles_usable(const GridDev& g) {
   return true;
 }
 
-// sum rows of the tile pass: 4 per CTA (one per tile slot along x)
-int tile_blocks(const GridDev& g) {
+int tile_total(const GridDev& g) {
   int nt[3];
   tile_counts(g, nt);
-  return ((nt[0] + 3) / 4) * nt[1] * nt[2] * 4;
+  return nt[0] * nt[1] * nt[2];
 }
 
 size_t tile_scratch_bytes(const GridDev& g) {
@@ -249,22 +228,21 @@ TileScratch carve_tile_scratch(const GridDev& g, void* ws) {
   return s;
 }
 
-__global__ void __launch_bounds__(256) k_tiles_grp(GroupMap m, const TileArgs* __restrict__ args) {
+__global__ void __launch_bounds__(256) k_tiles_grp(GroupMap m, const StepArgs* __restrict__ args) {
   unsigned b;
   const VB vb = vb_group(m, b);
-  __shared__ TileArgs sA;
-  const TileArgs& A = cta_args(args, b, sA);
-  k_tiles_body(A.g, A.c, A.e, A.ts, A.nt[0], A.nt[1], A.state, A.counters, vb);
+  __shared__ StepArgs sA;
+  const StepArgs& A = cta_args(args, b, sA);
+  k_tiles_body(A.g, A.c, A.e, A.ts, A.nt[0], A.nt[1], A.cnt, A.stats, vb);
 }
-__global__ void __launch_bounds__(256) k_quiet_grp(GroupMap m, const TileArgs* __restrict__ args) {
+__global__ void __launch_bounds__(256) k_quiet_grp(GroupMap m, const StepArgs* __restrict__ args) {
   unsigned b;
   const VB vb = vb_group(m, b);
-  __shared__ TileArgs sA;
-  const TileArgs& A = cta_args(args, b, sA);
-  k_quiet_body(A.g, A.c, A.e, A.ts, A.nt[0], A.nt[1], A.nt[2], A.sums, vb);
+  __shared__ StepArgs sA;
+  k_quiet_body(cta_args(args, b, sA), vb);
 }
 
-cudaError_t launch_tiles_grp(const GroupMap& mt, const GroupMap& mq, const TileArgs* a, unsigned ct, unsigned cq,
+cudaError_t launch_tiles_grp(const GroupMap& mt, const GroupMap& mq, const StepArgs* a, unsigned ct, unsigned cq,
                              cudaStream_t st) {
   if (ct) k_tiles_grp<<<ct, dim3(32, 8), 0, st>>>(mt, a);
   prof_mark("group.tiles", st);
@@ -273,22 +251,16 @@ cudaError_t launch_tiles_grp(const GroupMap& mt, const GroupMap& mq, const TileA
   return cudaGetLastError();
 }
 
-unsigned quiet_blocks(const GridDev& g) {
-  int nt[3];
-  tile_counts(g, nt);
-  const long long T = (long long)nt[0] * nt[1] * nt[2];
+unsigned quiet_ctas(const GridDev& g) {
+  const long long T = tile_total(g);
   // one warp per tile, 8 per CTA
   return (unsigned)((T + 7) / 8 < 152 * 8 ? (T + 7) / 8 : 152 * 8);
 }
 
-cudaError_t launch_tiles(const GridDev& g, const double* c, const double* e, TileScratch ts, SumOut sums,
-                         uint8_t* state, int* counters, cudaStream_t st) {
-  int nt[3];
-  tile_counts(g, nt);
-  launch_pdl(k_tiles, dim3((unsigned)((nt[0] + 3) / 4), (unsigned)nt[1], (unsigned)nt[2]), dim3(32, 8), st,
-             g, c, e, ts, nt[0], nt[1], state, counters);
+cudaError_t launch_tiles(const StepArgs& A, cudaStream_t st) {
+  launch_pdl(k_tiles, dim3((unsigned)((A.nt[0] + 3) / 4), (unsigned)A.nt[1], (unsigned)A.nt[2]), dim3(32, 8), st, A);
   prof_mark("tiles", st);
-  launch_pdl(k_quiet, quiet_blocks(g), 256, st, g, c, e, ts, nt[0], nt[1], nt[2], sums);
+  launch_pdl(k_quiet, quiet_ctas(A.g), 256, st, A);
   prof_mark("tiles.quiet", st);
   return cudaGetLastError();
 }
