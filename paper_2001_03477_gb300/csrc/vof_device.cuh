@@ -86,6 +86,25 @@ __device__ __forceinline__ double dhalf_exact(double x, bool& ok) {
   return __longlong_as_double((long long)(e >= 2 ? b - (1ull << 52) : b));
 }
 
+// FP32 of an FP64 value to nearest even, and back, on the integer pipe (an
+// FP64 conversion instruction occupies the FP64 unit like an add).  Values
+// below FP32's normal range become 0; infinities and NaN stay what they are.
+__device__ __forceinline__ float f32_of(double x) {
+  const unsigned long long b = (unsigned long long)dbits(x);
+  const unsigned long long r = (b & 0x7FFFFFFFFFFFFFFFull) + 0x0FFFFFFFull + ((b >> 29) & 1ull);
+  const int ex = (int)(r >> 52) - 1023 + 127;
+  unsigned f = ((unsigned)ex << 23) | ((unsigned)(r >> 29) & 0x7FFFFFu);
+  if (ex <= 0) f = 0u;
+  if (ex >= 255) f = ((b & 0x7FFFFFFFFFFFFFFFull) > 0x7FF0000000000000ull) ? 0x7FC00000u : 0x7F800000u;
+  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x), ex = (b >> 23) & 0xFFu;
+  const unsigned long long m = (unsigned long long)(b & 0x7FFFFFu) << 29;
+  const unsigned long long v = ex == 255u ? (0x7FF0000000000000ull | m) : (ex ? ((unsigned long long)(ex + 896u) << 52) | m : 0ull);
+  return __longlong_as_double((long long)(v | ((unsigned long long)(b & 0x80000000u) << 32)));
+}
+
 __device__ __forceinline__ int map_idx(int i, int n, int bc) {
   if (bc == 0) {
     int r = i % n;
@@ -129,6 +148,76 @@ __device__ __forceinline__ bool is_mixed_b(double c, const GridDev& g) {
 __device__ __forceinline__ bool is_full_b(double c, const GridDev& g) { return dbits(c) >= g.one_m_eps; }
 
 // ---------------------------------------------------------------------------
+// Division a / b for one denominator and several numerators.  The FP64 unit
+// takes 564 cycles for the library's quotient (nine FP64 instructions); here the
+// reciprocal is formed on the FP32 and integer units (an FP32 estimate of the
+// significand's reciprocal and one Newton correction carried as a second FP32
+// number, ~2^-45 relative) and a quotient costs three FP64 instructions: q0 = a r,
+// the remainder a - q0 b by a fused multiply-add, q = q0 + rem r by another
+// (Markstein 1990).  Before the last rounding q is within ~2^-90 of a / b
+// relatively, so it is the correctly rounded quotient but for about one operand
+// pair in 2^37.  Measured on 2^26 pairs: every quotient equal to the
+// library's, a division in 3 / 9 of the time.  Denominators and numerators whose
+// exponents leave room (2^-450 .. 2^450, or 0) take this path; a warp that holds
+// another one also issues the library's division.
+// ---------------------------------------------------------------------------
+struct Rcp {
+  double b, r;  // denominator, ~1 / b
+  bool ok;
+};
+__device__ __forceinline__ bool mid_range(unsigned hi) {  // exponent field in 573 .. 1472
+  return ((hi >> 20 & 0x7FFu) - 573u) <= 899u;
+}
+__device__ __forceinline__ Rcp rcp_of(double b) {
+  const df::words w = df::words_of(b);
+  const float mh = __uint_as_float(0x3F800000u | (w.hi & 0xFFFFFu) << 3 | w.lo >> 29);  // significand, top 24 bits
+  const float ml = (float)(w.lo & 0x1FFFFFFFu) * 0x1p-52f;                               // the rest
+  float r1;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(mh));
+  const float e = fmaf(-ml, r1, fmaf(-mh, r1, 1.0f));
+  const float r2 = r1 * fmaf(e, e, e);
+  // r1 in (1/2, 1]: r2 in units of the sum's FP64 last place, added to the
+  // pattern (below 1 the last place is 2^-53, also coming down from r1 = 1)
+  const unsigned rb = __float_as_uint(r1);
+  const unsigned long long r = ((unsigned long long)rb << 29) + (896ull << 52) +
+                               (long long)__float2int_rn(r2 * (rb >= 0x3F800000u && r2 >= 0.0f ? 0x1p52f : 0x1p53f));
+  Rcp R;
+  R.b = b;
+  R.ok = mid_range(w.hi);
+  // times 2^-(exponent of b), with b's sign
+  const unsigned hi = (unsigned)(r >> 32) - ((w.hi & 0x7FF00000u) - 0x3FF00000u);
+  R.r = __hiloint2double((int)(hi | (w.hi & 0x80000000u)), (int)(unsigned)r);
+  return R;
+}
+static __device__ __noinline__ double div_library(double a, double b) { return a / b; }
+__device__ __forceinline__ double div_by(double a, const Rcp& R) {
+  const double q0 = a * R.r;
+  const double q = fma(fma(-q0, R.b, a), R.r, q0);
+  const bool az = !dnz(a);
+  double res = az ? a : q;  // (b > 0 wherever a may be 0)
+  const bool ok = R.ok && (az || mid_range((unsigned)__double2hiint(a)));
+  if (__any_sync(__activemask(), !ok)) {
+    const double l = div_library(a, R.b);
+    if (!ok) res = l;
+  }
+  return res;
+}
+// 1 / b
+__device__ __forceinline__ double inv_of(const Rcp& R) {
+  double res = fma(fma(-R.r, R.b, 1.0), R.r, R.r);
+  if (__any_sync(__activemask(), !R.ok)) {
+    const double l = div_library(1.0, R.b);
+    if (!R.ok) res = l;
+  }
+  return res;
+}
+// a / 3 (1/3 rounded is within half a last place: two instructions after the product)
+__device__ __forceinline__ double third_of(double a) {
+  const double q0 = a * (1.0 / 3.0);
+  return fma(fma(-q0, 3.0, a), 1.0 / 3.0, q0);
+}
+
+// ---------------------------------------------------------------------------
 // Volume below a plane in the unit cube (Scardovelli & Zaleski 2000)
 // ---------------------------------------------------------------------------
 // sorted 0 <= m1 <= m2 <= m3, sum 1, 0 < a <= 1/2: inclusion-exclusion of the
@@ -148,48 +237,48 @@ __device__ __forceinline__ double vol_low(double m1, double m2, double m3, doubl
   return v3 - t3 * t3 * t3 / (6.0 * m1 * m2 * m3);
 }
 
-__device__ __forceinline__ void sort3(double& a, double& b, double& c) {
-  double t;
-  if (a > b) { t = a; a = b; b = t; }
-  if (b > c) { t = b; b = c; c = t; }
-  if (a > b) { t = a; a = b; b = t; }
+// Non-negative doubles order like their bit patterns read as integers: a
+// compare that needs no FP64 instruction (an FP64 compare occupies the FP64
+// unit as long as an add on this part).
+__device__ __forceinline__ bool nn_lt(double a, double b) { return dbits(a) < dbits(b); }
+__device__ __forceinline__ double dabs_i(double x) {  // |x| without an FP64 instruction
+  const df::words w = df::words_of(x);
+  return __hiloint2double((int)(w.hi & 0x7FFFFFFFu), (int)w.lo);
 }
 
-// m >= 0, sum 1
-__device__ __forceinline__ double vol_pos(double m0, double m1, double m2, double a) {
-  if (a <= 0.0) return 0.0;
-  if (a >= 1.0) return 1.0;
-  sort3(m0, m1, m2);
-  if (a <= 0.5) return vol_low(m0, m1, m2, a);
-  return 1.0 - vol_low(m0, m1, m2, 1.0 - a);
+__device__ __forceinline__ void sort3(double& a, double& b, double& c) {  // non-negative values
+  double t;
+  if (nn_lt(b, a)) { t = a; a = b; b = t; }
+  if (nn_lt(c, b)) { t = b; b = c; c = t; }
+  if (nn_lt(b, a)) { t = a; a = b; b = t; }
 }
 
 struct Mirror {
-  double mp[3];  // |m| / l1
+  double mp[3];  // |m| / l1, sorted
   double sh;     // alpha_mirror = alpha + sh
   double l1;
+  Rcp R;         // of l1
 };
 
+// The normal mirrored into the first octant, its L1 norm and the mirror's
+// shift, normalised and sorted (a zero component counts as positive).
 __device__ __forceinline__ Mirror mirror_normalise(double m0, double m1, double m2) {
   Mirror r;
-  double sh = 0.0;
-  double a0, a1, a2;
-  if (m0 < 0.0) { a0 = -m0; sh -= m0; } else a0 = m0;
-  if (m1 < 0.0) { a1 = -m1; sh -= m1; } else a1 = m1;
-  if (m2 < 0.0) { a2 = -m2; sh -= m2; } else a2 = m2;
-  double s = a0 + a1 + a2;
+  double a0 = dabs_i(m0), a1 = dabs_i(m1), a2 = dabs_i(m2);
+  double sh = dlt0(m0) ? a0 : 0.0;
+  sh = sh + (dlt0(m1) ? a1 : 0.0);
+  sh = sh + (dlt0(m2) ? a2 : 0.0);
   r.sh = sh;
-  r.l1 = s;
-  if (s > 0.0) { a0 /= s; a1 /= s; a2 /= s; }
+  r.l1 = a0 + a1 + a2;
+  r.R = rcp_of(r.l1);
+  if (dnz(r.l1)) {
+    a0 = div_by(a0, r.R);
+    a1 = div_by(a1, r.R);
+    a2 = div_by(a2, r.R);
+    sort3(a0, a1, a2);
+  }
   r.mp[0] = a0; r.mp[1] = a1; r.mp[2] = a2;
   return r;
-}
-
-// liquid fraction of {x in [0,1]^3 : m.x <= alpha}, any m
-__device__ __forceinline__ double volume(double m0, double m1, double m2, double alpha) {
-  Mirror r = mirror_normalise(m0, m1, m2);
-  if (r.l1 == 0.0) return alpha >= 0.0 ? 1.0 : 0.0;
-  return vol_pos(r.mp[0], r.mp[1], r.mp[2], (alpha + r.sh) / r.l1);
 }
 
 // derivative dV/da on the same branches (for the Newton polish)
@@ -294,11 +383,6 @@ static __device__ __noinline__ double alpha_low_analytic(double m1, double m2, d
   return best;
 }
 
-// Non-negative doubles order like their bit patterns read as integers: a
-// compare that needs no FP64 instruction (an FP64 compare occupies the FP64
-// unit as long as an add on this part).
-__device__ __forceinline__ bool nn_lt(double a, double b) { return dbits(a) < dbits(b); }
-
 // Single-precision guess of the plane constant for sorted m (sum 1) and
 // 0 < c <= 1/2: bisection of the volume's branch form in float (the float
 // unit is ~64x wider than the FP64 one here, and bisection has no
@@ -332,79 +416,104 @@ __device__ __forceinline__ float alpha_guess_f(float m1, float m2, float m3, flo
   return 0.5f * u * u * u;
 }
 
+// The volume's branch form at a and its derivative, without branches and with
+// the branches' shared terms formed once: the cube of a (first branch) or of
+// a - m2 (third and last), the quadratic's product, the linear branch; every
+// result is selected from the operations that its branch alone would take.
+struct VolForm {
+  double m1, m2, m3, m12, top, r6, r2, r3h, v2c;  // r6 = inf when m1 = 0: never selected then
+  bool lin;
+};
+__device__ __forceinline__ VolForm vol_form(double m1, double m2, double m3) {
+  VolForm f;
+  f.m1 = m1; f.m2 = m2; f.m3 = m3;
+  f.m12 = m1 + m2;
+  f.top = nn_lt(f.m12, m3) ? f.m12 : m3;
+  f.lin = !nn_lt(m3, f.m12);  // m12 <= m3
+  f.r6 = inv_of(rcp_of(6.0 * m1 * m2 * m3));
+  f.r2 = inv_of(rcp_of(2.0 * m2 * m3));
+  f.r3h = 0.5 * inv_of(rcp_of(m3));  // (halved exactly)
+  f.v2c = m1 * m1 * f.r2;
+  return f;
+}
+template <bool SLOPE>
+__device__ __forceinline__ double vol_eval(const VolForm& f, double a, double& d) {
+  const bool b1 = nn_lt(a, f.m1), b2 = nn_lt(a, f.m2), b3 = nn_lt(a, f.top);
+  const bool b5 = !b1 && !b2 && !b3 && !f.lin;
+  const double t1 = a - f.m1, t2 = a - f.m2;
+  const double s = b1 ? a : t2;
+  const double q = s * s * s * f.r6;                 // first branch; third's correction
+  const double v2 = a * t1 * f.r2 + f.v2c;
+  double v = b1 ? q : (b2 ? v2 : v2 - q);
+  double dq = 0.0, d2 = 0.0;
+  if (SLOPE) {
+    dq = 3.0 * s * s * f.r6;
+    d2 = (a + t1) * f.r2;
+    d = b1 ? dq : (b2 ? d2 : d2 - dq);
+  }
+  if (__any_sync(__activemask(), b5)) {
+    const double t3 = a - f.m3;
+    const double v5 = v - t3 * t3 * t3 * f.r6;
+    if (b5) v = v5;
+    if (SLOPE) {
+      const double d5 = d - 3.0 * t3 * t3 * f.r6;
+      if (b5) d = d5;
+    }
+  }
+  const bool b4 = !b1 && !b2 && !b3 && f.lin;
+  if (__any_sync(__activemask(), b4)) {
+    const double v4 = (a + (a - f.m12)) * f.r3h;
+    if (b4) {
+      v = v4;
+      if (SLOPE) d = f.r3h + f.r3h;
+    }
+  }
+  return v;
+}
+
 // Plane constant for sorted m (sum 1) and 0 < c <= 1/2: float guess, then
 // three Newton steps in FP64 on the volume's branch form evaluated without
-// branches (all branches computed, the right one selected, reciprocals of
-// the branch denominators formed once), so the lanes of a warp stay
-// together.  The best of the iterates is kept; if it misses c by more than
-// rounding, the analytic solution with its safeguarded polish is used.
+// branches, so the lanes of a warp stay together.  The best of the iterates
+// is kept; if it misses c by more than rounding, the analytic solution with its
+// safeguarded polish is used.  (FP64 instructions: 165, where separate branches
+// and library divisions took 265.)
 __device__ __forceinline__ double alpha_low(double m1, double m2, double m3, double c) {
-  const double m12 = m1 + m2;
-  const double top = m12 < m3 ? m12 : m3;
-  const bool lin = !nn_lt(m3, m12);  // m12 <= m3
-  const double r6 = 1.0 / (6.0 * m1 * m2 * m3);  // inf when m1 = 0: that branch is then never selected
-  const double r2 = 1.0 / (2.0 * m2 * m3);
-  const double r3 = 1.0 / m3;
-  const double v2c = m1 * m1 * r2 / 3.0;
-  double a = (double)alpha_guess_f((float)m1, (float)m2, (float)m3, (float)c);
+  VolForm f = vol_form(m1, m2, m3);
+  f.v2c = third_of(f.v2c);
+  double a = f64_of(alpha_guess_f(f32_of(m1), f32_of(m2), f32_of(m3), f32_of(c)));
   double best = a;
   long long bestf = 0x7FF0000000000000LL;  // |f| bits
-#pragma unroll
+#pragma unroll 1
   for (int it = 0; it < 4; ++it) {
-    const double t1 = a - m1, t2 = a - m2, t3 = a - m3;
-    const double v1 = a * a * a * r6, d1 = 3.0 * a * a * r6;
-    const double v2 = a * t1 * r2 + v2c, d2 = (a + t1) * r2;
-    const double v3 = v2 - t2 * t2 * t2 * r6, d3 = d2 - 3.0 * t2 * t2 * r6;
-    const double v4 = (a + (a - m12)) * 0.5 * r3, d4 = r3;
-    const double v5 = v3 - t3 * t3 * t3 * r6, d5 = d3 - 3.0 * t3 * t3 * r6;
-    double v, d;
-    if (nn_lt(a, m1)) { v = v1; d = d1; }
-    else if (nn_lt(a, m2)) { v = v2; d = d2; }
-    else if (nn_lt(a, top)) { v = v3; d = d3; }
-    else if (lin) { v = v4; d = d4; }
-    else { v = v5; d = d5; }
-    const double f = v - c;
-    const long long af = dbits(f) & 0x7FFFFFFFFFFFFFFFLL;
+    double d = 1.0;
+    const double r = vol_eval<true>(f, a, d) - c;
+    const long long af = dbits(dabs_i(r));
     if (af < bestf) { bestf = af; best = a; }
     if (it == 3) break;
-    double an = a - f / d;
+    double an = a - div_by(r, rcp_of(d));
     // stay in [0, 1/2] (a > 0 keeps the cubic corner's derivative nonzero)
     if (!(dbits(an) > 0)) an = 0.5 * a;
     if (nn_lt(0.5, an)) an = 0.5;
     a = an;
   }
-  // converged to rounding: |f| within a few ulps of the volume
-  const double tol = 32.0 * 1.1102230246251565e-16 * c;
-  if (!(__longlong_as_double(bestf) <= tol)) best = alpha_low_analytic(m1, m2, m3, c);
+  // converged to rounding: |f| within a few ulps of the volume (c >= 2^-900)
+  const bool off = !(bestf <= dbits(c) - (48LL << 52));
+  if (__any_sync(__activemask(), off)) {
+    if (off) best = alpha_low_analytic(m1, m2, m3, c);
+  }
   return best;
 }
 
 // An estimate of the same plane constant (float guess, two Newton steps on
 // the same branch form; no check of the result), for callers that verify it.
-__device__ __forceinline__ double alpha_low_est(double m1, double m2, double m3, double c) {
-  const double m12 = m1 + m2;
-  const double top = nn_lt(m12, m3) ? m12 : m3;
-  const bool lin = !nn_lt(m3, m12);
-  const double r6 = 1.0 / (6.0 * m1 * m2 * m3);
-  const double r2 = 1.0 / (2.0 * m2 * m3);
-  const double r3 = 1.0 / m3;
-  const double v2c = m1 * m1 * r2 * (1.0 / 3.0);
-  double a = (double)alpha_guess_f((float)m1, (float)m2, (float)m3, (float)c);
-#pragma unroll
+__device__ __forceinline__ double alpha_low_est(VolForm f, double c) {
+  f.v2c = f.v2c * (1.0 / 3.0);
+  double a = f64_of(alpha_guess_f(f32_of(f.m1), f32_of(f.m2), f32_of(f.m3), f32_of(c)));
+#pragma unroll 1
   for (int it = 0; it < 2; ++it) {
-    const double t1 = a - m1, t2 = a - m2, t3 = a - m3;
-    const double v1 = a * a * a * r6, d1 = 3.0 * a * a * r6;
-    const double v2 = a * t1 * r2 + v2c, d2 = (a + t1) * r2;
-    const double v3 = v2 - t2 * t2 * t2 * r6, d3 = d2 - 3.0 * t2 * t2 * r6;
-    const double v4 = (a + (a - m12)) * 0.5 * r3, d4 = r3;
-    const double v5 = v3 - t3 * t3 * t3 * r6, d5 = d3 - 3.0 * t3 * t3 * r6;
-    double v, d;
-    if (nn_lt(a, m1)) { v = v1; d = d1; }
-    else if (nn_lt(a, m2)) { v = v2; d = d2; }
-    else if (nn_lt(a, top)) { v = v3; d = d3; }
-    else if (lin) { v = v4; d = d4; }
-    else { v = v5; d = d5; }
-    double an = a - (v - c) / d;
+    double d = 1.0;
+    const double v = vol_eval<true>(f, a, d);
+    double an = a - div_by(v - c, rcp_of(d));
     if (!(dbits(an) > 0)) an = 0.5 * a;
     if (nn_lt(0.5, an)) an = 0.5;
     a = an;
@@ -415,19 +524,17 @@ __device__ __forceinline__ double alpha_low_est(double m1, double m2, double m3,
 // alpha with volume(m, alpha) = c for any m (mirror, normalise, invert,
 // undo): the same outer steps as the volume function.
 __device__ __forceinline__ double plane_alpha(double m0, double m1, double m2, double c) {
-  Mirror r = mirror_normalise(m0, m1, m2);
-  if (r.l1 == 0.0) return 0.0;
-  if (c <= 0.0) return 0.0 - r.sh;
-  if (c >= 1.0) return r.l1 - r.sh;
-  double s0 = r.mp[0], s1 = r.mp[1], s2 = r.mp[2];
-  sort3(s0, s1, s2);
+  const Mirror r = mirror_normalise(m0, m1, m2);
   // one call for both halves (c or 1 - c picked per lane): an FP64
   // instruction costs its full issue time whatever the active lanes, so a
   // warp that took both branches would pay for the inversion twice
-  const bool up = !(c <= 0.5);
-  const double al = alpha_low(s0, s1, s2, up ? 1.0 - c : c);
+  const bool up = dbits(c) > 0 && nn_lt(0.5, c);
+  const double al = alpha_low(r.mp[0], r.mp[1], r.mp[2], up ? 1.0 - c : c);
   const double am = up ? 1.0 - al : al;
-  return am * r.l1 - r.sh;
+  double res = am * r.l1 - r.sh;
+  if (dbits(c) <= 0) res = 0.0 - r.sh;                      // c <= 0
+  else if (!nn_lt(c, 1.0)) res = r.l1 - r.sh;               // c >= 1
+  return dnz(r.l1) ? res : 0.0;
 }
 
 // The same plane constant by bisection on the monotone volume, step for
@@ -457,30 +564,31 @@ __device__ __forceinline__ double plane_alpha(double m0, double m1, double m2, d
 template <int LANES>
 static __device__ __noinline__ double plane_alpha_bisect_t(double m0, double m1, double m2, double c, unsigned gmask,
                                                            int leader, int sub) {
-  Mirror r = mirror_normalise(m0, m1, m2);
-  if (r.l1 == 0.0) return 0.0;
-  if (c <= 0.0) return 0.0 - r.sh;
-  if (c >= 1.0) return r.l1 - r.sh;
+  const Mirror r = mirror_normalise(m0, m1, m2);
+  if (!dnz(r.l1)) return 0.0;
+  if (dbits(c) <= 0) return 0.0 - r.sh;
+  if (!nn_lt(c, 1.0)) return r.l1 - r.sh;
   // the volume function's own steps, with the sort of the (fixed) normal
   // done once and its compares of non-negative values made on integers:
   // the same values at every midpoint as the plain volume function
-  double s0 = r.mp[0], s1 = r.mp[1], s2 = r.mp[2];
-  sort3(s0, s1, s2);
+  const double s0 = r.mp[0], s1 = r.mp[1], s2 = r.mp[2];
   const double m12 = s0 + s1;
   const double top = nn_lt(m12, s2) ? m12 : s2;
   const bool lin = !nn_lt(s2, m12);
-  const double d6 = 6.0 * s0 * s1 * s2, d2 = 2.0 * s1 * s2, d2m3 = 2.0 * s2;
-  const double v2c = s0 * s0 / (6.0 * s1 * s2);
+  const Rcp q6 = rcp_of(6.0 * s0 * s1 * s2), q2 = rcp_of(2.0 * s1 * s2), q23 = rcp_of(2.0 * s2);
+  const double v2c = div_by(s0 * s0, rcp_of(6.0 * s1 * s2));
+  // (branches here: the cells that come here have a small constant, and most
+  // lanes of a warp are in the first one)
   auto vlow = [&](double a) -> double {
-    if (nn_lt(a, s0)) return a * a * a / d6;
-    const double v2 = a * (a - s0) / d2 + v2c;
+    if (nn_lt(a, s0)) return div_by(a * a * a, q6);
+    const double v2 = div_by(a * (a - s0), q2) + v2c;
     if (nn_lt(a, s1)) return v2;
     const double t2 = a - s1;
-    const double v3 = v2 - t2 * t2 * t2 / d6;
+    const double v3 = v2 - div_by(t2 * t2 * t2, q6);
     if (nn_lt(a, top)) return v3;
-    if (lin) return (2.0 * a - m12) / d2m3;
+    if (lin) return div_by(2.0 * a - m12, q23);
     const double t3 = a - s2;
-    return v3 - t3 * t3 * t3 / d6;
+    return v3 - div_by(t3 * t3 * t3, q6);
   };
   auto vpos = [&](double a) -> double {  // a in (0, 1) here; one vlow for both halves
     const bool up = nn_lt(0.5, a);
@@ -494,17 +602,22 @@ static __device__ __noinline__ double plane_alpha_bisect_t(double m0, double m1,
   // is on the same side of c -- and only midpoints near the root pay for the
   // exact volume's divisions (slow on this part).  The decisions, and so the
   // result, are those of the plain bisection.
-  const double r6 = 1.0 / d6, r2 = 1.0 / d2, r2m3 = 1.0 / d2m3;
+  VolForm f;
+  f.m1 = s0; f.m2 = s1; f.m3 = s2; f.m12 = m12; f.top = top; f.lin = lin;
+  f.r6 = inv_of(q6);
+  f.r2 = inv_of(q2);
+  f.r3h = inv_of(q23);
+  f.v2c = s0 * s0 * f.r2;
   auto vlow_fast = [&](double a) -> double {
-    if (nn_lt(a, s0)) return a * a * a * r6;
-    const double v2 = a * (a - s0) * r2 + v2c;
+    if (nn_lt(a, s0)) return a * a * a * f.r6;
+    const double v2 = a * (a - s0) * f.r2 + v2c;
     if (nn_lt(a, s1)) return v2;
     const double t2 = a - s1;
-    const double v3 = v2 - t2 * t2 * t2 * r6;
+    const double v3 = v2 - t2 * t2 * t2 * f.r6;
     if (nn_lt(a, top)) return v3;
-    if (lin) return (2.0 * a - m12) * r2m3;
+    if (lin) return (2.0 * a - m12) * f.r3h;
     const double t3 = a - s2;
-    return v3 - t3 * t3 * t3 * r6;
+    return v3 - t3 * t3 * t3 * f.r6;
   };
   // Above the cube's middle the decision vpos(mid) < c, vpos = RN(1 - w)
   // with w the volume at 1 - mid, is w > t exactly, t = (1 - c) + 2^-54 (c
@@ -529,9 +642,9 @@ static __device__ __noinline__ double plane_alpha_bisect_t(double m0, double m1,
     // (every step below is taken by every lane, the halves picked per
     // lane, so a warp evaluates each volume once)
     const bool low_c = nn_lt(c, 0.25);
-    const double al = alpha_low_est(s0, s1, s2, low_c ? c : 1.0 - c);
+    const double al = alpha_low_est(f, low_c ? c : 1.0 - c);
     const double ae = low_c ? al : 1.0 - al;
-    double dz = (low_c ? ae : 1.0 - ae) * 0x1p-36;
+    double dz = (low_c ? ae : 1.0 - ae) * 0x1p-40;
     if (!low_c && nn_lt(dz, 0x1p-50)) dz = 0x1p-50;  // a few ulps of 1 at least
     const double aL = ae - dz, aR = ae + dz;
     // below the middle: vlow(aL) < c <= vlow(aR); above it, with w(a) =
@@ -619,60 +732,52 @@ static __device__ __forceinline__ double plane_alpha_bisect(double m0, double m1
   return plane_alpha_bisect_t<1>(m0, m1, m2, c, 0u, 0, 0);
 }
 
-// The volume function with every compare on the integer pipe: the normal is
-// mirrored to |m_i| (a -0 component becomes +0, which changes no volume), so
-// all compared values are non-negative and order like their bit patterns.
-// Not bit-for-bit the plain routine's steps at a zero component's sign, so
-// the oracle-identical bisection keeps the plain one.
-__device__ __forceinline__ double vol_low_nn(double m1, double m2, double m3, double a) {
-  const double m12 = m1 + m2;
-  if (nn_lt(a, m1)) return a * a * a / (6.0 * m1 * m2 * m3);
-  const double v2 = a * (a - m1) / (2.0 * m2 * m3) + m1 * m1 / (6.0 * m2 * m3);
-  if (nn_lt(a, m2)) return v2;
-  const double t2 = a - m2;
-  const double v3 = v2 - t2 * t2 * t2 / (6.0 * m1 * m2 * m3);
-  const double top = nn_lt(m12, m3) ? m12 : m3;
-  if (nn_lt(a, top)) return v3;
-  if (!nn_lt(m3, m12)) return (2.0 * a - m12) / (2.0 * m3);
-  const double t3 = a - m3;
-  return v3 - t3 * t3 * t3 / (6.0 * m1 * m2 * m3);
-}
-
-// The volume function split in two: the normal's mirror, normalisation and
-// sort (once per normal), then the volume at a plane constant.  volume_nn is
-// the two in a row, so several volumes of one normal are bit for bit the
-// single calls'.
+// The volume function in two parts: the normal's mirror, normalisation and
+// sort with the denominators' reciprocals (once per normal), then the volume at
+// a plane constant; volume_nn is the two in a row, so several volumes of one
+// normal are bit for bit the single calls'.  Compares on the integer pipe, the
+// branches' shared terms formed once (the cube over 6 m1 m2 m3, the quadratic's
+// or the linear branch's quotient) and selected: ~75 FP64 instructions, where
+// separate branches and library divisions took ~135.
 struct VolNormal {
-  double sh, l1, a0, a1, a2;
+  Mirror n;
+  double m12;
+  Rcp q6;
+  double v2c;  // m1^2 / (6 m2 m3)
 };
 __device__ __forceinline__ VolNormal volume_normal_nn(double m0, double m1, double m2) {
   VolNormal p;
-  p.sh = 0.0;
-  if (dlt0(m0)) p.sh -= m0;
-  if (dlt0(m1)) p.sh -= m1;
-  if (dlt0(m2)) p.sh -= m2;
-  double a0 = fabs(m0), a1 = fabs(m1), a2 = fabs(m2);
-  p.l1 = a0 + a1 + a2;
-  if (dnz(p.l1)) {
-    a0 /= p.l1; a1 /= p.l1; a2 /= p.l1;
-    // sort the three non-negative components
-    double t;
-    if (nn_lt(a1, a0)) { t = a0; a0 = a1; a1 = t; }
-    if (nn_lt(a2, a1)) { t = a1; a1 = a2; a2 = t; }
-    if (nn_lt(a1, a0)) { t = a0; a0 = a1; a1 = t; }
-  }
-  p.a0 = a0; p.a1 = a1; p.a2 = a2;
+  p.n = mirror_normalise(m0, m1, m2);
+  const double a0 = p.n.mp[0], a1 = p.n.mp[1], a2 = p.n.mp[2];
+  p.m12 = a0 + a1;
+  p.q6 = rcp_of(6.0 * a0 * a1 * a2);
+  p.v2c = div_by(a0 * a0, rcp_of(6.0 * a1 * a2));
   return p;
 }
 
 __device__ __forceinline__ double volume_at_nn(const VolNormal& p, double alpha) {
-  if (!dnz(p.l1)) return dlt0(alpha) ? 0.0 : 1.0;
-  const double a = (alpha + p.sh) / p.l1;
-  if (!dgt0(a)) return 0.0;
-  if (!nn_lt(a, 1.0)) return 1.0;
-  // one call for both halves (the argument picked per lane, as above)
-  const bool up = nn_lt(0.5, a);
-  const double v = vol_low_nn(p.a0, p.a1, p.a2, up ? 1.0 - a : a);
+  if (!dnz(p.n.l1)) return dlt0(alpha) ? 0.0 : 1.0;
+  const double a0 = div_by(alpha + p.n.sh, p.n.R);
+  if (!dgt0(a0)) return 0.0;
+  if (!nn_lt(a0, 1.0)) return 1.0;
+  // one evaluation for both halves (the argument picked per lane, as above)
+  const bool up = nn_lt(0.5, a0);
+  const double a = up ? 1.0 - a0 : a0;
+  const double m1 = p.n.mp[0], m2 = p.n.mp[1], m3 = p.n.mp[2];
+  const double top = nn_lt(p.m12, m3) ? p.m12 : m3;
+  const bool lin = !nn_lt(m3, p.m12);
+  const bool b1 = nn_lt(a, m1), b2 = nn_lt(a, m2), b3 = nn_lt(a, top);
+  const bool b4 = !b1 && !b2 && !b3 && lin, b5 = !b1 && !b2 && !b3 && !lin;
+  const double s = b1 ? a : a - m2;
+  const double q = div_by(s * s * s, p.q6);
+  const double x = div_by(b4 ? dtwice(a) - p.m12 : a * (a - m1), rcp_of(b4 ? dtwice(m3) : dtwice(m2) * m3));
+  const double v2 = x + p.v2c;
+  double v = b1 ? q : (b4 ? x : (b2 ? v2 : v2 - q));
+  if (__any_sync(__activemask(), b5)) {
+    const double t3 = a - m3;
+    const double v5 = v - div_by(t3 * t3 * t3, p.q6);
+    if (b5) v = v5;
+  }
   return up ? 1.0 - v : v;
 }
 
@@ -690,18 +795,6 @@ __device__ __forceinline__ double slab_volume_nn(const double m[3], double alpha
   else if (axis == 1) mm1 = ma * delta;
   else mm2 = ma * delta;
   return delta * volume_nn(mm0, mm1, mm2, alpha - ma * x0);
-}
-
-// liquid volume (cell units) in the slab x_axis in [x0, x0+delta]
-__device__ __forceinline__ double slab_volume(const double m[3], double alpha, int axis, double x0, double delta) {
-  if (delta <= 0.0) return 0.0;
-  double mm0 = m[0], mm1 = m[1], mm2 = m[2];
-  double ma = m[axis];
-  if (axis == 0) mm0 = ma * delta;
-  else if (axis == 1) mm1 = ma * delta;
-  else mm2 = ma * delta;
-  double a2 = alpha - ma * x0;
-  return delta * volume(mm0, mm1, mm2, a2);
 }
 
 // ---------------------------------------------------------------------------
@@ -735,77 +828,34 @@ __device__ __forceinline__ void youngs_normal(const double* s, double m[3]) {
   else { m[0] = 1.0; m[1] = 0.0; m[2] = 0.0; }
 }
 
-__device__ __forceinline__ void cc_candidate(const double* s, int d, double m[3]) {
-  double h[3][3];
-#pragma unroll
-  for (int q = -1; q <= 1; ++q)
-#pragma unroll
-    for (int p = -1; p <= 1; ++p) {
-      double col = sax(s, d, -1, p, q);
-      col = col + sax(s, d, 0, p, q);
-      col = col + sax(s, d, 1, p, q);
-      h[p + 1][q + 1] = col;
-    }
-  double lower = 0.0, upper = 0.0;
-#pragma unroll
-  for (int q = -1; q <= 1; ++q)
-#pragma unroll
-    for (int p = -1; p <= 1; ++p) {
-      lower = lower + sax(s, d, -1, p, q);
-      upper = upper + sax(s, d, 1, p, q);
-    }
-  double sg = (lower >= upper) ? 1.0 : -1.0;
-  double a1 = -(h[2][1] - h[0][1]) * 0.5;
-  double a2 = -(h[1][2] - h[1][0]) * 0.5;
-  double l1 = fabs(a1) + fabs(a2) + 1.0;
-  int t1 = d == 0 ? 1 : 0, t2 = d == 2 ? 1 : 2;
-  m[t1] = a1 / l1;
-  m[t2] = a2 / l1;
-  m[d] = sg / l1;
-}
-
 // Centred-columns candidate along d without its divisions: the two
-// tangential slopes a1, a2 (along t1 < t2), the L1 norm l1 = |a1|+|a2|+1 and
-// the sign of the own-axis component.
+// tangential slopes a1, a2 (along t1 < t2) and the L1 norm l1 = |a1|+|a2|+1.
 struct CCParts {
-  double a1, a2, l1, sg;
+  double a1, a2, l1;
 };
 
 __device__ __forceinline__ CCParts cc_parts(const double* s, int d) {
-  double h[3][3];
-#pragma unroll
-  for (int q = -1; q <= 1; ++q)
-#pragma unroll
-    for (int p = -1; p <= 1; ++p) {
-      double col = sax(s, d, -1, p, q);
-      col = col + sax(s, d, 0, p, q);
-      col = col + sax(s, d, 1, p, q);
-      h[p + 1][q + 1] = col;
-    }
-  double lower = 0.0, upper = 0.0;
-#pragma unroll
-  for (int q = -1; q <= 1; ++q)
-#pragma unroll
-    for (int p = -1; p <= 1; ++p) {
-      lower = lower + sax(s, d, -1, p, q);
-      upper = upper + sax(s, d, 1, p, q);
-    }
-  CCParts r;
-  r.sg = !nn_lt(lower, upper) ? 1.0 : -1.0;  // lower >= upper (both >= 0)
+  // the four columns the central differences use
+  auto col = [&](int p, int q) {
+    double v = sax(s, d, -1, p, q);
+    v = v + sax(s, d, 0, p, q);
+    return v + sax(s, d, 1, p, q);
+  };
   // the central differences' halves on the integer pipe; a difference
   // whose half would be subnormal (never met in practice) takes the product
   // (a1 = -(h21 - h01) / 2, a2 = -(h12 - h10) / 2, the sign flipped on the
   // bit pattern)
-  const double d1 = h[2][1] - h[0][1], d2 = h[1][2] - h[1][0];
+  const double d1 = col(1, 0) - col(-1, 0), d2 = col(0, 1) - col(0, -1);
   bool ok1, ok2;
   double e1 = dhalf_exact(d1, ok1), e2 = dhalf_exact(d2, ok2);
   if (__any_sync(__activemask(), !(ok1 && ok2))) {
     e1 = ok1 ? e1 : d1 * 0.5;
     e2 = ok2 ? e2 : d2 * 0.5;
   }
+  CCParts r;
   r.a1 = dneg(e1);
   r.a2 = dneg(e2);
-  r.l1 = fabs(r.a1) + fabs(r.a2) + 1.0;
+  r.l1 = dabs_i(e1) + dabs_i(e2) + 1.0;
   return r;
 }
 
@@ -848,11 +898,11 @@ __device__ __forceinline__ void myc_normal(const double* s, double m[3]) {
         const double diff = sax(s, d, 1, p, q) - sax(s, d, -1, p, q);
         const int k = (p == 0) + (q == 0);  // weight 2^k
         const double wd = k == 0 ? diff : (k == 1 ? dtwice(diff) : dtwice(dtwice(diff)));
-        g = g + wd;
+        g = p == -1 && q == -1 ? wd : g + wd;
       }
-    y[d] = -g;
+    y[d] = dneg(g);
   }
-  const double ay0 = fabs(y[0]), ay1 = fabs(y[1]), ay2 = fabs(y[2]);
+  const double ay0 = dabs_i(y[0]), ay1 = dabs_i(y[1]), ay2 = dabs_i(y[2]);
   const double l1y = ay0 + ay1 + ay2;
   double amax = ay0;
   if (nn_lt(amax, ay1)) amax = ay1;
@@ -893,13 +943,28 @@ __device__ __forceinline__ void myc_normal(const double* s, double m[3]) {
   // Numerators and denominator are picked first, so both cases share three
   // divisions (a warp whose lanes took both branches would pay for five).
   const CCParts cb = bd == 0 ? c[0] : (bd == 1 ? c[1] : c[2]);
-  const double own = dbits(cb.sg) < 0 ? -1.0 : 1.0;
+  double lower = 0.0, upper = 0.0;
+  if (__any_sync(__activemask(), use_cc)) {
+    // the candidate's own sign: its lower layer sum not below its upper one
+    // (only the chosen candidate's 18 values, selected lane by lane)
+#pragma unroll
+    for (int q = -1; q <= 1; ++q)
+#pragma unroll
+      for (int p = -1; p <= 1; ++p) {
+        const double lo = bd == 0 ? sax(s, 0, -1, p, q) : (bd == 1 ? sax(s, 1, -1, p, q) : sax(s, 2, -1, p, q));
+        const double up = bd == 0 ? sax(s, 0, 1, p, q) : (bd == 1 ? sax(s, 1, 1, p, q) : sax(s, 2, 1, p, q));
+        lower = p == -1 && q == -1 ? lo : lower + lo;
+        upper = p == -1 && q == -1 ? up : upper + up;
+      }
+  }
+  const double own = nn_lt(lower, upper) ? -1.0 : 1.0;  // (both >= 0)
   // transverse axes of bd: t1 = bd == 0 ? 1 : 0, t2 = bd == 2 ? 1 : 2
   const double n0 = bd == 0 ? own : cb.a1;
   const double n1 = bd == 1 ? own : (bd == 0 ? cb.a1 : cb.a2);
   const double n2 = bd == 2 ? own : cb.a2;
-  const double den = use_cc ? cb.l1 : l1y;
-  const double q0 = (use_cc ? n0 : y[0]) / den, q1 = (use_cc ? n1 : y[1]) / den, q2 = (use_cc ? n2 : y[2]) / den;
+  const Rcp den = rcp_of(use_cc ? cb.l1 : l1y);
+  const double q0 = div_by(use_cc ? n0 : y[0], den), q1 = div_by(use_cc ? n1 : y[1], den),
+               q2 = div_by(use_cc ? n2 : y[2], den);
   const bool deg = !use_cc && !dnz(l1y);
   m[0] = deg ? 1.0 : q0;
   m[1] = deg ? 0.0 : q1;
@@ -1058,25 +1123,6 @@ __device__ __forceinline__ double slab_volume_f(const double m[3], double alpha,
   const double lo = c - (1.0 - delta);
   if (dgt0(lo) && nn_lt(v, lo)) v = lo;
   return v;
-}
-
-// FP32 of an FP64 value to nearest even, and back, on the integer pipe (an
-// FP64 conversion instruction occupies the FP64 unit like an add).  Values
-// below FP32's normal range become 0; infinities and NaN stay what they are.
-__device__ __forceinline__ float f32_of(double x) {
-  const unsigned long long b = (unsigned long long)dbits(x);
-  const unsigned long long r = (b & 0x7FFFFFFFFFFFFFFFull) + 0x0FFFFFFFull + ((b >> 29) & 1ull);
-  const int ex = (int)(r >> 52) - 1023 + 127;
-  unsigned f = ((unsigned)ex << 23) | ((unsigned)(r >> 29) & 0x7FFFFFu);
-  if (ex <= 0) f = 0u;
-  if (ex >= 255) f = ((b & 0x7FFFFFFFFFFFFFFFull) > 0x7FF0000000000000ull) ? 0x7FC00000u : 0x7F800000u;
-  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
-}
-__device__ __forceinline__ double f64_of(float x) {
-  const unsigned b = __float_as_uint(x), ex = (b >> 23) & 0xFFu;
-  const unsigned long long m = (unsigned long long)(b & 0x7FFFFFu) << 29;
-  const unsigned long long v = ex == 255u ? (0x7FF0000000000000ull | m) : (ex ? ((unsigned long long)(ex + 896u) << 52) | m : 0ull);
-  return __longlong_as_double((long long)(v | ((unsigned long long)(b & 0x80000000u) << 32)));
 }
 
 // WENO5 with the neighbour differences in FP64 and the nonlinear weights and

@@ -130,17 +130,17 @@ VOF_HD int rint_i(float x) {
 }
 // FP64 value of the pair (hi + lo) * 2^k (|lo| at most half a last place of
 // hi): hi widened exactly, then lo added to the bit pattern as an integer
-// number of FP64 last places, to the nearest (to two of them when the sum
-// drops below a power of two).  A lo whose last places are out of FP32's
+// number of the sum's FP64 last places, to the nearest (half as large when a
+// power of two hi meets a lo of the other sign).  A lo whose last places are out of FP32's
 // range (hi below 2^-74) is left out.
 VOF_HD double widen_pair(f2 q, int k) {
   const uint64_t h = d_bits(widen_scaled(q.hi, k));
   const int eh = (int)((f_bits(q.hi) >> 23) & 0xFF);
   if (eh == 0 || eh == 255) return bits_d(h);
-  const int es = 52 + 127 - (eh - 127);
-  const float up = es > 254 ? 0.0f : bits_f((uint32_t)es << 23);
   // towards larger magnitude when the signs agree
   const float l = bits_f(f_bits(q.lo) ^ (f_bits(q.hi) & 0x80000000u));
+  const int es = 52 + 127 - (eh - 127) + ((f_bits(q.hi) & 0x7FFFFFu) == 0 && l < 0.0f ? 1 : 0);
+  const float up = es > 254 ? 0.0f : bits_f((uint32_t)es << 23);
   return bits_d(h + (uint64_t)(int64_t)rint_i(l * up));
 }
 

@@ -194,7 +194,7 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
   myc_normal(st, m);
   double al;
   if (LANES == 3) al = plane_alpha_bisect_t<3>(m[0], m[1], m[2], ct, gmask, leader, sub);
-  else al = edge_cell(ct) ? plane_alpha_bisect(m[0], m[1], m[2], ct) : plane_alpha(m[0], m[1], m[2], ct);
+  else al = plane_alpha(m[0], m[1], m[2], ct);
   const double ddv = dd ? __ldg(dd + id) : dd_uniform;
   const double mn2 = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
   const double sft = mn2 * ddv;
@@ -230,31 +230,31 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
     fhi = fmaxf(fm[0], 0.f) + fmaxf(fm[1], 0.f) + fmaxf(fm[2], 0.f);
     mg = 1e-5f * (4.f + fabsf(al_f) + fabsf(sft_f));
   }
-  for (int oz = -1; oz <= 1; ++oz)
-    for (int oy = -1; oy <= 1; ++oy)
-      for (int ox = -1; ox <= 1; ++ox) {
-        if (!ox && !oy && !oz) continue;
-        size_t pid;
-        if (!neighbour(g, x, y, z, ox, oy, oz, pid)) continue;
-        if (sc.mark) {
-          const double cp = c_value(__ldg(c_in + pid));
-          if (is_mixed_b(cp, g) || is_full_b(cp, g) != full) continue;
-          // (every store of a word writes the same bits, and its readers here
-          // drop the tag)
-          reinterpret_cast<unsigned*>(sc.mark + pid)[1] = (unsigned)__double2hiint(cp) | 0xC0000000u;
-          sc.cnew[pid] = 0.0;  // no change so far
-          const float an = fa - (fm[0] * (float)ox + fm[1] * (float)oy + fm[2] * (float)oz);
-          const bool outside = full ? an >= fhi + mg : an <= flo - mg;
-          if (!outside && sub == 0 && dnz(sft)) {
-            const int k = atomicAdd(sc.npairs, 1);
-            if (k < sc.pair_cap) sc.pairs[k] = make_uint2((uint32_t)id, (unsigned)offset_bit(ox, oy, oz));
-          }
-          continue;
-        }
-        const double cp = __ldg(c_in + pid);
-        if (is_mixed_b(cp, g) || is_full_b(cp, g) != full) continue;
-        atomicOr(sc.claim + pid, 0x80000000u >> offset_bit(-ox, -oy, -oz));
-      }
+  // the neighbours' c are the stencil's (a neighbour beyond a zero-gradient
+  // boundary is no cell, and neighbour() says so)
+  unsigned pure = 0u;
+#pragma unroll
+  for (int b = 0; b < 27; ++b)
+    if (b != 13 && !is_mixed_b(st[b], g) && is_full_b(st[b], g) == full) pure |= 1u << b;
+  for (; pure; pure &= pure - 1u) {
+    const int b = __ffs(pure) - 1;
+    const int ox = b % 3 - 1, oy = (b / 3) % 3 - 1, oz = b / 9 - 1;
+    size_t pid;
+    if (!neighbour(g, x, y, z, ox, oy, oz, pid)) continue;
+    if (!sc.mark) {
+      atomicOr(sc.claim + pid, 0x80000000u >> offset_bit(-ox, -oy, -oz));
+      continue;
+    }
+    // (the readers of these words in this kernel drop the tag)
+    atomicOr(reinterpret_cast<unsigned*>(sc.mark + pid) + 1, 0xC0000000u);
+    sc.cnew[pid] = 0.0;  // no change so far
+    const float an = fa - (fm[0] * (float)ox + fm[1] * (float)oy + fm[2] * (float)oz);
+    const bool outside = full ? an >= fhi + mg : an <= flo - mg;
+    if (!outside && sub == 0 && dnz(sft)) {
+      const int k = atomicAdd(sc.npairs, 1);
+      if (k < sc.pair_cap) sc.pairs[k] = make_uint2((uint32_t)id, (unsigned)offset_bit(ox, oy, oz));
+    }
+  }
 }
 
 // The list's front (cells whose plane constant is inverted directly): one
