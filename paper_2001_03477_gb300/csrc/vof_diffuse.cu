@@ -28,13 +28,26 @@
 //
 // Kernels: k_dif_mlist (list of the mixed cells), k_dif_planes (MYC normal
 // and plane constant of each listed cell), k_dif_classify (per cell: its
-// class; every cell whose sides all couple by k_p / h^2 takes its diagonal
-// from a per-phase table), k_dif_irregular (the listed cells next to the
-// interface or a heated wall: the six couplings and the diagonal), k_dif_jacobi (one Jacobi sweep; the
-// system is strictly diagonally dominant -- C_p / dt sits on the diagonal
-// alone -- so the iteration converges; on every fourth sweep the largest
-// change is reduced per CTA and read on the host), k_dif_store (e' from T').
+// class and T at the start), k_dif_irregular (the listed cells next to the
+// interface or a heated wall: their couplings), the Jacobi sweeps -- the
+// system is strictly diagonally dominant (C_p / dt sits on the diagonal alone),
+// so the iteration converges; on every fourth sweep the largest change is
+// reduced -- and the store of e'.
+//
+// Phase heat capacity: the sweeps iterate on the change d = T - T0 of each node,
+//   d' = B sum d_nb + s,  B = k_p / h^2 / diagonal,  s = B sum (T0_nb - T0),
+// (the same iterates T, since C_p / dt and the couplings add up to the
+// diagonal), s formed once in FP64 (k_dif_first: it is also the first sweep),
+// d, B and s held as pairs of FP32 numbers (48 bits of the change itself, whose
+// rounding stays below an ulp of T), over the power of two next to the largest
+// T.  What bounds a sweep on this part is the
+// FP64 unit: 8 FP64 instructions per cell took 45 us at 128^3 (76 cycles of an
+// SM partition each); the pairs' FP32 instructions take 22 us (its reads come from L2).  The sweeps
+// are queued in batches without waiting: each starts by reading the last
+// check's result and leaves its buffers alone once that was within tol.
+// Mixture heat capacity: the FP64 form, every cell's diagonal stored.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -47,6 +60,7 @@ namespace {
 
 constexpr int kDifThreads = 256;
 constexpr int kDifCTAs = 152 * 8;
+constexpr int kDifPlaneThreads = 64;  // few cells, long FP64 chains: spread over the SMs
 constexpr double kThetaEps = 1e-3;
 
 __device__ __forceinline__ size_t dcid(const GridDev& g, int x, int y, int z) {
@@ -96,7 +110,7 @@ k_dif_mlist(GridDev g, const double* __restrict__ c, uint32_t* __restrict__ mlis
 
 // MYC normal and plane constant of each listed mixed cell (lanes dense over
 // the list: the FP64 work of a warp serves 32 cells)
-__global__ void __launch_bounds__(kDifThreads)
+__global__ void __launch_bounds__(kDifPlaneThreads)
 k_dif_planes(GridDev g, const double* __restrict__ c, const uint32_t* __restrict__ mlist,
              const int* __restrict__ count, double4* __restrict__ plane) {
   const int nm = *count;
@@ -182,6 +196,9 @@ struct DifConst {
   double kq[2];
   double cdt[2];
   double rdiag[2][7];
+  double B[2][7];    // kq * rdiag
+  float2 Bf[2][7];   // the same as pairs of FP32 numbers
+  int e0;            // largest exponent field of T_sat and the walls' T
 };
 
 // Cell classes: bits 0..5 the sides (-x, +x, -y, +y, -z, +z) with a
@@ -193,15 +210,28 @@ struct DifConst {
 constexpr uint8_t kDifLiq = 0x40, kDifIrr = 0x80;
 
 struct DifVec {
-  double* off;    // [6 N]: coupling to the neighbour (face order -x, +x, -y, +y, -z, +z); kDifIrr cells only
-  double* diag;   // [N] reciprocal of the diagonal; kDifIrr cells (all cells with the mixture heat capacity)
-  double* rhs;    // [N]; kDifIrr cells (all cells with the mixture heat capacity)
-  double* T0;     // [N] T at the start (the first iterate)
+  double* off;    // [6 N]: coupling to the neighbour (face order -x, +x, -y, +y, -z, +z), kDifIrr cells
+                  // only; with the phase heat capacity over the diagonal, as a pair of FP32 numbers
+  double* diag;   // [N] reciprocal of the diagonal (mixture heat capacity)
+  double* rhs;    // [N] right side (mixture)
+  double* T0;     // [N] T at the start (the first iterate of the mixture form)
   double* Ta;     // [N] the two later Jacobi iterates
   double* Tb;
-  double* part;   // [1] the largest change of a checked sweep
+  unsigned long long* part;  // [kDifChecks] the largest change of each checked sweep of a batch (bits)
   uint8_t* cls;   // [N] cell class
+  // phase form: pairs, high and low parts in arrays of their own, x rows padded
+  // to an even length px (two cells of a row are one aligned 8-byte access)
+  float* s;       // [2][px ny nz]: s, also the first iterate d
+  float* d[2];    // the two later iterates
+  int px;
+  size_t pn;      // px ny nz: the low parts' offset
+  int* tmax;      // largest exponent field of a finite T0
 };
+// the pairs hold d / 2^k
+__device__ __forceinline__ int dif_scale(const DifVec& v, const DifConst& K) { return max(*v.tmax, K.e0) - 1023; }
+__device__ __forceinline__ size_t pad_id(const GridDev& g, const DifVec& v, int x, int y, int z) {
+  return ((size_t)z * g.n[1] + y) * v.px + x;
+}
 
 constexpr long long kHalfBits = 0x3FE0000000000000LL;  // 0.5: c >= 1/2 on the integer pipe (c >= +0)
 
@@ -228,11 +258,6 @@ __device__ __forceinline__ void dif_sides(const GridDev& g, const double* __rest
   }
 }
 
-// Per cell: its class and T; every cell that couples by k_p / h^2 on all
-// sides also gets its right side (and, with the mixture heat capacity, its
-// diagonal); the others -- next to the interface or a heated wall -- are
-// listed for k_dif_irregular (one atomic per warp; the list's order varies
-// from run to run, and nothing depends on it).
 // the sweep's CTAs: 32 x 8 cells of every plane each, enough z shares for
 // a few waves
 static dim3 dif_sweep_grid(const GridDev& g) {
@@ -241,6 +266,11 @@ static dim3 dif_sweep_grid(const GridDev& g) {
   return dim3(gx, gy, gz);
 }
 
+// Per cell: its class and T; with the mixture heat capacity every cell that
+// couples by k_p / h^2 on all sides also gets its right side and diagonal; the
+// others -- next to the interface or a heated wall -- are listed for
+// k_dif_irregular (one atomic per warp; the list's order varies from run to
+// run, and nothing depends on it).
 template <bool PHASE>
 __global__ void __launch_bounds__(kDifThreads)
 k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict__ e, DifVec v, DifWalls walls,
@@ -249,6 +279,7 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
   if (y >= g.n[1]) return;  // whole warps (a warp is one row segment)
   const bool in_x = x < g.n[0];
   const int lane = threadIdx.x;
+  int tmax = 0;
   for (int z = blockIdx.z; z < g.n[2]; z += gridDim.z) {
     const size_t i = ((size_t)z * g.n[1] + y) * g.n[0] + x;
     bool irr = false;
@@ -261,6 +292,8 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
       dif_sides(g, c, walls, x, y, z, liq, inm, same, hot_wall);
       const int li = liq ? 1 : 0;
       v.T0[i] = T0;
+      const int ex = (int)((dbits(T0) >> 52) & 0x7FF);
+      if (ex != 0x7FF) tmax = max(tmax, ex);
       irr = hot_wall || same != inm;
       v.cls[i] = (uint8_t)(inm | (liq ? kDifLiq : 0) | (irr ? kDifIrr : 0));
       if (!irr && !PHASE) {
@@ -284,7 +317,27 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
     base = __shfl_sync(0xffffffffu, base, __ffs(mask) - 1);
     if (irr) ilist[base + __popc(mask & ((1u << lane) - 1u))] = (uint32_t)i;
   }
+  if constexpr (PHASE) {
+    tmax = __reduce_max_sync(0xffffffffu, tmax);
+    if (lane == 0 && tmax > *(volatile int*)v.tmax) atomicMax(v.tmax, tmax);  // (few warps find it larger)
+  }
 }
+
+// x / 2^k as a pair of FP32 numbers (48 bits)
+__device__ __forceinline__ float2 pair_of(double x, int k) {
+  const df::f2 p = df::split_scaled(df::words_of(x), k);
+  return make_float2(p.hi, p.lo);
+}
+// f 2^k (0 below the FP64 normal range; infinities and NaN kept)
+__device__ __forceinline__ double wide_of(float f, int k) {
+  const unsigned b = __float_as_uint(f), ef = (b >> 23) & 0xFFu;
+  int ex = ef == 255u ? 2047 : (int)ef + 896 + k;
+  unsigned long long m = (unsigned long long)(b & 0x7FFFFFu) << 29;
+  if (ex > 2046 && ef != 255u) { ex = 2047; m = 0; }
+  if (ef == 0u || ex <= 0) { ex = 0; m = 0; }
+  return __longlong_as_double((long long)(((unsigned long long)(b & 0x80000000u) << 32) | ((unsigned long long)ex << 52) | m));
+}
+__device__ __forceinline__ df::f2 f2_of(float2 p) { return df::f2{p.x, p.y}; }
 
 // Per listed cell (lanes dense over the list): the six couplings (heights
 // or plane distances on the interface sides), the diagonal and the right
@@ -294,7 +347,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
                 const double* __restrict__ c, const double* __restrict__ e, const double4* __restrict__ plane,
                 DifVec v, DifWalls walls, int phase_cp, DifConst K, const uint32_t* __restrict__ ilist,
                 const int* __restrict__ icount) {
-  const int ni = *icount;
+  const int ni = *icount, ks = dif_scale(v, K);
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ni; k += gridDim.x * blockDim.x) {
     const size_t i = ilist[k];
     int x, y, z;
@@ -308,13 +361,19 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
     const int li = liq ? 1 : 0;
     const double cdt = phase_cp ? K.cdt[li] : (g.Cp_l * cv + g.Cp_g * (1.0 - cv)) * inv_dt;
     double diag = cdt, rhs = cdt * T0;
+    double off[6], gain = 0.0;  // gain: the heat conducted at T0 over its own unit (phase form)
+    auto nb_T = [&](int f) {     // T0 of the neighbour across side f
+      int q[3] = {x, y, z};
+      q[f >> 1] = step_coord(q[f >> 1], (f & 1) ? 1 : -1, g.n[f >> 1], g.bc[f >> 1]);
+      return v.T0[dcid(g, q[0], q[1], q[2])];
+    };
     const double kp = liq ? k_l : k_g;
     // a same-phase neighbour couples by k_p / h^2 (no division); only the
     // interface and heated-wall sides need their own distances
     const double kq = kp * (inv_h * inv_h);
 #pragma unroll
     for (int axis = 0; axis < 3; ++axis) {
-      double cs[2], cq[2], cst[2], d[2];
+      double cs[2], cq[2], cst[2], d[2], Tfix[2] = {0.0, 0.0};
       bool reg[2];  // the side's distance is h (same phase or a wall without flux)
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
@@ -323,6 +382,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
         if (!(inm & (1u << f)) && walls.on[f]) {  // a wall at fixed T, half a cell away
           const double Tw = walls.T[f];
           cs[side] = 2.0 * inv_h; cq[side] = 0.0; cst[side] = Tw * 2.0 * inv_h; d[side] = 0.5 * h;
+          Tfix[side] = Tw;
           reg[side] = false;
         } else if (!(inm & (1u << f))) {  // a wall: no flux
           cs[side] = 0.0; cq[side] = 0.0; cst[side] = 0.0; d[side] = h;
@@ -331,6 +391,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
         } else {
           const double th = interface_theta(g, c, plane, x, y, z, axis, side ? 1 : -1, liq) * h;
           cs[side] = 1.0 / th; cq[side] = 0.0; cst[side] = g.T_sat / th; d[side] = th;
+          Tfix[side] = g.T_sat;
           reg[side] = false;
         }
       }
@@ -340,40 +401,66 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
         for (int side = 0; side < 2; ++side) {
           const double o = dnz(cq[side]) ? kq : 0.0;
           diag += o;
-          v.off[6 * i + 2 * axis + side] = o;
+          off[2 * axis + side] = o;
+          if (phase_cp && dnz(o)) gain += o * (nb_T(2 * axis + side) - T0);
         }
       } else {
         const double kd = kp / (0.5 * (d[0] + d[1]));
 #pragma unroll
         for (int side = 0; side < 2; ++side) {
           diag += kd * cs[side];
-          v.off[6 * i + 2 * axis + side] = kd * cq[side];
+          off[2 * axis + side] = kd * cq[side];
           rhs += kd * cst[side];
+          if (phase_cp) {
+            // towards a fixed temperature (T_Gamma, T_w) or the neighbour's
+            if (dnz(cq[side])) gain += kd * cq[side] * (nb_T(2 * axis + side) - T0);
+            else if (dnz(cs[side])) gain += kd * cs[side] * (Tfix[side] - T0);
+          }
         }
       }
     }
-    v.diag[i] = 1.0 / diag;  // stored as its reciprocal: the sweeps multiply
-    v.rhs[i] = rhs;
+    const double rd = 1.0 / diag;  // stored as its reciprocal: the sweeps multiply
+    if (phase_cp) {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) reinterpret_cast<float2*>(v.off)[6 * i + f] = pair_of(off[f] * rd, 0);
+      const float2 sp = pair_of(gain * rd, ks);
+      const size_t ip = pad_id(g, v, x, y, z);
+      v.s[ip] = sp.x;
+      v.s[v.pn + ip] = sp.y;
+    } else {
+#pragma unroll
+      for (int f = 0; f < 6; ++f) v.off[6 * i + f] = off[f];
+      v.diag[i] = rd;
+      v.rhs[i] = rhs;
+    }
   }
 }
 
-// The Jacobi update of one cell from its neighbours' values t0..t5 (sides
-// not in the grid skipped): (rhs + sum off T_nb) / diag, the right side
-// C_p / dt T0 and the couplings k_p / h^2 unless the cell's are stored.  Not
-// inlined, and called only by warps with a cell that needs it, so that the
-// other warps issue none of its FP64 instructions.
+// Checks of a batch of sweeps: at most kDifChecks; a sweep reads the slot of
+// the check before it.
+constexpr int kDifChecks = 32;
+
+// A check's result within tol (both non-negative: compared as integers).
+__device__ __forceinline__ bool dif_done(const unsigned long long* __restrict__ prev, double tol) {
+  return prev && *prev <= (unsigned long long)dbits(tol);
+}
+
+// The Jacobi update of one cell of the mixture form from its neighbours'
+// values t0..t5 (sides not in the grid skipped): (rhs + sum off T_nb) / diag,
+// the couplings k_p / h^2 unless the cell's are stored.  Not inlined, and called
+// only by warps with a cell that needs it, so that the other warps issue none
+// of its FP64 instructions.
 static __device__ __noinline__ double dif_row(unsigned cls, const double* __restrict__ off6,
                                               const double* __restrict__ rhs_i, const double* __restrict__ diag_i,
-                                              double kq, double cdt, double rdt, double T0, int phase_cp, double t0,
-                                              double t1, double t2, double t3, double t4, double t5) {
+                                              double kq, double t0, double t1, double t2, double t3, double t4,
+                                              double t5) {
   const bool irr = (cls & kDifIrr) != 0;
-  const bool stored = irr || !phase_cp;
-  double acc = stored ? __ldg(rhs_i) : cdt * T0;
+  double acc = __ldg(rhs_i);
   const double tn[6] = {t0, t1, t2, t3, t4, t5};
 #pragma unroll
   for (int f = 0; f < 6; ++f)
     if (cls & (1u << f)) acc = fma(irr ? __ldg(off6 + f) : kq, tn[f], acc);
-  return acc * (stored ? __ldg(diag_i) : rdt);
+  return acc * __ldg(diag_i);
 }
 
 // Neighbour index of cell i at (x, y, z) across side f (its class bit set):
@@ -391,9 +478,9 @@ __device__ __forceinline__ size_t dif_nb(const GridDev& g, size_t i, int x, int 
   }
 }
 
-// One Jacobi sweep Tout = (rhs + sum off T_nb(in)) / diag; with CHECK the
-// largest |Tout - Tin| into *change (non-negative doubles order like their
-// bits: an integer atomic max, the same whatever the order).  A cell
+// One Jacobi sweep of the mixture form, Tout = (rhs + sum off T_nb(in)) / diag;
+// with CHECK the largest |Tout - Tin| into *change (non-negative doubles order
+// like their bits: an integer atomic max, the same whatever the order).  A cell
 // coupled by k_p / h^2 whose own and neighbours' values all equal its T0 is
 // the sweep's fixed point, (C_p/dt T0 + n k_p/h^2 T0) / (C_p/dt + n k_p/h^2)
 // = T0, and keeps T0 without arithmetic.  CTAs of 32 x 8 threads over x and
@@ -401,7 +488,8 @@ __device__ __forceinline__ size_t dif_nb(const GridDev& g, size_t i, int x, int 
 template <bool CHECK>
 __global__ void __launch_bounds__(kDifThreads)
 k_dif_jacobi(GridDev g, DifVec v, DifConst K, const double* __restrict__ Tin, double* __restrict__ Tout,
-             unsigned long long* __restrict__ change, int phase_cp) {
+             const unsigned long long* __restrict__ prev, double tol, unsigned long long* __restrict__ change) {
+  if (dif_done(prev, tol)) return;
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
   double dmax = 0.0;
   if (x < g.n[0] && y < g.n[1]) {
@@ -421,10 +509,8 @@ k_dif_jacobi(GridDev g, DifVec v, DifConst K, const double* __restrict__ Tin, do
       }
       double t = T0;
       if (__any_sync(__activemask(), !fixed)) {
-        const int li = (cls & kDifLiq) ? 1 : 0;
-        const double r = dif_row(cls, v.off + 6 * i, v.rhs + i, v.diag + i, li ? K.kq[1] : K.kq[0],
-                                 li ? K.cdt[1] : K.cdt[0], K.rdiag[li][__popc(cls & 63u)], T0, phase_cp, tn[0],
-                                 tn[1], tn[2], tn[3], tn[4], tn[5]);
+        const double r = dif_row(cls, v.off + 6 * i, v.rhs + i, v.diag + i, (cls & kDifLiq) ? K.kq[1] : K.kq[0],
+                                 tn[0], tn[1], tn[2], tn[3], tn[4], tn[5]);
         if (!fixed) t = r;
       }
       Tout[i] = t;
@@ -439,22 +525,203 @@ k_dif_jacobi(GridDev g, DifVec v, DifConst K, const double* __restrict__ Tin, do
 }
 
 
-__global__ void k_dif_store(GridDev g, const double* __restrict__ c, const DifVec v, const double* __restrict__ T,
-                            double* __restrict__ e, size_t N, int phase_cp) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
-    const double Tn = T[i];
-    if (phase_cp) {
-      // e' = e + C_p,node (T' - T0); a node whose T came back unchanged
-      // keeps its e
-      const double T0 = __ldg(v.T0 + i);
-      if (dbits(Tn) == dbits(T0)) continue;
-      const double Cd = (__ldg(v.cls + i) & kDifLiq) ? g.Cp_l : g.Cp_g;
-      e[i] = e[i] + Cd * (Tn - T0);
-    } else {
-      const double cv = __ldg(c + i);
-      const double Cp = g.Cp_l * cv + g.Cp_g * (1.0 - cv);
-      e[i] = Cp * Tn;
+// largest change of the warp's lanes (over 2^k) into *change: FP64 bits
+__device__ __forceinline__ void dif_change(float m, int k, unsigned long long* change) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(change, (unsigned long long)dbits(wide_of(m, k)));
+}
+
+// Offsets to a cell's neighbours across the sides in the grid (wrapped across a
+// periodic boundary); has: bit f set where side f is in the grid.
+struct DifSides {
+  long long o[6];
+  unsigned has;
+};
+__device__ __forceinline__ void dif_lateral(const GridDev& g, int x, int y, long long row, DifSides& d) {
+  const int nx = g.n[0], ny = g.n[1];
+  d.o[0] = x > 0 ? -1 : nx - 1;
+  d.o[1] = x < nx - 1 ? 1 : 1 - nx;
+  d.o[2] = y > 0 ? -row : (ny - 1) * row;
+  d.o[3] = y < ny - 1 ? row : (1 - ny) * row;
+  d.has = (x > 0 || g.bc[0] == 0 ? 1u : 0u) | (x < nx - 1 || g.bc[0] == 0 ? 2u : 0u) |
+          (y > 0 || g.bc[1] == 0 ? 4u : 0u) | (y < ny - 1 || g.bc[1] == 0 ? 8u : 0u);
+}
+__device__ __forceinline__ unsigned dif_vertical(const GridDev& g, int z, long long plane, long long (&o)[6]) {
+  const int nz = g.n[2];
+  o[4] = z > 0 ? -plane : (nz - 1) * plane;
+  o[5] = z < nz - 1 ? plane : (1 - nz) * plane;
+  return (z > 0 || g.bc[2] == 0 ? 16u : 0u) | (z < nz - 1 || g.bc[2] == 0 ? 32u : 0u);
+}
+
+// First sweep of the phase form: d = s = B sum (T0_nb - T0) in FP64 (an
+// irregular cell's is k_dif_irregular's).  Cells of uniform T take no FP64.
+template <bool CHECK>
+__global__ void __launch_bounds__(kDifThreads)
+k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ change) {
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+  const bool in = x < g.n[0] && y < g.n[1];
+  const long long plane = (long long)g.n[0] * g.n[1];
+  const int ks = dif_scale(v, K);
+  DifSides sd;
+  dif_lateral(g, x, y, g.n[0], sd);
+  float dmax = 0.f;
+  for (int z = blockIdx.z; z < g.n[2]; z += gridDim.z) {
+    const unsigned has = sd.has | dif_vertical(g, z, plane, sd.o);
+    const size_t i = in ? ((size_t)z * g.n[1] + y) * g.n[0] + x : 0;
+    const unsigned cls = in ? __ldg(v.cls + i) : kDifIrr;
+    const bool irr = (cls & kDifIrr) != 0;
+    float2 r = make_float2(0.f, 0.f);
+    bool vary = false;
+    double T0 = 0.0, tn[6];
+    if (!irr) T0 = __ldg(v.T0 + i);
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      tn[f] = T0;
+      if (!irr && (has & (1u << f))) tn[f] = __ldg(v.T0 + (long long)i + sd.o[f]);
+      vary = vary || dbits(tn[f]) != dbits(T0);
     }
+    if (__any_sync(0xffffffffu, vary)) {
+      double a = tn[0] - T0;
+#pragma unroll
+      for (int f = 1; f < 6; ++f) a += tn[f] - T0;
+      const double sv = a * K.B[(cls & kDifLiq) ? 1 : 0][__popc(cls & 63u)];
+      if (vary) r = pair_of(sv, ks);
+    }
+    if (in) {
+      const size_t ip = pad_id(g, v, x, y, z);
+      if (!irr) {
+        v.s[ip] = r.x;
+        v.s[v.pn + ip] = r.y;
+      } else if (CHECK) {
+        r.x = v.s[ip];
+      }
+    }
+    if (CHECK) dmax = fmaxf(dmax, fabsf(r.x));
+  }
+  if constexpr (CHECK) dif_change(dmax, ks, change);
+}
+
+// One later sweep of the phase form, d' = sum B_nb d_nb + s, two cells of a row
+// per thread: every packed instruction serves both.  A cell whose own s and
+// neighbours' d are all 0 keeps 0 without arithmetic.
+template <bool CHECK>
+__global__ void __launch_bounds__(kDifThreads)
+k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, float* __restrict__ dout,
+            const unsigned long long* __restrict__ prev, double tol, unsigned long long* __restrict__ change) {
+  pdl_wait();
+  using namespace df;
+  if (dif_done(prev, tol)) return;
+  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+  const int x = (blockIdx.x * 32 + threadIdx.x) * 2, y = blockIdx.y * 8 + threadIdx.y;
+  const bool in = x < nx && y < ny, in1 = x + 1 < nx && y < ny;
+  const float* __restrict__ dlo = din + v.pn;
+  const long long row = v.px, plane = row * ny;
+  // sides of the pair: the outer x neighbours, y and z (those two cells share)
+  const bool px = g.bc[0] == 0;
+  const bool hasL = x > 0 || px, hasR = (in1 ? x + 1 : x) < nx - 1 || px;
+  const int oL = x > 0 ? -1 : nx - 1, oR = in1 ? (x + 2 < nx ? 2 : -x) : -x;
+  const bool hasS = y > 0 || g.bc[1] == 0, hasN = y < ny - 1 || g.bc[1] == 0;
+  const long long oS = y > 0 ? -row : (ny - 1) * row, oN = y < ny - 1 ? row : (1 - ny) * row;
+  float dmax = 0.f;
+  for (int z = blockIdx.z; z < nz; z += gridDim.z) {
+    const bool hasB = z > 0 || g.bc[2] == 0, hasT = z < nz - 1 || g.bc[2] == 0;
+    const long long oB = z > 0 ? -plane : (nz - 1) * plane, oT = z < nz - 1 ? plane : (1 - nz) * plane;
+    const long long ip = in ? z * plane + y * row + x : 0;
+    const float2 zero = make_float2(0.f, 0.f);
+    auto two = [&](const float* a, bool ok, long long o) {
+      return ok ? __ldg(reinterpret_cast<const float2*>(a + ip + o)) : zero;
+    };
+    auto one = [&](const float* a, bool ok, long long o) { return ok ? __ldg(a + ip + o) : 0.f; };
+    const float2 sh = two(v.s, in, 0), sl = two(v.s + v.pn, in, 0);
+    float2 ch = two(din, in, 0), cl = two(dlo, in, 0);
+    if (!in1) ch.y = cl.y = 0.f;  // (the padding)
+    const float2 Sh = two(din, in && hasS, oS), Sl = two(dlo, in && hasS, oS);
+    const float2 Nh = two(din, in && hasN, oN), Nl = two(dlo, in && hasN, oN);
+    const float2 Bh = two(din, in && hasB, oB), Bl = two(dlo, in && hasB, oB);
+    const float2 Th = two(din, in && hasT, oT), Tl = two(dlo, in && hasT, oT);
+    const float Lh = one(din, in && hasL, oL), Ll = one(dlo, in && hasL, oL);
+    const float Rh = one(din, in && hasR, oR), Rl = one(dlo, in && hasR, oR);
+    const unsigned c0 = in ? __ldg(v.cls + ((size_t)z * ny + y) * nx + x) : 0u;
+    const unsigned c1 = in1 ? __ldg(v.cls + ((size_t)z * ny + y) * nx + x + 1) : 0u;
+    auto fb = [](float f) { return __float_as_uint(f); };
+    // (a pair's high part is 0 exactly where the pair is; the padding's values
+    // reach no cell)
+    const unsigned any = (fb(sh.x) | fb(ch.x) | fb(Sh.x) | fb(Nh.x) | fb(Bh.x) | fb(Th.x) | fb(Lh) | fb(Rh) |
+                          (in1 ? fb(sh.y) | fb(ch.y) | fb(Sh.y) | fb(Nh.y) | fb(Bh.y) | fb(Th.y) : 0u)) & 0x7FFFFFFFu;
+    float2 rh = zero, rl = zero;
+    if (__any_sync(0xffffffffu, any != 0u)) {
+      // left and right neighbours of both cells: (L, c0), (c1, R); a lone last
+      // cell's right neighbour is R
+      const f2x2 W = {vset(Lh, ch.x), vset(Ll, cl.x)};
+      const f2x2 E = {vset(in1 ? ch.y : Rh, Rh), vset(in1 ? cl.y : Rl, Rl)};
+      f2x2 t = two_sum(W.hi, E.hi);
+      v2 lo = vadd(vadd(W.lo, E.lo), t.lo);
+      auto more = [&](float2 h, float2 l) {
+        t = two_sum(t.hi, vset(h.x, h.y));
+        lo = vadd(lo, vadd(vset(l.x, l.y), t.lo));
+      };
+      more(Sh, Sl);
+      more(Nh, Nl);
+      more(Bh, Bl);
+      more(Th, Tl);
+      const float2 B0 = K.Bf[(c0 & kDifLiq) ? 1 : 0][__popc(c0 & 63u)], B1 = K.Bf[(c1 & kDifLiq) ? 1 : 0][__popc(c1 & 63u)];
+      const f2x2 r = add_c(mul(fast_two_sum(t.hi, lo), f2x2{vset(B0.x, B1.x), vset(B0.y, B1.y)}),
+                           f2x2{vset(sh.x, sh.y), vset(sl.x, sl.y)});
+      vget(r.hi, rh.x, rh.y);
+      vget(r.lo, rl.x, rl.y);
+      if (__any_sync(0xffffffffu, ((c0 | c1) & kDifIrr) != 0u)) {
+        // cells next to the interface or a heated wall: their own couplings
+        const size_t i = ((size_t)z * ny + y) * nx + x;
+        const float2 n0[6] = {make_float2(Lh, Ll), in1 ? make_float2(ch.y, cl.y) : make_float2(Rh, Rl),
+                              make_float2(Sh.x, Sl.x), make_float2(Nh.x, Nl.x), make_float2(Bh.x, Bl.x), make_float2(Th.x, Tl.x)};
+        const float2 n1[6] = {make_float2(ch.x, cl.x), make_float2(Rh, Rl), make_float2(Sh.y, Sl.y),
+                              make_float2(Nh.y, Nl.y), make_float2(Bh.y, Bl.y), make_float2(Th.y, Tl.y)};
+        f2 e0 = f2{sh.x, sl.x}, e1 = f2{sh.y, sl.y};
+        const float2* off = reinterpret_cast<const float2*>(v.off) + 6 * i;
+#pragma unroll
+        for (int f = 0; f < 6; ++f) {
+          if ((c0 & kDifIrr) && (c0 & (1u << f))) e0 = add_c(mul(f2_of(__ldg(off + f)), f2_of(n0[f])), e0);
+          if ((c1 & kDifIrr) && (c1 & (1u << f))) e1 = add_c(mul(f2_of(__ldg(off + 6 + f)), f2_of(n1[f])), e1);
+        }
+        if (c0 & kDifIrr) { rh.x = e0.hi; rl.x = e0.lo; }
+        if (c1 & kDifIrr) { rh.y = e1.hi; rl.y = e1.lo; }
+      }
+    }
+    if (in) {
+      *reinterpret_cast<float2*>(dout + ip) = rh;
+      *reinterpret_cast<float2*>(dout + v.pn + ip) = rl;
+    }
+    if (CHECK) {
+      dmax = fmaxf(dmax, fabsf((rh.x - ch.x) + (rl.x - cl.x)));
+      if (in1) dmax = fmaxf(dmax, fabsf((rh.y - ch.y) + (rl.y - cl.y)));
+    }
+  }
+  if constexpr (CHECK) dif_change(dmax, dif_scale(v, K), change);
+}
+
+// e' = e + C_p,node d; a node without change keeps its e
+__global__ void __launch_bounds__(kDifThreads)
+k_dif_store_phase(GridDev g, const DifVec v, DifConst K, const float* __restrict__ d, double* __restrict__ e) {
+  const int ks = dif_scale(v, K);
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+  if (x >= g.n[0] || y >= g.n[1]) return;
+  for (int z = blockIdx.z; z < g.n[2]; z += gridDim.z) {
+    const size_t i = ((size_t)z * g.n[1] + y) * g.n[0] + x, ip = pad_id(g, v, x, y, z);
+    const float hi = __ldg(d + ip), lo = __ldg(d + v.pn + ip);
+    if (hi == 0.f && lo == 0.f) continue;
+    const double Cd = (__ldg(v.cls + i) & kDifLiq) ? g.Cp_l : g.Cp_g;
+    e[i] = e[i] + Cd * (wide_of(hi, ks) + wide_of(lo, ks));
+  }
+}
+
+// e' = C_p(c) T' (mixture form)
+__global__ void k_dif_store(GridDev g, const double* __restrict__ c, const double* __restrict__ T,
+                            double* __restrict__ e, size_t N) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
+    const double cv = __ldg(c + i);
+    const double Cp = g.Cp_l * cv + g.Cp_g * (1.0 - cv);
+    e[i] = Cp * T[i];
   }
 }
 
@@ -473,7 +740,7 @@ DifLayout dif_layout(size_t N) {
   L.T0 = o; o += a(N * 8);
   L.Ta = o; o += a(N * 8);
   L.Tb = o; o += a(N * 8);
-  L.part = o; o += 256;  // the largest change (bits of a non-negative double)
+  L.part = o; o += a(kDifChecks * 8);  // the checks' largest changes (bits of non-negative doubles)
   L.cls = o; o += a(N);
   L.mlist = o; o += a(N * 4);
   L.count = o; o += 256;
@@ -500,16 +767,24 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   v.T0 = reinterpret_cast<double*>(ws + L.T0);
   v.Ta = reinterpret_cast<double*>(ws + L.Ta);
   v.Tb = reinterpret_cast<double*>(ws + L.Tb);
-  v.part = reinterpret_cast<double*>(ws + L.part);
+  v.part = reinterpret_cast<unsigned long long*>(ws + L.part);
   v.cls = reinterpret_cast<uint8_t*>(ws + L.cls);
+  // the padded pairs (px / nx <= 2 cell arrays each): s in diag's and rhs's
+  // place, the iterates in the planes' (not read any more when they are written)
+  v.px = (g.n[0] + 1) & ~1;
+  v.pn = (size_t)v.px * g.n[1] * g.n[2];
+  v.s = reinterpret_cast<float*>(ws + L.diag);
+  v.d[0] = reinterpret_cast<float*>(ws + L.plane);
+  v.d[1] = v.d[0] + 2 * v.pn;
   uint32_t* mlist = reinterpret_cast<uint32_t*>(ws + L.mlist);
   int* count = reinterpret_cast<int*>(ws + L.count);
+  v.tmax = count + 2;
   *status = 0;
   const int grid = (int)std::min<size_t>((N + kDifThreads - 1) / kDifThreads, (size_t)kDifCTAs);
-  cudaError_t err = cudaMemsetAsync(count, 0, 2 * sizeof(int), st);
+  cudaError_t err = cudaMemsetAsync(count, 0, 3 * sizeof(int), st);
   if (err != cudaSuccess) return err;
   k_dif_mlist<<<grid, kDifThreads, 0, st>>>(g, c, mlist, count, N);
-  k_dif_planes<<<grid, kDifThreads, 0, st>>>(g, c, mlist, count, plane);
+  k_dif_planes<<<kDifCTAs, kDifPlaneThreads, 0, st>>>(g, c, mlist, count, plane);
   prof_mark("diffuse.planes", st);
   DifWalls walls;
   for (int f = 0; f < 6; ++f) {
@@ -526,9 +801,15 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
     double d = K.cdt[p];
     for (int n = 0; n <= 6; ++n) {
       K.rdiag[p][n] = 1.0 / d;
+      K.B[p][n] = K.kq[p] * K.rdiag[p][n];
+      K.Bf[p][n].x = (float)K.B[p][n];
+      K.Bf[p][n].y = (float)(K.B[p][n] - (double)K.Bf[p][n].x);
       d += K.kq[p];
     }
   }
+  auto exponent = [](double x) { return std::isfinite(x) && x != 0.0 ? std::max(0, std::ilogb(x) + 1023) : 0; };
+  K.e0 = exponent(g.T_sat);
+  for (int f = 0; f < 6; ++f) K.e0 = std::max(K.e0, exponent(walls.T[f]));
   // the cells next to the interface or a heated wall are listed in the
   // mixed-cell list's storage (k_dif_planes is done with it)
   uint32_t* ilist = mlist;
@@ -538,38 +819,73 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   k_dif_irregular<<<grid, kDifThreads, 0, st>>>(g, h, inv_h, inv_dt, k_l, k_g, c, e, plane, v, walls, phase_cp, K,
                                                  ilist, count + 1);
   prof_mark("diffuse.assemble", st);
-  unsigned long long* chg = reinterpret_cast<unsigned long long*>(v.part);
-  // T0 is the first iterate; Ta and Tb take turns after it
-  const double* Tin = v.T0;
-  double* Tout = v.Ta;
-  double* Tnext = v.Tb;
-  int it = 0;
-  double change = 0.0;
+  // Sweeps in batches, each with its checks' slots cleared first: a sweep
+  // queued behind a check that was within tol returns at once (its slot stays
+  // 0, so the ones behind it do too), and the host reads a batch's slots
+  // together.  The batches grow, cut short where the last checks' rate says
+  // when tol will be met.
+  unsigned long long* slot = v.part;
+  // the iterates: T0, then Ta and Tb in turn (phase form: s, the first sweep's
+  // result, then d[0] and d[1])
+  double* buf[2] = {v.Ta, v.Tb};
+  int it = 0, batch = 2;
+  double change = 0.0, before = 0.0;
   bool done = false;
+  auto iterate = [&](int n) -> double* { return n == 0 ? v.T0 : buf[n & 1]; };  // the n-th sweep's result
+  auto iterate_d = [&](int n) -> float* { return n <= 1 ? v.s : v.d[n & 1]; };
+  // two cells of a row per thread
+  const dim3 pgrid((unsigned)((g.n[0] + 63) / 64), sgrid.y,
+                   (unsigned)std::max(1, std::min(g.n[2], (int)(152u * 16u / std::max(1u, (unsigned)((g.n[0] + 63) / 64) * sgrid.y)))));
   while (!done && it < max_iter) {
-    const bool check = (it + 1) % 4 == 0 || it + 1 == max_iter;
-    if (check) {
-      err = cudaMemsetAsync(chg, 0, sizeof(unsigned long long), st);
-      if (err != cudaSuccess) return err;
-      k_dif_jacobi<true><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, Tin, Tout, chg, phase_cp);
-    } else {
-      k_dif_jacobi<false><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, Tin, Tout, chg, phase_cp);
+    err = cudaMemsetAsync(slot, 0, kDifChecks * sizeof(unsigned long long), st);
+    if (err != cudaSuccess) return err;
+    int nc = 0;
+    const unsigned long long* prev = nullptr;
+    int at[kDifChecks];
+    while (it < max_iter && nc < batch) {
+      const bool check = (it + 1) % 4 == 0 || it + 1 == max_iter;
+      unsigned long long* chg = check ? slot + nc : nullptr;
+      const double* in = iterate(it);
+      double* out = iterate(it + 1);
+      if (phase_cp && it == 0) {
+        if (check) k_dif_first<true><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, chg);
+        else k_dif_first<false><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, chg);
+      } else if (phase_cp) {
+        const float* di = iterate_d(it);
+        float* dd = iterate_d(it + 1);
+        if (check) launch_pdl(k_dif_sweep<true>, pgrid, dim3(32, 8), st, g, v, K, di, dd, prev, tol, chg);
+        else launch_pdl(k_dif_sweep<false>, pgrid, dim3(32, 8), st, g, v, K, di, dd, prev, tol, chg);
+      } else {
+        if (check) k_dif_jacobi<true><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, in, out, prev, tol, chg);
+        else k_dif_jacobi<false><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, in, out, prev, tol, chg);
+      }
+      ++it;
+      if (check) {
+        at[nc] = it;
+        prev = slot + nc++;
+      }
     }
-    Tin = Tout;
-    std::swap(Tout, Tnext);
-    ++it;
-    if (check) {
-      unsigned long long hb = 0ull;
-      err = cudaMemcpyAsync(&hb, chg, sizeof(hb), cudaMemcpyDeviceToHost, st);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(st);
-      if (err != cudaSuccess) return err;
-      std::memcpy(&change, &hb, sizeof(change));
+    unsigned long long hb[kDifChecks];
+    err = cudaMemcpyAsync(hb, slot, nc * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
+    if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+    if (err != cudaSuccess) return err;
+    for (int k = 0; k < nc && !done; ++k) {
+      before = change;
+      std::memcpy(&change, &hb[k], sizeof(change));
       done = change <= tol;
+      if (done) it = at[k];
+    }
+    batch = batch * 2 < kDifChecks ? batch * 2 : kDifChecks;
+    if (!done && change > 0.0 && before > change) {
+      // checks until tol at the last pair's rate
+      const double more = std::log(change / tol) / std::log(before / change);
+      if (more + 1.0 < (double)batch) batch = (int)more + 1;
     }
   }
   prof_mark("diffuse.jacobi", st);
   if (!done) *status = 2;
-  k_dif_store<<<grid, kDifThreads, 0, st>>>(g, c, v, Tin, e, N, phase_cp);
+  if (phase_cp) k_dif_store_phase<<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, iterate_d(it), e);
+  else k_dif_store<<<grid, kDifThreads, 0, st>>>(g, c, iterate(it), e, N);
   prof_mark("diffuse.store", st);
   if (iters_out) *iters_out = it;
   if (change_out) *change_out = change;
