@@ -15,17 +15,25 @@
 // as preconditioner; then u~ = -(dt / rho_f) (p~_R - p~_L) / h on every face
 // with a sub-domain cell on one side and no liquid cell or wall.
 //
-// Kernels: k_ext_init / k_ext_dilate (layer codes, full grid, 1 B per
-// cell), k_ext_list (compact the unknowns), k_ext_assemble (the six
-// couplings and the source of each unknown, CG start), the CG iterations,
-// and k_ext_faces (the face correction, full face grid per axis).  The CG
-// iterations run in one cooperative launch, k_ext_cg: its CTAs pass three
-// grid barriers per iteration (after the matrix product, the update and the
-// new direction) and test the residual every iteration on the device; where
-// a cooperative launch of that size is refused, the same three phases run as
-// the kernels k_ext_spmv, k_ext_update, k_ext_dir with a host test every 8
-// iterations.  Inner products are per-CTA partial sums that every CTA adds
-// up in the same fixed order, so all CTAs use the same scalars.
+// Kernels: k_ext_init (stream c: a code per cell, the mixed cells listed),
+// k_ext_layer (the two gas layers, from the list of the layer before: the
+// unknowns), k_ext_assemble (the six couplings and the source of each
+// unknown), the CG iterations, and k_ext_faces (the correction on the faces of
+// the unknowns).  Everything after the stream works on the list; whole-grid
+// dilations, listing and face passes took 50 + 82 us at 160^3.
+//
+// The CG iterations run in one cooperative launch, k_ext_cg, one grid barrier
+// each: the single-reduction form of Chronopoulos and Gear (1989) keeps s = M p
+// by recurrence, so that both inner products belong to the same point of the
+// iteration, and every thread forms its neighbours' new residuals again from
+// their records {r, w, s, 1 / diag} (one 32-byte sector each; the owner's
+// arithmetic) instead of waiting for them.  What bounds an iteration is the
+// barrier and the chain of its sums (~15,000 unknowns are one per thread): the
+// two-barrier form took 18.7 us per iteration at 160^3.  Where a cooperative
+// launch of that size is refused, the standard iteration runs as the kernels
+// k_ext_spmv, k_ext_update, k_ext_dir with a host test every 8 iterations.
+// Inner products are per-CTA partial sums that every CTA adds up in the same
+// fixed order, so all CTAs use the same scalars.
 #include <algorithm>
 #include <vector>
 
@@ -38,11 +46,15 @@ namespace {
 
 constexpr uint8_t kOut = 255;  // pure liquid
 constexpr uint8_t kGas = 254;  // pure gas beyond the layers reached so far
+constexpr uint8_t kLayer = 2;  // pure gas of the two layers (unknowns, with the mixed cells' 0)
 constexpr int kExtThreads = 256;    // grid-wide cell and face kernels
 constexpr int kSolveThreads = 256;   // the CG kernels: one CTA per SM (few warps per FP64 sum tree)
 constexpr int kExtCTAs = 152;
 constexpr int kNoNb = -1;       // no-slip face (liquid cell or wall)
 constexpr int kFreeNb = -2;     // free-flow face (p~ = 0 beyond)
+// counters: [0] unknowns, [1] free-flow faces, [2], [3], [4] mixed cells, first
+// and second layer
+constexpr int kCntMixed = 2, kCnts = 5;
 
 // face neighbour of (x, y, z) along `axis` in direction d (+-1): false
 // across a zero-gradient wall
@@ -65,110 +77,69 @@ __device__ __forceinline__ size_t cid(const GridDev& g, int x, int y, int z) {
 
 __device__ __forceinline__ bool is_gas_b(double c, const GridDev& g) { return dbits(c) <= g.eps_bits; }
 
-__global__ void k_ext_init(GridDev g, const double* __restrict__ c, uint8_t* __restrict__ code, size_t N) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
-    const double cv = __ldg(c + i);
-    code[i] = is_mixed_b(cv, g) ? (uint8_t)0 : (is_gas_b(cv, g) ? kGas : kOut);
-  }
-}
-
-// gas cells next (across a face) to layer L - 1 join layer L
-__global__ void k_ext_dilate(GridDev g, uint8_t* __restrict__ code, int L, size_t N) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
-    if (code[i] != kGas) continue;
-    int x, y, z;
-    cell_xyz(g, i, x, y, z);
-    bool hit = false;
-    for (int axis = 0; axis < 3 && !hit; ++axis)
-      for (int d = -1; d <= 1 && !hit; d += 2) {
-        int qx, qy, qz;
-        if (face_nb(g, x, y, z, axis, d, qx, qy, qz) && code[cid(g, qx, qy, qz)] == (uint8_t)(L - 1)) hit = true;
-      }
-    if (hit) code[i] = (uint8_t)L;
-  }
-}
-
-__device__ __forceinline__ void warp_append_ext(bool take, uint32_t v, uint32_t* list, int* counter, int* slot) {
+// entries appended to a list by a warp, one atomic
+__device__ __forceinline__ int warp_append_ext(bool take, uint32_t v, uint32_t* list, int* counter) {
   const unsigned mask = __ballot_sync(0xffffffffu, take);
-  *slot = -1;
-  if (!mask) return;
+  if (!mask) return -1;
   const int lane = threadIdx.x & 31;
   int base = 0;
   if (lane == __ffs(mask) - 1) base = atomicAdd(counter, __popc(mask));
   base = __shfl_sync(0xffffffffu, base, __ffs(mask) - 1);
-  if (take) {
-    *slot = base + __popc(mask & ((1u << lane) - 1u));
-    list[*slot] = v;
-  }
+  if (!take) return -1;
+  const int slot = base + __popc(mask & ((1u << lane) - 1u));
+  list[slot] = v;
+  return slot;
 }
 
-// the unknowns: every sub-domain cell (layer 0, 1, 2), and the map from
-// cells to unknowns (-1 outside)
-__global__ void k_ext_list(const uint8_t* __restrict__ code, uint32_t* __restrict__ list, int* __restrict__ map,
-                           int* __restrict__ counter, size_t N) {
+// code of every cell; the mixed cells are the first unknowns (list, map)
+__global__ void __launch_bounds__(kExtThreads)
+k_ext_init(GridDev g, const double* __restrict__ c, uint8_t* __restrict__ code, uint32_t* __restrict__ list,
+           int* __restrict__ map, int* __restrict__ counters, size_t N) {
   const size_t stride = (size_t)gridDim.x * blockDim.x;
-  const size_t n_iter = (N + stride - 1) / stride;
+  const size_t n_iter = (N + stride - 1) / stride;  // whole warps iterate together
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (size_t it = 0; it < n_iter; ++it, i += stride) {
-    const bool take = i < N && code[i] <= 2;
-    int slot;
-    warp_append_ext(take, (uint32_t)i, list, counter, &slot);
-    if (i < N) map[i] = slot;
+    bool mx = false;
+    if (i < N) {
+      const double cv = __ldg(c + i);
+      mx = is_mixed_b(cv, g);
+      code[i] = mx ? (uint8_t)0 : (is_gas_b(cv, g) ? kGas : kOut);
+    }
+    const int slot = warp_append_ext(mx, (uint32_t)i, list, counters + kCntMixed);
+    if (mx) map[i] = slot;
   }
 }
 
-// area of the plane m . x = alpha inside the unit cube: the cut polygon
-// projected on the coordinate plane normal to m's largest component,
-// vertices ordered by angle about their mean, shoelace area, divided by
-// that component of the unit normal
-__device__ double cut_area(const double m[3], double alpha) {
-  double px[24], py[24];
-  const double am0 = fabs(m[0]), am1 = fabs(m[1]), am2 = fabs(m[2]);
-  const int dom = (am0 >= am1 && am0 >= am2) ? 0 : (am1 >= am2 ? 1 : 2);
-  const int ia = dom == 0 ? 1 : 0, ib = dom == 2 ? 1 : 2;
-  int np = 0;
-  for (int ax = 0; ax < 3; ++ax) {
-    const int b1 = (ax + 1) % 3, b2 = (ax + 2) % 3;
-    for (int u = 0; u < 2; ++u)
-      for (int v = 0; v < 2; ++v) {
-        double p0[3], p1[3];
-        p0[ax] = 0.0; p0[b1] = u; p0[b2] = v;
-        p1[ax] = 1.0; p1[b1] = u; p1[b2] = v;
-        const double f0 = (m[0] * p0[0] + m[1] * p0[1] + m[2] * p0[2]) - alpha;
-        const double f1 = (m[0] * p1[0] + m[1] * p1[1] + m[2] * p1[2]) - alpha;
-        if (f0 == 0.0 && np < 24) { px[np] = p0[ia]; py[np] = p0[ib]; ++np; }
-        if (f1 == 0.0 && np < 24) { px[np] = p1[ia]; py[np] = p1[ib]; ++np; }
-        if (((f0 < 0.0 && f1 > 0.0) || (f0 > 0.0 && f1 < 0.0)) && np < 24) {
-          const double t = f0 / (f0 - f1);
-          double q[3] = {p0[0], p0[1], p0[2]};
-          q[ax] = t;
-          px[np] = q[ia]; py[np] = q[ib]; ++np;
+// The gas cells next (across a face) to the unknowns of the layer before (the
+// mixed cells; then the first layer) join the list behind them.  One bit mask
+// per claim: kGas becomes kLayer, and the thread that sees kGas lists the cell.
+__global__ void __launch_bounds__(kExtThreads)
+k_ext_layer(GridDev g, uint8_t* __restrict__ code, uint32_t* __restrict__ list, int* __restrict__ map,
+            int* __restrict__ counters, int layer) {
+  const int nm = counters[kCntMixed], n1 = layer == 1 ? 0 : counters[kCntMixed + 1];
+  const int b = layer == 1 ? 0 : nm, n = nm + n1;  // the sources; the new entries start at n
+  // eight threads per source, six of them a face each
+  const long long stride = (long long)gridDim.x * blockDim.x, total = 8ll * (n - b);
+  for (long long j0 = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); j0 < total; j0 += stride) {
+    const long long j = j0 + (threadIdx.x & 31);
+    const int f = (int)(j & 7);
+    bool take = false;
+    size_t q = 0;
+    if (j < total && f < 6) {
+      int x, y, z, qx, qy, qz;
+      cell_xyz(g, list[b + (j >> 3)], x, y, z);
+      if (face_nb(g, x, y, z, f >> 1, (f & 1) ? 1 : -1, qx, qy, qz)) {
+        q = cid(g, qx, qy, qz);
+        if (code[q] == kGas) {  // (it may have been claimed since: the mask keeps kLayer)
+          const int sh = 8 * (int)(q & 3);
+          const unsigned old = atomicAnd(reinterpret_cast<unsigned*>(code + (q & ~(size_t)3)), ~((unsigned)(kGas ^ kLayer) << sh));
+          take = ((old >> sh) & 0xFFu) == kGas;
         }
       }
-  }
-  if (np < 3) return 0.0;
-  double cx = 0.0, cy = 0.0;
-  for (int q = 0; q < np; ++q) { cx += px[q]; cy += py[q]; }
-  cx /= np; cy /= np;
-  double ang[24];
-  for (int q = 0; q < np; ++q) ang[q] = atan2(py[q] - cy, px[q] - cx);
-  for (int a = 1; a < np; ++a) {  // insertion sort by angle
-    const double ka = ang[a], kx = px[a], ky = py[a];
-    int b = a - 1;
-    while (b >= 0 && ang[b] > ka) {
-      ang[b + 1] = ang[b]; px[b + 1] = px[b]; py[b + 1] = py[b];
-      --b;
     }
-    ang[b + 1] = ka; px[b + 1] = kx; py[b + 1] = ky;
+    const int slot = warp_append_ext(take, (uint32_t)q, list + n, counters + kCntMixed + layer);
+    if (take) map[q] = n + slot;
   }
-  double s = 0.0;
-  for (int q = 0; q < np; ++q) {
-    const int r = q + 1 == np ? 0 : q + 1;
-    s += (px[q] - cx) * (py[r] - cy) - (px[r] - cx) * (py[q] - cy);
-  }
-  const double len = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
-  const double nd = fabs(m[dom]) / len;
-  return 0.5 * fabs(s) / nd;
 }
 
 // Fixed-order sums of the per-CTA partials (the same values in every CTA):
@@ -199,21 +170,6 @@ __device__ __forceinline__ void sum_partials_k(const double* const (&part)[K], i
 #pragma unroll
   for (int k = 0; k < K; ++k) out[k] = res[k];
 }
-// The same sums in warp 0 alone (valid in its lane 0), for a scalar step
-// that lane 0 takes before sharing the result.
-template <int K, bool L2>
-__device__ __forceinline__ void warp0_sums(const double* const (&part)[K], int n, double (&out)[K]) {
-#pragma unroll
-  for (int k = 0; k < K; ++k) out[k] = 0.0;
-  for (int i = threadIdx.x; i < n; i += 32)
-#pragma unroll
-    for (int k = 0; k < K; ++k) out[k] += L2 ? __ldcg(part[k] + i) : part[k][i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int k = 0; k < K; ++k) out[k] += __shfl_down_sync(0xffffffffu, out[k], o);
-}
-
 // A CTA's partial sums of K values in a fixed order (the threads' values
 // staged in shared memory; warp 0 sums them, each lane its entries lane,
 // lane + 32, ... in order, then a shuffle tree: few FP64 instructions per
@@ -247,6 +203,11 @@ __device__ __forceinline__ void block_partial(double v, double* __restrict__ out
   block_partial_k<1>(vv, o);
 }
 
+// one unknown's state of the cooperative solver: a 32-byte sector
+struct __align__(32) ExtRec {
+  double r, w, s, rdiag;
+};
+
 struct ExtVec {
   int* nb;        // [6 n]: neighbour unknown, kNoNb, or kFreeNb
   double* beta;   // [6 n]
@@ -255,20 +216,37 @@ struct ExtVec {
   double* x;      // p~
   double* r;
   double* d;
-  double* d2;     // the cooperative solver's second direction buffer (the two take turns)
   double* q;
-  double* part;   // [5][kExtCTAs]: b.b, r.z (two, alternating), d.q, r.r
-  int* counters;  // [0] unknowns, [1] free-flow faces
+  ExtRec* rec[2]; // the cooperative solver's records, the two taking turns (in r, q and their
+  int cap;        // spare's place, for up to cap unknowns)
+  double* part;   // [6][kExtCTAs]: b.b, r.z (two, alternating), d.q, r.r; cooperative: two sets of three
+  int* counters;  // [kCnts]
 };
 
-__global__ void __launch_bounds__(kExtThreads)  // (heavy per unknown: no register cap)
+// area of the plane m . x = alpha inside the unit cube: |m|_2 dV/dalpha, the
+// slope of the volume's branch form (a polygon's vertices sorted by angle took
+// ~800 FP64 instructions)
+__device__ __forceinline__ double cut_area(const double m[3], double alpha) {
+  const Mirror r = mirror_normalise(m[0], m[1], m[2]);
+  if (!dnz(r.l1)) return 0.0;
+  const double a0 = div_by(alpha + r.sh, r.R);
+  const double a = nn_lt(0.5, a0) ? 1.0 - a0 : a0;
+  if (!dgt0(a)) return 0.0;
+  double slope = 0.0;
+  (void)vol_eval<true>(vol_form(r.mp[0], r.mp[1], r.mp[2]), a, slope);
+  return div_by(slope, r.R) * sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+}
+
+constexpr int kAsmThreads = 64;  // few unknowns, long chains: spread over the SMs
+__global__ void __launch_bounds__(kAsmThreads)  // (heavy per unknown: no register cap)
 k_ext_assemble(GridDev g, double h, double dt, double rho_l, double rho_g, const double* __restrict__ c,
                const double* __restrict__ mdot, const uint8_t* __restrict__ code, const int* __restrict__ map,
                const uint32_t* __restrict__ list, ExtVec v, unsigned char* __restrict__ cg_state) {
-  const int n = v.counters[0];
+  const int n = v.counters[kCntMixed] + v.counters[kCntMixed + 1] + v.counters[kCntMixed + 2];
   if (blockIdx.x == 0 && threadIdx.x < 32) reinterpret_cast<unsigned long long*>(cg_state)[threadIdx.x] = 0ull;
-  double bb = 0.0, rz = 0.0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) v.counters[0] = n;  // read by the kernels after this one
   int free_faces = 0;
+  const Rcp rhh = rcp_of(h * h);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint32_t id = list[i];
     int x, y, z;
@@ -286,7 +264,7 @@ k_ext_assemble(GridDev g, double h, double dt, double rho_l, double rho_g, const
         if (qc != kOut) {
           const double cf = 0.5 * (cp + __ldg(c + qid));
           const double rho = rho_l * cf + rho_g * (1.0 - cf);
-          beta = (dt / rho) / (h * h);
+          beta = div_by(div_by(dt, rcp_of(rho)), rhh);
           nb = qc <= 2 ? map[qid] : kFreeNb;
           if (nb == kFreeNb) ++free_faces;
         }
@@ -315,27 +293,38 @@ k_ext_assemble(GridDev g, double h, double dt, double rho_l, double rho_g, const
     v.diag[i] = dsum;
     v.rdiag[i] = rd;
     v.x[i] = 0.0;
-    v.r[i] = b;
-    const double zi = b * rd;
-    v.d[i] = zi;
-    bb = fma(b, b, bb);
-    rz = fma(b, zi, rz);
+    if (n <= v.cap) {
+      v.rec[0][i] = ExtRec{b, 0.0, 0.0, rd};
+    } else {
+      v.r[i] = b;
+      v.d[i] = b * rd;
+    }
   }
   if (free_faces) atomicAdd(v.counters + 1, free_faces);
+}
+
+// b . b and r . z of the start (the kernel-per-phase solver)
+__global__ void __launch_bounds__(kSolveThreads) k_ext_start(ExtVec v) {
+  const int n = v.counters[0];
+  double bb = 0.0, rz = 0.0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double b = v.r[i];
+    bb = fma(b, b, bb);
+    rz = fma(b, v.d[i], rz);
+  }
   const double pv[2] = {bb, rz};
   double* const po[2] = {v.part, v.part + kExtCTAs};
   block_partial_k<2>(pv, po);
 }
 
-// The element arithmetic of one CG iteration (both forms of the solver use
-// it): q = M d with its partial d . q; x += alpha d, r -= alpha q, z = r /
+// The element arithmetic of one iteration of the kernel-per-phase solver: q = M d with its partial d . q; x += alpha d, r -= alpha q, z = r /
 // diag with the partials r . z and r . r; d = z + beta d.
-__device__ __forceinline__ double ext_spmv_elem(const ExtVec& v, int i, bool l2) {
+__device__ __forceinline__ double ext_spmv_elem(const ExtVec& v, int i) {
   double q = v.diag[i] * v.d[i];
 #pragma unroll
   for (int f = 0; f < 6; ++f) {
     const int nb = v.nb[6 * (size_t)i + f];
-    if (nb >= 0) q = fma(-v.beta[6 * (size_t)i + f], l2 ? __ldcg(v.d + nb) : v.d[nb], q);  // another CTA's
+    if (nb >= 0) q = fma(-v.beta[6 * (size_t)i + f], v.d[nb], q);
   }
   v.q[i] = q;
   return q;
@@ -346,7 +335,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_ext_spmv(ExtVec v) {
   const int n = v.counters[0];
   double dq = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    dq = fma(v.d[i], ext_spmv_elem(v, i, false), dq);
+    dq = fma(v.d[i], ext_spmv_elem(v, i), dq);
   block_partial(dq, v.part + 3 * kExtCTAs);
 }
 
@@ -389,14 +378,12 @@ __global__ void __launch_bounds__(kSolveThreads) k_ext_dir(ExtVec v, int cur) {
 
 // Device state of the persistent solver (in the workspace; the assemble
 // kernel clears it).
-constexpr int kBarGroup = 32;  // CTAs per first-level arrival counter
 struct ExtCG {
-  unsigned arrive;  // grid barrier: groups arrived at the current barrier
+  unsigned arrive;  // grid barrier: CTAs arrived at the current barrier
   unsigned gen;     // grid barrier: barriers completed
   int iters;        // iterations done
-  int flag;         // 1 converged, 2 iteration limit, 3 a barrier wait gave up
+  int flag;         // 1 converged, 2 iteration limit, 3 a barrier wait gave up, 4 not solved here
   double res;       // |r| at the end
-  unsigned sub[(kExtCTAs + kBarGroup - 1) / kBarGroup];  // CTAs arrived, per group
 };
 static_assert(sizeof(ExtCG) <= 256, "the solver state lives in 256 bytes of the workspace");
 
@@ -406,11 +393,11 @@ __device__ __forceinline__ unsigned long long ext_now_ns() {
   return t;
 }
 
-// Grid barrier of a cooperative launch (all CTAs resident): each CTA
-// arrives on its group's counter, the last of a group on the top counter,
-// and the last group starts the next generation (two short chains of
-// atomics instead of one of all CTAs).  The wait is bounded (1 s): on
-// expiry the CTA records DEV_WAIT and returns false, and the solver stops.
+// Grid barrier of a cooperative launch (all CTAs resident): the last of the
+// CTAs to arrive starts the next generation, which the others poll (an atomic
+// and a load from L2; a tree of counters and a sleeping poll took longer).  The
+// wait is bounded (1 s): on expiry the CTA records DEV_WAIT and returns false,
+// and the solver stops.
 __device__ __forceinline__ bool ext_grid_barrier(ExtCG* cg, int* status) {
   __shared__ int ok_s;
   __syncthreads();
@@ -419,15 +406,7 @@ __device__ __forceinline__ bool ext_grid_barrier(ExtCG* cg, int* status) {
     volatile unsigned* vgen = &cg->gen;
     const unsigned g0 = *vgen;
     __threadfence();  // this CTA's writes, and g0, before its arrival
-    const unsigned grp = blockIdx.x / kBarGroup, ngrp = (gridDim.x + kBarGroup - 1) / kBarGroup;
-    const unsigned gsize = min((unsigned)kBarGroup, gridDim.x - grp * kBarGroup);
-    bool last = false;
-    if (atomicAdd(&cg->sub[grp], 1u) == gsize - 1) {
-      atomicExch(&cg->sub[grp], 0u);
-      __threadfence();
-      last = atomicAdd(&cg->arrive, 1u) == ngrp - 1;
-    }
-    if (last) {
+    if (atomicAdd(&cg->arrive, 1u) == gridDim.x - 1) {
       atomicExch(&cg->arrive, 0u);
       __threadfence();
       atomicAdd(&cg->gen, 1u);
@@ -439,7 +418,6 @@ __device__ __forceinline__ bool ext_grid_barrier(ExtCG* cg, int* status) {
           if (status) atomicOr(status, DEV_WAIT);
           break;
         }
-        __nanosleep(32);
       }
     }
     __threadfence();  // the other CTAs' writes before this CTA reads them
@@ -449,169 +427,197 @@ __device__ __forceinline__ bool ext_grid_barrier(ExtCG* cg, int* status) {
   return ok_s != 0;
 }
 
-// The CG iterations in one launch, two grid barriers per iteration: the
-// direction d_k = z_k + beta_k d_(k-1) (d_0 = z_0) is formed where the
-// matrix product needs it -- each thread its own elements, written to the
-// other of two buffers, and the neighbours' again from their r and previous
-// d, the same arithmetic, so the values are the owners' -- and the product,
-// its partial d . q, then (after a barrier) alpha, x += alpha d, r -=
-// alpha q and the partials r . z, r . r (then a barrier) follow; beta and
-// |r| are formed from those partials at the top of the next iteration.  The
-// same element arithmetic, partial slots and grid as k_ext_spmv,
-// k_ext_update and k_ext_dir, so both forms of the solver give the same
-// iterates.  The iteration's scalars are formed once per CTA by thread 0
-// and shared; partials written by other CTAs are read from L2.
+__device__ __forceinline__ ExtRec rec_l2(const ExtRec* p) {  // written by other CTAs of this launch: from L2
+  const double2 a = __ldcg(reinterpret_cast<const double2*>(p)), b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
+  return ExtRec{a.x, a.y, b.x, b.y};
+}
+
+// One pass per iteration (the first, with alpha = beta = 0, only forms u = r /
+// diag, w = M u and the inner products of the start):
+//   s <- w + beta s, r <- r - alpha s, u = r / diag, w = M u,
+//   p <- u_old + beta p, x <- x + alpha p;  gamma = r.u, delta = w.u, |r|^2
+// then beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha).
 __global__ void __launch_bounds__(kSolveThreads)
 k_ext_cg(ExtVec v, ExtCG* cg, double tol, int max_iter, int* status) {
-  // [0] alpha, [1] beta, [2] r.z, [3] |r|, [4] target
-  __shared__ double scal[5];
+  __shared__ double red[3][kSolveThreads];
+  __shared__ double tot[3];
   const int n = v.counters[0];
-  if (threadIdx.x < 32) {
-    const double* pp[2] = {v.part, v.part + kExtCTAs};
-    double s2[2];
-    warp0_sums<2, true>(pp, kExtCTAs, s2);
-    if (threadIdx.x == 0) {
-      scal[2] = s2[1];
-      scal[3] = sqrt(s2[0]);
-      scal[4] = tol * scal[3];
-    }
+  if (n == 0 || v.counters[1] == 0 || n > v.cap) {  // the same in every CTA
+    if (blockIdx.x == 0 && threadIdx.x == 0) cg->flag = 4;
+    return;
   }
-  __syncthreads();
-  double rz = scal[2];  // r.z, carried between phases
-  double res = scal[3];
-  const double target = scal[4];
-  double* dcur = v.d;   // d_(k-1); d_0 itself in the first iteration
-  double* dnew = v.d2;  // d_k
-  int cur = 0, it = 0;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // unknown i is CTA i mod grid's: a few thousand of them reach every SM, and
+  // its partitions' FP64 units share them; the first of a thread keeps its
+  // couplings in registers
+  const int i0 = blockIdx.x + gridDim.x * threadIdx.x, step = gridDim.x * blockDim.x;
+  const int rows = min(kSolveThreads / 32, ((n - 1) / (int)gridDim.x) / 32 + 1);  // warps with unknowns
+  int nb0[6];
+  double be0[6], dg0 = 0.0;
+#pragma unroll
+  for (int f = 0; f < 6; ++f) {
+    nb0[f] = i0 < n ? v.nb[6 * (size_t)i0 + f] : kNoNb;
+    be0[f] = i0 < n ? v.beta[6 * (size_t)i0 + f] : 0.0;
+  }
+  if (i0 < n) dg0 = v.diag[i0];
+  double alpha = 0.0, beta = 0.0, gamma = 0.0, rr = 0.0, limit = 0.0;
+  int cur = 0, it = -1;
   bool ok = true;
-  double beta = 0.0;
-  while (res > target && it < max_iter) {  // the same values in every CTA
-    const bool first = it == 0;
-    // d_k and q = M d_k, partial d_k . q
-    double dq = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      const double di = first ? dcur[i] : fma(beta, dcur[i], v.r[i] * v.rdiag[i]);
-      dnew[i] = di;
-      double q = v.diag[i] * di;
+  for (;;) {
+    const ExtRec* __restrict__ in = v.rec[cur];
+    ExtRec* __restrict__ out = v.rec[cur ^ 1];
+    double gm = 0.0, dl = 0.0, r2 = 0.0;
+    for (int i = i0; i < n; i += step) {
+      ExtRec o = rec_l2(in + i), q[6];
+      const bool kept = i == i0;
+      int nb[6];
 #pragma unroll
       for (int f = 0; f < 6; ++f) {
-        const int nb = v.nb[6 * (size_t)i + f];
-        if (nb >= 0) {
-          const double dn = first ? __ldcg(dcur + nb)
-                                  : fma(beta, __ldcg(dcur + nb), __ldcg(v.r + nb) * __ldcg(v.rdiag + nb));
-          q = fma(-v.beta[6 * (size_t)i + f], dn, q);
+        nb[f] = kept ? nb0[f] : v.nb[6 * (size_t)i + f];
+        q[f] = nb[f] >= 0 ? rec_l2(in + nb[f]) : ExtRec{0.0, 0.0, 0.0, 0.0};
+      }
+      if (it >= 0) {
+        // (the direction: z of the iteration before, the owner's only)
+        const double p = it == 0 ? o.r * o.rdiag : fma(beta, v.d[i], o.r * o.rdiag);
+        v.d[i] = p;
+        v.x[i] = fma(alpha, p, v.x[i]);
+      }
+      o.s = fma(beta, o.s, o.w);
+      o.r = fma(-alpha, o.s, o.r);
+      const double u = o.r * o.rdiag;
+      double w = (kept ? dg0 : v.diag[i]) * u;
+#pragma unroll
+      for (int f = 0; f < 6; ++f) {
+        if (__any_sync(__activemask(), nb[f] >= 0)) {
+          const double un = fma(-alpha, fma(beta, q[f].s, q[f].w), q[f].r) * q[f].rdiag;
+          const double be = kept ? be0[f] : v.beta[6 * (size_t)i + f];
+          if (nb[f] >= 0) w = fma(-be, un, w);
         }
       }
-      v.q[i] = q;
-      dq = fma(di, q, dq);
+      o.w = w;
+      out[i] = o;
+      gm = fma(o.r, u, gm);
+      dl = fma(w, u, dl);
+      r2 = fma(o.r, o.r, r2);
     }
-    block_partial(dq, v.part + 3 * kExtCTAs);
-    if (!(ok = ext_grid_barrier(cg, status))) break;
-    // alpha = r.z / d.q; x += alpha d; r -= alpha q; partial r.z and r.r
-    if (threadIdx.x < 32) {
-      const double* pp[1] = {v.part + 3 * kExtCTAs};
-      double dqs[1];
-      warp0_sums<1, true>(pp, kExtCTAs, dqs);
-      if (threadIdx.x == 0) scal[0] = dqs[0] > 0.0 ? rz / dqs[0] : 0.0;
-    }
+    // the CTA's partial sums, one quantity per warp, in a fixed order
+    red[0][threadIdx.x] = gm;
+    red[1][threadIdx.x] = dl;
+    red[2][threadIdx.x] = r2;
+    // (the reciprocals of the scalars before, while others arrive)
+    const Rcp Rg = rcp_of(gamma), Ra = rcp_of(alpha);
     __syncthreads();
-    {
-      const double alpha = scal[0];
-      double rzn = 0.0, rr = 0.0;
-      for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        v.x[i] = fma(alpha, dnew[i], v.x[i]);
-        const double r = fma(-alpha, v.q[i], v.r[i]);
-        v.r[i] = r;
-        rzn = fma(r, r * v.rdiag[i], rzn);
-        rr = fma(r, r, rr);
-      }
-      const double pv[2] = {rzn, rr};
-      double* const po[2] = {v.part + (2 - cur) * kExtCTAs, v.part + 4 * kExtCTAs};
-      block_partial_k<2>(pv, po);
+    double* part = v.part + 3 * cur * kExtCTAs;  // the passes alternate: a slow CTA may still read the last
+    if (warp < 3) {
+      double t = red[warp][lane];
+      for (int j = 1; j < rows; ++j) t += red[warp][lane + 32 * j];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (lane == 0) part[warp * kExtCTAs + blockIdx.x] = t;
     }
     if (!(ok = ext_grid_barrier(cg, status))) break;
-    // beta = r.z new / r.z old, |r|
-    if (threadIdx.x < 32) {
-      const double* pp[2] = {v.part + (2 - cur) * kExtCTAs, v.part + 4 * kExtCTAs};
-      double s2[2];
-      warp0_sums<2, true>(pp, kExtCTAs, s2);
-      if (threadIdx.x == 0) {
-        scal[1] = rz > 0.0 ? s2[0] / rz : 0.0;
-        scal[2] = s2[0];
-        scal[3] = sqrt(s2[1]);
+    if (warp < 3) {
+      double t = 0.0;
+#pragma unroll
+      for (int j = 0; j < (kExtCTAs + 31) / 32; ++j) {
+        const int b = lane + 32 * j;
+        if (b < kExtCTAs) t += __ldcg(part + warp * kExtCTAs + b);
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+      if (lane == 0) tot[warp] = t;
     }
     __syncthreads();
-    beta = scal[1];
-    rz = scal[2];
-    res = scal[3];
-    double* t = dcur;  // the buffers take turns
-    dcur = dnew;
-    dnew = t;
+    const double g1 = tot[0], d1 = tot[1];
+    rr = tot[2];
     cur ^= 1;
     ++it;
+    if (it == 0) {
+      limit = tol * tol * rr;  // (|r| against tol |b| without a square root)
+      beta = 0.0;
+      alpha = d1 > 0.0 ? div_by(g1, rcp_of(d1)) : 0.0;
+    } else {
+      beta = gamma > 0.0 ? div_by(g1, Rg) : 0.0;
+      const double den = alpha > 0.0 ? d1 - beta * div_by(g1, Ra) : 0.0;
+      alpha = den > 0.0 ? div_by(g1, rcp_of(den)) : 0.0;
+    }
+    gamma = g1;
+    if (!(rr > limit) || it >= max_iter) break;  // the same values in every CTA
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     cg->iters = it;
-    cg->res = res;
-    cg->flag = !ok ? 3 : (res > target ? 2 : 1);
+    cg->res = sqrt(rr);
+    cg->flag = !ok ? 3 : (rr > limit ? 2 : 1);
   }
 }
 
-// the face correction along AX over the whole face grid of that axis
-template <int AX>
+// The face correction u~ = -(dt / rho_f) (p~_R - p~_L) / h on the faces of the
+// unknowns, one (unknown, face) per thread: a face between two unknowns is its
+// left cell's, any other face its unknown's; a face to a liquid cell or a wall
+// has none.  Across a periodic boundary the face is stored twice.
+struct ExtOut {
+  double* u[3];
+  double* ut[3];
+};
+// zeros in the arrays of u~ (three memsets one after the other took 45 us at
+// 160^3)
+__global__ void __launch_bounds__(kExtThreads) k_ext_zero(GridDev g, ExtOut out) {
+  const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2], stride = (size_t)gridDim.x * blockDim.x;
+  for (int ax = 0; ax < 3; ++ax) {
+    double* __restrict__ p = out.ut[ax];
+    if (!p) continue;
+    const size_t n = N / (size_t)g.n[ax] * (size_t)(g.n[ax] + 1);
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) p[i] = 0.0;
+  }
+}
 __global__ void __launch_bounds__(kExtThreads)
 k_ext_faces(GridDev g, double h, double dt, double rho_l, double rho_g, const double* __restrict__ c,
-            const uint8_t* __restrict__ code, const int* __restrict__ map, const double* __restrict__ x,
-            double* __restrict__ uf, double* __restrict__ ut) {
-  const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const int fx = nx + (AX == 0), fy = ny + (AX == 1), fz = nz + (AX == 2);
-  const size_t nf = (size_t)fx * fy * fz;
-  const int n_ax = g.n[AX];
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += (size_t)gridDim.x * blockDim.x) {
-    const uint32_t ii = (uint32_t)i;
-    int a = (int)(ii % (uint32_t)fx);
-    const uint32_t rest = ii / (uint32_t)fx;
-    int b = (int)(rest % (uint32_t)fy);
-    int cc = (int)(rest / (uint32_t)fy);
-    // face index f along AX, between cells f - 1 and f
-    const int f = AX == 0 ? a : (AX == 1 ? b : cc);
-    double val = 0.0;
-    bool has = true;
-    int fl = f - 1, fr = f;
-    if (f == 0 || f == n_ax) {
-      if (g.bc[AX] != 0) has = false;  // a wall: no-slip
-      else { fl = n_ax - 1; fr = 0; }
-    }
-    if (has) {
-      int lx = a, ly = b, lz = cc, rx = a, ry = b, rz = cc;
-      if (AX == 0) { lx = fl; rx = fr; }
-      else if (AX == 1) { ly = fl; ry = fr; }
-      else { lz = fl; rz = fr; }
-      const size_t L = cid(g, lx, ly, lz), R = cid(g, rx, ry, rz);
-      const uint8_t cl = code[L], cr = code[R];
-      if ((cl <= 2 || cr <= 2) && cl != kOut && cr != kOut) {
-        const double pl = cl <= 2 ? x[map[L]] : 0.0;
-        const double pr = cr <= 2 ? x[map[R]] : 0.0;
-        const double cf = 0.5 * (__ldg(c + L) + __ldg(c + R));
-        const double rho = rho_l * cf + rho_g * (1.0 - cf);
-        val = -(dt / rho) * (pr - pl) / h;
-      }
-    }
-    if (ut) ut[i] = val;
-    if (uf) uf[i] += val;
+            const uint8_t* __restrict__ code, const int* __restrict__ map, const uint32_t* __restrict__ list,
+            const int* __restrict__ counters, const double* __restrict__ xs, ExtOut out) {
+  const long long total = 8ll * counters[0];  // (two of eight threads idle: no division by 6)
+  for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < total; j += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(j >> 3), f = (int)(j & 7), axis = f >> 1;
+    if (f >= 6) continue;
+    const bool right = (f & 1) != 0;
+    const size_t id = list[i];
+    int x, y, z, qx, qy, qz;
+    cell_xyz(g, id, x, y, z);
+    if (!face_nb(g, x, y, z, axis, right ? 1 : -1, qx, qy, qz)) continue;  // a wall: no-slip
+    const size_t q = cid(g, qx, qy, qz);
+    const uint8_t cq = code[q];
+    if (cq == kOut || (!right && cq <= kLayer)) continue;
+    const double own = xs[i], oth = cq <= kLayer ? xs[map[q]] : 0.0;
+    const double cf = 0.5 * (__ldg(c + (right ? id : q)) + __ldg(c + (right ? q : id)));
+    const double rho = rho_l * cf + rho_g * (1.0 - cf);
+    const double pl = right ? own : oth, pr = right ? oth : own;
+    const double val = div_by(-div_by(dt, rcp_of(rho)) * (pr - pl), rcp_of(h));
+    const int n = g.n[axis];
+    int p[3] = {x, y, z};
+    p[axis] += right ? 1 : 0;
+    auto put = [&](int fp) {
+      int s[3] = {p[0], p[1], p[2]};
+      s[axis] = fp;
+      const size_t at = axis == 0 ? ((size_t)s[2] * g.n[1] + s[1]) * (n + 1) + s[0]
+                                  : (axis == 1 ? ((size_t)s[2] * (n + 1) + s[1]) * g.n[0] + s[0]
+                                               : ((size_t)s[2] * g.n[1] + s[1]) * g.n[0] + s[0]);
+      if (out.ut[axis]) out.ut[axis][at] = val;
+      if (out.u[axis]) out.u[axis][at] += val;
+    };
+    put(p[axis]);
+    if (g.bc[axis] == 0 && p[axis] == n) put(0);
+    if (g.bc[axis] == 0 && p[axis] == 0) put(n);
   }
 }
 
 struct ExtLayout {
-  size_t code, map, list, nb, beta, diag, rdiag, x, r, d, d2, q, part, counters, cg, total;
+  size_t code, map, list, nb, beta, diag, rdiag, x, r, d, q, part, counters, cg, total;
 };
 
 ExtLayout ext_layout(size_t N) {
   auto a = [](size_t b) { return (b + 255) & ~(size_t)255; };
   ExtLayout L;
   size_t o = 0;
-  L.code = o; o += a(N);
+  L.code = o; o += a(N + 3);
   L.map = o; o += a(N * 4);
   L.list = o; o += a(N * 4);
   L.nb = o; o += a(N * 6 * 4);
@@ -619,12 +625,11 @@ ExtLayout ext_layout(size_t N) {
   L.diag = o; o += a(N * 8);
   L.rdiag = o; o += a(N * 8);
   L.x = o; o += a(N * 8);
-  L.r = o; o += a(N * 8);
   L.d = o; o += a(N * 8);
-  L.d2 = o; o += a(N * 8);
-  L.q = o; o += a(N * 8);
-  L.part = o; o += a(5 * kExtCTAs * 8);
-  L.counters = o; o += a(4 * 4);
+  L.r = o; o += a(N * 8);
+  L.q = o; o += 2 * a(N * 8);  // (and a spare: the cooperative solver's records take all three)
+  L.part = o; o += a(6 * kExtCTAs * 8);
+  L.counters = o; o += a(kCnts * 4);
   L.cg = o; o += 256;
   L.total = o;
   return L;
@@ -652,21 +657,44 @@ cudaError_t launch_velocity_extension(const GridDev& g, double h, const double* 
   vec.x = reinterpret_cast<double*>(ws + L.x);
   vec.r = reinterpret_cast<double*>(ws + L.r);
   vec.d = reinterpret_cast<double*>(ws + L.d);
-  vec.d2 = reinterpret_cast<double*>(ws + L.d2);
   vec.q = reinterpret_cast<double*>(ws + L.q);
   vec.part = reinterpret_cast<double*>(ws + L.part);
   vec.counters = reinterpret_cast<int*>(ws + L.counters);
   *status = 0;
-  cudaError_t err = cudaMemsetAsync(vec.counters, 0, 4 * sizeof(int), st);
+  cudaError_t err = cudaMemsetAsync(vec.counters, 0, kCnts * sizeof(int), st);
   if (err != cudaSuccess) return err;
   const int grid_cells = (int)std::min<size_t>((N + kExtThreads - 1) / kExtThreads, (size_t)152 * 16);
-  k_ext_init<<<grid_cells, kExtThreads, 0, st>>>(g, c, code, N);
-  for (int layer = 1; layer <= 2; ++layer) k_ext_dilate<<<grid_cells, kExtThreads, 0, st>>>(g, code, layer, N);
-  k_ext_list<<<grid_cells, kExtThreads, 0, st>>>(code, list, map, vec.counters, N);
+  k_ext_init<<<grid_cells, kExtThreads, 0, st>>>(g, c, code, list, map, vec.counters, N);
+  k_ext_layer<<<kExtCTAs * 4, kExtThreads, 0, st>>>(g, code, list, map, vec.counters, 1);
+  k_ext_layer<<<kExtCTAs * 4, kExtThreads, 0, st>>>(g, code, list, map, vec.counters, 2);
   prof_mark("ext.layers", st);
+  // one cooperative launch when all kExtCTAs CTAs fit at once (the grid
+  // barriers need them resident); else three kernels per iteration
+  int dev = 0, nsm = 0, per_sm = 0, coop = 0;
+  const bool one = cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+                   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ext_cg, kSolveThreads, 0) == cudaSuccess &&
+                   coop && (long long)per_sm * nsm >= kExtCTAs;
+  // the records of up to 3/8 N unknowns fit (interface layers hold far fewer
+  // cells than that but on tiny grids); more go the other way
+  vec.cap = one ? (int)(3 * N / 8) : 0;
+  vec.rec[0] = reinterpret_cast<ExtRec*>(ws + L.r);
+  vec.rec[1] = vec.rec[0] + vec.cap;
   unsigned char* cg_state = reinterpret_cast<unsigned char*>(ws + L.cg);
-  k_ext_assemble<<<kExtCTAs, kExtThreads, 0, st>>>(g, h, dt, rho_l, rho_g, c, mdot, code, map, list, vec, cg_state);
+  k_ext_assemble<<<kExtCTAs * 8, kAsmThreads, 0, st>>>(g, h, dt, rho_l, rho_g, c, mdot, code, map, list, vec, cg_state);
   prof_mark("ext.assemble", st);
+  ExtCG hcg{};
+  if (one) {
+    ExtCG* cg = reinterpret_cast<ExtCG*>(cg_state);
+    int* dstat = device_status_ptr();
+    void* args[] = {&vec, &cg, &tol, &max_iter, &dstat};
+    err = cudaLaunchCooperativeKernel((const void*)k_ext_cg, dim3(kExtCTAs), dim3(kSolveThreads), args, 0, st);
+    if (err != cudaSuccess) return err;
+    prof_mark("ext.cg", st);
+    err = cudaMemcpyAsync(&hcg, cg, sizeof(ExtCG), cudaMemcpyDeviceToHost, st);
+    if (err != cudaSuccess) return err;
+  }
   int host_counts[2] = {0, 0};
   err = cudaMemcpyAsync(host_counts, vec.counters, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
   if (err == cudaSuccess) err = cudaStreamSynchronize(st);
@@ -684,37 +712,18 @@ cudaError_t launch_velocity_extension(const GridDev& g, double h, const double* 
   };
   int it = 0;
   double res = 0.0;
-  bool n_done = false;  // solved by the cooperative launch
-  if (n > 0) {
-    if (host_counts[1] == 0) {
-      *status = 1;  // nothing fixes p~
-      return cudaSuccess;
-    }
-    // one cooperative launch when all kExtCTAs CTAs fit at once (the grid
-    // barriers need them resident); else the three kernels per iteration
-    int dev = 0, nsm = 0, per_sm = 0, coop = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ext_cg, kSolveThreads, 0) == cudaSuccess && coop &&
-        (long long)per_sm * nsm >= kExtCTAs) {
-      ExtCG* cg = reinterpret_cast<ExtCG*>(cg_state);
-      int* dstat = device_status_ptr();
-      void* args[] = {&vec, &cg, &tol, &max_iter, &dstat};
-      err = cudaLaunchCooperativeKernel((const void*)k_ext_cg, dim3(kExtCTAs), dim3(kSolveThreads), args, 0, st);
-      if (err != cudaSuccess) return err;
-      prof_mark("ext.cg", st);
-      ExtCG hcg{};
-      err = cudaMemcpyAsync(&hcg, cg, sizeof(ExtCG), cudaMemcpyDeviceToHost, st);
-      if (err == cudaSuccess) err = cudaStreamSynchronize(st);
-      if (err != cudaSuccess) return err;
-      it = hcg.iters;
-      res = hcg.res;
-      if (hcg.flag != 1) *status = 2;  // not converged (or a barrier wait gave up: DEV_WAIT is set)
-      n_done = true;
-    }
+  if (n > 0 && host_counts[1] == 0) {
+    *status = 1;  // nothing fixes p~
+    return cudaSuccess;
   }
-  if (n > 0 && !n_done) {
+  const bool solved = one && n <= vec.cap;
+  if (solved && n > 0) {
+    it = hcg.iters;
+    res = hcg.res;
+    if (hcg.flag != 1) *status = 2;  // not converged (or a barrier wait gave up: DEV_WAIT is set)
+  }
+  if (n > 0 && !solved) {
+    k_ext_start<<<kExtCTAs, kSolveThreads, 0, st>>>(vec);
     double bb = 0.0;
     err = host_sum(0, &bb);
     if (err != cudaSuccess) return err;
@@ -737,9 +746,10 @@ cudaError_t launch_velocity_extension(const GridDev& g, double h, const double* 
     prof_mark("ext.cg", st);
     if (res > target) *status = 2;  // not converged within max_iter
   }
-  k_ext_faces<0><<<grid_cells, kExtThreads, 0, st>>>(g, h, dt, rho_l, rho_g, c, code, map, vec.x, u, ut);
-  k_ext_faces<1><<<grid_cells, kExtThreads, 0, st>>>(g, h, dt, rho_l, rho_g, c, code, map, vec.x, v, vt);
-  k_ext_faces<2><<<grid_cells, kExtThreads, 0, st>>>(g, h, dt, rho_l, rho_g, c, code, map, vec.x, w, wt);
+  ExtOut out{{u, v, w}, {ut, vt, wt}};
+  if (ut || vt || wt) k_ext_zero<<<152 * 8, kExtThreads, 0, st>>>(g, out);
+  if (n > 0)
+    k_ext_faces<<<kExtCTAs * 4, kExtThreads, 0, st>>>(g, h, dt, rho_l, rho_g, c, code, map, list, vec.counters, vec.x, out);
   prof_mark("ext.faces", st);
   if (iters_out) *iters_out = it;
   if (res_out) *res_out = res;

@@ -61,3 +61,27 @@ def test_diffusion_scales_by_powers_of_two(P, power):
                                  wall_T={(1, -1): 320.0 * s})
         out.append((e.cpu().numpy() / s, r))
     assert np.array_equal(out[0][0], out[1][0]) and np.isfinite(out[0][0]).all()
+
+
+@pytest.mark.parametrize("shape,bc", [((7, 8, 9), (0, 0, 0)), ((6, 5, 12), (1, 0, 1)), ((24, 20, 22), (1, 1, 1))])
+def test_extension_with_many_and_few_unknowns(P, shape, bc):
+    """Tiny boxes whose unknowns outnumber the one-launch solver's records (the
+    kernel-per-phase solver takes them) and a larger one, against the oracle's
+    direct solve."""
+    import torch
+    import oracle as O
+    from oracle.extension import velocity_extension
+    nz, ny, nx = shape
+    z, y, x = np.meshgrid(*[np.arange(n) + 0.5 for n in shape], indexing="ij")
+    r = np.sqrt((x - 0.5 * nx) ** 2 + (y - 0.5 * ny) ** 2 + (z - 0.47 * nz) ** 2)
+    c = np.clip(0.25 * min(shape) + 0.5 - r, 0.0, 1.0)  # a drop in gas
+    mdot = np.where((c > 1e-12) & (c < 1 - 1e-12), 1e-3 * (1 + 0.1 * np.cos(x + y)), 0.0)
+    og = O.Grid(nx, ny, nz, bc, 0.1, 1.0, 1.0, 0.0)
+    ref = velocity_extension(og, c, mdot, 10.0, 1.0, 0.01)[:3]
+    g = P.Grid(nx, ny, nz, bc, 0.1, 1.0, 1.0, 0.0)
+    out = [torch.empty(g.face_shape(a), dtype=torch.float64, device="cuda") for a in range(3)]
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+    P.vof_velocity_extension(g, dev(c), dev(mdot), 10.0, 1.0, 0.01, ut=out[0], vt=out[1], wt=out[2])
+    scale = max(np.abs(np.asarray(ref[a])).max() for a in range(3))
+    for a in range(3):
+        assert np.abs(out[a].cpu().numpy() - np.asarray(ref[a])).max() <= 1e-9 * scale
