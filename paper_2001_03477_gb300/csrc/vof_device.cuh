@@ -556,14 +556,13 @@ __device__ __forceinline__ double plane_alpha(double m0, double m1, double m2, d
 // (a - m3)^3 / d6 <= 0.04 v5) the rounding analysis gives ~14 ulps, so a
 // 64-ulp margin decides.
 //
-// LANES = 3: three lanes of a warp (lanes leader .. leader + 2, mask gmask,
-// sub = lane - leader) share one cell and take two levels per round -- the
-// midpoint and both midpoints of the level after it, each lane deciding
-// one, so a round costs one volume per lane -- with the same midpoints and
-// decisions as the one-lane loop.
-template <int LANES>
-static __device__ __noinline__ double plane_alpha_bisect_t(double m0, double m1, double m2, double c, unsigned gmask,
-                                                           int leader, int sub) {
+// Three lanes of a warp (lanes leader .. leader + 2, mask gmask, sub = lane -
+// leader) share one cell and take two levels per round -- the midpoint and
+// both midpoints of the level after it, each lane deciding one, so a round
+// costs one volume per lane -- with the midpoints and decisions of the plain
+// loop.
+static __device__ __noinline__ double plane_alpha_bisect3(double m0, double m1, double m2, double c, unsigned gmask,
+                                                          int leader, int sub) {
   const Mirror r = mirror_normalise(m0, m1, m2);
   if (!dnz(r.l1)) return 0.0;
   if (dbits(c) <= 0) return 0.0 - r.sh;
@@ -694,32 +693,23 @@ static __device__ __noinline__ double plane_alpha_bisect_t(double m0, double m1,
     if (nn_lt(up ? margin_high : margin_low, fabs(d))) return up ? dgt0(d) : dlt0(d);
     return nn_lt(vpos(mid), c);
   };
-  if (LANES == 1) {
-    for (; it < 200; ++it) {
-      double mid = lo + 0.5 * (hi - lo);
-      if (!(nn_lt(lo, mid) && nn_lt(mid, hi))) break;
-      if (below_at(mid)) lo = mid;
-      else hi = mid;
-    }
-  } else {
-    while (it < 200) {
-      const double mid = lo + 0.5 * (hi - lo);
-      if (!(nn_lt(lo, mid) && nn_lt(mid, hi))) break;
-      // the next level's midpoint after either decision, as the loop above
-      // would compute it from its new bracket
-      const double midL = lo + 0.5 * (mid - lo), midR = mid + 0.5 * (hi - mid);
-      const bool b = below_at(sub == 0 ? mid : (sub == 1 ? midL : midR));
-      const bool bA = __shfl_sync(gmask, b, leader), bL = __shfl_sync(gmask, b, leader + 1),
-                 bR = __shfl_sync(gmask, b, leader + 2);
-      if (bA) lo = mid;
-      else hi = mid;
-      if (++it >= 200) break;
-      const double m2n = bA ? midR : midL;
-      if (!(nn_lt(lo, m2n) && nn_lt(m2n, hi))) break;
-      if (bA ? bR : bL) lo = m2n;
-      else hi = m2n;
-      ++it;
-    }
+  while (it < 200) {
+    const double mid = lo + 0.5 * (hi - lo);
+    if (!(nn_lt(lo, mid) && nn_lt(mid, hi))) break;
+    // the next level's midpoint after either decision, as the loop above
+    // would compute it from its new bracket
+    const double midL = lo + 0.5 * (mid - lo), midR = mid + 0.5 * (hi - mid);
+    const bool b = below_at(sub == 0 ? mid : (sub == 1 ? midL : midR));
+    const bool bA = __shfl_sync(gmask, b, leader), bL = __shfl_sync(gmask, b, leader + 1),
+               bR = __shfl_sync(gmask, b, leader + 2);
+    if (bA) lo = mid;
+    else hi = mid;
+    if (++it >= 200) break;
+    const double m2n = bA ? midR : midL;
+    if (!(nn_lt(lo, m2n) && nn_lt(m2n, hi))) break;
+    if (bA ? bR : bL) lo = m2n;
+    else hi = m2n;
+    ++it;
   }
   // lo and hi are 0 or 1 only at a bracket end never left (vpos's end cases)
   const double vlo = dbits(lo) == 0 ? 0.0 : vpos(lo);
@@ -727,9 +717,6 @@ static __device__ __noinline__ double plane_alpha_bisect_t(double m0, double m1,
   const long long el = dbits(vlo - c) & 0x7FFFFFFFFFFFFFFFLL, eh = dbits(vhi - c) & 0x7FFFFFFFFFFFFFFFLL;
   double am = (eh < el) ? hi : lo;
   return am * r.l1 - r.sh;
-}
-static __device__ __forceinline__ double plane_alpha_bisect(double m0, double m1, double m2, double c) {
-  return plane_alpha_bisect_t<1>(m0, m1, m2, c, 0u, 0, 0);
 }
 
 // The volume function in two parts: the normal's mirror, normalisation and

@@ -79,29 +79,22 @@ __device__ __forceinline__ const T& cta_args(const T* __restrict__ args, unsigne
   return smem;
 }
 
-// Sums.  Every kernel that sums produces one row of kNSums values per CTA,
-// in one layout:
+// Sums, in one layout of kNSums values: a time step's rows (one per tile,
+// reduced later in a fixed order), and what a CTA of a stand-alone kernel adds
+// to the caller's diagnostics:
 //   [kSumC] sum of c contributions   [kSumE] sum of e contributions
 //   [kSumClip] clipped volume of the sweeps
 //   [kSumShDc] shift: sum Delta c    [kSumUnpl] shift: volume clamped away
 //   [kSumShDe] shift: sum Delta e
-// and either writes it to partials[block * stride] (deterministic, reduced
-// later in a fixed order) or, when partials == nullptr, adds each value k
-// with map[k] >= 0 to diag[map[k]] with an atomic (nothing when diag is
-// null too).
+// each value k with map[k] >= 0 by an atomic to diag[map[k]] (nothing when diag
+// is null).
 enum { kSumC = 0, kSumE, kSumClip, kSumShDc, kSumUnpl, kSumShDe, kNSums };
 struct SumOut {
-  double* partials;
-  int stride;
   double* diag;
   signed char map[kNSums];
 };
-__host__ __device__ inline SumOut sums_to_partials(double* p, int stride) {
-  SumOut s{p, stride, nullptr, {-1, -1, -1, -1, -1, -1}};
-  return s;
-}
 inline SumOut sums_to_diag(double* diag, const signed char (&map)[kNSums]) {
-  SumOut s{nullptr, kNSums, diag, {map[0], map[1], map[2], map[3], map[4], map[5]}};
+  SumOut s{diag, {map[0], map[1], map[2], map[3], map[4], map[5]}};
   return s;
 }
 

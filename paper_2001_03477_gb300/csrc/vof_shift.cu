@@ -86,7 +86,7 @@ __device__ __forceinline__ void k_shift_stream_body(const GridDev& g, const doub
   const size_t w = (size_t)row * vb.gy + vb.by;  // list of this warp
   const int cap = nx < kWarpCells ? nx : kWarpCells;
   uint32_t* list = sc.list + w * cap;
-  const bool do_sums = sums.partials || sums.diag;
+  const bool do_sums = sums.diag != nullptr;
   int n = 0, ne = 0;
   double v[kNSums] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   const bool uni_moving = dnz(dd_uniform);
@@ -148,7 +148,7 @@ __device__ __forceinline__ void k_shift_stream_body(const GridDev& g, const doub
       bn += __popc(mn);
     }
   }
-  block_sums(v, sums, vb.bx + vb.gx * vb.by);
+  block_sums(v, sums);
 }
 
 __global__ void __launch_bounds__(256)
@@ -193,7 +193,7 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
   double m[3];
   myc_normal(st, m);
   double al;
-  if (LANES == 3) al = plane_alpha_bisect_t<3>(m[0], m[1], m[2], ct, gmask, leader, sub);
+  if (LANES == 3) al = plane_alpha_bisect3(m[0], m[1], m[2], ct, gmask, leader, sub);
   else al = plane_alpha(m[0], m[1], m[2], ct);
   const double ddv = dd ? __ldg(dd + id) : dd_uniform;
   const double mn2 = sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
@@ -488,7 +488,7 @@ __device__ __forceinline__ void k_shift_sums_body(const GridDev& g, const double
   v[kSumShDc] = acc[0];
   v[kSumUnpl] = acc[1];
   v[kSumShDe] = acc[2];
-  block_sums(v, sums, vb.bx);
+  block_sums(v, sums);
 }
 
 __global__ void __launch_bounds__(256)

@@ -5,14 +5,13 @@
 
 namespace vofgb {
 
-// Sums v[] over the block (up to 32 warps) in a fixed order and writes the
-// row to out.partials, or adds the mapped nonzero values to out.diag with
-// atomics.  Whole warps of zeros skip the FP64 shuffle tree (FP64 adds are
+// Sums v[] over the block (up to 32 warps) in a fixed order and adds the
+// mapped nonzero values to out.diag with atomics.  Whole warps of zeros skip the FP64 shuffle tree (FP64 adds are
 // the scarce operation on this part, and most warps of most kernels sum
 // zeros).  Every thread of the block must call it.
-__device__ __forceinline__ void block_sums(double (&v)[kNSums], const SumOut& out, unsigned block_lin) {
+__device__ __forceinline__ void block_sums(double (&v)[kNSums], const SumOut& out) {
   __shared__ double red[kNSums][32];
-  if (!out.partials && !out.diag) return;  // uniform over the block
+  if (!out.diag) return;  // uniform over the block
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nw = (int)(blockDim.x * blockDim.y * blockDim.z) >> 5;
   const int lane = tid & 31, warp = tid >> 5;
@@ -38,10 +37,7 @@ __device__ __forceinline__ void block_sums(double (&v)[kNSums], const SumOut& ou
       } else {
         x = 0.0;
       }
-      if (lane == 0) {
-        if (out.partials) out.partials[(size_t)block_lin * out.stride + k] = x;
-        else if (out.map[k] >= 0 && dnz(x)) atomicAdd(out.diag + out.map[k], x);
-      }
+      if (lane == 0 && out.map[k] >= 0 && dnz(x)) atomicAdd(out.diag + out.map[k], x);
     }
   }
 }

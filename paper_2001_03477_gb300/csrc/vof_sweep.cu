@@ -635,7 +635,7 @@ __device__ __forceinline__ void k_update_body(const GridDev& g, const double* c_
   else
     update_groups<AX, ENERGY, false>(g, c_in, e_in, c_out, e_out, uf, state, theta, sc, nsub, cap, ngrp, vb, pre,
                                      lst, v);
-  block_sums(v, sc.sums, vb.bx);
+  block_sums(v, sc.sums);
 }
 
 template <int AX, bool ENERGY>
