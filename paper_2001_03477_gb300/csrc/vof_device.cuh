@@ -986,7 +986,7 @@ __device__ __forceinline__ void myc_normal(const double* s, double m[3]) {
 __device__ __forceinline__ void myc_normal_f(const double* sd, double m[3]) {
   float s[27];
 #pragma unroll
-  for (int i = 0; i < 27; ++i) s[i] = (float)sd[i];
+  for (int i = 0; i < 27; ++i) s[i] = f32_of(sd[i]);
   auto at = [&](int d, int r, int p, int q) -> float {
     int o0, o1, o2;
     if (d == 0) { o0 = r; o1 = p; o2 = q; }
@@ -1044,11 +1044,8 @@ __device__ __forceinline__ void myc_normal_f(const double* sd, double m[3]) {
     myc_normal(sd, m);
     return;
   }
-  if (bdom <= ymax) {
-    m[0] = best[0]; m[1] = best[1]; m[2] = best[2];
-  } else {
-    m[0] = y[0] / l1y; m[1] = y[1] / l1y; m[2] = y[2] / l1y;
-  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) m[d] = f64_of(bdom <= ymax ? best[d] : y[d] / l1y);
 }
 
 __device__ __forceinline__ float vol_low_f(float m1, float m2, float m3, float a) {

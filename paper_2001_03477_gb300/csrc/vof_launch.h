@@ -24,6 +24,14 @@ namespace vofgb {
 // kernel's waiting CTAs on the SMs that happened to be free, unevenly, and the
 // step took 1.05 ms instead of 0.83 ms (0.88 ms with plain launches).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A pointer whose loads stay behind the wait: to the compiler, data that a
+// kernel only reads (const, restrict) is the same before and after it, and such
+// a load of what the grid ahead writes may otherwise move up.
+template <typename T>
+__device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p) : : "memory");
+  return p;
+}
 
 template <typename... KArgs, typename... Args>
 inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {

@@ -19,7 +19,9 @@
 // evaluated in FP64 with the same BF16 weights to FP32 accumulation error.
 // Gradient contractions use two-term splits (hi + lo) of both operands.
 //
-// Tensor-core use (one CTA of 128 threads per tile of 128 stencils):
+// Tensor-core use (one CTA per tile of 128 stencils, 2 threads per row in the
+// forward pass and 4 in training: each layer is a short chain of MMAs between
+// long element-wise ones -- erf, the splits -- whose latency more warps hide):
 //   * operands in shared memory in the canonical K-major layout without
 //     swizzle: 8-row x 16-byte core matrices, K-adjacent core matrices 128 B
 //     apart (leading byte offset), 8-row groups KC x 128 B apart (stride
@@ -33,6 +35,8 @@
 //     tensor memory and returns.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "../../include/vofgb.h"
 #include "vof_launch.h"
 
@@ -41,7 +45,9 @@ namespace mlp {
 
 constexpr int kIn = 27, kK1 = 32, kH = 64, kOut = 3, kN3 = 16;
 constexpr int kRows = 128;
-constexpr int kThreads = 128;
+constexpr int kInferThreads = 256;   // 2 per row
+constexpr int kTrainThreads = 512;   // 4 per row
+constexpr int kChooseThreads = 128;  // 4 warps on 32 cells
 
 // master parameter vector (FP32), the order of the C ABI
 constexpr int oW1 = 0;                  // W1[64][27]
@@ -161,8 +167,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 // numerics
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float gelu(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-__device__ __forceinline__ float gelu_grad(float x) {
-  return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * __expf(-0.5f * x * x) * 0.39894228040143268f;
+// GELU and its derivative, one erf
+__device__ __forceinline__ float gelu_both(float x, float& grad) {
+  const float e = 1.0f + erff(x * 0.70710678118654752f);
+  grad = 0.5f * e + x * __expf(-0.5f * x * x) * 0.39894228040143268f;
+  return 0.5f * x * e;
+}
+// the network's input 2 c - 1, rounded once to FP32, from c's FP32 pair (the
+// FP64 form takes two instructions of 76 cycles)
+__device__ __forceinline__ float input_of(double c) {
+  const df::f2 p = df::split_scaled(df::words_of(c), 0);
+  const float a = 2.0f * p.hi, s = a - 1.0f, b = s - a;
+  return s + (2.0f * p.lo + ((a - (s - b)) + (-1.0f - b)));
 }
 
 __device__ __forceinline__ uint16_t bf16_bits(float x) {
@@ -194,22 +210,76 @@ __device__ __forceinline__ void st_row8(unsigned char* img, int r, int k0, int K
 }
 
 // FP32 plane geometry of the fallback test ----------------------------------
-// volume below the plane m.x <= a in the unit cube (any signs of m)
-__device__ __forceinline__ float volume_f(float m0, float m1, float m2, float a) {
-  if (m0 < 0.f) { a -= m0; m0 = -m0; }
-  if (m1 < 0.f) { a -= m1; m1 = -m1; }
-  if (m2 < 0.f) { a -= m2; m2 = -m2; }
+// x / d, correctly rounded, from r = 1 / d (correctly rounded): the quotient's
+// remainder corrects it (Markstein)
+__device__ __forceinline__ float quot(float x, float d, float r) {
+  const float q = x * r;
+  return fmaf(fmaf(-q, d, x), r, q);
+}
+// What the volumes below one plane's shifts share: the normal mirrored to
+// m >= 0, normalised and sorted, the branches' divisors with their reciprocals
+struct PlaneF {
+  float n0, n1, n2;  // the negative components (or 0): the shift's mirror
+  float r;           // 1 / (m0 + m1 + m2)
+  float m1, m2, m3, m12, top, d6, r6, d2, r2, d3, r3, cube;
+  bool lin, none, tiny;
+};
+__device__ __forceinline__ PlaneF plane_f(float m0, float m1, float m2) {
+  PlaneF p;
+  p.n0 = fminf(m0, 0.f);
+  p.n1 = fminf(m1, 0.f);
+  p.n2 = fminf(m2, 0.f);
+  m0 = fabsf(m0);
+  m1 = fabsf(m1);
+  m2 = fabsf(m2);
   const float l1 = m0 + m1 + m2;
-  if (!(l1 > 0.f)) return a >= 0.f ? 1.f : 0.f;
-  const float r = 1.f / l1;
-  m0 *= r; m1 *= r; m2 *= r; a *= r;
-  if (a <= 0.f) return 0.f;
-  if (a >= 1.f) return 1.f;
+  p.none = !(l1 > 0.f);
+  p.r = 1.f / l1;
+  m0 *= p.r; m1 *= p.r; m2 *= p.r;
   float t;
   if (m1 < m0) { t = m0; m0 = m1; m1 = t; }
   if (m2 < m1) { t = m1; m1 = m2; m2 = t; }
   if (m1 < m0) { t = m0; m0 = m1; m1 = t; }
-  return a <= 0.5f ? vol_low_f(m0, m1, m2, a) : 1.f - vol_low_f(m0, m1, m2, 1.f - a);
+  p.m1 = m0; p.m2 = m1; p.m3 = m2;
+  p.m12 = m0 + m1;
+  p.top = p.m12 < m2 ? p.m12 : m2;
+  p.lin = p.m12 <= m2;
+  p.d6 = 6.f * m0 * m1 * m2;
+  p.d2 = 2.f * m1 * m2;
+  p.d3 = 2.f * m2;
+  p.r6 = 1.f / p.d6;
+  p.r2 = 1.f / p.d2;
+  p.r3 = 1.f / p.d3;
+  p.cube = m0 * m0 / (6.f * m1 * m2);
+  // products that leave the range where the corrected quotients round as
+  // divisions do (a component below ~1e-20): those take the divisions
+  p.tiny = !(p.d6 > 1e-20f);
+  return p;
+}
+// volume below the plane m.x <= a in the unit cube
+__device__ __forceinline__ float volume_f(const PlaneF& p, float a) {
+  a = ((a - p.n0) - p.n1) - p.n2;
+  const float a0 = a;
+  a *= p.r;
+  const float b = a <= 0.5f ? a : 1.f - a;
+  // every branch's operations, its own selected (no divergent paths): the cube
+  // of b (first branch) or b - m2, the quadratic, and past `top` the linear
+  // branch's or the third cube's quotient
+  const float t2 = b - p.m2, t3 = b - p.m3;
+  const bool first = b < p.m1, past = b >= p.top, lin = past && p.lin;
+  const float x = first ? b : t2, x3 = x * x * x;
+  const float y = p.lin ? 2.f * b - p.m12 : t3 * t3 * t3;
+  const float q6 = quot(x3, p.d6, p.r6);
+  const float qy = quot(y, p.lin ? p.d3 : p.d6, p.lin ? p.r3 : p.r6);
+  const float v2 = quot(b * (b - p.m1), p.d2, p.r2) + p.cube;
+  const float v3 = v2 - q6;
+  float v = first ? q6 : (b < p.m2 ? v2 : (lin ? qy : (past ? v3 - qy : v3)));
+  if (p.tiny) v = vol_low_f(p.m1, p.m2, p.m3, b);
+  v = a <= 0.5f ? v : 1.f - v;
+  if (a <= 0.f) v = 0.f;
+  if (a >= 1.f) v = 1.f;
+  if (p.none) v = a0 >= 0.f ? 1.f : 0.f;
+  return v;
 }
 
 // plane constant with volume_f(m, a) = c (m L1-normalised)
@@ -228,22 +298,25 @@ __device__ __forceinline__ float alpha_f(float m0, float m1, float m2, float c) 
   return a - sh;
 }
 
-// RMS over the 26 neighbours of (volume of the plane with normal m through
-// the central cell's plane constant) - c; s: the stencil (x fastest)
-__device__ __forceinline__ float plane_residual(const float* s, float m0, float m1, float m2) {
+// The plane with normal m (any length) through the central cell's plane constant
+// for c: its residual is the RMS over the 26 neighbours of volume - c.
+struct PlaneFit {
+  float m0, m1, m2, al;
+  PlaneF p;
+};
+__device__ __forceinline__ PlaneFit plane_fit(float m0, float m1, float m2, float c) {
+  PlaneFit f;
   const float l1 = fabsf(m0) + fabsf(m1) + fabsf(m2);
   const float r = 1.f / l1;
-  m0 *= r; m1 *= r; m2 *= r;
-  const float al = alpha_f(m0, m1, m2, s[13]);
-  float acc = 0.f;
-#pragma unroll
-  for (int k = 0; k < 27; ++k) {
-    if (k == 13) continue;
-    const float ox = (float)(k % 3 - 1), oy = (float)((k / 3) % 3 - 1), oz = (float)(k / 9 - 1);
-    const float d = volume_f(m0, m1, m2, al - (m0 * ox + m1 * oy + m2 * oz)) - s[k];
-    acc += d * d;
-  }
-  return sqrtf(acc * (1.f / 26.f));
+  f.m0 = m0 * r; f.m1 = m1 * r; f.m2 = m2 * r;
+  f.al = alpha_f(f.m0, f.m1, f.m2, c);
+  f.p = plane_f(f.m0, f.m1, f.m2);
+  return f;
+}
+// volume - ck at neighbour k (x fastest)
+__device__ __forceinline__ float fit_at(const PlaneFit& f, int k, float ck) {
+  const float ox = (float)(k % 3 - 1), oy = (float)((k / 3) % 3 - 1), oz = (float)(k / 9 - 1);
+  return volume_f(f.p, f.al - (f.m0 * ox + f.m1 * oy + f.m2 * oz)) - ck;
 }
 
 // ---------------------------------------------------------------------------
@@ -253,6 +326,11 @@ __device__ __forceinline__ float plane_residual(const float* s, float m0, float 
 struct SrcX {
   const double* X;
   __device__ __forceinline__ double at(long i, int k) const { return __ldg(X + 27 * i + k); }
+  struct Cell {
+    const double* x;
+    __device__ __forceinline__ double at(int k) const { return __ldg(x + k); }
+  };
+  __device__ __forceinline__ Cell cell(long i) const { return Cell{X + 27 * i}; }
 };
 // the mixed-cell list of a sweep: stencil of cell gmix[i] with the boundary
 // conditions' index mapping
@@ -271,6 +349,27 @@ struct SrcGrid {
     const double w = __ldg(c + ((size_t)zz * g.n[1] + yy) * g.n[0] + xx);
     return __hiloint2double((int)((unsigned)__double2hiint(w) & mask), __double2loint(w));
   }
+  // one cell, for neighbours k that vary at run time
+  struct Cell {
+    const SrcGrid& s;
+    int x, y, z;
+    __device__ __forceinline__ static int near(int p, int n, int bc) {  // p in -1 .. n
+      if (p < 0) return bc ? 0 : p + n;
+      return p < n ? p : (bc ? n - 1 : p - n);
+    }
+    __device__ __forceinline__ double at(int k) const {
+      const GridDev& g = s.g;
+      const int xx = near(x + k % 3 - 1, g.n[0], g.bc[0]), yy = near(y + (k / 3) % 3 - 1, g.n[1], g.bc[1]),
+                zz = near(z + k / 9 - 1, g.n[2], g.bc[2]);
+      const double w = __ldg(s.c + ((size_t)zz * g.n[1] + yy) * g.n[0] + xx);
+      return __hiloint2double((int)((unsigned)__double2hiint(w) & s.mask), __double2loint(w));
+    }
+  };
+  __device__ __forceinline__ Cell cell(long i) const {
+    Cell q{*this, 0, 0, 0};
+    cell_xyz(g, gmix[i], q.x, q.y, q.z);
+    return q;
+  }
 };
 
 // ---------------------------------------------------------------------------
@@ -282,7 +381,6 @@ struct InferSmem {
   float bias[kH + kH + kN3];
   uint64_t bar;
   uint32_t tmem;
-  int abort;
 };
 
 constexpr uint32_t kInferCols = 128;  // tensor-memory columns per CTA
@@ -325,50 +423,65 @@ __device__ __forceinline__ bool layer_done(InferSmem& S, uint32_t& ph) {
   return all != 0;
 }
 
-// MODE 0: network output y[n][3] (FP32) for explicit stencils.
-// MODE 1: learned normal with MYC fallback for explicit stencils:
-//         m[n][3] (L1-normalised, FP64) and flag[n] (1: MYC used).
-// MODE 2: the same normal for the mixed cells of a sweep, into the planes
-//         of the sweep scratch (m0, m1, m2; the plane constant follows).
-template <int MODE, class Src>
-__global__ void __launch_bounds__(kThreads)
+// Where the network's output of stencil i goes: y[n][3], the first 12 of m[n]'s
+// 24 bytes, or the plane slot of the cell (k_mlp_choose turns the latter two
+// into normals).
+struct OutY {
+  float* y;
+  __device__ __forceinline__ float* at(long i) const { return y + 3 * i; }
+};
+struct OutM {
+  double* m;
+  __device__ __forceinline__ double* at(long i) const { return m + 3 * i; }
+};
+struct OutPlane {
+  double* plane;
+  const uint32_t* gmix;
+  __device__ __forceinline__ double* at(long i) const { return plane + 4 * (size_t)gmix[i]; }
+};
+
+// Forward pass.  Two threads per row: thread (r, half) takes 16 of the 32 inputs
+// and 32 of the 64 units of each hidden layer.
+template <class Src, class Out>
+__global__ void __launch_bounds__(kInferThreads)
 k_mlp_infer(Src src, const int* __restrict__ count_dev, long n_host, const unsigned char* __restrict__ params,
-            float* __restrict__ y_out, double* __restrict__ m_out, uint8_t* __restrict__ flag_out,
-            double* __restrict__ plane_out, int* __restrict__ nfallback, int* __restrict__ status) {
+            Out out, int* __restrict__ status) {
   extern __shared__ unsigned char smem_raw[];
   InferSmem& S = *reinterpret_cast<InferSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = t >> 5, row = t & (kRows - 1), half = t >> 7;
   const long n = count_dev ? (long)*count_dev : n_host;
   const long ntiles = (n + kRows - 1) / kRows;
   if ((long)blockIdx.x >= ntiles) return;  // uniform across the CTA
 
   // weights and biases (the images are already in the canonical layout)
-  for (uint32_t o = t * 16; o < kInferWBytes; o += kThreads * 16)
+  for (uint32_t o = t * 16; o < kInferWBytes; o += kInferThreads * 16)
     *reinterpret_cast<uint4*>(S.w + o) = __ldg(reinterpret_cast<const uint4*>(params + o));
-  for (int i = t; i < kH + kH + kN3; i += kThreads) S.bias[i] = __ldg(reinterpret_cast<const float*>(params + pB) + i);
-  if (t == 0) {
-    mbar_init(&S.bar, 1);
-    S.abort = 0;
-  }
+  if (t < kH + kH + kN3) S.bias[t] = __ldg(reinterpret_cast<const float*>(params + pB) + t);
+  if (t == 0) mbar_init(&S.bar, 1);
   if (warp == 0) tmem_alloc(&S.tmem, kInferCols);
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
   const uint32_t tm = S.tmem;
-  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;  // this warp's tensor-memory lanes
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;  // this warp's tensor-memory lanes
   uint32_t ph = 0;
   bool ok = true;
 
   for (long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    const long i = tile * kRows + t;
+    const long i = tile * kRows + row;
     const bool live = i < n;
     // layer 1 input: 2 c - 1 (K padded to 32 with zeros)
     {
-      float v[32];
+      float v[16];
+      if (half == 0) {
 #pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = (live && k < kIn) ? (float)(2.0 * src.at(i, k) - 1.0) : 0.f;
+        for (int k = 0; k < 16; ++k) v[k] = live ? input_of(src.at(i, k)) : 0.f;
+      } else {
 #pragma unroll
-      for (int k0 = 0; k0 < 32; k0 += 8) put_act3(S, t, k0, 4, v + k0);
+        for (int k = 16; k < 32; ++k) v[k - 16] = (live && k < kIn) ? input_of(src.at(i, k < kIn ? k : 0)) : 0.f;
+      }
+      put_act3(S, row, 16 * half, 4, v);
+      put_act3(S, row, 16 * half + 8, 4, v + 8);
     }
     fence_async_smem();
     tc_before_sync();
@@ -379,95 +492,38 @@ k_mlp_infer(Src src, const int* __restrict__ count_dev, long n_host, const unsig
       umma_commit(&S.bar);
     }
     if (!(ok = layer_done(S, ph))) break;
-    // layer 1 -> 2: z1 = D + b1, GELU, three pieces
+    // z = D + b, GELU, three pieces: layer 1 -> 2, then 2 -> 3
+#pragma unroll 1
+    for (int layer = 0; layer < 2; ++layer) {
+#pragma unroll 1
+      for (int j0 = 0; j0 < kH / 2; j0 += 16) {
+        const int c0 = half * (kH / 2) + j0;
+        float v[16];
+        tmem_ld16(tm + lane_base + layer * kH + c0, v);
 #pragma unroll
-    for (int c0 = 0; c0 < kH; c0 += 16) {
-      float v[16];
-      tmem_ld16(tm + lane_base + c0, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = gelu(v[j] + S.bias[c0 + j]);
-      put_act3(S, t, c0, 8, v);
-      put_act3(S, t, c0 + 8, 8, v + 8);
+        for (int j = 0; j < 16; ++j) v[j] = gelu(v[j] + S.bias[layer * kH + c0 + j]);
+        put_act3(S, row, c0, 8, v);
+        put_act3(S, row, c0 + 8, 8, v + 8);
+      }
+      fence_async_smem();
+      tc_before_sync();
+      __syncthreads();
+      if (t == 0) {
+        tc_after_sync();
+        if (layer == 0) issue_layer(tm + kH, S.act[0], kRows * kH * 2, 3, S.w + pW2, kH, kH);
+        else issue_layer(tm + 0, S.act[0], kRows * kH * 2, 3, S.w + pW3, kH, kN3);
+        umma_commit(&S.bar);
+      }
+      if (!(ok = layer_done(S, ph))) break;
     }
-    fence_async_smem();
-    tc_before_sync();
-    __syncthreads();
-    if (t == 0) {
-      tc_after_sync();
-      issue_layer(tm + 64, S.act[0], kRows * kH * 2, 3, S.w + pW2, kH, kH);
-      umma_commit(&S.bar);
-    }
-    if (!(ok = layer_done(S, ph))) break;
+    if (!ok) break;
+    if (half == 0) {
+      float y[16];
+      tmem_ld16(tm + lane_base + 0, y);
+      if (live) {
+        float* o = reinterpret_cast<float*>(out.at(i));
 #pragma unroll
-    for (int c0 = 0; c0 < kH; c0 += 16) {
-      float v[16];
-      tmem_ld16(tm + lane_base + 64 + c0, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = gelu(v[j] + S.bias[kH + c0 + j]);
-      put_act3(S, t, c0, 8, v);
-      put_act3(S, t, c0 + 8, 8, v + 8);
-    }
-    fence_async_smem();
-    tc_before_sync();
-    __syncthreads();
-    if (t == 0) {
-      tc_after_sync();
-      issue_layer(tm + 0, S.act[0], kRows * kH * 2, 3, S.w + pW3, kH, kN3);
-      umma_commit(&S.bar);
-    }
-    if (!(ok = layer_done(S, ph))) break;
-    float y[16];
-    tmem_ld16(tm + lane_base + 0, y);
-    const float y0 = y[0] + S.bias[2 * kH + 0], y1 = y[1] + S.bias[2 * kH + 1], y2 = y[2] + S.bias[2 * kH + 2];
-    if (live) {
-      if constexpr (MODE == 0) {
-        y_out[3 * i + 0] = y0;
-        y_out[3 * i + 1] = y1;
-        y_out[3 * i + 2] = y2;
-      } else {
-        double sd[27];
-        float sf[27];
-#pragma unroll
-        for (int k = 0; k < 27; ++k) {
-          sd[k] = src.at(i, k);
-          sf[k] = (float)sd[k];
-        }
-        // the fallback: MYC as the sweeps of this precision compute it
-        // (explicit stencils: the precision form's)
-        double mm[3];
-        if constexpr (MODE == 2) {
-          if (src.g.f32) myc_normal_f(sd, mm);
-          else myc_normal(sd, mm);
-        } else {
-          myc_normal_f(sd, mm);
-        }
-        const float rm = plane_residual(sf, (float)mm[0], (float)mm[1], (float)mm[2]);
-        const float l1 = fabsf(y0) + fabsf(y1) + fabsf(y2);
-        const float rn = plane_residual(sf, y0, y1, y2);
-        // keep the network's normal only when its residual is a number
-        // within the bound (a zero or non-finite output falls back)
-        const bool use_mlp = l1 > 0.f && rn <= kFallbackRatio * rm + kFallbackTol;
-        double m0 = mm[0], m1 = mm[1], m2 = mm[2];
-        if (use_mlp) {
-          const double dl1 = (double)fabsf(y0) + (double)fabsf(y1) + (double)fabsf(y2);
-          m0 = (double)y0 / dl1;
-          m1 = (double)y1 / dl1;
-          m2 = (double)y2 / dl1;
-        } else if (nfallback) {
-          atomicAdd(nfallback, 1);
-        }
-        if constexpr (MODE == 1) {
-          m_out[3 * i + 0] = m0;
-          m_out[3 * i + 1] = m1;
-          m_out[3 * i + 2] = m2;
-          if (flag_out) flag_out[i] = use_mlp ? 0 : 1;
-        } else {
-          const size_t id = src.gmix[i];
-          double* pl = plane_out + 4 * id;
-          pl[0] = m0;
-          pl[1] = m1;
-          pl[2] = m2;
-        }
+        for (int q = 0; q < 3; ++q) o[q] = y[q] + S.bias[2 * kH + q];
       }
     }
     // the next tile's layer-1 MMAs overwrite columns 0..63 read above
@@ -479,6 +535,103 @@ k_mlp_infer(Src src, const int* __restrict__ count_dev, long n_host, const unsig
   __syncthreads();
   tc_after_sync();
   if (warp == 0) tmem_dealloc(tm, kInferCols);
+}
+
+// The network's outputs (already at out) into normals, with the MYC fallback: four
+// warps on 32 cells (lane = cell), whatever the tile of the forward pass.  A
+// sweep's few thousand cells are one warp each per SM partition, so the time is
+// the longest chain of one warp: 57 us with a thread per cell (the two
+// residuals' 52 volumes in straight-line code), 26 us here, where warps 2 and 3 take the
+// network's residual, half the neighbours each, while warp 0 forms the MYC normal;
+// then all four take MYC's; the squares are summed in the neighbours' order.
+// MYC as the sweeps of the precision compute it (explicit stencils: the precision
+// form's).
+template <bool GRID, class Src, class Out>
+__global__ void __launch_bounds__(kChooseThreads)
+k_mlp_choose(Src src, const int* __restrict__ count_dev, long n_host, Out out, uint8_t* __restrict__ flag_out,
+             int* __restrict__ nfallback) {
+  __shared__ double s_c[27][32];
+  __shared__ double s_m[3][32];
+  __shared__ float s_y[3][32], s_d[2][27][32], s_r[32];
+  pdl_wait();
+  const long n = count_dev ? (long)*count_dev : n_host;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (long b = (long)blockIdx.x * 32; b < n; b += (long)gridDim.x * 32) {
+    const long i = min(b + lane, n - 1);  // (lanes past the end repeat the last cell)
+    {
+      const auto cell = src.cell(i);
+#pragma unroll
+      for (int j = 0; j < 7; ++j) {
+        const int k = warp + 4 * j;
+        if (k < 27) s_c[k][lane] = cell.at(k);
+      }
+      if (warp == 0) {
+        const float* o = reinterpret_cast<const float*>(out.at(i));
+        s_y[0][lane] = o[0];
+        s_y[1][lane] = o[1];
+        s_y[2][lane] = o[2];
+      }
+    }
+    __syncthreads();
+    const float cc = f32_of(s_c[13][lane]);
+    auto residual = [&](int which, float m0, float m1, float m2, int k0, int dk) {
+      const PlaneFit f = plane_fit(m0, m1, m2, cc);
+#pragma unroll 2
+      for (int k = k0; k < 27; k += dk) s_d[which][k][lane] = fit_at(f, k, f32_of(s_c[k][lane]));
+    };
+    if (warp == 0) {
+      double sd[27], mm[3];
+#pragma unroll
+      for (int k = 0; k < 27; ++k) sd[k] = s_c[k][lane];
+      if constexpr (GRID) {
+        if (src.g.f32) myc_normal_f(sd, mm);
+        else myc_normal(sd, mm);
+      } else {
+        myc_normal_f(sd, mm);
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) s_m[q][lane] = mm[q];
+    } else if (warp >= 2) {
+      residual(1, s_y[0][lane], s_y[1][lane], s_y[2][lane], warp - 2, 2);
+    }
+    __syncthreads();
+    residual(0, f32_of(s_m[0][lane]), f32_of(s_m[1][lane]), f32_of(s_m[2][lane]), warp, 4);
+    __syncthreads();
+    float res = 0.f;
+    if (warp < 2) {
+#pragma unroll
+      for (int k = 0; k < 27; ++k)
+        if (k != 13) res += s_d[warp][k][lane] * s_d[warp][k][lane];
+      res = sqrtf(res * (1.f / 26.f));
+      if (warp == 1) s_r[lane] = res;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const float y0 = s_y[0][lane], y1 = s_y[1][lane], y2 = s_y[2][lane];
+      const float l1 = fabsf(y0) + fabsf(y1) + fabsf(y2);
+      // keep the network's normal only when its residual is a number
+      // within the bound (a zero or non-finite output falls back)
+      const bool use_mlp = l1 > 0.f && s_r[lane] <= kFallbackRatio * res + kFallbackTol;
+      double m[3] = {s_m[0][lane], s_m[1][lane], s_m[2][lane]};
+      if (use_mlp) {
+        const double a0 = f64_of(y0), a1 = f64_of(y1), a2 = f64_of(y2);
+        const Rcp R = rcp_of((dabs_i(a0) + dabs_i(a1)) + dabs_i(a2));
+        m[0] = div_by(a0, R);
+        m[1] = div_by(a1, R);
+        m[2] = div_by(a2, R);
+      }
+      const bool live = b + lane < n;
+      const unsigned back = __ballot_sync(0xffffffffu, live && !use_mlp);
+      if (nfallback && lane == 0 && back) atomicAdd(nfallback, __popc(back));
+      if (live) {
+        double* o = out.at(i);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) o[q] = m[q];
+        if (!GRID && flag_out) flag_out[i] = use_mlp ? 0 : 1;
+      }
+    }
+    __syncthreads();  // (the next cells overwrite the tables)
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -521,7 +674,6 @@ __global__ void k_mlp_pack(const float* __restrict__ master, unsigned char* __re
 // tile's gradient written to its own row of partial sums (reduced in tile
 // order by the Adam kernel: deterministic).
 // ---------------------------------------------------------------------------
-constexpr int kZs = kH + 1;  // row stride of the FP32 pre-activations (no bank conflicts)
 constexpr int kTB = 96;      // rows of the transposed B operand: a1 (64) then a0 (32)
 constexpr uint32_t kTrainCols = 256;
 
@@ -529,8 +681,6 @@ struct TrainSmem {
   alignas(1024) unsigned char act[3][kRows * kH * 2];  // A pieces; later [a1; a0]^T pieces (2 x 24 KB)
   alignas(1024) unsigned char at[2][kRows * kRows * 2];  // [g_z2; g_z1]^T pieces (rows: unit, K: sample)
   alignas(1024) unsigned char w[kPackedBytes];
-  float z1[kRows * kZs];
-  float z2[kRows * kZs];
   float red[4][kOut * kH + kOut + 1];  // per-warp dW3, db3, loss
   uint64_t bar;
   uint32_t tmem;
@@ -570,27 +720,77 @@ __device__ __forceinline__ void put2_t(unsigned char* img, uint32_t piece_bytes,
   *reinterpret_cast<uint16_t*>(img + piece_bytes + canon(row, s, KC)) = l;
 }
 
+// Sums of NV values over the 32 lanes, all at once: each step folds the values
+// in half and adds the other lane's share, so that 48 sums take 48 shuffles and
+// not 240.  Value j's sum ends in the lanes whose index bits pick it: out(j, v)
+// is called by one lane per value.  The additions are those of the shuffle tree
+// 16, 8, 4, 2, 1 of a single value.
+template <int NV, class F>
+__device__ __forceinline__ void warp_sums(float (&v)[NV], int lane, F out) {
+  static_assert(NV % 16 == 0, "four folds");
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int o = 16 >> s, m = NV >> (s + 1);
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < m; ++j) {
+      const float keep = up ? v[m + j] : v[j], send = up ? v[j] : v[m + j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  // lane bits 4..1 have picked the value's block of NV / 16
+  const int base = ((lane >> 4) & 1) * (NV / 2) + ((lane >> 3) & 1) * (NV / 4) + ((lane >> 2) & 1) * (NV / 8) +
+                   ((lane >> 1) & 1) * (NV / 16);
+#pragma unroll
+  for (int j = 0; j < NV / 16; ++j) {
+    const float x = v[j] + __shfl_xor_sync(0xffffffffu, v[j], 1);
+    if ((lane & 1) == 0) out(base + j, x);
+  }
+}
+
 // X[ntrain][27] stencils, N[ntrain][3] unit normals; batch = gridDim.x * 128
 // samples drawn with replacement by splitmix64(seed, step, slot).
 // partial[tile][kParams] gradients of the batch-mean loss, loss_part[tile].
-__global__ void __launch_bounds__(kThreads, 1)
+// Four threads per row: thread (row, quarter) holds 16 units of each hidden
+// layer (activations and derivatives in registers) and 8 of the inputs.  A
+// batch has fewer tiles than the part has SMs: a step's time is one tile's
+// chain: a step of 8192 took 64 us with one thread per row (one warp per SM
+// partition), 28 us now.
+__global__ void __launch_bounds__(kTrainThreads, 1)
 k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntrain, unsigned long long seed,
             long step, const unsigned char* __restrict__ params, float* __restrict__ partial,
             float* __restrict__ loss_part, const long* __restrict__ idx_fixed, int* __restrict__ status) {
   extern __shared__ unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, row = t & (kRows - 1), quarter = t >> 7;
   const int B = gridDim.x * kRows;
   const float invB = 1.0f / (float)B;
-  for (uint32_t o = t * 16; o < kPackedBytes; o += kThreads * 16)
+  for (uint32_t o = t * 16; o < kPackedBytes; o += kTrainThreads * 16)
     *reinterpret_cast<uint4*>(S.w + o) = __ldg(reinterpret_cast<const uint4*>(params + o));
   if (t == 0) mbar_init(&S.bar, 1);
   if (warp == 0) tmem_alloc(&S.tmem, kTrainCols);
+  // sample
+  const long slot = (long)blockIdx.x * kRows + row;
+  const long si = idx_fixed ? idx_fixed[slot]
+                            : (long)(mix64(seed ^ mix64((uint64_t)step * 0x100000001B3ull + (uint64_t)slot)) %
+                                     (uint64_t)ntrain);
+  // the feature after the 27 inputs is a constant 1 with zero weight: it
+  // carries the bias gradients through the weight-gradient contraction
+  float x[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int k = 8 * quarter + j;
+    x[j] = k < kIn ? input_of(__ldg(X + 27 * si + k)) : (k == kIn ? 1.f : 0.f);
+  }
+  float nn[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) nn[q] = f32_of(__ldg(N + 3 * si + q));
   tc_before_sync();
   __syncthreads();
   tc_after_sync();
   const uint32_t tm = S.tmem;
-  const uint32_t lb = (uint32_t)(warp * 32) << 16;
+  const uint32_t lb = (uint32_t)((warp & 3) * 32) << 16;
+  const int u0 = 16 * quarter;  // this thread's units
   const float* bias = reinterpret_cast<const float*>(S.w + pB);
   const float* w3f = reinterpret_cast<const float*>(S.w + pW3F);
   uint32_t ph = 0;
@@ -599,19 +799,9 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
   constexpr uint32_t kActPiece = kRows * kH * 2;
   constexpr uint32_t kAtPiece = kRows * kRows * 2;
   constexpr uint32_t kBtPiece = kTB * kRows * 2;
+  float a1[16], d1[16], a2[16], d2[16];  // GELU and its derivative of z1, z2
 
-  // sample
-  const long slot = (long)blockIdx.x * kRows + t;
-  const long si = idx_fixed ? idx_fixed[slot]
-                            : (long)(mix64(seed ^ mix64((uint64_t)step * 0x100000001B3ull + (uint64_t)slot)) %
-                                     (uint64_t)ntrain);
-  float x[32];
-#pragma unroll
-  for (int k = 0; k < 32; ++k) x[k] = k < kIn ? (float)(2.0 * __ldg(X + 27 * si + k) - 1.0) : (k == kIn ? 1.f : 0.f);
-  // the feature after the 27 inputs is a constant 1 with zero weight: it
-  // carries the bias gradients through the weight-gradient contraction
-#pragma unroll
-  for (int k0 = 0; k0 < 32; k0 += 8) put3(act, kActPiece, t, k0, 4, x + k0);
+  put3(act, kActPiece, row, 8 * quarter, 4, x);
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -621,19 +811,11 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
     umma_commit(&S.bar);
   }
   if (!(ok = train_wait(S, ph))) goto done;
+  tmem_ld16(tm + lb + u0, a1);
 #pragma unroll
-  for (int c0 = 0; c0 < kH; c0 += 16) {
-    float v[16];
-    tmem_ld16(tm + lb + c0, v);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float z = v[j] + bias[c0 + j];
-      S.z1[t * kZs + c0 + j] = z;
-      v[j] = gelu(z);
-    }
-    put3(act, kActPiece, t, c0, 8, v);
-    put3(act, kActPiece, t, c0 + 8, 8, v + 8);
-  }
+  for (int j = 0; j < 16; ++j) a1[j] = gelu_both(a1[j] + bias[u0 + j], d1[j]);
+  put3(act, kActPiece, row, u0, 8, a1);
+  put3(act, kActPiece, row, u0 + 8, 8, a1 + 8);
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -643,19 +825,11 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
     umma_commit(&S.bar);
   }
   if (!(ok = train_wait(S, ph))) goto done;
+  tmem_ld16(tm + lb + 64 + u0, a2);
 #pragma unroll
-  for (int c0 = 0; c0 < kH; c0 += 16) {
-    float v[16];
-    tmem_ld16(tm + lb + 64 + c0, v);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float z = v[j] + bias[kH + c0 + j];
-      S.z2[t * kZs + c0 + j] = z;
-      v[j] = gelu(z);
-    }
-    put3(act, kActPiece, t, c0, 8, v);
-    put3(act, kActPiece, t, c0 + 8, 8, v + 8);
-  }
+  for (int j = 0; j < 16; ++j) a2[j] = gelu_both(a2[j] + bias[kH + u0 + j], d2[j]);
+  put3(act, kActPiece, row, u0, 8, a2);
+  put3(act, kActPiece, row, u0 + 8, 8, a2 + 8);
   fence_async_smem();
   tc_before_sync();
   __syncthreads();
@@ -667,14 +841,12 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
   if (!(ok = train_wait(S, ph))) goto done;
   {
     // loss and its gradient at the output: yh = y / |y|_2, loss = |yh - n|^2
+    // (the row's four threads alike)
     float yv[16];
     tmem_ld16(tm + lb + 0, yv);
-    float y[3], nn[3];
+    float y[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      y[q] = yv[q] + bias[2 * kH + q];
-      nn[q] = (float)__ldg(N + 3 * si + q);
-    }
+    for (int q = 0; q < 3; ++q) y[q] = yv[q] + bias[2 * kH + q];
     const float ny = sqrtf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2]);
     float yh[3], gyh[3], gy[3];
     float loss = 0.f, dotp = 0.f;
@@ -691,38 +863,32 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
     // g_z2 = (g_y W3) * gelu'(z2): the A operand of g_a1 (three pieces, rows
     // = samples) and rows 0..63 of the transposed A of the weight gradients;
     // dW3, db3 and the loss by warp sums
+    float g[16];
 #pragma unroll
-    for (int c0 = 0; c0 < kH; c0 += 8) {
-      float g8[8];
+    for (int j = 0; j < 16; ++j) {
+      const int k = u0 + j;
+      g[j] = (gy[0] * w3f[k] + gy[1] * w3f[kH + k] + gy[2] * w3f[2 * kH + k]) * d2[j];
+      put2_t(S.at[0], kAtPiece, k, row, 16, g[j]);
+    }
+    put3(act, kActPiece, row, u0, 8, g);
+    put3(act, kActPiece, row, u0 + 8, 8, g + 8);
+    float pr[48];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int k = c0 + j;
-        const float z = S.z2[t * kZs + k];
-        const float ga = gy[0] * w3f[k] + gy[1] * w3f[kH + k] + gy[2] * w3f[2 * kH + k];
-        g8[j] = ga * gelu_grad(z);
-        put2_t(S.at[0], kAtPiece, k, t, 16, g8[j]);
-        const float a2 = gelu(z);
+    for (int q = 0; q < 3; ++q)
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          float pr = gy[q] * a2;
+      for (int j = 0; j < 16; ++j) pr[16 * q + j] = gy[q] * a2[j];
+    float* red = S.red[warp & 3];
+    warp_sums<48>(pr, lane, [&](int j, float s) { red[(j >> 4) * kH + u0 + (j & 15)] = s; });
+    if (quarter == 0) {
+      const float b4[4] = {gy[0], gy[1], gy[2], loss};
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) pr += __shfl_xor_sync(0xffffffffu, pr, o);
-          if (lane == 0) S.red[warp][q * kH + k] = pr;
-        }
+      for (int q = 0; q < 4; ++q) {
+        float s = b4[q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) red[kOut * kH + q] = s;
       }
-      put3(act, kActPiece, t, c0, 8, g8);
     }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      float pr = gy[q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) pr += __shfl_xor_sync(0xffffffffu, pr, o);
-      if (lane == 0) S.red[warp][kOut * kH + q] = pr;
-    }
-    float ls = loss;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, o);
-    if (lane == 0) S.red[warp][kOut * kH + kOut] = ls;
   }
   fence_async_smem();
   tc_before_sync();
@@ -740,20 +906,15 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
     // feature (rows 64..95), two pieces each, in the activation buffer
     // (free now: the MMAs that read it are complete)
     unsigned char* bt = S.act[0];
+    float v[16];
+    tmem_ld16(tm + lb + u0, v);
 #pragma unroll
-    for (int c0 = 0; c0 < kH; c0 += 16) {
-      float v[16];
-      tmem_ld16(tm + lb + c0, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int k = c0 + j;
-        const float z = S.z1[t * kZs + k];
-        put2_t(S.at[0], kAtPiece, kH + k, t, 16, v[j] * gelu_grad(z));
-        put2_t(bt, kBtPiece, k, t, 16, gelu(z));
-      }
+    for (int j = 0; j < 16; ++j) {
+      put2_t(S.at[0], kAtPiece, kH + u0 + j, row, 16, v[j] * d1[j]);
+      put2_t(bt, kBtPiece, u0 + j, row, 16, a1[j]);
     }
 #pragma unroll
-    for (int k = 0; k < 32; ++k) put2_t(bt, kBtPiece, kH + k, t, 16, x[k]);
+    for (int j = 0; j < 8; ++j) put2_t(bt, kBtPiece, kH + 8 * quarter + j, row, 16, x[j]);
   }
   fence_async_smem();
   tc_before_sync();
@@ -777,29 +938,31 @@ k_mlp_train(const double* __restrict__ X, const double* __restrict__ N, long ntr
   if (!(ok = train_wait(S, ph))) goto done;
   {
     float* prow = partial + (size_t)blockIdx.x * kParams;
-    // row t of the accumulator: t < 64 is unit t of layer 2, else unit
-    // t - 64 of layer 1
+    // row r of the accumulator: r < 64 is unit r of layer 2, else unit
+    // r - 64 of layer 1; a quarter takes the blocks u0 and u0 + 64 of columns
 #pragma unroll
-    for (int c0 = 0; c0 < kTB; c0 += 16) {
+    for (int cb = 0; cb < kTB; cb += 64) {
+      const int c0 = cb + u0;
+      if (c0 >= kTB) continue;  // (uniform in a warp)
       float v[16];
       tmem_ld16(tm + lb + 64 + c0, v);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         const int col = c0 + j;
-        if (t < kH) {
-          if (col < kH) prow[oW2 + t * kH + col] = v[j];
-          else if (col == kH + kIn) prow[oB2 + t] = v[j];
+        if (row < kH) {
+          if (col < kH) prow[oW2 + row * kH + col] = v[j];
+          else if (col == kH + kIn) prow[oB2 + row] = v[j];
         } else {
-          if (col >= kH && col < kH + kIn) prow[oW1 + (t - kH) * kIn + (col - kH)] = v[j];
-          else if (col == kH + kIn) prow[oB1 + (t - kH)] = v[j];
+          if (col >= kH && col < kH + kIn) prow[oW1 + (row - kH) * kIn + (col - kH)] = v[j];
+          else if (col == kH + kIn) prow[oB1 + (row - kH)] = v[j];
         }
       }
     }
     // dW3, db3, loss: the four warps' sums in order
-    for (int q = t; q < kOut * kH + kOut + 1; q += kThreads) {
-      const float v = ((S.red[0][q] + S.red[1][q]) + S.red[2][q]) + S.red[3][q];
-      if (q < kOut * kH) prow[oW3 + q] = v;
-      else if (q < kOut * kH + kOut) prow[oB3 + q - kOut * kH] = v;
+    if (t < kOut * kH + kOut + 1) {
+      const float v = ((S.red[0][t] + S.red[1][t]) + S.red[2][t]) + S.red[3][t];
+      if (t < kOut * kH) prow[oW3 + t] = v;
+      else if (t < kOut * kH + kOut) prow[oB3 + t - kOut * kH] = v;
       else loss_part[blockIdx.x] = v * invB;
     }
   }
@@ -811,21 +974,27 @@ done:
   if (warp == 0) tmem_dealloc(tm, kTrainCols);
 }
 
+constexpr int kAdamThreads = 64;  // 6147 parameters over the SMs
 // Adam on the FP32 master parameters from the tiles' partial gradients
 // (summed in tile order), then the packed BF16 images of the new values;
 // loss_out (nullable) = the batch-mean loss.
-__global__ void k_mlp_adam(float* __restrict__ master, float* __restrict__ mom, float* __restrict__ vel,
+__global__ void __launch_bounds__(kAdamThreads) k_mlp_adam(float* __restrict__ master, float* __restrict__ mom, float* __restrict__ vel,
                            const float* __restrict__ partial, const float* __restrict__ loss_part, int ntiles,
                            long step, float lr, float beta1, float beta2, float eps, unsigned char* __restrict__ P,
                            float* __restrict__ grad_out, float* __restrict__ loss_out) {
+  pdl_wait();
+  partial = after_wait(partial);
+  loss_part = after_wait(loss_part);
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q == 0 && loss_out) {
+  if (q == (int)(gridDim.x * blockDim.x) - 1 && loss_out) {  // (a thread without a parameter)
     float l = 0.f;
+#pragma unroll 16
     for (int b = 0; b < ntiles; ++b) l += loss_part[b];
     *loss_out = l;
   }
   if (q >= kParams) return;
   float g = 0.f;
+#pragma unroll 16  // (the loads of 16 tiles in flight; the sum stays in tile order)
   for (int b = 0; b < ntiles; ++b) g += partial[(size_t)b * kParams + q];
   if (grad_out) grad_out[q] = g;
   if (!(lr > 0.f)) return;  // gradient only
@@ -850,15 +1019,14 @@ int mlp_param_count() { return mlp::kParams; }
 static size_t infer_smem() { return sizeof(mlp::InferSmem) + 1024; }
 static size_t train_smem() { return sizeof(mlp::TrainSmem) + 1024; }
 
-template <int MODE, class Src>
-static cudaError_t launch_infer_t(const Src& src, const int* count_dev, long n_host, long max_n,
-                                  const void* params, float* y, double* m, uint8_t* flag, double* plane,
-                                  int* nfallback, cudaStream_t st) {
+template <class Src, class Out>
+static cudaError_t launch_infer_t(const Src& src, const Out& out, const int* count_dev, long n_host, long max_n,
+                                  const void* params, cudaStream_t st) {
   static bool attr_set[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(mlp::k_mlp_infer<MODE, Src>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(mlp::k_mlp_infer<Src, Out>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)infer_smem());
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
@@ -866,10 +1034,20 @@ static cudaError_t launch_infer_t(const Src& src, const int* count_dev, long n_h
   const long tiles = (max_n + mlp::kRows - 1) / mlp::kRows;
   long grid = tiles < 152 * 3 ? tiles : 152 * 3;
   if (grid < 1) grid = 1;
-  mlp::k_mlp_infer<MODE, Src><<<(unsigned)grid, mlp::kThreads, infer_smem(), st>>>(
-      src, count_dev, n_host, static_cast<const unsigned char*>(params), y, m, flag, plane, nfallback,
-      device_status_ptr());
-  prof_mark(MODE == 2 ? "mlp.normals" : "mlp.infer", st);
+  mlp::k_mlp_infer<Src, Out><<<(unsigned)grid, mlp::kInferThreads, infer_smem(), st>>>(
+      src, count_dev, n_host, static_cast<const unsigned char*>(params), out, device_status_ptr());
+  prof_mark("mlp.infer", st);
+  return cudaGetLastError();
+}
+
+template <bool GRID, class Src, class Out>
+static cudaError_t launch_choose_t(const Src& src, const Out& out, const int* count_dev, long n_host, long max_n,
+                                   uint8_t* flag, int* nfallback, cudaStream_t st) {
+  const long ctas = std::min<long>((max_n + 31) / 32, 152 * 8);
+  using mlp::k_mlp_choose;
+  launch_pdl(k_mlp_choose<GRID, Src, Out>, dim3((unsigned)std::max<long>(ctas, 1)), dim3(mlp::kChooseThreads), st,
+             src, count_dev, n_host, out, flag, nfallback);
+  prof_mark("mlp.normals", st);
   return cudaGetLastError();
 }
 
@@ -881,21 +1059,26 @@ cudaError_t launch_mlp_pack(const float* master, void* packed, cudaStream_t st) 
 }
 
 cudaError_t launch_mlp_forward(const void* params, const double* X, long n, float* y, cudaStream_t st) {
-  return launch_infer_t<0>(mlp::SrcX{X}, nullptr, n, n, params, y, nullptr, nullptr, nullptr, nullptr, st);
+  return launch_infer_t(mlp::SrcX{X}, mlp::OutY{y}, nullptr, n, n, params, st);
 }
 
 cudaError_t launch_mlp_normals(const void* params, const double* X, long n, double* m, uint8_t* flag,
                                int* nfallback, cudaStream_t st) {
-  return launch_infer_t<1>(mlp::SrcX{X}, nullptr, n, n, params, nullptr, m, flag, nullptr, nfallback, st);
+  const mlp::SrcX src{X};
+  const mlp::OutM out{m};
+  const cudaError_t err = launch_infer_t(src, out, nullptr, n, n, params, st);
+  return err != cudaSuccess ? err : launch_choose_t<false>(src, out, nullptr, n, n, flag, nfallback, st);
 }
 
 cudaError_t launch_mlp_sweep_normals(const GridDev& g, const double* c, bool tagged, const uint32_t* list,
                                      int* counters, double* plane, cudaStream_t st) {
-  const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-  mlp::SrcGrid src{g, c, list, tagged ? 0x3FFFFFFFu : 0xFFFFFFFFu};
+  const long N = (long)g.n[0] * g.n[1] * g.n[2];
+  const mlp::SrcGrid src{g, c, list, tagged ? 0x3FFFFFFFu : 0xFFFFFFFFu};
+  const mlp::OutPlane out{plane, list};
   // the mixed-cell count (counters[0]) is read on the device; fallbacks are
   // counted in counters[3]
-  return launch_infer_t<2>(src, counters, 0, (long)N, g.mlp_params, nullptr, nullptr, nullptr, plane, counters + 3, st);
+  const cudaError_t err = launch_infer_t(src, out, counters, 0, N, g.mlp_params, st);
+  return err != cudaSuccess ? err : launch_choose_t<true>(src, out, counters, 0, N, nullptr, counters + 3, st);
 }
 
 cudaError_t launch_mlp_train_step(const double* X, const double* N, long ntrain, int batch, unsigned long long seed,
@@ -912,14 +1095,14 @@ cudaError_t launch_mlp_train_step(const double* X, const double* N, long ntrain,
     attr_set[dev] = true;
   }
   const int tiles = batch / mlp::kRows;
-  mlp::k_mlp_train<<<tiles, mlp::kThreads, train_smem(), st>>>(X, N, ntrain, seed, step,
+  mlp::k_mlp_train<<<tiles, mlp::kTrainThreads, train_smem(), st>>>(X, N, ntrain, seed, step,
                                                               static_cast<const unsigned char*>(packed), partial,
                                                               loss_part, idx_fixed, device_status_ptr());
   prof_mark("mlp.train", st);
-  mlp::k_mlp_adam<<<(mlp::kParams + 255) / 256, 256, 0, st>>>(master, mom, vel, partial, loss_part, tiles, step, lr,
-                                                               beta1, beta2, eps,
-                                                               static_cast<unsigned char*>(packed), grad_out,
-                                                               loss_out);
+  using mlp::k_mlp_adam;
+  launch_pdl(k_mlp_adam, dim3(mlp::kParams / mlp::kAdamThreads + 1), dim3(mlp::kAdamThreads), st, master, mom, vel,
+             (const float*)partial, (const float*)loss_part, tiles, step, lr, beta1, beta2, eps,
+             static_cast<unsigned char*>(packed), grad_out, loss_out);
   prof_mark("mlp.adam", st);
   return cudaGetLastError();
 }
