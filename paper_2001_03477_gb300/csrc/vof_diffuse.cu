@@ -604,14 +604,18 @@ k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ ch
 
 // One later sweep of the phase form, d' = sum B_nb d_nb + s, two cells of a row
 // per thread: every packed instruction serves both.  A cell whose own s and
-// neighbours' d are all 0 keeps 0 without arithmetic.
+// neighbours' d are all 0 keeps 0 without arithmetic.  (z walked in consecutive
+// planes held in registers, for a third of the reads of d, took 25 us at 128^3
+// against 22: the loads' latency bounds it, and that form keeps fewer warps.)
 template <bool CHECK>
 __global__ void __launch_bounds__(kDifThreads)
 k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, float* __restrict__ dout,
             const unsigned long long* __restrict__ prev, double tol, unsigned long long* __restrict__ change) {
   pdl_wait();
   using namespace df;
-  if (dif_done(prev, tol)) return;
+  din = after_wait(din);
+  v.s = after_wait(v.s);
+  if (dif_done(after_wait(prev), tol)) return;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
   const int x = (blockIdx.x * 32 + threadIdx.x) * 2, y = blockIdx.y * 8 + threadIdx.y;
   const bool in = x < nx && y < ny, in1 = x + 1 < nx && y < ny;
