@@ -286,7 +286,6 @@ bool step_box(const vof_grid* g, double* c, double* e, const double* u, const do
   A.rows = reinterpret_cast<double*>(ws + L.off_rows);
   A.ts = carve_tile_scratch(d, ws + L.off_tiles);
   tile_counts(d, A.nt);
-  A.usable = tiles_usable(d) ? 1 : 0;
   A.stats = reinterpret_cast<int*>(ws + L.off_stats);
   A.cnt = reinterpret_cast<int*>(ws + L.off_stats + 128);
   A.status = device_status_ptr();

@@ -201,7 +201,6 @@ struct TileScratch {
   uint8_t* quiet;
 };
 void tile_counts(const GridDev& g, int nt[3]);
-bool tiles_usable(const GridDev& g);
 int tile_total(const GridDev& g);
 size_t tile_scratch_bytes(const GridDev& g);
 TileScratch carve_tile_scratch(const GridDev& g, void* ws);
@@ -234,7 +233,6 @@ struct StepArgs {
   double* rows;          // [tiles][kNSums] sum rows
   TileScratch ts;
   int nt[3];
-  int usable;            // quiet tiles may be skipped (tiles_usable)
   int* cnt;              // [kStepCounters]
   int* stats;            // [VOF_NCOUNTS] work counts, by axis
   int* status;

@@ -98,3 +98,21 @@ def test_chains_equal_standalone_calls(P, dense):
     n = 200
     c, e, vel = fields((n, n, n), (0, 1, 0), 5, dense)
     check(P, P.Grid(n, n, n, (0, 1, 0), 1.0, 900.0, 1.5, 1.0), c, e, vel, 1.0, -0.02)
+
+
+@pytest.mark.parametrize("shape", [(41, 34, 26), (26, 41, 25), (33, 18, 50)])
+@pytest.mark.parametrize("at", [0.0, 4.5, -2.5, -6.5, -10.5, 11.0])
+def test_quiet_tiles_across_a_short_last_tile(P, shape, at):
+    """Periodic axes whose last tile holds one or two cells: a small drop near
+    the wrap leaves quiet tiles whose three-cell halo spans that tile."""
+    import torch
+    nx, ny, nz = shape
+    z, y, x = torch.meshgrid(*[torch.arange(n, dtype=torch.float64, device="cuda") + 0.5 for n in (nz, ny, nx)], indexing="ij")
+    d2 = 0.0
+    for q, n, o in ((x, nx, at), (y, ny, 0.3 * at), (z, nz, -at)):
+        d = (q - o) % n
+        d2 = d2 + torch.minimum(d, n - d) ** 2
+    c = (3.2 - d2.sqrt()).clamp(0.0, 1.0)
+    vel = fields((nz, ny, nx), (0, 0, 0), 3, False)[2]
+    g = P.Grid(nx, ny, nz, (0, 0, 0), 1.0, 900.0, 1.5, 1.0)
+    check(P, g, c, 900.0 * c + 1.5 * (1.0 - c), vel, 1.0, 0.02)
