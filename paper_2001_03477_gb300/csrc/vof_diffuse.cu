@@ -42,7 +42,8 @@
 // rounding stays below an ulp of T), over the power of two next to the largest
 // T.  What bounds a sweep on this part is the
 // FP64 unit: 8 FP64 instructions per cell took 45 us at 128^3 (76 cycles of an
-// SM partition each); the pairs' FP32 instructions take 22 us (its reads come from L2).  The sweeps
+// SM partition each); the pairs' FP32 instructions take 20.6 us (two cells of a row in one 16-byte
+// block; 22 us with high and low parts in arrays of their own).  The sweeps
 // are queued in batches without waiting: each starts by reading the last
 // check's result and leaves its buffers alone once that was within tol.
 // Mixture heat capacity: the FP64 form, every cell's diagonal stored.
@@ -219,18 +220,18 @@ struct DifVec {
   double* Tb;
   unsigned long long* part;  // [kDifChecks] the largest change of each checked sweep of a batch (bits)
   uint8_t* cls;   // [N] cell class
-  // phase form: pairs, high and low parts in arrays of their own, x rows padded
-  // to an even length px (two cells of a row are one aligned 8-byte access)
-  float* s;       // [2][px ny nz]: s, also the first iterate d
-  float* d[2];    // the two later iterates
+  // phase form: two cells of a row (x even, x + 1) in 16 bytes, {hi, hi, lo, lo},
+  // a row of px such blocks
+  float4* s;      // [px ny nz]: s, also the first iterate d
+  float4* d[2];   // the two later iterates
   int px;
-  size_t pn;      // px ny nz: the low parts' offset
   int* tmax;      // largest exponent field of a finite T0
 };
 // the pairs hold d / 2^k
 __device__ __forceinline__ int dif_scale(const DifVec& v, const DifConst& K) { return max(*v.tmax, K.e0) - 1023; }
-__device__ __forceinline__ size_t pad_id(const GridDev& g, const DifVec& v, int x, int y, int z) {
-  return ((size_t)z * g.n[1] + y) * v.px + x;
+// the high part of cell (x, y, z) in array a; the low part is two floats on
+__device__ __forceinline__ float* part_of(const GridDev& g, const DifVec& v, float4* a, int x, int y, int z) {
+  return reinterpret_cast<float*>(a + ((size_t)z * g.n[1] + y) * v.px + (x >> 1)) + (x & 1);
 }
 
 constexpr long long kHalfBits = 0x3FE0000000000000LL;  // 0.5: c >= 1/2 on the integer pipe (c >= +0)
@@ -342,7 +343,7 @@ __device__ __forceinline__ df::f2 f2_of(float2 p) { return df::f2{p.x, p.y}; }
 // Per listed cell (lanes dense over the list): the six couplings (heights
 // or plane distances on the interface sides), the diagonal and the right
 // side.
-__global__ void __launch_bounds__(kDifThreads)
+__global__ void __launch_bounds__(kDifPlaneThreads)
 k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, double k_g,
                 const double* __restrict__ c, const double* __restrict__ e, const double4* __restrict__ plane,
                 DifVec v, DifWalls walls, int phase_cp, DifConst K, const uint32_t* __restrict__ ilist,
@@ -424,9 +425,9 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
 #pragma unroll
       for (int f = 0; f < 6; ++f) reinterpret_cast<float2*>(v.off)[6 * i + f] = pair_of(off[f] * rd, 0);
       const float2 sp = pair_of(gain * rd, ks);
-      const size_t ip = pad_id(g, v, x, y, z);
-      v.s[ip] = sp.x;
-      v.s[v.pn + ip] = sp.y;
+      float* const at = part_of(g, v, v.s, x, y, z);
+      at[0] = sp.x;
+      at[2] = sp.y;
     } else {
 #pragma unroll
       for (int f = 0; f < 6; ++f) v.off[6 * i + f] = off[f];
@@ -589,12 +590,12 @@ k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ ch
       if (vary) r = pair_of(sv, ks);
     }
     if (in) {
-      const size_t ip = pad_id(g, v, x, y, z);
+      float* const at = part_of(g, v, v.s, x, y, z);
       if (!irr) {
-        v.s[ip] = r.x;
-        v.s[v.pn + ip] = r.y;
+        at[0] = r.x;
+        at[2] = r.y;
       } else if (CHECK) {
-        r.x = v.s[ip];
+        r.x = at[0];
       }
     }
     if (CHECK) dmax = fmaxf(dmax, fabsf(r.x));
@@ -609,7 +610,7 @@ k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ ch
 // against 22: the loads' latency bounds it, and that form keeps fewer warps.)
 template <bool CHECK>
 __global__ void __launch_bounds__(kDifThreads)
-k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, float* __restrict__ dout,
+k_dif_sweep(GridDev g, DifVec v, DifConst K, const float4* __restrict__ din, float4* __restrict__ dout,
             const unsigned long long* __restrict__ prev, double tol, unsigned long long* __restrict__ change) {
   pdl_wait();
   using namespace df;
@@ -617,43 +618,47 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, floa
   v.s = after_wait(v.s);
   if (dif_done(after_wait(prev), tol)) return;
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-  const int x = (blockIdx.x * 32 + threadIdx.x) * 2, y = blockIdx.y * 8 + threadIdx.y;
+  const int xb = blockIdx.x * 32 + threadIdx.x, x = 2 * xb, y = blockIdx.y * 8 + threadIdx.y;
   const bool in = x < nx && y < ny, in1 = x + 1 < nx && y < ny;
-  const float* __restrict__ dlo = din + v.pn;
-  const long long row = v.px, plane = row * ny;
+  const int row = v.px;
+  const long long plane = (long long)row * ny;
   // sides of the pair: the outer x neighbours, y and z (those two cells share)
-  const bool px = g.bc[0] == 0;
-  const bool hasL = x > 0 || px, hasR = (in1 ? x + 1 : x) < nx - 1 || px;
-  const int oL = x > 0 ? -1 : nx - 1, oR = in1 ? (x + 2 < nx ? 2 : -x) : -x;
+  const bool wrap = g.bc[0] == 0;
+  const bool hasL = x > 0 || wrap, hasR = (in1 ? x + 1 : x) < nx - 1 || wrap;
+  const int oL = x > 0 ? -1 : (nx - 1) >> 1, oR = x + 2 < nx ? 1 : -xb;  // blocks of the outer neighbours
+  const bool oddL = x > 0 || (nx & 1) == 0;                             // and L's place in its block (R's is the first)
   const bool hasS = y > 0 || g.bc[1] == 0, hasN = y < ny - 1 || g.bc[1] == 0;
-  const long long oS = y > 0 ? -row : (ny - 1) * row, oN = y < ny - 1 ? row : (1 - ny) * row;
+  const long long oS = y > 0 ? -row : (ny - 1) * (long long)row, oN = y < ny - 1 ? row : (1 - ny) * (long long)row;
   float dmax = 0.f;
   for (int z = blockIdx.z; z < nz; z += gridDim.z) {
     const bool hasB = z > 0 || g.bc[2] == 0, hasT = z < nz - 1 || g.bc[2] == 0;
     const long long oB = z > 0 ? -plane : (nz - 1) * plane, oT = z < nz - 1 ? plane : (1 - nz) * plane;
-    const long long ip = in ? z * plane + y * row + x : 0;
-    const float2 zero = make_float2(0.f, 0.f);
-    auto two = [&](const float* a, bool ok, long long o) {
-      return ok ? __ldg(reinterpret_cast<const float2*>(a + ip + o)) : zero;
-    };
-    auto one = [&](const float* a, bool ok, long long o) { return ok ? __ldg(a + ip + o) : 0.f; };
-    const float2 sh = two(v.s, in, 0), sl = two(v.s + v.pn, in, 0);
-    float2 ch = two(din, in, 0), cl = two(dlo, in, 0);
-    if (!in1) ch.y = cl.y = 0.f;  // (the padding)
-    const float2 Sh = two(din, in && hasS, oS), Sl = two(dlo, in && hasS, oS);
-    const float2 Nh = two(din, in && hasN, oN), Nl = two(dlo, in && hasN, oN);
-    const float2 Bh = two(din, in && hasB, oB), Bl = two(dlo, in && hasB, oB);
-    const float2 Th = two(din, in && hasT, oT), Tl = two(dlo, in && hasT, oT);
-    const float Lh = one(din, in && hasL, oL), Ll = one(dlo, in && hasL, oL);
-    const float Rh = one(din, in && hasR, oR), Rl = one(dlo, in && hasR, oR);
-    const unsigned c0 = in ? __ldg(v.cls + ((size_t)z * ny + y) * nx + x) : 0u;
-    const unsigned c1 = in1 ? __ldg(v.cls + ((size_t)z * ny + y) * nx + x + 1) : 0u;
+    const long long ip = in ? z * plane + (long long)y * row + xb : 0;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto at = [&](const float4* a, bool ok, long long o) { return ok ? __ldg(a + ip + o) : zero; };
+    const float4 s4 = at(v.s, in, 0);
+    float4 c4 = at(din, in, 0);
+    if (!in1) c4.y = c4.w = 0.f;  // (the padding)
+    const float4 S4 = at(din, in && hasS, oS), N4 = at(din, in && hasN, oN);
+    const float4 B4 = at(din, in && hasB, oB), T4 = at(din, in && hasT, oT);
+    const float4 L4 = at(din, in && hasL, oL), R4 = at(din, in && hasR, oR);
+    const float2 sh = make_float2(s4.x, s4.y), sl = make_float2(s4.z, s4.w);
+    const float2 ch = make_float2(c4.x, c4.y), cl = make_float2(c4.z, c4.w);
+    const float2 Sh = make_float2(S4.x, S4.y), Sl = make_float2(S4.z, S4.w);
+    const float2 Nh = make_float2(N4.x, N4.y), Nl = make_float2(N4.z, N4.w);
+    const float2 Bh = make_float2(B4.x, B4.y), Bl = make_float2(B4.z, B4.w);
+    const float2 Th = make_float2(T4.x, T4.y), Tl = make_float2(T4.z, T4.w);
+    const float Lh = oddL ? L4.y : L4.x, Ll = oddL ? L4.w : L4.z;
+    const float Rh = R4.x, Rl = R4.z;
+    const size_t ic = ((size_t)z * ny + y) * nx + x;
+    const unsigned c0 = in ? __ldg(v.cls + ic) : 0u;
+    const unsigned c1 = in1 ? __ldg(v.cls + ic + 1) : 0u;
     auto fb = [](float f) { return __float_as_uint(f); };
     // (a pair's high part is 0 exactly where the pair is; the padding's values
     // reach no cell)
     const unsigned any = (fb(sh.x) | fb(ch.x) | fb(Sh.x) | fb(Nh.x) | fb(Bh.x) | fb(Th.x) | fb(Lh) | fb(Rh) |
                           (in1 ? fb(sh.y) | fb(ch.y) | fb(Sh.y) | fb(Nh.y) | fb(Bh.y) | fb(Th.y) : 0u)) & 0x7FFFFFFFu;
-    float2 rh = zero, rl = zero;
+    float2 rh = make_float2(0.f, 0.f), rl = rh;
     if (__any_sync(0xffffffffu, any != 0u)) {
       // left and right neighbours of both cells: (L, c0), (c1, R); a lone last
       // cell's right neighbour is R
@@ -676,13 +681,12 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, floa
       vget(r.lo, rl.x, rl.y);
       if (__any_sync(0xffffffffu, ((c0 | c1) & kDifIrr) != 0u)) {
         // cells next to the interface or a heated wall: their own couplings
-        const size_t i = ((size_t)z * ny + y) * nx + x;
         const float2 n0[6] = {make_float2(Lh, Ll), in1 ? make_float2(ch.y, cl.y) : make_float2(Rh, Rl),
                               make_float2(Sh.x, Sl.x), make_float2(Nh.x, Nl.x), make_float2(Bh.x, Bl.x), make_float2(Th.x, Tl.x)};
         const float2 n1[6] = {make_float2(ch.x, cl.x), make_float2(Rh, Rl), make_float2(Sh.y, Sl.y),
                               make_float2(Nh.y, Nl.y), make_float2(Bh.y, Bl.y), make_float2(Th.y, Tl.y)};
         f2 e0 = f2{sh.x, sl.x}, e1 = f2{sh.y, sl.y};
-        const float2* off = reinterpret_cast<const float2*>(v.off) + 6 * i;
+        const float2* off = reinterpret_cast<const float2*>(v.off) + 6 * ic;
 #pragma unroll
         for (int f = 0; f < 6; ++f) {
           if ((c0 & kDifIrr) && (c0 & (1u << f))) e0 = add_c(mul(f2_of(__ldg(off + f)), f2_of(n0[f])), e0);
@@ -692,10 +696,7 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, floa
         if (c1 & kDifIrr) { rh.y = e1.hi; rl.y = e1.lo; }
       }
     }
-    if (in) {
-      *reinterpret_cast<float2*>(dout + ip) = rh;
-      *reinterpret_cast<float2*>(dout + v.pn + ip) = rl;
-    }
+    if (in) dout[ip] = make_float4(rh.x, rh.y, rl.x, rl.y);
     if (CHECK) {
       dmax = fmaxf(dmax, fabsf((rh.x - ch.x) + (rl.x - cl.x)));
       if (in1) dmax = fmaxf(dmax, fabsf((rh.y - ch.y) + (rl.y - cl.y)));
@@ -706,13 +707,14 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float* __restrict__ din, floa
 
 // e' = e + C_p,node d; a node without change keeps its e
 __global__ void __launch_bounds__(kDifThreads)
-k_dif_store_phase(GridDev g, const DifVec v, DifConst K, const float* __restrict__ d, double* __restrict__ e) {
+k_dif_store_phase(GridDev g, const DifVec v, DifConst K, float4* d, double* __restrict__ e) {
   const int ks = dif_scale(v, K);
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
   if (x >= g.n[0] || y >= g.n[1]) return;
   for (int z = blockIdx.z; z < g.n[2]; z += gridDim.z) {
-    const size_t i = ((size_t)z * g.n[1] + y) * g.n[0] + x, ip = pad_id(g, v, x, y, z);
-    const float hi = __ldg(d + ip), lo = __ldg(d + v.pn + ip);
+    const size_t i = ((size_t)z * g.n[1] + y) * g.n[0] + x;
+    const float* const at = part_of(g, v, d, x, y, z);
+    const float hi = at[0], lo = at[2];
     if (hi == 0.f && lo == 0.f) continue;
     const double Cd = (__ldg(v.cls + i) & kDifLiq) ? g.Cp_l : g.Cp_g;
     e[i] = e[i] + Cd * (wide_of(hi, ks) + wide_of(lo, ks));
@@ -773,13 +775,13 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   v.Tb = reinterpret_cast<double*>(ws + L.Tb);
   v.part = reinterpret_cast<unsigned long long*>(ws + L.part);
   v.cls = reinterpret_cast<uint8_t*>(ws + L.cls);
-  // the padded pairs (px / nx <= 2 cell arrays each): s in diag's and rhs's
+  // the pairs' blocks (up to two cell arrays each): s in diag's and rhs's
   // place, the iterates in the planes' (not read any more when they are written)
-  v.px = (g.n[0] + 1) & ~1;
-  v.pn = (size_t)v.px * g.n[1] * g.n[2];
-  v.s = reinterpret_cast<float*>(ws + L.diag);
-  v.d[0] = reinterpret_cast<float*>(ws + L.plane);
-  v.d[1] = v.d[0] + 2 * v.pn;
+  v.px = (g.n[0] + 1) / 2;
+  const size_t pn = (size_t)v.px * g.n[1] * g.n[2];
+  v.s = reinterpret_cast<float4*>(ws + L.diag);
+  v.d[0] = reinterpret_cast<float4*>(ws + L.plane);
+  v.d[1] = v.d[0] + pn;
   uint32_t* mlist = reinterpret_cast<uint32_t*>(ws + L.mlist);
   int* count = reinterpret_cast<int*>(ws + L.count);
   v.tmax = count + 2;
@@ -820,7 +822,7 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   const dim3 sgrid = dif_sweep_grid(g);
   if (phase_cp) k_dif_classify<true><<<sgrid, dim3(32, 8), 0, st>>>(g, c, e, v, walls, inv_dt, K, ilist, count + 1);
   else k_dif_classify<false><<<sgrid, dim3(32, 8), 0, st>>>(g, c, e, v, walls, inv_dt, K, ilist, count + 1);
-  k_dif_irregular<<<grid, kDifThreads, 0, st>>>(g, h, inv_h, inv_dt, k_l, k_g, c, e, plane, v, walls, phase_cp, K,
+  k_dif_irregular<<<kDifCTAs, kDifPlaneThreads, 0, st>>>(g, h, inv_h, inv_dt, k_l, k_g, c, e, plane, v, walls, phase_cp, K,
                                                  ilist, count + 1);
   prof_mark("diffuse.assemble", st);
   // Sweeps in batches, each with its checks' slots cleared first: a sweep
@@ -836,7 +838,7 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   double change = 0.0, before = 0.0;
   bool done = false;
   auto iterate = [&](int n) -> double* { return n == 0 ? v.T0 : buf[n & 1]; };  // the n-th sweep's result
-  auto iterate_d = [&](int n) -> float* { return n <= 1 ? v.s : v.d[n & 1]; };
+  auto iterate_d = [&](int n) -> float4* { return n <= 1 ? v.s : v.d[n & 1]; };
   // two cells of a row per thread
   const dim3 pgrid((unsigned)((g.n[0] + 63) / 64), sgrid.y,
                    (unsigned)std::max(1, std::min(g.n[2], (int)(152u * 16u / std::max(1u, (unsigned)((g.n[0] + 63) / 64) * sgrid.y)))));
@@ -855,8 +857,8 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
         if (check) k_dif_first<true><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, chg);
         else k_dif_first<false><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, chg);
       } else if (phase_cp) {
-        const float* di = iterate_d(it);
-        float* dd = iterate_d(it + 1);
+        const float4* di = iterate_d(it);
+        float4* dd = iterate_d(it + 1);
         if (check) launch_pdl(k_dif_sweep<true>, pgrid, dim3(32, 8), st, g, v, K, di, dd, prev, tol, chg);
         else launch_pdl(k_dif_sweep<false>, pgrid, dim3(32, 8), st, g, v, K, di, dd, prev, tol, chg);
       } else {
