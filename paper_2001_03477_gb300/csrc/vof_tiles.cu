@@ -118,8 +118,8 @@ __device__ __forceinline__ double times_cells(int n, long long v) {
   return r;
 }
 
-// One warp per tile: quiet flag (a lane for each of the tile and its 26
-// neighbours, up to 64 with the far ones).  A quiet tile's sum row is (cells) x value; any other
+// One warp per tile: quiet flag (lanes 0..26 check the tile and its 26
+// neighbours at once; the far ones, where there are any, in two rounds).  A quiet tile's sum row is (cells) x value; any other
 // tile joins the active list, and its mixed cells the first stage's list
 // (one atomic per tile and list; both orders vary from run to run).
 __device__ __forceinline__ void k_quiet_body(const StepArgs& A, const VB vb) {
@@ -134,26 +134,38 @@ __device__ __forceinline__ void k_quiet_body(const StepArgs& A, const VB vb) {
   // cells are read) spread over the SMs
   for (long long t = vb.bx + (long long)vb.gx * (threadIdx.x >> 5); t < nt; t += (long long)vb.gx * wpb) {
     const int tx = (int)(t % ntx), ty = (int)((t / ntx) % nty), tz = (int)(t / ((long long)ntx * nty));
-    // the tile itself, then its neighbours: the o-th at offset (o % 3 - 1, o / 3
-    // % 3 - 1, o / 9 - 1), or with a fourth choice, the far one, along an axis
-    // that has it; one beyond a zero-gradient boundary counts as equal
-    const size_t self = ((size_t)tz * nty + ty) * ntx + tx;
-    const bool uni = ts.uni[self] != 0;
-    const long long cr = dbits(ts.vc[self]), er = dbits(ts.ve[self]);
-    const bool pure = cr == 0 || cr == 0x3FF0000000000000LL;
+    // lane o < 27: the tile at offset (o % 3 - 1, o / 3 % 3 - 1, o / 9 - 1);
+    // one beyond a zero-gradient boundary counts as equal
+    bool nb_ok = true, nb_uni = true;
+    long long nb_c = 0, nb_e = 0;
+    auto look = [&](int px, int py, int pz) {
+      nb_ok = (px | py | pz) >= 0;
+      if (nb_ok) {
+        const size_t u = ((size_t)pz * nty + py) * ntx + px;
+        nb_uni = ts.uni[u] != 0;
+        nb_c = dbits(ts.vc[u]);
+        nb_e = dbits(ts.ve[u]);
+      }
+    };
+    if (lane < 27)
+      look(tile_nb(tx + lane % 3 - 1, ntx, g.bc[0]), tile_nb(ty + (lane / 3) % 3 - 1, nty, g.bc[1]),
+           tile_nb(tz + lane / 9 - 1, ntz, g.bc[2]));
+    const bool uni = __shfl_sync(kFullT, nb_uni ? 1 : 0, 13) != 0;  // lane 13: the tile itself
+    const long long cr = __shfl_sync(kFullT, nb_c, 13), er = __shfl_sync(kFullT, nb_e, 13);
+    bool same = lane >= 27 || !nb_ok || (nb_uni && nb_c == cr && nb_e == er);
     const int fx = tile_far(tx, ntx, g.n[0], g.bc[0]), fy = tile_far(ty, nty, g.n[1], g.bc[1]),
               fz = tile_far(tz, ntz, g.n[2], g.bc[2]);
-    const int kx = fx >= 0 ? 4 : 3, ky = fy >= 0 ? 4 : 3, kz = fz >= 0 ? 4 : 3;
-    bool same = true;
-    for (int o = lane; o < kx * ky * kz; o += 32) {
-      const int ox = o % kx, oy = (o / kx) % ky, oz = o / (kx * ky);
-      const int px = ox == 3 ? fx : tile_nb(tx + ox - 1, ntx, g.bc[0]), py = oy == 3 ? fy : tile_nb(ty + oy - 1, nty, g.bc[1]),
-                pz = oz == 3 ? fz : tile_nb(tz + oz - 1, ntz, g.bc[2]);
-      if ((px | py | pz) < 0) continue;
-      const size_t u = ((size_t)pz * nty + py) * ntx + px;
-      same = same && ts.uni[u] != 0 && dbits(ts.vc[u]) == cr && dbits(ts.ve[u]) == er;
+    if (fx >= 0 || fy >= 0 || fz >= 0) {  // a far neighbour is a fourth choice along its axis
+      const int kx = fx >= 0 ? 4 : 3, ky = fy >= 0 ? 4 : 3, kz = fz >= 0 ? 4 : 3;
+      for (int o = lane; o < kx * ky * kz; o += 32) {
+        const int ox = o % kx, oy = (o / kx) % ky, oz = o / (kx * ky);
+        look(ox == 3 ? fx : tile_nb(tx + ox - 1, ntx, g.bc[0]), oy == 3 ? fy : tile_nb(ty + oy - 1, nty, g.bc[1]),
+             oz == 3 ? fz : tile_nb(tz + oz - 1, ntz, g.bc[2]));
+        same = same && (!nb_ok || (nb_uni && nb_c == cr && nb_e == er));
+      }
     }
     const bool all = __all_sync(kFullT, same);
+    const bool pure = cr == 0 || cr == 0x3FF0000000000000LL;
     const bool q = uni && pure && all;
     const int x0 = tx * kTile, y0 = ty * kTile, z0 = tz * kTile;
     if (lane == 0) ts.quiet[t] = q ? 1 : 0;
