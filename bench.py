@@ -134,12 +134,14 @@ def measured_peak_gbs():
         return 6800.0, "fallback"
 
 
-# FP64 flops of one face of kernel F (pure donor; fused multiply-adds count
-# two): a = u lambda (1), F = c a (1), WENO5 face value (3 candidate
-# polynomials 15, 3 smoothness indicators 33, weights and their normalised
-# combination 21, the folded 1/6: 1), G = T_f C_pl F + T_f C_pg (a - F) (6)
-FACE_FLOP = 78
-FACE_SOURCES = ("paper_2001_03477_gb300/csrc/vof_sweep.cu", "paper_2001_03477_gb300/csrc/vof_device.cuh")
+# FP64 work of k_walk per face and cell (pure, fused multiply-adds count two
+# flop): T = e / C_p 1, the difference of T 1, a = u lambda 1, T_f = v0 +
+# correction / 6 2, G = (T_f C_p) a 2, Theta = C_p T 1, e' = (e + (G_l - Theta
+# a_l)) - (G_r - Theta a_r) 6: 14 flop in 13 instructions.  The WENO5
+# correction itself (64 of the method's 78 flop) runs in pairs of FP32 numbers.
+FACE_FLOP, FACE_INSTR = 14, 13
+FACE_SOURCES = ("paper_2001_03477_gb300/csrc/vof_fused.cu", "paper_2001_03477_gb300/csrc/vof_sweep.cuh",
+                "paper_2001_03477_gb300/csrc/vof_df.cuh", "paper_2001_03477_gb300/csrc/vof_device.cuh")
 
 
 def sources_sha1(paths):
@@ -152,9 +154,9 @@ def sources_sha1(paths):
 
 
 def faces_traffic_from_profile():
-    """DRAM bytes per launch of kernel F (k_faces) from the committed ncu
-    summary, if it was taken on the current sources of that kernel; None
-    otherwise."""
+    """DRAM bytes per launch of the step's face kernel (k_walk) from the
+    committed ncu summary, if it was taken on the current sources of that
+    kernel; None otherwise."""
     path = os.path.join(ROOT, "profiles", "k_faces_traffic.json.txt")
     try:
         with open(path) as f:
@@ -252,9 +254,10 @@ def run_gpu(args):
     kernels_per_step = sum(1 for name, _ in launches if "memset" not in name) // reps
     peak, peak_kind = measured_peak_gbs()
     counts = P.vof_step_work_counts(g, st.workspace, stream)
-    # the dominant kernel: k_faces (its three launches take the largest share
-    # of the step); FP64-ALU bound: it evaluates every listed face once
-    faces_ms = sum(kern_ms.get(f"sweep_{a}.faces", 0.0) for a in "xyz")
+    # the dominant kernel: k_walk (its three launches take the largest share
+    # of the step); bound by the instructions of the faces it evaluates, FP64
+    # and others
+    faces_ms = sum(kern_ms.get(f"sweep_{a}.walk", 0.0) for a in "xyz")
     faces_per_step = sum(counts["faces"])
     step_ms_prof = sum(kern_ms.values())
     fp64_achieved = FACE_FLOP * faces_per_step / (faces_ms * 1e-3) / 1e12 if faces_ms > 0 else 0.0
@@ -346,7 +349,7 @@ def run_gpu(args):
                            (wl.c.nbytes + wl.e.nbytes + h2d) / 1e9),
                        "algorithmic_bytes_per_cell_step": STEP_BYTES_PER_CELL,
                        "hbm_roofline_frac_step": round(value / world * STEP_BYTES_PER_CELL / peak, 4)},
-            "roofline": {"bound": "alu", "kernel": "k_faces (sweep x, y, z)", "achieved": round(fp64_achieved, 4),
+            "roofline": {"bound": "alu", "kernel": "k_walk (sweep x, y, z)", "achieved": round(fp64_achieved, 4),
                          "peak": round(fp64_peak, 4),
                          "unit": "TFLOP/s",
                          "frac": round(fp64_achieved / fp64_peak, 4),
@@ -357,6 +360,7 @@ def run_gpu(args):
                          "fp64_probe": fp64,
                          "peak_derived_tflops": round(fp64_peak_tflops(clocks["sm_max_mhz"] if clocks else None), 4),
                          "flop_per_face": FACE_FLOP, "faces_per_launch": round(faces_per_step / 3),
+                         "fp64_issue_frac": round(fp64_achieved / fp64_peak * 2 * FACE_INSTR / FACE_FLOP, 4),
                          "ms_per_launch": round(faces_ms / 3, 5),
                          "share_of_step": round(faces_ms / step_ms_prof, 4) if step_ms_prof > 0 else None,
                          "hbm_frac_step": round(value / world * STEP_BYTES_PER_CELL / peak, 4), "hbm_peak_gbs": peak,
@@ -523,7 +527,7 @@ def fp64_rate(P, dev, stream, iters=20000, blocks=152 * 8):
 def dense_roofline(P, st, g, c, e, u, v, w, dt, stream, fp64_peak, hbm_peak, value, reps=3):
     """The FP64 step's kernels on a workload where T varies everywhere (no
     quiet tiles): per-launch times of `reps` steps (CUDA events recorded by
-    the library after each launch), faces evaluated, and k_faces' FP64 rate
+    the library after each launch), faces evaluated, and k_walk's FP64 rate
     against the measured peak; the step against the HBM ledger."""
     import torch
     torch.cuda.synchronize()
@@ -535,11 +539,12 @@ def dense_roofline(P, st, g, c, e, u, v, w, dt, stream, fp64_peak, hbm_peak, val
     for name, t in launches:
         kms[name] = kms.get(name, 0.0) + t / reps
     counts = P.vof_step_work_counts(g, st.workspace, stream)
-    faces_ms = sum(kms.get(f"sweep_{a}.faces", 0.0) for a in "xyz")
+    faces_ms = sum(kms.get(f"sweep_{a}.walk", 0.0) for a in "xyz")
     faces = sum(counts["faces"])
     ach = FACE_FLOP * faces / (faces_ms * 1e-3) / 1e12 if faces_ms > 0 else 0.0
-    return {"kernel": "k_faces (sweep x, y, z)", "bound": "alu", "unit": "TFLOP/s", "achieved": round(ach, 4),
+    return {"kernel": "k_walk (sweep x, y, z)", "bound": "alu", "unit": "TFLOP/s", "achieved": round(ach, 4),
             "peak": round(fp64_peak, 4), "frac": round(ach / fp64_peak, 4), "flop_per_face": FACE_FLOP,
+            "fp64_issue_frac": round(ach / fp64_peak * 2 * FACE_INSTR / FACE_FLOP, 4),
             "faces_per_launch": round(faces / 3), "ms_per_launch": round(faces_ms / 3, 5),
             "share_of_step": round(faces_ms / sum(kms.values()), 4),
             "hbm_frac_step": round(value * STEP_BYTES_PER_CELL / hbm_peak, 4), "work_counts": counts,
@@ -816,7 +821,7 @@ def batched_form(dev, nbox=4096, nsub=4, steps=5):
     cell, generated on all host cores).  The grouped form (vof_group_*: one
     launch per kernel of the step over all boxes, the CTA granularity picked
     by the autotuner on a sample) timed directly and as a CUDA-graph replay;
-    beside it vof_batched_step over lane streams (~21 launches per box).
+    beside it vof_batched_step over lane streams (12 launches per box).
     CUDA events on the launching stream."""
     import multiprocessing as mp
     import torch
@@ -921,7 +926,7 @@ def batched_form(dev, nbox=4096, nsub=4, steps=5):
                       "value": round(cells / (direct_ms * 1e-3) / 1e9, 4), "ms_per_step": round(direct_ms, 3),
                       "value_graph_replay": round(cells / (graph_ms * 1e-3) / 1e9, 4),
                       "graph_capture_and_instantiate_s": round(inst_s, 2),
-                      "launches_per_step": "about 21 per box (one vof_step each)",
+                      "launches_per_step": "12 per box (one vof_step each)",
                       "finite": bool(np.isfinite(sums).all())},
             "input_generation_s": round(gen_s, 1)}
 

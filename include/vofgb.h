@@ -305,7 +305,7 @@ VOF_API vof_status vof_batched_step(const vof_box* boxes, int nbox, long step_in
  * the caller's buffer and writes, once, every kernel's per-box arguments
  * and the CTA -> box maps of the grouped launches into the same buffer
  * (synchronising `stream`); vof_group_step() then runs a time step of every
- * box with ~22 launches on `stream` whatever the number of boxes: each CTA
+ * box with 13 launches on `stream` whatever the number of boxes: each CTA
  * finds its box and its block within that box's own launch shape, so every
  * box computes exactly what vof_step() computes on it (the same kernels, sum
  * rows and reductions: bit-identical results).  No host work per box; the
@@ -315,7 +315,7 @@ VOF_API vof_status vof_batched_step(const vof_box* boxes, int nbox, long step_in
  *                 grouped: VOF_EINVAL)
  *   sums          device double[nbox][VOF_NSUMS] or NULL: each box's step
  *                 sums, written by every vof_group_step()
- *   work_per_cta  cells per CTA of the grid-stride kernels (planes, faces,
+ *   work_per_cta  cells per CTA of the grid-stride kernels (mixed cells,
  *                 shift lists; >= 32): the grouped launches' granularity
  *                 (results do not depend on it; the autotuner picks it)
  *   workspace     device, 256-byte aligned, vof_group_workspace_bytes()
