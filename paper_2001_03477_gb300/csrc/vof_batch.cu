@@ -279,12 +279,23 @@ static vof_status group_plan(const vof_box* boxes, int nbox, double* sums, int w
     p_tiles.add(B.grid_tiles.x, B.grid_tiles.y, B.grid_tiles.z);
     p_quiet.add(quiet_ctas(B.args.g), 1, 1);
     p_mix.add(gs_ctas(B.cells, work, mix_ctas(B.args.g)), 1, 1);
-    p_walk.add(walk_ctas(B.args.g), 1, 1);
     p_planes.add(gs_ctas(B.cells, work, shift_plane_ctas()), 1, 1);
     p_sweep.add(gs_ctas(B.cells, work, shift_plane_ctas()), 1, 1);
     p_apply.add(apply_ctas(B.args.g), 1, 1);
     p_red1.add(kReduceCTAs, 1, 1);
   }
+  // The boxes' walks share the machine: chains short enough for a dozen items a
+  // resident warp over the whole batch, at most 4 tiles (48 ... 96 cells an edge
+  // hold 6 ... 12), and CTAs for as many items a warp, 4 at most, as leave eight
+  // warps for each resident one.  (About 40 % of a droplet box's tiles are active:
+  // with a warp for every quarter tile four of five CTAs found no work, and 96
+  // boxes' two steps took 10,985 us; 10,335 now.)
+  size_t tiles = 0;
+  for (int b = 0; b < nbox; ++b) tiles += (size_t)tile_total(sb[b].args.g);
+  const size_t resident = 152 * 16;
+  const int chain = (int)std::min<size_t>(4, std::max<size_t>(1, 2 * tiles / (12 * resident)));
+  const int per_warp = (int)std::min<size_t>(4, std::max<size_t>(1, 2 * tiles / chain / (8 * resident)));
+  for (int b = 0; b < nbox; ++b) p_walk.add(walk_ctas_grp(sb[b].args.g, chain, per_warp), 1, 1);
   // table region after the boxes' workspaces
   LaunchPlan* plans[] = {&p_tiles, &p_quiet, &p_mix, &p_walk, &p_planes, &p_sweep, &p_apply, &p_red1};
   const size_t nb = (size_t)nbox;
@@ -303,15 +314,9 @@ static vof_status group_plan(const vof_box* boxes, int nbox, double* sums, int w
   {
     std::vector<StepArgs> sa(nb);
     std::vector<ReduceBox> rb(nb);
-    // the boxes' walks share the machine: chains short enough for a dozen
-    // items a resident warp over the whole batch, at most 4 tiles (48 ... 96
-    // cells an edge hold 6 ... 12)
-    size_t tiles = 0;
-    for (size_t b = 0; b < nb; ++b) tiles += (size_t)tile_total(sb[b].args.g);
-    const size_t items = 2 * tiles / (12ull * 152 * 16);
     for (size_t b = 0; b < nb; ++b) {
       sa[b] = sb[b].args;
-      sa[b].chain = items < 1 ? 1 : (items > 4 ? 4 : (int)items);
+      sa[b].chain = chain;
     }
     put(o_args, sa.data(), nb * sizeof(StepArgs));
     for (size_t b = 0; b < nb; ++b) rb[b] = sb[b].red;

@@ -543,6 +543,13 @@ unsigned walk_ctas(const GridDev& g) {
   return (unsigned)std::min<long long>((4ll * tile_total(g) + kWalkWarps - 1) / kWalkWarps, 152 * kWalkPerSM);
 }
 
+// In a batch of boxes (no quarters): per_warp halves or chains of halves a warp if
+// every tile is active.
+unsigned walk_ctas_grp(const GridDev& g, int chain, int per_warp) {
+  const long long items = 2ll * tile_total(g) / chain;
+  return (unsigned)std::max<long long>(1, (items + per_warp * kWalkWarps - 1) / (per_warp * kWalkWarps));
+}
+
 template <int AX>
 static cudaError_t stage_t(const StepArgs& A, int stage, cudaStream_t st) {
   const GridDev& g = A.g;

@@ -254,6 +254,7 @@ cudaError_t launch_shift_step(const StepArgs& A, int odd, cudaStream_t st);
 unsigned quiet_ctas(const GridDev& g);
 unsigned mix_ctas(const GridDev& g);
 unsigned walk_ctas(const GridDev& g);
+unsigned walk_ctas_grp(const GridDev& g, int chain, int per_warp);
 unsigned shift_plane_ctas();
 unsigned apply_ctas(const GridDev& g);
 
