@@ -164,8 +164,12 @@ k_shift_stream(GridDev g, const double* __restrict__ c_in, const double* __restr
 // reaches.  LANES = 3: the three lanes leader .. leader + 2 (mask gmask) of
 // one cell share its bisection (edge cells); every lane computes the same
 // values, and the stores and the claims' atomic ORs repeat them harmlessly.
-template <int LANES>
-__device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double* __restrict__ c_in,
+// STEP: a time step's shift, whose c words (c_in = sc.mark) carry tag bits and
+// are tagged further by other threads of this launch: their loads are ordinary
+// ones (a read-only load promises nothing for memory that the kernel writes);
+// either state of the two tag bits is dropped.
+template <int LANES, bool STEP>
+__device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double* c_in,
                                                  const double* __restrict__ dd, double dd_uniform,
                                                  const ShiftScratch& sc, size_t id, unsigned gmask, int leader,
                                                  int sub) {
@@ -181,13 +185,10 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
 #pragma unroll
       for (int ox = 0; ox < 3; ++ox) {
         const int xx = map_idx(x + ox - 1, g.n[0], g.bc[0]);
-        st[(oz * 3 + oy) * 3 + ox] = __ldg(c_in + cell_id(g, xx, yy, zz));
+        const double* p = c_in + cell_id(g, xx, yy, zz);
+        st[(oz * 3 + oy) * 3 + ox] = STEP ? c_value(*p) : __ldg(p);
       }
     }
-  }
-  if (sc.mark) {  // a time step's c words carry tag bits
-#pragma unroll
-    for (int i = 0; i < 27; ++i) st[i] = c_value(st[i]);
   }
   const double ct = st[13];
   double m[3];
@@ -222,7 +223,7 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
   // which FP32 decides with a margin far above its rounding; the exact test and
   // the volumes are k_shift_sweep's.
   float fm[3] = {0.f, 0.f, 0.f}, fa = 0.f, flo = 0.f, fhi = 0.f, mg = 0.f;
-  if (sc.mark) {
+  if (STEP) {
     fm[0] = f32_of(m[0]); fm[1] = f32_of(m[1]); fm[2] = f32_of(m[2]);
     const float al_f = f32_of(al), sft_f = f32_of(sft);
     fa = al_f + sft_f;
@@ -241,7 +242,7 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
     const int ox = b % 3 - 1, oy = (b / 3) % 3 - 1, oz = b / 9 - 1;
     size_t pid;
     if (!neighbour(g, x, y, z, ox, oy, oz, pid)) continue;
-    if (!sc.mark) {
+    if (!STEP) {
       atomicOr(sc.claim + pid, 0x80000000u >> offset_bit(-ox, -oy, -oz));
       continue;
     }
@@ -262,20 +263,21 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
 // per warp, three lanes each, the warps' chunks taken from the grid's last
 // warp down -- warps the front leaves idle, on SMs of their own -- so the
 // bisections' long FP64 chains run side by side.
-__device__ __forceinline__ void k_shift_planes_body(const GridDev& g, const double* __restrict__ c_in, const double* __restrict__ dd, double dd_uniform, const ShiftScratch& sc, const VB vb) {
+template <bool STEP>
+__device__ __forceinline__ void k_shift_planes_body(const GridDev& g, const double* c_in, const double* __restrict__ dd, double dd_uniform, const ShiftScratch& sc, const VB vb) {
   const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
   const int nn = sc.counters[0], ne = sc.counters[1];
   const int lane = threadIdx.x & 31;
   const int stride = vb.gx * blockDim.x;
   for (int i = vb.bx * blockDim.x + threadIdx.x; i < nn; i += stride)
-    shift_plane_cell<1>(g, c_in, dd, dd_uniform, sc, sc.gmix[i], 0u, 0, 0);
+    shift_plane_cell<1, STEP>(g, c_in, dd, dd_uniform, sc, sc.gmix[i], 0u, 0, 0);
   const int nw = (int)(vb.gx * (blockDim.x >> 5)), gw = (int)((vb.bx * blockDim.x + threadIdx.x) >> 5);
   const int nchunk = (ne + 9) / 10;
   for (int wc = nw - 1 - gw; wc < nchunk; wc += nw) {
     const int j = wc * 10 + lane / 3;
     if (lane >= 30 || j >= ne) continue;
     const int leader = (lane / 3) * 3;
-    shift_plane_cell<3>(g, c_in, dd, dd_uniform, sc, sc.gmix[N - 1 - (size_t)j], 7u << leader, leader,
+    shift_plane_cell<3, STEP>(g, c_in, dd, dd_uniform, sc, sc.gmix[N - 1 - (size_t)j], 7u << leader, leader,
                         lane - leader);
   }
 }
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(kListThreads)
 k_shift_planes(GridDev g, const double* __restrict__ c_in, const double* __restrict__ dd, double dd_uniform,
                ShiftScratch sc) {
   pdl_wait();
-  k_shift_planes_body(g, c_in, dd, dd_uniform, sc, vb_self());
+  k_shift_planes_body<false>(g, c_in, dd, dd_uniform, sc, vb_self());
 }
 
 // Per moving mixed cell (same list, after all claims are in): the receivers
@@ -625,7 +627,7 @@ __device__ __forceinline__ ShiftScratch step_shift_scratch(const StepArgs& A) {
 
 __global__ void __launch_bounds__(kListThreads) k_shift_mark(StepArgs A) {
   pdl_wait();
-  k_shift_planes_body(A.g, A.s_c, A.dd, A.dd_uniform, step_shift_scratch(A), vb_self());
+  k_shift_planes_body<true>(A.g, A.s_c, A.dd, A.dd_uniform, step_shift_scratch(A), vb_self());
 }
 
 // the change by one neighbour's plane (m, al, shift sft) extended into the
@@ -827,7 +829,7 @@ __global__ void __launch_bounds__(kListThreads) k_shift_mark_grp(GroupMap m, con
   const VB vb = vb_group(m, b);
   __shared__ StepArgs sA;
   const StepArgs& A = cta_args(args, b, sA);
-  k_shift_planes_body(A.g, A.s_c, A.dd, A.dd_uniform, step_shift_scratch(A), vb);
+  k_shift_planes_body<true>(A.g, A.s_c, A.dd, A.dd_uniform, step_shift_scratch(A), vb);
 }
 __global__ void __launch_bounds__(kListThreads) k_shift_sweep_grp(GroupMap m, const StepArgs* __restrict__ args) {
   unsigned b;
