@@ -80,9 +80,12 @@ __device__ __forceinline__ void k_tiles_body(const GridDev& g, const double* __r
   }
 }
 
+// (c and e are read at addresses known from the start, and the grid ahead on the
+// stream may be what writes them: the step before without sums, a program's own
+// kernel)
 __global__ void __launch_bounds__(256) k_tiles(StepArgs A) {
   pdl_wait();
-  k_tiles_body(A.g, A.c, A.e, A.ts, A.nt[0], A.nt[1], A.cnt, A.stats, vb_self());
+  k_tiles_body(A.g, after_wait(A.c), after_wait(A.e), A.ts, A.nt[0], A.nt[1], A.cnt, A.stats, vb_self());
 }
 
 // neighbour tile index along one axis: -1 when it lies beyond a

@@ -42,3 +42,23 @@ def test_words_tagged_by_the_same_kernel_are_read_by_ordinary_loads():
     assert re.search(r"__ldg\(dd \+ id\)", body)
     for kernel, form in (("k_shift_mark", "true"), ("k_shift_mark_grp", "true"), ("k_shift_planes", "false")):
         assert f"k_shift_planes_body<{form}>(" in function(text, kernel)[1], kernel
+
+
+def test_step_reads_the_fields_behind_its_wait():
+    """The step's first kernel streams c and e, which the grid ahead may write,
+    at addresses that depend on nothing loaded; the step's other kernels load
+    their lists' lengths first."""
+    text = source("vof_tiles.cu")
+    body = function(text, "k_tiles")[1]
+    assert re.search(r"pdl_wait\(\);\s*k_tiles_body\(A\.g, after_wait\(A\.c\), after_wait\(A\.e\),", body)
+
+
+def test_the_step_kernels_wait_first():
+    """By name: every kernel of a time step starts with the wait."""
+    for name, kernels in (("vof_tiles.cu", ("k_tiles", "k_quiet")), ("vof_fused.cu", ("k_mix", "k_walk")),
+                          ("vof_shift.cu", ("k_shift_mark", "k_shift_sweep", "k_shift_apply", "k_reduce_fused"))):
+        text = source(name)
+        for k in kernels:
+            body = re.sub(r"__shared__[^;]*;", "", function(text, k)[1])
+            assert body.split(";")[0].strip() == "pdl_wait()", k
+            assert re.search(r"launch_pdl\(" + k + r"\b", text), k
