@@ -292,7 +292,7 @@ bool step_box(const vof_grid* g, double* c, double* e, const double* u, const do
   A.dd = dd;
   A.dd_uniform = dd_uniform;
   A.pairs = reinterpret_cast<uint2*>(A.theta);
-  A.pair_cap = (int)B.cells;
+  A.pair_cap = (unsigned)B.cells;
   A.chain = 0;
   B.grid_tiles = dim3((unsigned)((A.nt[0] + 3) / 4), (unsigned)A.nt[1], (unsigned)A.nt[2]);
   B.red = ReduceBox{A.rows, L.ntiles, sums, reinterpret_cast<double*>(ws + L.off_red)};

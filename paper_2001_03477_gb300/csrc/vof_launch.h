@@ -184,8 +184,8 @@ struct ShiftScratch {
   double* mark;   // nullable: the tagged c words (c_in), where receivers are marked instead of
                   // claimed; then also the pairs whose plane may enter the receiver
   uint2* pairs;
-  int pair_cap;
-  int* npairs;
+  unsigned pair_cap;
+  unsigned* npairs;
 };
 
 // The shift's kernels: stream (lists; out of place also copies; sums c, e
@@ -239,7 +239,7 @@ struct StepArgs {
   const double* dd;
   double dd_uniform;
   uint2* pairs;          // [N] the shift's (source, neighbour) pairs (Theta's storage)
-  int pair_cap;
+  unsigned pair_cap;
   int chain;             // 0: one grid; else the walks' chain length in a batch of boxes
 };
 

@@ -172,7 +172,7 @@ template <int LANES, bool STEP>
 __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double* c_in,
                                                  const double* __restrict__ dd, double dd_uniform,
                                                  const ShiftScratch& sc, size_t id, unsigned gmask, int leader,
-                                                 int sub) {
+                                                 int sub, bool& room) {
   int x, y, z;
   decode(g, id, x, y, z);
   double st[27];
@@ -251,9 +251,12 @@ __device__ __forceinline__ void shift_plane_cell(const GridDev& g, const double*
     sc.cnew[pid] = 0.0;  // no change so far
     const float an = fa - (fm[0] * (float)ox + fm[1] * (float)oy + fm[2] * (float)oz);
     const bool outside = full ? an >= fhi + mg : an <= flo - mg;
-    if (!outside && sub == 0 && dnz(sft)) {
-      const int k = atomicAdd(sc.npairs, 1);
-      if (k < sc.pair_cap) sc.pairs[k] = make_uint2((uint32_t)id, (unsigned)offset_bit(ox, oy, oz));
+    // (a thread that has met a full list adds no more: the count stays within
+    // the cap and one a thread, below 2^32 for the cap's 2^31 - 1 at most)
+    if (!outside && sub == 0 && room && dnz(sft)) {
+      const unsigned k = atomicAdd(sc.npairs, 1u);
+      room = k < sc.pair_cap;
+      if (room) sc.pairs[k] = make_uint2((uint32_t)id, (unsigned)offset_bit(ox, oy, oz));
     }
   }
 }
@@ -268,9 +271,10 @@ __device__ __forceinline__ void k_shift_planes_body(const GridDev& g, const doub
   const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
   const int nn = sc.counters[0], ne = sc.counters[1];
   const int lane = threadIdx.x & 31;
+  bool room = true;  // in the list of pairs, as far as this thread knows
   const int stride = vb.gx * blockDim.x;
   for (int i = vb.bx * blockDim.x + threadIdx.x; i < nn; i += stride)
-    shift_plane_cell<1, STEP>(g, c_in, dd, dd_uniform, sc, sc.gmix[i], 0u, 0, 0);
+    shift_plane_cell<1, STEP>(g, c_in, dd, dd_uniform, sc, sc.gmix[i], 0u, 0, 0, room);
   const int nw = (int)(vb.gx * (blockDim.x >> 5)), gw = (int)((vb.bx * blockDim.x + threadIdx.x) >> 5);
   const int nchunk = (ne + 9) / 10;
   for (int wc = nw - 1 - gw; wc < nchunk; wc += nw) {
@@ -278,7 +282,7 @@ __device__ __forceinline__ void k_shift_planes_body(const GridDev& g, const doub
     if (lane >= 30 || j >= ne) continue;
     const int leader = (lane / 3) * 3;
     shift_plane_cell<3, STEP>(g, c_in, dd, dd_uniform, sc, sc.gmix[N - 1 - (size_t)j], 7u << leader, leader,
-                        lane - leader);
+                        lane - leader, room);
   }
 }
 
@@ -621,7 +625,7 @@ __device__ __forceinline__ ShiftScratch step_shift_scratch(const StepArgs& A) {
   s.mark = A.s_c;
   s.pairs = A.pairs;
   s.pair_cap = A.pair_cap;
-  s.npairs = A.cnt + 2;
+  s.npairs = reinterpret_cast<unsigned*>(A.cnt + 2);
   return s;
 }
 
@@ -657,9 +661,10 @@ __device__ __forceinline__ double swept_change(const double4& pl, double sft, bo
 __device__ __forceinline__ void sweep_pairs_body(const StepArgs& A, const VB vb) {
   const GridDev& g = A.g;
   const size_t N = (size_t)g.n[0] * g.n[1] * g.n[2];
-  const int np = A.cnt[2], nn = A.cnt[12], ne = A.cnt[13];
+  const unsigned np = (unsigned)A.cnt[2];
+  const int nn = A.cnt[12], ne = A.cnt[13];
   const bool listed = np <= A.pair_cap;
-  const long long total = listed ? np : 27ll * (nn + ne);
+  const long long total = listed ? (long long)np : 27ll * (nn + ne);
   for (long long i = (long long)vb.bx * blockDim.x + threadIdx.x; i < total; i += (long long)vb.gx * blockDim.x) {
     size_t id;
     int b;
