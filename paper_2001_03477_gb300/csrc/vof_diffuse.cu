@@ -38,13 +38,21 @@
 //   d' = B sum d_nb + s,  B = k_p / h^2 / diagonal,  s = B sum (T0_nb - T0),
 // (the same iterates T, since C_p / dt and the couplings add up to the
 // diagonal), s formed once in FP64 (k_dif_first: it is also the first sweep),
-// d, B and s held as pairs of FP32 numbers (48 bits of the change itself, whose
-// rounding stays below an ulp of T), over the power of two next to the largest
-// T.  What bounds a sweep on this part is the
+// d, B and s held as pairs of FP32 numbers (48 bits of the change itself), over
+// the power of two next to the largest T.  What bounds a sweep on this part is the
 // FP64 unit: 8 FP64 instructions per cell took 45 us at 128^3 (76 cycles of an
 // SM partition each); the pairs' FP32 instructions take 20.6 us (two cells of a row in one 16-byte
-// block; 22 us with high and low parts in arrays of their own).  The sweeps
-// are queued in batches without waiting: each starts by reading the last
+// block; 22 us with high and low parts in arrays of their own).
+// A pair of the change is as accurate as an FP64 T only while the change is small
+// beside T.  Every iterate lies between the smallest and the largest of the T0,
+// of T_Gamma where a cell sees an interface and of the walls' T, so |d| is at most
+// their range R, and the rule is 16 R <= the smallest of them (all positive): the
+// energies' errors against long double are then 0.2 to 0.4 of the FP64 sweeps'
+// (16^3 box, diffusion numbers 0.05 to 20; R = T / 8: up to 0.65 in the mean and as
+// large at most; R = T: 1.4 to 24 times).  Other calls sweep T itself in FP64.  The
+// kernels decide on the device: the first batch's sweeps in pairs return at once
+// where the rule says FP64, and the host reads it with that batch's checks.
+// The sweeps are queued in batches without waiting: each starts by reading the last
 // check's result and leaves its buffers alone once that was within tol.
 // Mixture heat capacity: the FP64 form, every cell's diagonal stored.
 #include <algorithm>
@@ -199,7 +207,7 @@ struct DifConst {
   double rdiag[2][7];
   double B[2][7];    // kq * rdiag
   float2 Bf[2][7];   // the same as pairs of FP32 numbers
-  int e0;            // largest exponent field of T_sat and the walls' T
+  int wlo, whi;      // smallest and largest high word of the heated walls' T
 };
 
 // Cell classes: bits 0..5 the sides (-x, +x, -y, +y, -z, +z) with a
@@ -212,23 +220,38 @@ constexpr uint8_t kDifLiq = 0x40, kDifIrr = 0x80;
 
 struct DifVec {
   double* off;    // [6 N]: coupling to the neighbour (face order -x, +x, -y, +y, -z, +z), kDifIrr cells
-                  // only; with the phase heat capacity over the diagonal, as a pair of FP32 numbers
-  double* diag;   // [N] reciprocal of the diagonal (mixture heat capacity)
-  double* rhs;    // [N] right side (mixture)
-  double* T0;     // [N] T at the start (the first iterate of the mixture form)
+                  // only; in pairs over the diagonal, as a pair of FP32 numbers
+  double* diag;   // [N] reciprocal of the diagonal; kDifIrr cells (all cells with the mixture heat capacity)
+  double* rhs;    // [N] right side; likewise
+  double* T0;     // [N] T at the start (the first iterate in FP64)
   double* Ta;     // [N] the two later Jacobi iterates
   double* Tb;
-  unsigned long long* part;  // [kDifChecks] the largest change of each checked sweep of a batch (bits)
+  unsigned long long* part;  // [kDifChecks] the largest change of each checked sweep of a batch (bits),
+                             // [kDifChecks]: infinity where the sweeps run in pairs, else 0
   uint8_t* cls;   // [N] cell class
-  // phase form: two cells of a row (x even, x + 1) in 16 bytes, {hi, hi, lo, lo},
+  // in pairs: two cells of a row (x even, x + 1) in 16 bytes, {hi, hi, lo, lo},
   // a row of px such blocks
   float4* s;      // [px ny nz]: s, also the first iterate d
   float4* d[2];   // the two later iterates
   int px;
-  int* tmax;      // largest exponent field of a finite T0
+  int* range;     // [0] the largest high word of a T, [1] 0x7FFFFFFF minus the smallest (unsigned maximum)
 };
+// high words (as signed integers: positive values in order, any negative one
+// below them) of the smallest and the largest T of the system
+__device__ __forceinline__ int dif_lo(const DifVec& v, const DifConst& K) { 
+  return min((int)(0x7FFFFFFFu - (unsigned)v.range[1]), K.wlo);
+}
+__device__ __forceinline__ int dif_hi(const DifVec& v, const DifConst& K) { return max(v.range[0], K.whi); }
+// the rule for pairs (an infinite or NaN T fails it: hi is its high word, or lo
+// is negative)
+__device__ __forceinline__ bool dif_pairs(const DifVec& v, const DifConst& K) {
+  const int lo = dif_lo(v, K), hi = dif_hi(v, K);
+  if (lo < 0x00100000 || hi >= 0x7FE00000) return false;
+  const double a = __hiloint2double(lo, 0), b = __hiloint2double(hi + 1, 0);  // around all of them
+  return 16.0 * (b - a) <= a;
+}
 // the pairs hold d / 2^k
-__device__ __forceinline__ int dif_scale(const DifVec& v, const DifConst& K) { return max(*v.tmax, K.e0) - 1023; }
+__device__ __forceinline__ int dif_scale(const DifVec& v, const DifConst& K) { return (dif_hi(v, K) >> 20) - 1023; }
 // the high part of cell (x, y, z) in array a; the low part is two floats on
 __device__ __forceinline__ float* part_of(const GridDev& g, const DifVec& v, float4* a, int x, int y, int z) {
   return reinterpret_cast<float*>(a + ((size_t)z * g.n[1] + y) * v.px + (x >> 1)) + (x & 1);
@@ -280,7 +303,12 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
   if (y >= g.n[1]) return;  // whole warps (a warp is one row segment)
   const bool in_x = x < g.n[0];
   const int lane = threadIdx.x;
-  int tmax = 0;
+  int thi = 0;
+  unsigned tlo = 0u;
+  auto in_range = [&](double T) {
+    thi = max(thi, __double2hiint(T));
+    tlo = max(tlo, 0x7FFFFFFFu - (unsigned)__double2hiint(T));
+  };
   for (int z = blockIdx.z; z < g.n[2]; z += gridDim.z) {
     const size_t i = ((size_t)z * g.n[1] + y) * g.n[0] + x;
     bool irr = false;
@@ -293,8 +321,8 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
       dif_sides(g, c, walls, x, y, z, liq, inm, same, hot_wall);
       const int li = liq ? 1 : 0;
       v.T0[i] = T0;
-      const int ex = (int)((dbits(T0) >> 52) & 0x7FF);
-      if (ex != 0x7FF) tmax = max(tmax, ex);
+      in_range(T0);
+      if (same != inm) in_range(g.T_sat);
       irr = hot_wall || same != inm;
       v.cls[i] = (uint8_t)(inm | (liq ? kDifLiq : 0) | (irr ? kDifIrr : 0));
       if (!irr && !PHASE) {
@@ -319,8 +347,12 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
     if (irr) ilist[base + __popc(mask & ((1u << lane) - 1u))] = (uint32_t)i;
   }
   if constexpr (PHASE) {
-    tmax = __reduce_max_sync(0xffffffffu, tmax);
-    if (lane == 0 && tmax > *(volatile int*)v.tmax) atomicMax(v.tmax, tmax);  // (few warps find it larger)
+    thi = __reduce_max_sync(0xffffffffu, thi);
+    tlo = __reduce_max_sync(0xffffffffu, tlo);
+    volatile int* r = v.range;
+    unsigned* ru = reinterpret_cast<unsigned*>(v.range);
+    if (lane == 0 && thi > r[0]) atomicMax(v.range, thi);  // (few warps find it larger)
+    if (lane == 0 && tlo > (unsigned)r[1]) atomicMax(ru + 1, tlo);
   }
 }
 
@@ -340,6 +372,16 @@ __device__ __forceinline__ double wide_of(float f, int k) {
 }
 __device__ __forceinline__ df::f2 f2_of(float2 p) { return df::f2{p.x, p.y}; }
 
+// Checks of a batch of sweeps: at most kDifChecks; a sweep reads the slot of
+// the check before it (the first ones of a call, in pairs, whether the rule
+// lets them run).
+constexpr int kDifChecks = 31;
+
+// A check's result within tol (both non-negative: compared as integers).
+__device__ __forceinline__ bool dif_done(const unsigned long long* __restrict__ prev, double tol) {
+  return prev && *prev <= (unsigned long long)dbits(tol);
+}
+
 // Per listed cell (lanes dense over the list): the six couplings (heights
 // or plane distances on the interface sides), the diagonal and the right
 // side.
@@ -348,7 +390,10 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
                 const double* __restrict__ c, const double* __restrict__ e, const double4* __restrict__ plane,
                 DifVec v, DifWalls walls, int phase_cp, DifConst K, const uint32_t* __restrict__ ilist,
                 const int* __restrict__ icount) {
-  const int ni = *icount, ks = dif_scale(v, K);
+  const int ni = *icount;
+  const bool pairs = phase_cp && dif_pairs(v, K);
+  const int ks = dif_scale(v, K);
+  if (blockIdx.x == 0 && threadIdx.x == 0) v.part[kDifChecks] = pairs ? 0x7FF0000000000000ull : 0ull;
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < ni; k += gridDim.x * blockDim.x) {
     const size_t i = ilist[k];
     int x, y, z;
@@ -362,7 +407,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
     const int li = liq ? 1 : 0;
     const double cdt = phase_cp ? K.cdt[li] : (g.Cp_l * cv + g.Cp_g * (1.0 - cv)) * inv_dt;
     double diag = cdt, rhs = cdt * T0;
-    double off[6], gain = 0.0;  // gain: the heat conducted at T0 over its own unit (phase form)
+    double off[6], gain = 0.0;  // gain: the heat conducted at T0 over its own unit (pairs)
     auto nb_T = [&](int f) {     // T0 of the neighbour across side f
       int q[3] = {x, y, z};
       q[f >> 1] = step_coord(q[f >> 1], (f & 1) ? 1 : -1, g.n[f >> 1], g.bc[f >> 1]);
@@ -403,7 +448,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
           const double o = dnz(cq[side]) ? kq : 0.0;
           diag += o;
           off[2 * axis + side] = o;
-          if (phase_cp && dnz(o)) gain += o * (nb_T(2 * axis + side) - T0);
+          if (pairs && dnz(o)) gain += o * (nb_T(2 * axis + side) - T0);
         }
       } else {
         const double kd = kp / (0.5 * (d[0] + d[1]));
@@ -412,7 +457,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
           diag += kd * cs[side];
           off[2 * axis + side] = kd * cq[side];
           rhs += kd * cst[side];
-          if (phase_cp) {
+          if (pairs) {
             // towards a fixed temperature (T_Gamma, T_w) or the neighbour's
             if (dnz(cq[side])) gain += kd * cq[side] * (nb_T(2 * axis + side) - T0);
             else if (dnz(cs[side])) gain += kd * cs[side] * (Tfix[side] - T0);
@@ -421,7 +466,7 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
       }
     }
     const double rd = 1.0 / diag;  // stored as its reciprocal: the sweeps multiply
-    if (phase_cp) {
+    if (pairs) {
 #pragma unroll
       for (int f = 0; f < 6; ++f) reinterpret_cast<float2*>(v.off)[6 * i + f] = pair_of(off[f] * rd, 0);
       const float2 sp = pair_of(gain * rd, ks);
@@ -437,31 +482,23 @@ k_dif_irregular(GridDev g, double h, double inv_h, double inv_dt, double k_l, do
   }
 }
 
-// Checks of a batch of sweeps: at most kDifChecks; a sweep reads the slot of
-// the check before it.
-constexpr int kDifChecks = 32;
-
-// A check's result within tol (both non-negative: compared as integers).
-__device__ __forceinline__ bool dif_done(const unsigned long long* __restrict__ prev, double tol) {
-  return prev && *prev <= (unsigned long long)dbits(tol);
-}
-
-// The Jacobi update of one cell of the mixture form from its neighbours'
-// values t0..t5 (sides not in the grid skipped): (rhs + sum off T_nb) / diag,
-// the couplings k_p / h^2 unless the cell's are stored.  Not inlined, and called
-// only by warps with a cell that needs it, so that the other warps issue none
-// of its FP64 instructions.
+// The Jacobi update of one cell in FP64 from its neighbours' values t0..t5
+// (sides not in the grid skipped): (rhs + sum off T_nb) / diag, the right side
+// C_p / dt T0 and the couplings k_p / h^2 unless the cell's are stored.  Not
+// inlined, and called only by warps with a cell that needs it, so that the
+// other warps issue none of its FP64 instructions.
+template <bool PHASE>
 static __device__ __noinline__ double dif_row(unsigned cls, const double* __restrict__ off6,
                                               const double* __restrict__ rhs_i, const double* __restrict__ diag_i,
-                                              double kq, double t0, double t1, double t2, double t3, double t4,
-                                              double t5) {
-  const bool irr = (cls & kDifIrr) != 0;
-  double acc = __ldg(rhs_i);
+                                              double kq, double cdt, double rdt, double T0, double t0, double t1,
+                                              double t2, double t3, double t4, double t5) {
+  const bool irr = (cls & kDifIrr) != 0, stored = irr || !PHASE;
+  double acc = stored ? __ldg(rhs_i) : cdt * T0;
   const double tn[6] = {t0, t1, t2, t3, t4, t5};
 #pragma unroll
   for (int f = 0; f < 6; ++f)
     if (cls & (1u << f)) acc = fma(irr ? __ldg(off6 + f) : kq, tn[f], acc);
-  return acc * __ldg(diag_i);
+  return acc * (stored ? __ldg(diag_i) : rdt);
 }
 
 // Neighbour index of cell i at (x, y, z) across side f (its class bit set):
@@ -479,14 +516,14 @@ __device__ __forceinline__ size_t dif_nb(const GridDev& g, size_t i, int x, int 
   }
 }
 
-// One Jacobi sweep of the mixture form, Tout = (rhs + sum off T_nb(in)) / diag;
-// with CHECK the largest |Tout - Tin| into *change (non-negative doubles order
-// like their bits: an integer atomic max, the same whatever the order).  A cell
+// One Jacobi sweep in FP64, Tout = (rhs + sum off T_nb(in)) / diag; with CHECK
+// the largest |Tout - Tin| into *change (non-negative doubles order like their
+// bits: an integer atomic max, the same whatever the order).  A cell
 // coupled by k_p / h^2 whose own and neighbours' values all equal its T0 is
 // the sweep's fixed point, (C_p/dt T0 + n k_p/h^2 T0) / (C_p/dt + n k_p/h^2)
 // = T0, and keeps T0 without arithmetic.  CTAs of 32 x 8 threads over x and
 // y, each walking its share of the z planes (no index division).
-template <bool CHECK>
+template <bool CHECK, bool PHASE>
 __global__ void __launch_bounds__(kDifThreads)
 k_dif_jacobi(GridDev g, DifVec v, DifConst K, const double* __restrict__ Tin, double* __restrict__ Tout,
              const unsigned long long* __restrict__ prev, double tol, unsigned long long* __restrict__ change) {
@@ -510,8 +547,10 @@ k_dif_jacobi(GridDev g, DifVec v, DifConst K, const double* __restrict__ Tin, do
       }
       double t = T0;
       if (__any_sync(__activemask(), !fixed)) {
-        const double r = dif_row(cls, v.off + 6 * i, v.rhs + i, v.diag + i, (cls & kDifLiq) ? K.kq[1] : K.kq[0],
-                                 tn[0], tn[1], tn[2], tn[3], tn[4], tn[5]);
+        const int li = (cls & kDifLiq) ? 1 : 0;
+        const double r = dif_row<PHASE>(cls, v.off + 6 * i, v.rhs + i, v.diag + i, li ? K.kq[1] : K.kq[0],
+                                        li ? K.cdt[1] : K.cdt[0], K.rdiag[li][__popc(cls & 63u)], T0, tn[0], tn[1],
+                                        tn[2], tn[3], tn[4], tn[5]);
         if (!fixed) t = r;
       }
       Tout[i] = t;
@@ -555,11 +594,12 @@ __device__ __forceinline__ unsigned dif_vertical(const GridDev& g, int z, long l
   return (z > 0 || g.bc[2] == 0 ? 16u : 0u) | (z < nz - 1 || g.bc[2] == 0 ? 32u : 0u);
 }
 
-// First sweep of the phase form: d = s = B sum (T0_nb - T0) in FP64 (an
-// irregular cell's is k_dif_irregular's).  Cells of uniform T take no FP64.
+// First sweep in pairs: d = s = B sum (T0_nb - T0) in FP64 (an irregular cell's
+// is k_dif_irregular's).  Cells of uniform T take no FP64.
 template <bool CHECK>
 __global__ void __launch_bounds__(kDifThreads)
 k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ change) {
+  if (v.part[kDifChecks] == 0ull) return;  // not in pairs: s has no place of its own then
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
   const bool in = x < g.n[0] && y < g.n[1];
   const long long plane = (long long)g.n[0] * g.n[1];
@@ -603,7 +643,7 @@ k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ ch
   if constexpr (CHECK) dif_change(dmax, ks, change);
 }
 
-// One later sweep of the phase form, d' = sum B_nb d_nb + s, two cells of a row
+// One later sweep in pairs, d' = sum B_nb d_nb + s, two cells of a row
 // per thread: every packed instruction serves both.  A cell whose own s and
 // neighbours' d are all 0 keeps 0 without arithmetic.  (z walked in consecutive
 // planes held in registers, for a third of the reads of d, took 25 us at 128^3
@@ -707,7 +747,7 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float4* __restrict__ din, flo
 
 // e' = e + C_p,node d; a node without change keeps its e
 __global__ void __launch_bounds__(kDifThreads)
-k_dif_store_phase(GridDev g, const DifVec v, DifConst K, float4* d, double* __restrict__ e) {
+k_dif_store_pairs(GridDev g, const DifVec v, DifConst K, float4* d, double* __restrict__ e) {
   const int ks = dif_scale(v, K);
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
   if (x >= g.n[0] || y >= g.n[1]) return;
@@ -721,10 +761,18 @@ k_dif_store_phase(GridDev g, const DifVec v, DifConst K, float4* d, double* __re
   }
 }
 
-// e' = C_p(c) T' (mixture form)
-__global__ void k_dif_store(GridDev g, const double* __restrict__ c, const double* __restrict__ T,
+// From an iterate in FP64: e' = e + C_p,node (T' - T0) (phase; a node whose T came
+// back unchanged keeps its e), e' = C_p(c) T' (mixture)
+template <bool PHASE>
+__global__ void k_dif_store(GridDev g, const double* __restrict__ c, const DifVec v, const double* __restrict__ T,
                             double* __restrict__ e, size_t N) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
+    if constexpr (PHASE) {
+      const double Tn = T[i], T0 = __ldg(v.T0 + i);
+      if (dbits(Tn) == dbits(T0)) continue;
+      e[i] = e[i] + ((__ldg(v.cls + i) & kDifLiq) ? g.Cp_l : g.Cp_g) * (Tn - T0);
+      continue;
+    }
     const double cv = __ldg(c + i);
     const double Cp = g.Cp_l * cv + g.Cp_g * (1.0 - cv);
     e[i] = Cp * T[i];
@@ -746,7 +794,7 @@ DifLayout dif_layout(size_t N) {
   L.T0 = o; o += a(N * 8);
   L.Ta = o; o += a(N * 8);
   L.Tb = o; o += a(N * 8);
-  L.part = o; o += a(kDifChecks * 8);  // the checks' largest changes (bits of non-negative doubles)
+  L.part = o; o += a((kDifChecks + 1) * 8);  // the checks' largest changes (bits of non-negative doubles)
   L.cls = o; o += a(N);
   L.mlist = o; o += a(N * 4);
   L.count = o; o += 256;
@@ -784,10 +832,10 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   v.d[1] = v.d[0] + pn;
   uint32_t* mlist = reinterpret_cast<uint32_t*>(ws + L.mlist);
   int* count = reinterpret_cast<int*>(ws + L.count);
-  v.tmax = count + 2;
+  v.range = count + 2;
   *status = 0;
   const int grid = (int)std::min<size_t>((N + kDifThreads - 1) / kDifThreads, (size_t)kDifCTAs);
-  cudaError_t err = cudaMemsetAsync(count, 0, 3 * sizeof(int), st);
+  cudaError_t err = cudaMemsetAsync(count, 0, 4 * sizeof(int), st);
   if (err != cudaSuccess) return err;
   k_dif_mlist<<<grid, kDifThreads, 0, st>>>(g, c, mlist, count, N);
   k_dif_planes<<<kDifCTAs, kDifPlaneThreads, 0, st>>>(g, c, mlist, count, plane);
@@ -813,9 +861,15 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
       d += K.kq[p];
     }
   }
-  auto exponent = [](double x) { return std::isfinite(x) && x != 0.0 ? std::max(0, std::ilogb(x) + 1023) : 0; };
-  K.e0 = exponent(g.T_sat);
-  for (int f = 0; f < 6; ++f) K.e0 = std::max(K.e0, exponent(walls.T[f]));
+  K.wlo = 0x7FFFFFFF;
+  K.whi = 0;
+  for (int f = 0; f < 6; ++f) {
+    if (!walls.on[f]) continue;
+    long long b;
+    std::memcpy(&b, &walls.T[f], sizeof(b));
+    K.wlo = std::min(K.wlo, (int)(b >> 32));
+    K.whi = std::max(K.whi, (int)(b >> 32));
+  }
   // the cells next to the interface or a heated wall are listed in the
   // mixed-cell list's storage (k_dif_planes is done with it)
   uint32_t* ilist = mlist;
@@ -831,10 +885,11 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   // together.  The batches grow, cut short where the last checks' rate says
   // when tol will be met.
   unsigned long long* slot = v.part;
-  // the iterates: T0, then Ta and Tb in turn (phase form: s, the first sweep's
+  // the iterates: T0, then Ta and Tb in turn (in pairs: s, the first sweep's
   // result, then d[0] and d[1])
   double* buf[2] = {v.Ta, v.Tb};
   int it = 0, batch = 2;
+  bool pairs = phase_cp != 0;  // until the first batch's results say otherwise
   double change = 0.0, before = 0.0;
   bool done = false;
   auto iterate = [&](int n) -> double* { return n == 0 ? v.T0 : buf[n & 1]; };  // the n-th sweep's result
@@ -846,24 +901,25 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
     err = cudaMemsetAsync(slot, 0, kDifChecks * sizeof(unsigned long long), st);
     if (err != cudaSuccess) return err;
     int nc = 0;
-    const unsigned long long* prev = nullptr;
+    const unsigned long long* prev = pairs && it == 0 ? slot + kDifChecks : nullptr;
     int at[kDifChecks];
     while (it < max_iter && nc < batch) {
       const bool check = (it + 1) % 4 == 0 || it + 1 == max_iter;
       unsigned long long* chg = check ? slot + nc : nullptr;
       const double* in = iterate(it);
       double* out = iterate(it + 1);
-      if (phase_cp && it == 0) {
+      if (pairs && it == 0) {
         if (check) k_dif_first<true><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, chg);
         else k_dif_first<false><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, chg);
-      } else if (phase_cp) {
+      } else if (pairs) {
         const float4* di = iterate_d(it);
         float4* dd = iterate_d(it + 1);
         if (check) launch_pdl(k_dif_sweep<true>, pgrid, dim3(32, 8), st, g, v, K, di, dd, prev, tol, chg);
         else launch_pdl(k_dif_sweep<false>, pgrid, dim3(32, 8), st, g, v, K, di, dd, prev, tol, chg);
       } else {
-        if (check) k_dif_jacobi<true><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, in, out, prev, tol, chg);
-        else k_dif_jacobi<false><<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, in, out, prev, tol, chg);
+        auto sweep = phase_cp ? (check ? k_dif_jacobi<true, true> : k_dif_jacobi<false, true>)
+                              : (check ? k_dif_jacobi<true, false> : k_dif_jacobi<false, false>);
+        sweep<<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, in, out, prev, tol, chg);
       }
       ++it;
       if (check) {
@@ -871,10 +927,15 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
         prev = slot + nc++;
       }
     }
-    unsigned long long hb[kDifChecks];
-    err = cudaMemcpyAsync(hb, slot, nc * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st);
+    unsigned long long hb[kDifChecks + 1];
+    err = cudaMemcpyAsync(hb, slot, sizeof(hb), cudaMemcpyDeviceToHost, st);
     if (err == cudaSuccess) err = cudaStreamSynchronize(st);
     if (err != cudaSuccess) return err;
+    if (pairs && hb[kDifChecks] == 0ull) {  // nothing has run: from the start, in FP64
+      pairs = false;
+      it = 0;
+      continue;
+    }
     for (int k = 0; k < nc && !done; ++k) {
       before = change;
       std::memcpy(&change, &hb[k], sizeof(change));
@@ -890,8 +951,9 @@ cudaError_t launch_heat_diffusion(const GridDev& g, double h, const double* c, d
   }
   prof_mark("diffuse.jacobi", st);
   if (!done) *status = 2;
-  if (phase_cp) k_dif_store_phase<<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, iterate_d(it), e);
-  else k_dif_store<<<grid, kDifThreads, 0, st>>>(g, c, iterate(it), e, N);
+  if (pairs) k_dif_store_pairs<<<sgrid, dim3(32, 8), 0, st>>>(g, v, K, iterate_d(it), e);
+  else if (phase_cp) k_dif_store<true><<<grid, kDifThreads, 0, st>>>(g, c, v, iterate(it), e, N);
+  else k_dif_store<false><<<grid, kDifThreads, 0, st>>>(g, c, v, iterate(it), e, N);
   prof_mark("diffuse.store", st);
   if (iters_out) *iters_out = it;
   if (change_out) *change_out = change;
