@@ -565,11 +565,26 @@ k_dif_jacobi(GridDev g, DifVec v, DifConst K, const double* __restrict__ Tin, do
 }
 
 
+// The larger of two non-negative pairs (each its high part rounded, so that they
+// order by high part, then low part); a NaN is left out.
+__device__ __forceinline__ void dif_larger(df::f2& m, df::f2 d) {
+  if (d.hi > m.hi || (d.hi == m.hi && d.lo > m.lo)) m = d;
+}
+// |a - b| of two pairs
+__device__ __forceinline__ df::f2 dif_apart(df::f2 a, df::f2 b) {
+  df::f2 d = df::two_sum(a.hi, -b.hi);
+  d = df::fast_two_sum(d.hi, d.lo + (a.lo - b.lo));
+  return d.hi < 0.f ? df::neg(d) : d;
+}
 // largest change of the warp's lanes (over 2^k) into *change: FP64 bits
-__device__ __forceinline__ void dif_change(float m, int k, unsigned long long* change) {
+__device__ __forceinline__ void dif_change(df::f2 m, int k, unsigned long long* change) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(change, (unsigned long long)dbits(wide_of(m, k)));
+  for (int o = 16; o > 0; o >>= 1)
+    dif_larger(m, df::f2{__shfl_down_sync(0xffffffffu, m.hi, o), __shfl_down_sync(0xffffffffu, m.lo, o)});
+  if ((threadIdx.x & 31) != 0 || !(m.hi > 0.f)) return;
+  // (a change near the ends of FP64's range is put together by an addition)
+  const double x = k > -800 && k < 800 ? df::widen_pair(m, k) : wide_of(m.hi, k) + wide_of(m.lo, k);
+  atomicMax(change, (unsigned long long)dbits(x));
 }
 
 // Offsets to a cell's neighbours across the sides in the grid (wrapped across a
@@ -606,7 +621,7 @@ k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ ch
   const int ks = dif_scale(v, K);
   DifSides sd;
   dif_lateral(g, x, y, g.n[0], sd);
-  float dmax = 0.f;
+  df::f2 dmax = {0.f, 0.f};
   for (int z = blockIdx.z; z < g.n[2]; z += gridDim.z) {
     const unsigned has = sd.has | dif_vertical(g, z, plane, sd.o);
     const size_t i = in ? ((size_t)z * g.n[1] + y) * g.n[0] + x : 0;
@@ -635,10 +650,10 @@ k_dif_first(GridDev g, DifVec v, DifConst K, unsigned long long* __restrict__ ch
         at[0] = r.x;
         at[2] = r.y;
       } else if (CHECK) {
-        r.x = at[0];
+        r = make_float2(at[0], at[2]);
       }
     }
-    if (CHECK) dmax = fmaxf(dmax, fabsf(r.x));
+    if (CHECK) dif_larger(dmax, dif_apart(f2_of(r), df::f2{0.f, 0.f}));
   }
   if constexpr (CHECK) dif_change(dmax, ks, change);
 }
@@ -669,7 +684,7 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float4* __restrict__ din, flo
   const bool oddL = x > 0 || (nx & 1) == 0;                             // and L's place in its block (R's is the first)
   const bool hasS = y > 0 || g.bc[1] == 0, hasN = y < ny - 1 || g.bc[1] == 0;
   const long long oS = y > 0 ? -row : (ny - 1) * (long long)row, oN = y < ny - 1 ? row : (1 - ny) * (long long)row;
-  float dmax = 0.f;
+  f2 dmax = {0.f, 0.f};
   for (int z = blockIdx.z; z < nz; z += gridDim.z) {
     const bool hasB = z > 0 || g.bc[2] == 0, hasT = z < nz - 1 || g.bc[2] == 0;
     const long long oB = z > 0 ? -plane : (nz - 1) * plane, oT = z < nz - 1 ? plane : (1 - nz) * plane;
@@ -699,7 +714,8 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float4* __restrict__ din, flo
     const unsigned any = (fb(sh.x) | fb(ch.x) | fb(Sh.x) | fb(Nh.x) | fb(Bh.x) | fb(Th.x) | fb(Lh) | fb(Rh) |
                           (in1 ? fb(sh.y) | fb(ch.y) | fb(Sh.y) | fb(Nh.y) | fb(Bh.y) | fb(Th.y) : 0u)) & 0x7FFFFFFFu;
     float2 rh = make_float2(0.f, 0.f), rl = rh;
-    if (__any_sync(0xffffffffu, any != 0u)) {
+    const bool work = __any_sync(0xffffffffu, any != 0u);
+    if (work) {
       // left and right neighbours of both cells: (L, c0), (c1, R); a lone last
       // cell's right neighbour is R
       const f2x2 W = {vset(Lh, ch.x), vset(Ll, cl.x)};
@@ -737,9 +753,9 @@ k_dif_sweep(GridDev g, DifVec v, DifConst K, const float4* __restrict__ din, flo
       }
     }
     if (in) dout[ip] = make_float4(rh.x, rh.y, rl.x, rl.y);
-    if (CHECK) {
-      dmax = fmaxf(dmax, fabsf((rh.x - ch.x) + (rl.x - cl.x)));
-      if (in1) dmax = fmaxf(dmax, fabsf((rh.y - ch.y) + (rl.y - cl.y)));
+    if (CHECK && work) {
+      dif_larger(dmax, dif_apart(f2{rh.x, rl.x}, f2{ch.x, cl.x}));
+      if (in1) dif_larger(dmax, dif_apart(f2{rh.y, rl.y}, f2{ch.y, cl.y}));
     }
   }
   if constexpr (CHECK) dif_change(dmax, dif_scale(v, K), change);

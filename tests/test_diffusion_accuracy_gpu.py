@@ -27,9 +27,9 @@ def P():
     return P
 
 
-def sweeps(T0, Tw, fourier, real):
-    """e / C_p after SWEEPS Jacobi sweeps of gas in a box of zero-gradient walls,
-    the lower x wall at Tw (None: no heated wall), in the number type given."""
+def sweeps(T0, Tw, fourier, real, count=SWEEPS):
+    """T after `count` Jacobi sweeps of gas in a box of zero-gradient walls, the
+    lower x wall at Tw (None: no heated wall), in the number type given."""
     f = lambda v: real(v)  # noqa: E731
     T0 = T0.astype(real)
     dt = fourier * H * H * CP / K_G
@@ -51,7 +51,7 @@ def sweeps(T0, Tw, fourier, real):
     for o in off:
         diag = diag + o
     T = T0.copy()
-    for _ in range(SWEEPS):
+    for _ in range(count):
         a = rhs
         for q, (axis, s) in enumerate((ax, s) for ax in range(3) for s in (-1, 1)):
             a = a + off[q] * np.roll(T, -s, axis)
@@ -88,3 +88,21 @@ def test_no_further_off_than_fp64_sweeps(P, name, fourier):
         assert err.status == P.VOF_ESOLVE
     off = float(np.abs(e.cpu().numpy() / CP - exact).max())
     assert off <= 3 * plain + 4 * np.spacing(float(exact.max()))
+
+
+@pytest.mark.parametrize("budget,tol", [(1, 1e3), (2, 1e3), (3, 1e3), (1000, 1.0), (1000, 1e-2), (1000, 1e-4)])
+@pytest.mark.parametrize("name", ["small change", "cold gas, hot wall"])
+def test_reported_change_is_the_sweeps(P, name, budget, tol):
+    """The change of the last sweep, to the rounding of FP64 temperatures: both
+    iterates carry at most 16 ulps of the largest T each."""
+    import torch
+    shape = (3, 4, 9)
+    T0, Tw = start(name, shape)
+    g = P.Grid(shape[2], shape[1], shape[0], (1, 1, 1), H, 4e6, CP, 300.0)
+    e = torch.from_numpy(CP * T0).cuda()
+    it, change = P.vof_heat_diffusion(g, torch.zeros(shape, dtype=torch.float64, device="cuda"), e, 0.68, K_G,
+                                      0.8 * H * H * CP / K_G, tol=tol, max_iter=budget, wall_T={(0, -1): Tw})
+    last, before = (sweeps(T0, Tw, 0.8, np.longdouble, n) for n in (it, it - 1))
+    want = float(np.abs(last - before).max())
+    assert 1 <= it <= budget and change <= tol
+    assert abs(change - want) <= 32 * np.spacing(float(np.abs(last).max()))
