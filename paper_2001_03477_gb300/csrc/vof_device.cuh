@@ -148,46 +148,59 @@ __device__ __forceinline__ bool is_mixed_b(double c, const GridDev& g) {
 __device__ __forceinline__ bool is_full_b(double c, const GridDev& g) { return dbits(c) >= g.one_m_eps; }
 
 // ---------------------------------------------------------------------------
-// Division a / b for one denominator and several numerators.  The FP64 unit
-// takes 564 cycles for the library's quotient (nine FP64 instructions); here the
-// reciprocal is formed on the FP32 and integer units (an FP32 estimate of the
-// significand's reciprocal and one Newton correction carried as a second FP32
-// number, ~2^-45 relative) and a quotient costs three FP64 instructions: q0 = a r,
-// the remainder a - q0 b by a fused multiply-add, q = q0 + rem r by another
-// (Markstein 1990).  Before the last rounding q is within ~2^-90 of a / b
-// relatively, so it is the correctly rounded quotient but for about one operand
-// pair in 2^37.  Measured on 2^26 pairs: every quotient equal to the
-// library's, a division in 3 / 9 of the time.  Denominators and numerators whose
+// Division a / b for one denominator and several numerators, correctly rounded.
+// The FP64 unit takes 564 cycles for the library's quotient (nine FP64
+// instructions); here the reciprocal r of the significand is formed on the FP32 and
+// integer units -- an FP32 estimate, one Newton correction as a second FP32 number
+// (~2^-45 relative together), then the exact remainder 2^105 - B R of the integer
+// significands, which fits 64 bits, settles the last bits -- and a quotient costs
+// three FP64 instructions: q0 = a r, the remainder a - q0 b by a fused multiply-add,
+// q = q0 + rem r by another.  r is the correctly rounded reciprocal, so q is the
+// correctly rounded quotient for every pair (Markstein 1990), and 1 / b is r itself.
+// (With r good to 2^-45 alone, quotients next to the middle of two numbers, 1 / (2
+// - 2^-52) for one, came out on the wrong side.)  Denominators and numerators whose
 // exponents leave room (2^-450 .. 2^450, or 0) take this path; a warp that holds
 // another one also issues the library's division.
 // ---------------------------------------------------------------------------
 struct Rcp {
-  double b, r;  // denominator, ~1 / b
+  double b, r;  // denominator, 1 / b rounded
   bool ok;
 };
 __device__ __forceinline__ bool mid_range(unsigned hi) {  // exponent field in 573 .. 1472
   return ((hi >> 20 & 0x7FFu) - 573u) <= 899u;
 }
+// (NEAR: r to ~2^-45, without the integer remainder's ~100 cycles, and div_by's
+// quotient within 2^-90 before its rounding: for the steps of an iteration)
+template <bool NEAR = false>
 __device__ __forceinline__ Rcp rcp_of(double b) {
   const df::words w = df::words_of(b);
   const float mh = __uint_as_float(0x3F800000u | (w.hi & 0xFFFFFu) << 3 | w.lo >> 29);  // significand, top 24 bits
   const float ml = (float)(w.lo & 0x1FFFFFFFu) * 0x1p-52f;                               // the rest
   float r1;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(mh));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(mh));  // within 1 ulp
+  r1 = fmaxf(r1, 0.5f);
   const float e = fmaf(-ml, r1, fmaf(-mh, r1, 1.0f));
   const float r2 = r1 * fmaf(e, e, e);
-  // r1 in (1/2, 1]: r2 in units of the sum's FP64 last place, added to the
-  // pattern (below 1 the last place is 2^-53, also coming down from r1 = 1)
-  const unsigned rb = __float_as_uint(r1);
-  const unsigned long long r = ((unsigned long long)rb << 29) + (896ull << 52) +
-                               (long long)__float2int_rn(r2 * (rb >= 0x3F800000u && r2 >= 0.0f ? 0x1p52f : 0x1p53f));
-  Rcp R;
-  R.b = b;
-  R.ok = mid_range(w.hi);
+  // r1 + r2 in (1/2, 1] as R units of 2^-53, within ~2^8; B: b's significand
+  const unsigned long long B = (unsigned long long)((w.hi & 0xFFFFFu) | 0x100000u) << 32 | w.lo;
+  unsigned long long R = ((unsigned long long)(__float_as_uint(r1) - 0x3E800000u) << 29) +
+                         (unsigned long long)(long long)__float2int_rn(r2 * 0x1p53f);
+  if (!NEAR) {
+    long long rem = -(long long)(B * R);  // 2^105 - B R, its low 64 bits: |.| < 2^62
+    const int c = __float2int_rn((float)(int)(rem >> 32) * (r1 * 0x1p-20f));  // rem / B, within 1/2 + 2^-13
+    rem -= (long long)c * (long long)B;
+    R += (unsigned long long)(long long)c;
+    if (2 * rem > (long long)B) ++R;
+    else if (2 * rem < -(long long)B) --R;  // (never half way: 2^106 has no odd factor)
+  }
+  const unsigned long long r = R + (1021ull << 52);  // (R = 2^53 carries into the exponent: 1)
+  Rcp q;
+  q.b = b;
+  q.ok = mid_range(w.hi);
   // times 2^-(exponent of b), with b's sign
   const unsigned hi = (unsigned)(r >> 32) - ((w.hi & 0x7FF00000u) - 0x3FF00000u);
-  R.r = __hiloint2double((int)(hi | (w.hi & 0x80000000u)), (int)(unsigned)r);
-  return R;
+  q.r = __hiloint2double((int)(hi | (w.hi & 0x80000000u)), (int)(unsigned)r);
+  return q;
 }
 static __device__ __noinline__ double div_library(double a, double b) { return a / b; }
 __device__ __forceinline__ double div_by(double a, const Rcp& R) {
@@ -204,14 +217,14 @@ __device__ __forceinline__ double div_by(double a, const Rcp& R) {
 }
 // 1 / b
 __device__ __forceinline__ double inv_of(const Rcp& R) {
-  double res = fma(fma(-R.r, R.b, 1.0), R.r, R.r);
+  double res = R.r;
   if (__any_sync(__activemask(), !R.ok)) {
     const double l = div_library(1.0, R.b);
     if (!R.ok) res = l;
   }
   return res;
 }
-// a / 3 (1/3 rounded is within half a last place: two instructions after the product)
+// a / 3, likewise (1/3 is a rounded reciprocal: two instructions after the product)
 __device__ __forceinline__ double third_of(double a) {
   const double q0 = a * (1.0 / 3.0);
   return fma(fma(-q0, 3.0, a), 1.0 / 3.0, q0);
@@ -490,7 +503,7 @@ __device__ __forceinline__ double alpha_low(double m1, double m2, double m3, dou
     const long long af = dbits(dabs_i(r));
     if (af < bestf) { bestf = af; best = a; }
     if (it == 3) break;
-    double an = a - div_by(r, rcp_of(d));
+    double an = a - div_by(r, rcp_of<true>(d));
     // stay in [0, 1/2] (a > 0 keeps the cubic corner's derivative nonzero)
     if (!(dbits(an) > 0)) an = 0.5 * a;
     if (nn_lt(0.5, an)) an = 0.5;
@@ -513,7 +526,7 @@ __device__ __forceinline__ double alpha_low_est(VolForm f, double c) {
   for (int it = 0; it < 2; ++it) {
     double d = 1.0;
     const double v = vol_eval<true>(f, a, d);
-    double an = a - div_by(v - c, rcp_of(d));
+    double an = a - div_by(v - c, rcp_of<true>(d));
     if (!(dbits(an) > 0)) an = 0.5 * a;
     if (nn_lt(0.5, an)) an = 0.5;
     a = an;

@@ -505,7 +505,7 @@ k_ext_cg(ExtVec v, ExtCG* cg, double tol, int max_iter, int* status) {
     red[1][threadIdx.x] = dl;
     red[2][threadIdx.x] = r2;
     // (the reciprocals of the scalars before, while others arrive)
-    const Rcp Rg = rcp_of(gamma), Ra = rcp_of(alpha);
+    const Rcp Rg = rcp_of<true>(gamma), Ra = rcp_of<true>(alpha);
     __syncthreads();
     double* part = v.part + 3 * cur * kExtCTAs;  // the passes alternate: a slow CTA may still read the last
     if (warp < 3) {
@@ -535,11 +535,11 @@ k_ext_cg(ExtVec v, ExtCG* cg, double tol, int max_iter, int* status) {
     if (it == 0) {
       limit = tol * tol * rr;  // (|r| against tol |b| without a square root)
       beta = 0.0;
-      alpha = d1 > 0.0 ? div_by(g1, rcp_of(d1)) : 0.0;
+      alpha = d1 > 0.0 ? div_by(g1, rcp_of<true>(d1)) : 0.0;
     } else {
       beta = gamma > 0.0 ? div_by(g1, Rg) : 0.0;
       const double den = alpha > 0.0 ? d1 - beta * div_by(g1, Ra) : 0.0;
-      alpha = den > 0.0 ? div_by(g1, rcp_of(den)) : 0.0;
+      alpha = den > 0.0 ? div_by(g1, rcp_of<true>(den)) : 0.0;
     }
     gamma = g1;
     if (!(rr > limit) || it >= max_iter) break;  // the same values in every CTA
