@@ -349,10 +349,10 @@ k_dif_classify(GridDev g, const double* __restrict__ c, const double* __restrict
   if constexpr (PHASE) {
     thi = __reduce_max_sync(0xffffffffu, thi);
     tlo = __reduce_max_sync(0xffffffffu, tlo);
-    volatile int* r = v.range;
-    unsigned* ru = reinterpret_cast<unsigned*>(v.range);
-    if (lane == 0 && thi > r[0]) atomicMax(v.range, thi);  // (few warps find it larger)
-    if (lane == 0 && tlo > (unsigned)r[1]) atomicMax(ru + 1, tlo);
+    if (lane < 2) {  // (few warps find either larger)
+      const unsigned key = lane ? tlo : (unsigned)thi;
+      if (key > *(volatile unsigned*)(v.range + lane)) atomicMax(reinterpret_cast<unsigned*>(v.range) + lane, key);
+    }
   }
 }
 
