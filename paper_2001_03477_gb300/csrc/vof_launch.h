@@ -111,22 +111,20 @@ inline SumOut sums_to_diag(double* diag, const signed char (&map)[kNSums]) {
 // such a tile changes in any of the step's three sweeps (each sweep's 7-cell
 // window stays inside the uniform box, and the cells of the box outside the
 // tile that the earlier sweeps' windows reach are themselves no-ops), and none
-// is mixed when the shift runs, so the streaming kernels of an in-place step
-// skip them.  quiet == nullptr: no tile is skipped.
+// is mixed when the shift runs, so the step's kernels skip them.
 constexpr int kTile = 8;
 
 // Scratch of one sweep (kernel A -> kernels M, F, U): T of the cells whose
 // (c, e) differs from the previous cell of their line (kernel F adds the
 // listed others), the per-warp lists of cells that are not no-ops with their
-// counts, per-CTA partial sums of the clipped volume (or, when partial is
-// null, atomics into diag), per-warp staging of mixed cells and run ends,
-// the grid-wide lists of mixed cells and of face items with their counters,
+// counts, where the clipped volume goes, per-warp staging of mixed cells and
+// run ends, the grid-wide lists of mixed cells and of face items with their counters,
 // the planes of the mixed cells and the face fluxes F, G.
 struct SweepScratch {
   double* T;
   uint32_t* list;
   int* count;
-  SumOut sums;       // per-CTA sums of kernel U: Delta c, Delta e, clipped volume
+  SumOut sums;       // kernel U: the clipped volume
   uint32_t* mlist;   // per-warp staging lists of mixed cells
   uint32_t* rlist;   // per-warp staging lists of run ends
   int* counters;     // [0] mixed cells, [1] face items at the front, [2] at the
@@ -178,7 +176,7 @@ struct ShiftScratch {
   double* cnew;   // [N] shifted volume of a moving mixed cell
   uint32_t* own;  // [N]
   // reach and claim are written (and cleared) by the stream kernel for
-  // every cell it visits; the cells of quiet tiles it skips are never read
+  // every cell
   uint8_t* reach; // [N] 1: moving mixed cell with shift < 0, 2: > 0, else 0
   uint32_t* claim;  // [N] receivers: bit 31 - b set by the reaching neighbour at offset index b
   double* mark;   // nullable: the tagged c words (c_in), where receivers are marked instead of
@@ -279,12 +277,8 @@ struct ReduceJob {
   int nblocks, stride, k0, nk;
   double* out;
 };
-constexpr int kMaxReduceJobs = 4;
-constexpr int kMaxReduceK = 8;      // outputs per job at most
-constexpr int kReduceCTAs = 152;    // first-level CTAs per job
-struct ReduceJobs {
-  ReduceJob job[kMaxReduceJobs];
-};
+constexpr int kMaxReduceK = 8;      // outputs at most
+constexpr int kReduceCTAs = 152;    // first-level CTAs
 size_t reduce_scratch_bytes();
 // one job's two levels in one launch; *ticket is zero before and after
 cudaError_t launch_reduce_fused(const ReduceJob& job, double* scratch, int* ticket, cudaStream_t st);

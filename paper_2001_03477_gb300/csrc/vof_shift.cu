@@ -975,12 +975,11 @@ __device__ __forceinline__ void reduce2_body(const ReduceJob& J, const double* p
 // finishes last (a ticket, zero at the start and left zero) the second
 // level -- the same arithmetic and order as the grouped pair k_reduce1_grp
 // and k_reduce2_grp below, so a box sums to the same bits either way.
-__global__ void __launch_bounds__(kReduceThreads) k_reduce_fused(ReduceJobs jobs, double* __restrict__ scratch,
+__global__ void __launch_bounds__(kReduceThreads) k_reduce_fused(ReduceJob J, double* __restrict__ scratch,
                                                                  int* __restrict__ ticket) {
   __shared__ double red[kMaxReduceK][kReduceThreads];
   __shared__ int last;
   pdl_wait();
-  const ReduceJob J = jobs.job[0];
   reduce1_body(J, blockIdx.x, gridDim.x, scratch + (size_t)blockIdx.x * kMaxReduceK, red);
   __threadfence();  // this CTA's partials before its ticket
   __syncthreads();
@@ -994,7 +993,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_fused(ReduceJobs jobs
 }
 
 // grouped: the first level over (box, part) CTAs, the second one CTA per box,
-// in the same order as a box's own reduction (job 0, kReduceCTAs parts)
+// in the same order as a box's own reduction (kReduceCTAs parts)
 __global__ void __launch_bounds__(kReduceThreads) k_reduce1_grp(GroupMap m, const ReduceBox* __restrict__ rb) {
   __shared__ double red[kMaxReduceK][kReduceThreads];
   unsigned b;
@@ -1019,13 +1018,11 @@ cudaError_t launch_reduce_grp(const GroupMap& m1, const ReduceBox* rb, unsigned 
   return cudaGetLastError();
 }
 
-size_t reduce_scratch_bytes() { return (size_t)kMaxReduceJobs * kReduceCTAs * kMaxReduceK * sizeof(double); }
+size_t reduce_scratch_bytes() { return (size_t)kReduceCTAs * kMaxReduceK * sizeof(double); }
 
 cudaError_t launch_reduce_fused(const ReduceJob& job, double* scratch, int* ticket, cudaStream_t st) {
   if (job.nk > kMaxReduceK) return cudaErrorInvalidValue;
-  ReduceJobs jobs{};
-  jobs.job[0] = job;
-  launch_pdl(k_reduce_fused, kReduceCTAs, kReduceThreads, st, jobs, scratch, ticket);
+  launch_pdl(k_reduce_fused, kReduceCTAs, kReduceThreads, st, job, scratch, ticket);
   prof_mark("reduce", st);
   return cudaGetLastError();
 }

@@ -16,8 +16,7 @@
 // J = 1 + (a_r - a_l) its stretch.
 //
 // Four kernels per sweep:
-//   A (stream): walks the grid lines (skipping quiet tiles in an in-place
-//     step), copies the cells that provably do not change (no-op cells,
+//   A (stream): walks the grid lines, copies the cells that provably do not change (no-op cells,
 //     below) to the output when out of place, and lists the other cells per
 //     warp in a fixed order, plus grid-wide lists of the mixed cells and of
 //     the faces to evaluate (left face of every listed cell, right face of
@@ -545,8 +544,8 @@ k_faces(GridDev g, const double* __restrict__ c_in, const double* __restrict__ e
 // it may update in place (c_out == c_in, e_out == e_in); kernel A then
 // copies nothing.
 // ---------------------------------------------------------------------------
-// The groups of lists this CTA takes, cell by cell; v accumulates the
-// CTA's contributions to the sums in a fixed order.
+// The groups of lists this CTA takes, cell by cell; v accumulates the clipped
+// volume in a fixed order.
 template <int AX, bool ENERGY, bool LAG>
 __device__ __forceinline__ void update_groups(const GridDev& g, const double* c_in, const double* e_in, double* c_out,
                                               double* e_out, const double* __restrict__ uf,
@@ -605,15 +604,11 @@ __device__ __forceinline__ void update_groups(const GridDev& g, const double* c_
       const bool cc = dirty ? ((stv >> 1) & 1) != 0 : dgthalf(c);
       const double2 r = update_c(c, Fl, al, Fr, ar, cc, LAG);
       c_out[id] = r.x;
-      if (!same_bits(r.x, c) || dnz(r.y)) {
-        v[kSumClip] += r.y;
-        v[kSumC] += r.x - c;
-      }
+      if (dnz(r.y)) v[kSumClip] += r.y;
       if (ENERGY) {
         const double th = dirty ? theta[id] : theta_now(g, T, c, cc, LAG);
         const double en = (e + (Gl - th * al)) - (Gr - th * ar);
         e_out[id] = en;
-        v[kSumE] += en - e;
         if (!LAG && state && !dirty && (!deq(r.x, c) || !deq(en, e))) {
           state[id] = (uint8_t)(1 | (cc ? 2 : 0));
           theta[id] = th;
