@@ -220,12 +220,15 @@ VOF_API vof_status vof_phase_change_shift(const vof_grid* g, const double* c_in,
  * One full time step of the method (Sec. 3.1 steps 1-2: Step 1 the split
  * VOF sweeps of Sec. 3.3.1 with the thermal energy fluxed in tandem, Sec.
  * 3.4.1, Eq. disc_et_adv; Step 2 the interface shift of Sec. 3.3.2) on the
- * caller's stream: zero the frozen state, three
+ * caller's stream: three
  * (g->scheme: Weymouth-Yue or Lagrangian-explicit)
  * sweeps in Strang-alternated order (x,y,z on even step_index, z,y,x on odd),
- * then the shift; c and e are updated in place (every sweep and the shift
- * read and write them directly; the workspace holds the frozen state, the
- * per-sweep lists, planes and face fluxes, and the partial sums).
+ * then the shift; c and e are updated in place.  While the step's kernels
+ * run, c and e hold intermediate states, and words of c also carry two flag
+ * bits above the value (such a word is no volume fraction): other work reads
+ * them only after the step's has completed, and after VOF_ECUDA their
+ * contents are undefined.  (The workspace holds a second pair of fields, the
+ * frozen Theta, lists, planes and donor volumes, and the partial sums.)
  *   u, v, w        face velocities
  *   dd, dd_uniform as for vof_phase_change_shift
  *   sums           device double[VOF_NSUMS] (nullable), OVERWRITTEN with
@@ -315,9 +318,11 @@ VOF_API vof_status vof_batched_step(const vof_box* boxes, int nbox, long step_in
  *                 grouped: VOF_EINVAL)
  *   sums          device double[nbox][VOF_NSUMS] or NULL: each box's step
  *                 sums, written by every vof_group_step()
- *   work_per_cta  cells per CTA of the grid-stride kernels (mixed cells,
- *                 shift lists; >= 32): the grouped launches' granularity
- *                 (results do not depend on it; the autotuner picks it)
+ *   work_per_cta  cells per CTA of the grid-stride kernels (>= 32): the
+ *                 grouped launches' granularity (results do not depend on
+ *                 it; the autotuner picks it).  The kernels over the mixed
+ *                 cells take at most 1024 cells per CTA whatever it says; the
+ *                 tile, walk and write-back kernels size themselves
  *   workspace     device, 256-byte aligned, vof_group_workspace_bytes()
  *                 bytes; it holds the boxes' workspaces and the tables while
  *                 the group lives.  Fields must not overlap it or each other.

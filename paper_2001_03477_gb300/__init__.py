@@ -787,7 +787,8 @@ class Group:
     """A batch of boxes stepped with one launch per kernel of the time step
     (vof_group_*): the boxes' workspaces and the launch tables live in one
     device buffer (allocated through torch); `step()` runs vof_group_step.
-    `work_per_cta`: cells per CTA of the grid-stride kernels."""
+    `work_per_cta`: cells per CTA of the grid-stride kernels (at most 1024 in
+    those over the mixed cells)."""
 
     def __init__(self, boxes, work_per_cta=4096, device="cuda", stream=None):
         import torch
