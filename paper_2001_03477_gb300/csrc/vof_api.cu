@@ -212,7 +212,9 @@ vof_status vof_phase_change_shift(const vof_grid* g, const double* c_in, const d
 // active tiles | clipped volumes.  The step's last kernel sums every
 // active tile's cells, the tile pass the quiet ones', so one fixed-order
 // reduction of the rows gives the sums.  The size is at least that of the
-// stand-alone sweeps' and shift's scratch and a byte per cell behind the first five regions.
+// stand-alone sweeps' and shift's scratch behind the first five regions and a
+// byte per cell: a program's one buffer of vof_step_workspace_bytes() has always
+// served those calls too.
 struct StepLayout {
   size_t off_th, off_rows, off_red, off_stats, off_tiles, off_sc, off_se, off_fl, off_fr, off_gf, off_plane,
       off_l0, off_l1, off_tlist, off_clip, total;
