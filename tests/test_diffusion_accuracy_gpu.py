@@ -1,6 +1,7 @@
 """Accuracy of the heat diffusion where the change of T is as large as T itself
-(a hot wall on cold gas, a jump from 300 to 600), against the same sweeps in
-long double.
+(a hot wall on cold gas, a jump from 300 to 600), small beside it, and on both
+sides of the rule that chooses the sweeps' form, against the same sweeps in long
+double.
 
 Bound: the result may be no further off than plain FP64 sweeps of T.  Those are
 made here in numpy; the library's differ in the order of roundings (fused
@@ -67,11 +68,18 @@ def start(name, shape):
         return np.where(np.arange(shape[2]) < shape[2] // 2, 600.0, 300.0) * np.ones(shape), None
     if name == "hot wall":
         return np.full(shape, 300.0), 600.0
+    if name == "within the rule":  # for pairs: 16 times the range is at most the smallest T
+        return np.full(shape, 320.0), 339.9
+    if name == "beyond the rule":
+        return np.full(shape, 320.0), 340.1
+    if name == "below zero":
+        return -300.0 - 10.0 * rng.random(shape), -310.0
     return 300.0 + 10.0 * rng.random(shape), 310.0  # a change small beside T
 
 
 @pytest.mark.parametrize("fourier", [0.8, 5.0, 20.0])
-@pytest.mark.parametrize("name", ["cold gas, hot wall", "a jump of the size of T", "hot wall", "small change"])
+@pytest.mark.parametrize("name", ["cold gas, hot wall", "a jump of the size of T", "hot wall", "small change",
+                                  "within the rule", "beyond the rule", "below zero"])
 def test_no_further_off_than_fp64_sweeps(P, name, fourier):
     import torch
     shape = (4, 5, 22)
@@ -87,7 +95,7 @@ def test_no_further_off_than_fp64_sweeps(P, name, fourier):
     except P.VofError as err:  # the budget, unless no T changes any more
         assert err.status == P.VOF_ESOLVE
     off = float(np.abs(e.cpu().numpy() / CP - exact).max())
-    assert off <= 3 * plain + 4 * np.spacing(float(exact.max()))
+    assert off <= 3 * plain + 4 * np.spacing(float(np.abs(exact).max()))
 
 
 @pytest.mark.parametrize("budget,tol", [(1, 1e3), (2, 1e3), (3, 1e3), (1000, 1.0), (1000, 1e-2), (1000, 1e-4)])
