@@ -48,7 +48,7 @@
 // of T_Gamma where a cell sees an interface and of the walls' T, so |d| is at most
 // their range R, and the rule is 16 R <= the smallest of them (all positive): the
 // energies' errors against long double are then 0.2 to 0.4 of the FP64 sweeps'
-// (16^3 box, diffusion numbers 0.05 to 20; R = T / 8: up to 0.65 in the mean and as
+// (14^3 box, diffusion numbers 0.05 to 20; R = T / 8: up to 0.65 in the mean and as
 // large at most; R = T: 1.4 to 24 times).  Other calls sweep T itself in FP64 (128^3,
 // a hot wall on gas at 0: 42.7 us a sweep all in all, 20.4 in pairs).  The
 // kernels decide on the device: the first batch's sweeps in pairs return at once
